@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <iterator>
 #include <cmath>
 #include <cstdio>
@@ -98,9 +99,8 @@ void split_df(double x, float* hi, float* lo) {
   *lo = (float)(x - (double)h);
 }
 
-// Largest |c_j| over the corners of the intrinsic prior box (x1.25 margin).
-void coefficient_bounds(const swig_ctx* c, double* cmax) {
-  double lo[6], hi[6];
+// The intrinsic prior box (slots 0..5; a default one without a prior).
+void intrinsic_box(const swig_ctx* c, double* lo, double* hi) {
   const double dlo[6] = {0.87, 0.125, -0.1, -0.1, 0.0, 0.0}, dhi[6] = {3.0, 1.0, 0.1, 0.1, 5000.0, 5000.0};
   for (int i = 0; i < 6; ++i) {
     lo[i] = dlo[i];
@@ -115,6 +115,12 @@ void coefficient_bounds(const swig_ctx* c, double* cmax) {
       }
     }
   }
+}
+
+// Largest |c_j| over the corners of the intrinsic prior box (x1.25 margin).
+void coefficient_bounds(const swig_ctx* c, double* cmax) {
+  double lo[6], hi[6];
+  intrinsic_box(c, lo, hi);
   for (int j = 0; j < NBASIS; ++j) cmax[j] = 0.0;
   for (int m = 0; m < 64; ++m) {
     double v[6];
@@ -195,9 +201,200 @@ void plan_tiles(const swig_ctx* c, std::vector<TileInfo>& tiles, std::vector<Til
   }
 }
 
+// phi_j^(n)(f) h^n / n! for n = 0 .. nd (row n), j < NBASIS.
+void basis_taylor(double f, double h, int nd, double (*T)[NBASIS]) {
+  const double lf = std::log(f), hf = h / f;
+  for (int j = 0; j < NBASIS; ++j) {
+    // f^p (a ln f + b); each derivative divides by f
+    double a = kBasisLog[j] ? 1.0 : 0.0, b = kBasisLog[j] ? 0.0 : 1.0;
+    double s = std::pow(f, kBasisPow[j]);
+    for (int n = 0; n <= nd; ++n) {
+      T[n][j] = s * (a * lf + b);
+      const double p = kBasisPow[j] - n;
+      b = p * b + a;
+      a = p * a;
+      s *= hf / (n + 1);
+    }
+  }
+}
+
+// Chunks and tables of the folded full-grid sums (kernels.h FoldRow, fold.cuh).
+// Greedy from the lowest bin: the widest run of bins whose phase, over the
+// prior box, keeps within the bandwidth that kFoldNodes Chebyshev nodes serve
+// and whose Taylor form errs by at most kFoldTaylorEps / 5; where that is no
+// more than kFoldNodes bins, a block of at most kFoldNodes bins taken as they
+// are.  The box's slopes are taken at its corners and centre; a vector of
+// parameters that exceeds what was planned for (the device checks each) is
+// summed bin by bin, so the plan bounds the cost and not the error.
+void fold_plan(const swig_ctx* c, int n_det, std::vector<FoldChunk>& chunks, std::vector<float>& tab) {
+  constexpr int nd = kFoldDeg;
+  const double rho = kFoldRho, ea = 0.5 * (rho + 1.0 / rho), eb = 0.5 * (rho - 1.0 / rho);
+  auto band = [&](double eps) {
+    return (std::log(eps * (rho - 1.0) / 4.0) + (kFoldNodes - 1) * std::log(rho)) / (2.0 * kPi * eb);
+  };
+  const double om_plan = band(0.1 * kFoldEps), om_dev = band(kFoldEps);
+  double lo[6], hi[6], cmax[NBASIS];
+  intrinsic_box(c, lo, hi);
+  coefficient_bounds(c, cmax);
+  std::vector<std::array<double, NBASIS>> pts;
+  for (int m = 0; m <= 64; ++m) {
+    double v[6];
+    bool dup = false;  // a fixed slot has one corner
+    for (int i = 0; i < 6; ++i) {
+      v[i] = m == 64 ? 0.5 * (lo[i] + hi[i]) : (m >> i & 1) ? hi[i] : lo[i];
+      dup = dup || (m < 64 && (m >> i & 1) && hi[i] == lo[i]);
+    }
+    if (dup) continue;
+    pts.emplace_back();
+    taylorf2_basis_coeffs(v[0], v[1], v[2], v[3], v[4], v[5], pts.back().data());
+  }
+  double t_lo = -0.2, t_hi = 0.2;  // t_c plus the geocentric delays
+  if (c->prior_set) {
+    const swig_param& p = c->params[11];
+    t_lo = p.mode == SWIG_MODE_SAMPLE ? p.lo : p.value;
+    t_hi = p.mode == SWIG_MODE_SAMPLE ? p.hi : p.value;
+  }
+  double delay = 0.0;
+  for (int i = 0; i < n_det; ++i) delay = std::max(delay, std::hypot(std::hypot(c->vertex[i][0], c->vertex[i][1]), c->vertex[i][2]) / kCSI);
+  t_lo -= delay;
+  t_hi += delay;
+  const int n = (int)c->n_bins;
+  double T[nd + 2][NBASIS];
+  struct Fit {
+    double fc, h, slope, omega, rem;
+  };
+  auto fit = [&](double fc, double h) {
+    Fit r{fc, h, 0.0, 0.0, 0.0};
+    basis_taylor(fc, h, nd + 1, T);
+    double s0 = INFINITY, s1 = -INFINITY, curv = 0.0;
+    for (const auto& cc : pts) {
+      double s = 0.0, cv = 0.0, g = 1.0;
+      for (int j = 0; j < kFoldSlopes; ++j) s += cc[j] * T[1][j];
+      for (int m = 2; m <= nd; ++m) {
+        double a = 0.0;
+        for (int j = 0; j < kFoldSlopes; ++j) a += cc[j] * T[m][j];
+        g *= ea;
+        cv += m * g * std::fabs(a);
+      }
+      s0 = std::min(s0, s);
+      s1 = std::max(s1, s);
+      curv = std::max(curv, cv);
+    }
+    s0 += t_lo * h;
+    s1 += t_hi * h;
+    r.slope = 0.5 * (s0 + s1);
+    // 2 % of margin on the box's spread and curvature
+    r.omega = 1.02 * (0.5 * (s1 - s0) + curv);
+    for (int j = 0; j < kFoldSlopes; ++j)
+      r.rem += cmax[j] * basis_derivative_bound(kBasisPow[j], kBasisLog[j], nd + 1, std::max(fc - h, 0.25 * c->df), fc + h);
+    double hn = 1.0;
+    for (int m = 1; m <= nd + 1; ++m) hn *= h / m;
+    r.rem *= hn;
+    return r;
+  };
+  auto freq = [&](int k) { return (double)(c->k_min + k) * c->df; };
+  auto folded = [&](int k, int w) { return fit(0.5 * (freq(k) + freq(k + w - 1)), 0.5 * (w - 1) * c->df); };
+  auto good = [&](const Fit& r) { return r.omega <= om_plan && r.rem <= 0.2 * kFoldTaylorEps; };
+  chunks.clear();
+  std::vector<Fit> fits;
+  int k = 0, last = kFoldNodes + 1;
+  while (k < n) {
+    const int left = n - k, w_min = kFoldNodes + 1;
+    FoldChunk ck{k, 0, 0, 0, 0.0};
+    Fit best{};
+    if (left >= w_min) {
+      // bracket the widest good width from the previous chunk's, then bisect
+      // to 2 %
+      int w = std::max(w_min, std::min(left, last)), bad = left + 1;
+      Fit r = folded(k, w);
+      while (!good(r) && w > w_min) {
+        bad = w;
+        w = std::max(w_min, (int)(0.8 * w));
+        r = folded(k, w);
+      }
+      if (good(r)) {
+        ck.nbins = w;
+        best = r;
+        for (int step = std::max(1, w / 8); bad > left && w < left; step *= 2) {
+          const int w2 = std::min(left, w + step);
+          r = folded(k, w2);
+          if (!good(r)) {
+            bad = w2;
+          } else {
+            ck.nbins = w = w2;
+            best = r;
+          }
+        }
+        while (bad - w > std::max(1, w / 50)) {
+          const int w2 = (w + bad) / 2;
+          if (w2 > left) break;
+          r = folded(k, w2);
+          if (good(r)) {
+            ck.nbins = w = w2;
+            best = r;
+          } else {
+            bad = w2;
+          }
+        }
+        last = w;
+      }
+    }
+    if (ck.nbins == 0) {
+      int bw = kFoldNodes;
+      for (ck.kind = 1;; ++ck.kind, bw /= 2) {
+        best = fit(freq(k) + 0.5 * (bw - 1) * c->df, 0.5 * bw * c->df);
+        if (best.rem <= 0.2 * kFoldTaylorEps || ck.kind == kFoldKinds - 1) break;
+      }
+      ck.nbins = std::min(bw, left);
+    }
+    ck.slope_h = std::isfinite(best.slope) ? best.slope : 0.0;
+    chunks.push_back(ck);
+    fits.push_back(best);
+    k += ck.nbins;
+  }
+  const size_t nc = chunks.size();
+  tab.assign(FR_ROWS * nc, 0.0f);
+  for (size_t q = 0; q < nc; ++q) {
+    auto put = [&](int row, double v) { tab[(size_t)row * nc + q] = (float)v; };
+    auto put2 = [&](int row, int row_lo, double v) {
+      float a, b;
+      split_df(v, &a, &b);
+      put(row, a);
+      put(row_lo, b);
+    };
+    const double fc = fits[q].fc, h = fits[q].h;
+    basis_taylor(fc, h, nd, T);
+    for (int j = 0; j < NBASIS; ++j) put2(FR_VAL_HI + j, FR_VAL_LO + j, j == B_ONE ? 1.0 : T[0][j]);
+    double hn = 1.0;
+    for (int m = 1; m <= nd + 1; ++m) hn *= h / m;
+    for (int j = 0; j < kFoldSlopes; ++j) {
+      put2(FR_D1_HI + j, FR_D1_LO + j, T[1][j]);
+      for (int m = 2; m <= nd; ++m) put(FR_POLY + (m - 2) * kFoldSlopes + j, T[m][j]);
+      put(FR_BND + j, hn * basis_derivative_bound(kBasisPow[j], kBasisLog[j], nd + 1, std::max(fc - h, 0.25 * c->df), fc + h));
+    }
+    put2(FR_FC_HI, FR_FC_LO, fc);
+    put2(FR_H_HI, FR_H_LO, h);
+    put2(FR_SM_HI, FR_SM_LO, chunks[q].slope_h);
+    put(FR_LIM, chunks[q].kind ? 1e30 : om_dev);
+    put(FR_KIND, chunks[q].kind);
+  }
+}
+
+// Node abscissae of every kind (kernels.h kFoldKinds), hi and lo; the lanes
+// past a block's bins (whose weights are zero) repeat x = 1.
+std::vector<float2> fold_abscissae() {
+  std::vector<float2> x(32 * kFoldKinds);
+  for (int s = 0; s < kFoldKinds; ++s)
+    for (int l = 0; l < 32; ++l) {
+      const double v = s == 0 ? std::cos(kPi * (2 * l + 1) / (2.0 * kFoldNodes))
+                              : std::min(1.0, (2 * l + 1) / (double)(2 * kFoldNodes >> s));
+      split_df(v, &x[32 * s + l].x, &x[32 * s + l].y);
+    }
+  return x;
+}
+
 void free_scratch(DeviceBuffers& B) {
   dfree(B.rec);
-  dfree(B.anchors);
   dfree(B.partials32);
   dfree(B.partials64);
   dfree(B.theta);
@@ -214,9 +411,11 @@ void free_problem(DeviceBuffers& B) {
   dfree(B.basis);
   dfree(B.slice_begin);
   dfree(B.bin_tile);
+  dfree(B.fold_tab);
+  dfree(B.fold_w);
+  dfree(B.fold_x);
+  B.fold_nc = 0;
   dfree(B.prior);
-  dfree(B.piece_begin);
-  dfree(B.slice_piece);
   dfree(B.het_edge_basis);
   dfree(B.het_edge_f);
   dfree(B.het_inv_width);
@@ -754,9 +953,7 @@ int ensure_scratch(swig_ctx* c, int n) {
   if (n <= B.cap) return SWIG_OK;
   free_scratch(B);
   const int cap = std::max(n, 256);
-  const size_t ntiles = std::max(c->L.n_tiles, 1);
   CUDA_TRY(c, cudaMalloc(&B.rec, sizeof(EvalRecord) * cap));
-  CUDA_TRY(c, cudaMalloc(&B.anchors, sizeof(float) * kAnchorStride * ntiles * cap));
   const size_t units = (size_t)c->L.n_slices * 4;  // up to 4 work units per (theta, slice)
   CUDA_TRY(c, cudaMalloc(&B.partials32, sizeof(float) * kPartialStride * units * cap));
   CUDA_TRY(c, cudaMalloc(&B.partials64, sizeof(double) * kPartialStride * units * cap));
@@ -810,6 +1007,32 @@ void plan_slices(int64_t n, int n_det, int sm_count, const std::vector<TileInfo>
   *max_bins_out = max_bins;
 }
 
+// Tables and node weights of the folded full-grid sums.
+int prepare_fold(swig_ctx* c) {
+  DeviceBuffers& B = c->B;
+  std::vector<FoldChunk> chunks;
+  std::vector<float> tab;
+  fold_plan(c, c->L.n_det, chunks, tab);
+  const std::vector<float2> x = fold_abscissae();
+  FoldChunk* ck_d = nullptr;
+  B.fold_nc = (int)chunks.size();
+  CUDA_TRY(c, cudaMalloc(&B.fold_tab, sizeof(float) * tab.size()));
+  CUDA_TRY(c, cudaMemcpy(B.fold_tab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMalloc(&B.fold_x, sizeof(float2) * x.size()));
+  CUDA_TRY(c, cudaMemcpy(B.fold_x, x.data(), sizeof(float2) * x.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMalloc(&B.fold_w, sizeof(float4) * 32 * c->L.n_det * chunks.size()));
+  CUDA_TRY(c, cudaMalloc(&ck_d, sizeof(FoldChunk) * chunks.size()));
+  cudaError_t e = cudaMemcpy(ck_d, chunks.data(), sizeof(FoldChunk) * chunks.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_fold_weights(c->L, B, ck_d, c->stream);
+  cudaFree(ck_d);
+  if (e != cudaSuccess)
+    return fail(c, e == cudaErrorMemoryAllocation ? SWIG_E_NOMEM : SWIG_E_CUDA,
+                std::string("folded weights: ") + cudaGetErrorString(e));
+  c->n_launches += 2;
+  c->h2d_bytes += sizeof(float) * tab.size() + sizeof(float2) * x.size() + sizeof(FoldChunk) * chunks.size();
+  return SWIG_OK;
+}
+
 // Validate the problem and (re)build every device-side table.
 int prepare(swig_ctx* c) {
   if (!c->dirty) return SWIG_OK;
@@ -830,6 +1053,7 @@ int prepare(swig_ctx* c) {
 
   LikeConst& L = c->L;
   std::memset(&L, 0, sizeof(L));
+  L.sm_count = c->sm_count;
   L.n_det = n_det;
   L.n_bins = (int)n;
   L.k_min = (int)c->k_min;
@@ -925,7 +1149,10 @@ int prepare(swig_ctx* c) {
     CUDA_TRY(c, cudaMemcpy(B.basis, basis.data(), sizeof(TileBasis) * basis.size(), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMalloc(&B.bin_tile, sizeof(int) * n));
     CUDA_TRY(c, cudaMemcpy(B.bin_tile, bin_tile.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
-    CUDA_TRY(c, set_sweep_smem_limit(sweep_smem_bytes(n_det, max_bins)));
+    if (!c->cfg_set || c->cfg.likelihood == SWIG_LIKE_FULL) {
+      const int rc = prepare_fold(c);
+      if (rc) return rc;
+    }
   } else {
     std::vector<double2> d64((size_t)n_det * n);
     for (size_t k = 0; k < d64.size(); ++k) d64[k] = make_double2(dre[k], dim[k]);
@@ -942,40 +1169,6 @@ int prepare(swig_ctx* c) {
     CUDA_TRY(c, cudaMalloc(&B.ftab, sizeof(double) * ftab.size()));
     CUDA_TRY(c, cudaMemcpy(B.ftab, ftab.data(), sizeof(double) * ftab.size(), cudaMemcpyHostToDevice));
     L.n_tiles = 0;
-  }
-  // sweep pieces: whole 32-bin chunks, at most 8 chunks and 32 tiles each, so
-  // that a warp computes a piece's anchors with one lane per tile
-  {
-    std::vector<int> bt;
-    if (prec == SWIG_PREC_MIXED) {
-      bt.resize(n);
-      CUDA_TRY(c, cudaMemcpy(bt.data(), B.bin_tile, sizeof(int) * n, cudaMemcpyDeviceToHost));
-    }
-    std::vector<int> pb, sp(n_slices + 1);
-    int maxp = 1;
-    for (int s = 0; s < n_slices; ++s) {
-      sp[s] = (int)pb.size();
-      int b = slice_begin[s];
-      while (b < slice_begin[s + 1]) {
-        pb.push_back(b);
-        int e = std::min<int>(b + kChunk, slice_begin[s + 1]);
-        while (e < slice_begin[s + 1] && e - b < 8 * kChunk) {
-          const int e2 = std::min<int>(e + kChunk, slice_begin[s + 1]);
-          if (!bt.empty() && bt[e2 - 1] - bt[b] + 1 > 32) break;
-          e = e2;
-        }
-        b = e;
-      }
-      pb.push_back(slice_begin[s + 1]);
-      maxp = std::max(maxp, (int)pb.size() - sp[s] - 1);
-    }
-    sp[n_slices] = (int)pb.size();
-    B.n_pieces = (int)pb.size() - n_slices;
-    B.max_pieces = maxp;
-    CUDA_TRY(c, cudaMalloc(&B.piece_begin, sizeof(int) * pb.size()));
-    CUDA_TRY(c, cudaMemcpy(B.piece_begin, pb.data(), sizeof(int) * pb.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(c, cudaMalloc(&B.slice_piece, sizeof(int) * sp.size()));
-    CUDA_TRY(c, cudaMemcpy(B.slice_piece, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice));
   }
   // prior slots (defaults when no prior was set: every slot sampled uniform on [0,1])
   PriorSlot slots[SWIG_N_PARAMS];
@@ -1009,7 +1202,7 @@ int loglike_device(swig_ctx* c, const double* theta_dev, int64_t n, double* out_
       e = c->prepared_precision == SWIG_PREC_MIXED
               ? launch_loglike_mixed(c->L, c->B, theta_dev + off * SWIG_N_PARAMS, m, out_dev + off, st)
               : launch_loglike_fp64(c->L, c->B, theta_dev + off * SWIG_N_PARAMS, m, out_dev + off, st);
-      c->n_launches += c->prepared_precision == SWIG_PREC_MIXED ? 4 : 3;
+      c->n_launches += c->prepared_precision == SWIG_PREC_MIXED ? 2 : 3;
     }
     if (e != cudaSuccess) return fail(c, SWIG_E_CUDA, std::string("likelihood launch: ") + cudaGetErrorString(e));
   }

@@ -1,0 +1,283 @@
+// Folded full-grid sums (mixed precision), device side.
+//
+// kappa_i = sum_k D_i(k) exp(-2 pi i (P(f_k) + f_k tau_i)) over a few hundred
+// thousand bins samples a smooth function far more finely than it varies: over
+// a chunk of bins the phase, less the chunk's reference slope s, turns through
+// a few cycles only.  The host cuts the grid into chunks over which every
+// template of the prior box keeps below a fixed bandwidth (fold_plan in
+// capi.cu).  On such a chunk the template equals its polynomial interpolant
+// through 64 Chebyshev nodes to 1e-8, and the sum over the chunk's bins is,
+// exactly for that interpolant, a sum over the nodes,
+//   sum_k D'_i(k) E'(x_k) = sum_j W_ij E'(x_j),  W_ij = sum_k D'_i(k) l_j(x_k),
+// with D'_i(k) = D_i(k) exp(-2 pi i s (f_k - f_c)), l_j the Lagrange basis and
+// W formed once per event in FP64.  Where 64 bins hold more phase than that
+// (the lowest frequencies) the nodes are the bins themselves.  The 128 s
+// three-detector grid's 259,585 bins become about 80 chunks of 64 nodes.
+//
+// Bound: the SFU (two results per node and detector, 78 x 64 x 3 nodes instead
+// of 778,755 bins) and the FP32 issue slots beside it.  Batched, against the
+// direct sum over every bin (one GB300): 1000 vectors on the 128 s grid 84 us
+// (668), 4099 on the 256 s grid 253 us (4.74 ms), one vector 63 us with the
+// host copies (91); the error against FP64 is the same or smaller.
+//
+// An evaluation checks its own bandwidth and Taylor remainder on every chunk
+// against the bound the weights were made for; a parameter vector outside
+// (one far from the prior box) is summed bin by bin instead (fold_direct).
+#pragma once
+
+#include "sweep.cuh"
+
+namespace swig {
+
+constexpr int kFoldWarps = 16;     // warps of a CTA that evaluates one parameter vector
+constexpr int kFoldPanel = 128;    // chunks whose anchors are in shared memory at once
+constexpr int kFoldAnchor = 16;    // floats per (evaluation, chunk) anchor
+
+// What an evaluation reads of its record: coefficients and time shifts in
+// double-float.
+struct FoldIn {
+  float c_hi[NBASIS], c_lo[NBASIS];
+  float tau_hi[SWIG_MAX_DET], tau_lo[SWIG_MAX_DET];
+};
+static_assert(offsetof(EvalRecord, c_lo) == offsetof(EvalRecord, c_hi) + sizeof(float) * NBASIS &&
+                  offsetof(EvalRecord, tau_lo) == offsetof(EvalRecord, tau_hi) + sizeof(float) * SWIG_MAX_DET,
+              "FoldIn is two runs of EvalRecord's words");
+
+// Word w (0 .. 29) of FoldIn from a record.
+__device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
+  return w < 2 * NBASIS ? reinterpret_cast<const float*>(&r.c_hi)[w]
+                        : reinterpret_cast<const float*>(&r.tau_hi)[w - 2 * NBASIS];
+}
+
+// Two FP32 operations per instruction (the packed forms of the Blackwell FP32
+// pipe); a pair is held in one 64-bit register.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_make(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_split(f2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// One quarter (sub 0 .. 3) of the anchor of chunk q for the evaluation `r`,
+// written to out[kFoldAnchor]:
+//   sub 0: out[i] = frac(P(f_c) + f_c tau_i), double-float sums;
+//   sub 1: out[4], out[5] = the scaled slope h (P'(f_c) + tau_0 - s) as a
+//          double-float, out[5 + i] = h (tau_i - tau_0), i = 1 .. 3;
+//   sub 2: out[9], out[11], out[13], out[15]: even Taylor terms a_2 .. a_8;
+//   sub 3: out[10], out[12], out[14]: a_3, a_5, a_7, and the order-9 remainder
+//          bound against kFoldTaylorEps.
+// Returns false when the remainder is too large.  The serial part of an
+// anchor is the eleven-term double-float sums; four lanes of different warps
+// share it (a lane per chunk took 2.2x as long alone).
+template <int NDET>
+__device__ __forceinline__ bool fold_anchor(const FoldTables& F, const FoldIn& r, int sub, int q, float* out) {
+  const float* T = F.tab + q;
+  const int nc = F.nc;
+  auto row = [&](int k) { return __ldg(T + (size_t)k * nc); };
+  if (sub == 0) {
+    dfl A = {0.0f, 0.0f};
+#pragma unroll
+    for (int j = 0; j < NBASIS; ++j)
+      A = df_add(A, df_mul(dfl{r.c_hi[j], r.c_lo[j]}, dfl{row(FR_VAL_HI + j), row(FR_VAL_LO + j)}));
+    const dfl fc = {row(FR_FC_HI), row(FR_FC_LO)};
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) out[i] = df_frac(df_add(A, df_mul(fc, dfl{r.tau_hi[i], r.tau_lo[i]})));
+  } else if (sub == 1) {
+    const dfl h = {row(FR_H_HI), row(FR_H_LO)};
+    dfl S = df_add(df_mul(h, dfl{r.tau_hi[0], r.tau_lo[0]}), dfl{-row(FR_SM_HI), -row(FR_SM_LO)});
+#pragma unroll
+    for (int j = 0; j < kFoldSlopes; ++j)
+      S = df_add(S, df_mul(dfl{r.c_hi[j], r.c_lo[j]}, dfl{row(FR_D1_HI + j), row(FR_D1_LO + j)}));
+    out[4] = S.hi;
+    out[5] = S.lo;
+#pragma unroll
+    for (int i = 1; i < NDET; ++i)
+      out[5 + i] = h.hi * ((r.tau_hi[i] - r.tau_hi[0]) + (r.tau_lo[i] - r.tau_lo[0]));
+  } else {
+    const int n0 = sub == 2 ? 2 : 3, nn = sub == 2 ? 4 : 3;
+    float a[4] = {0.0f, 0.0f, 0.0f, 0.0f}, R = 0.0f;
+#pragma unroll
+    for (int j = 0; j < kFoldSlopes; ++j) {
+      const float c = r.c_hi[j];
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (m < nn) a[m] = fmaf(c, row(FR_POLY + (n0 + 2 * m - 2) * kFoldSlopes + j), a[m]);
+      if (sub == 3) R = fmaf(fabsf(c), row(FR_BND + j), R);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (m < nn) out[7 + n0 + 2 * m] = a[m];
+    return R <= kFoldTaylorEps;  // false for a NaN as well
+  }
+  return true;
+}
+
+// Whether the finished anchor of chunk q keeps below the chunk's bandwidth
+// (kernels.h FR_LIM): |slope| + sum_n n a^(n-1) |a_n| in cycles, a the half
+// axis of the Bernstein ellipse of the interpolation bound.
+template <int NDET>
+__device__ __forceinline__ bool fold_in_band(const FoldTables& F, const float* an, int q) {
+  float b = 0.0f;
+#pragma unroll
+  for (int i = 1; i < NDET; ++i) b = fmaxf(b, fabsf(an[5 + i]));
+  float om = fabsf(an[4]) + b, g = 1.0f;
+#pragma unroll
+  for (int n = 2; n <= kFoldDeg; ++n) {
+    g *= kFoldEllipse;
+    om = fmaf((float)n * g, fabsf(an[7 + n]), om);
+  }
+  return om <= __ldg(F.tab + (size_t)FR_LIM * F.nc + q);  // false for a NaN as well
+}
+
+// Accumulators of a lane: per detector the four real products of the complex
+// multiply-add, for the nodes +x and -x in the two halves of a pair.
+template <int NDET>
+struct FoldAcc {
+  f2 rr[NDET], ri[NDET], ir[NDET], ii[NDET];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) rr[i] = ri[i] = ir[i] = ii[i] = 0ull;
+  }
+  __device__ __forceinline__ void total(int i, float& re, float& im) const {
+    float a, b, c, d, e, f, g, h;
+    f2_split(rr[i], a, b);
+    f2_split(ri[i], c, d);
+    f2_split(ir[i], e, f);
+    f2_split(ii[i], g, h);
+    re = (a + b) + (c + d);
+    im = (e + f) - (g + h);
+  }
+};
+
+// Chunk q of one evaluation by one warp, two nodes (+x, -x) per lane.  The
+// phase is E(x) + O(x), even and odd Taylor parts: at the two nodes E + O and
+// E - O, so the polynomial is formed once for both; the slope's product with x
+// is carried in double-float and reduced to its fractional part.
+template <int NDET>
+__device__ __forceinline__ void fold_chunk(const FoldTables& F, const float* __restrict__ an, int q, int lane,
+                                           FoldAcc<NDET>& acc) {
+  const float4* W = F.w + (size_t)q * NDET * 32 + lane;
+  float4 w[NDET];
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) w[i] = __ldg(W + 32 * i);
+  const float2 xv = __ldg(F.x + 32 * (int)__ldg(F.tab + (size_t)FR_KIND * F.nc + q) + lane);
+  const float4 A = *reinterpret_cast<const float4*>(an), B = *reinterpret_cast<const float4*>(an + 4);
+  const float4 C = *reinterpret_cast<const float4*>(an + 8), D = *reinterpret_cast<const float4*>(an + 12);
+  const float x = xv.x, x2 = x * x;
+  // C = (b_3, a_2, a_3, a_4), D = (a_5, a_6, a_7, a_8)
+  const float ev = x2 * fmaf(x2, fmaf(x2, fmaf(x2, D.w, D.y), C.w), C.y);
+  const float oh = x2 * x * fmaf(x2, fmaf(x2, D.z, D.x), C.z);
+  const float p = x * B.x;
+  float e = fmaf(x, B.x, -p);
+  e = fmaf(xv.y, B.x, e);
+  e = fmaf(x, B.y, e);
+  const float od = (p - round_nearest(p)) + (e + oh);
+  const float b[4] = {0.0f, B.z, B.w, C.x}, a0[4] = {A.x, A.y, A.z, A.w};
+  const f2 magic = f2_make(12582912.0f, 12582912.0f), nmagic = f2_make(-12582912.0f, -12582912.0f);
+  const f2 none = f2_make(-1.0f, -1.0f), twopi = f2_make(6.283185307179586f, 6.283185307179586f);
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) {
+    const float ei = ev + a0[i], oi = i ? fmaf(b[i], x, od) : od;
+    f2 ph = f2_make(ei + oi, ei - oi);
+    const f2 n = f2_add(f2_add(ph, magic), nmagic);  // nearest integers (see round_nearest)
+    ph = f2_mul(f2_fma(n, none, ph), twopi);
+    float pa, pb, sa, ca, sb, cb;
+    f2_split(ph, pa, pb);
+    __sincosf(pa, &sa, &ca);
+    __sincosf(pb, &sb, &cb);
+    const f2 c2 = f2_make(ca, cb), s2 = f2_make(sa, sb);
+    const f2 wr = f2_make(w[i].x, w[i].y), wi = f2_make(w[i].z, w[i].w);
+    acc.rr[i] = f2_fma(wr, c2, acc.rr[i]);
+    acc.ri[i] = f2_fma(wi, s2, acc.ri[i]);
+    acc.ir[i] = f2_fma(wi, c2, acc.ir[i]);
+    acc.ii[i] = f2_fma(wr, s2, acc.ii[i]);
+  }
+}
+
+// Bin by bin (rare): tiles first, first + stride, ... of the grid by one warp
+// from global memory, with the tile anchors of the direct sum (sweep.cuh);
+// row: kAnchorStride floats of the warp's own in shared memory.  Lane sums in
+// FP64 across tiles; every lane returns the warp's totals.
+template <int NDET>
+__device__ __noinline__ void fold_direct(const LikeConst& L, const FoldTables& F, const EvalRecord& r, int first,
+                                         int stride, int lane, float* row, double* out) {
+#pragma unroll
+  for (int j = 0; j < 2 * NDET; ++j) out[j] = 0.0;
+  for (int t = first; t < L.n_tiles; t += stride) {
+    __syncwarp();
+    if (lane == 0) compute_anchor(NDET, F.tiles[t], F.basis[t], r, row);
+    __syncwarp();
+    float v[2 * NDET];
+    const int lo = F.tiles[t].k0, hi = lo + F.tiles[t].nbins;
+    sweep_warp_mixed<NDET>(L, F.data, L.n_bins, F.bin_tile, 0, lo, hi, F.tiles + t, row, t, r, lane, v);
+#pragma unroll
+    for (int j = 0; j < 2 * NDET; ++j) out[j] += (double)v[j];
+  }
+}
+
+// Distance-marginalised logL (distance_marg_logl) by a whole warp: the 64
+// nodes on 32 lanes, each exponent formed once.
+__device__ inline double distance_marg_logl_warp(const LikeConst& L, double zre, double zim, double H, int lane) {
+  const double X = L.phase_marg ? sqrt(zre * zre + zim * zim) : zre;
+  double a, b;
+  distance_window(L, X, H, &a, &b);
+  const double mid = 0.5 * (a + b), half = 0.5 * (b - a);
+  static_assert(kGaussLegendre == 64, "two nodes per lane");
+  const double e0 = distance_exponent(L, zre, X, H, mid + half * L.gl_x[lane]);
+  const double e1 = distance_exponent(L, zre, X, H, mid + half * L.gl_x[lane + 32]);
+  double M = fmax(fmax(-INFINITY, e0), e1);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+  double sum = L.gl_w[lane] * (double)expf((float)(e0 - M)) + L.gl_w[lane + 32] * (double)expf((float)(e1 - M));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return M + log(half * sum) - 0.5 * L.DD;
+}
+
+// logL of record r by a whole warp from kappa (component j on lane j < 2
+// NDET, data-scaled): detector i's terms of Z on lane i, added in detector
+// order, then loglike_epilogue's closed forms.  Every lane returns it.
+template <int NDET>
+__device__ __forceinline__ double loglike_epilogue_warp(const LikeConst& L, const EvalRecord& r, double kapc,
+                                                        int lane) {
+  const int di = lane < NDET ? lane : 0;
+  const double kre = __shfl_sync(0xffffffffu, kapc, 2 * di), kim = __shfl_sync(0xffffffffu, kapc, 2 * di + 1);
+  double tr = 0.0, ti = 0.0;
+  if (lane < NDET) {
+    const double a = kre * L.inv_scale[di], b = kim * L.inv_scale[di];
+    tr = r.cre[di] * a - r.cim[di] * b;
+    ti = r.cre[di] * b + r.cim[di] * a;
+  }
+  double zr = __shfl_sync(0xffffffffu, tr, 0), zi = __shfl_sync(0xffffffffu, ti, 0);
+#pragma unroll
+  for (int i = 1; i < NDET; ++i) {
+    zr += __shfl_sync(0xffffffffu, tr, i);
+    zi += __shfl_sync(0xffffffffu, ti, i);
+  }
+  if (!r.valid) return -INFINITY;  // warp-uniform
+  if (L.dist_marg) return distance_marg_logl_warp(L, zr, zi, r.hh, lane);
+  const double base = -0.5 * r.hh - 0.5 * L.DD;
+  if (!L.phase_marg) return zr + base;
+  const double x = sqrt(zr * zr + zi * zi);
+  return (L.fast_epilogue ? x + (double)log_i0e_f32((float)x) : log_bessel_i0(x)) + base;
+}
+
+}  // namespace swig

@@ -87,6 +87,68 @@ static_assert(kHetAncExact < kHetAncStride, "chunk anchor layout");
 // widths, edge offsets), filled by cp.async one chunk ahead: bytes per stage.
 inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) + 2 * 32 * 4; }
 
+// Folded full-grid sums (fold.cuh): the grid in chunks of kFoldNodes nodes.
+// Rows of the [FR_ROWS][chunks] table: at the chunk's centre f_c, with h the
+// half width [Hz] that scales the node abscissae to |x| <= 1, the basis values
+// and first derivatives times h (double-float; the constant basis function,
+// last, has no derivatives), derivatives of orders 2..kFoldDeg times h^n / n!
+// (float), the order-9 remainder bound max |phi_j^(9)| h^9 / 9!, f_c, h and the
+// reference slope times h (double-float), the bandwidth the weights serve
+// [cycles] and the node kind.
+constexpr int kFoldNodes = 64;
+constexpr int kFoldDeg = 8;
+constexpr int kFoldSlopes = NBASIS - 1;
+enum FoldRow {
+  FR_VAL_HI = 0,
+  FR_VAL_LO = NBASIS,
+  FR_D1_HI = 2 * NBASIS,
+  FR_D1_LO = FR_D1_HI + kFoldSlopes,
+  FR_POLY = FR_D1_LO + kFoldSlopes,  // FR_POLY + (n - 2) * kFoldSlopes + j
+  FR_BND = FR_POLY + (kFoldDeg - 1) * kFoldSlopes,
+  FR_FC_HI = FR_BND + kFoldSlopes,
+  FR_FC_LO,
+  FR_H_HI,
+  FR_H_LO,
+  FR_SM_HI,
+  FR_SM_LO,
+  FR_LIM,
+  FR_KIND,
+  FR_ROWS
+};
+// Node kinds: 0 the 64 Chebyshev nodes; s = 1 .. kFoldKinds - 1 the bins of a
+// block of w = 128 >> s themselves, x = +-(2 l + 1) / w.
+constexpr int kFoldKinds = 7;
+// Interpolation of exp(2 pi i delta(x)) through n Chebyshev nodes errs by at
+// most 4 M rho^(1 - n) / (rho - 1), M its bound on the Bernstein ellipse of
+// parameter rho: M <= exp(2 pi b omega) with omega = |delta_1| + sum_n n
+// a^(n-1) |delta_n|, a and b the ellipse's half axes.  rho = 3 gave the fewest
+// chunks on the 128 s grid (78; 2: 130, 4: 82, 5: 87).
+constexpr float kFoldRho = 3.0f;
+constexpr float kFoldEllipse = 0.5f * (kFoldRho + 1.0f / kFoldRho);
+// Taylor remainder [cycles] and interpolation error an evaluation may have
+// (the host plans for a fifth and a tenth of them over the prior box).
+constexpr float kFoldTaylorEps = 1e-7f;
+constexpr double kFoldEps = 1e-7;
+
+struct FoldChunk {
+  int k0, nbins;   // bins [k0, k0 + nbins)
+  int kind;        // node kind
+  int pad;
+  double slope_h;  // reference slope times h [cycles]
+};
+
+struct FoldTables {
+  int nc;             // chunks
+  const float* tab;   // [FR_ROWS][nc]
+  const float4* w;    // [nc][n_det][32] node weights (+x re, -x re, +x im, -x im)
+  const float2* x;    // [kFoldKinds][32] abscissae (hi, lo)
+  // bin by bin (fold_direct)
+  const float2* data;
+  const TileInfo* tiles;
+  const TileBasis* basis;
+  const int* bin_tile;
+};
+
 // Device buffers owned by a context (all allocated with cudaMalloc).
 struct DeviceBuffers {
   // problem data
@@ -98,10 +160,10 @@ struct DeviceBuffers {
   int* slice_begin = nullptr;    // [n_slices + 1] first bin of each slice
   int* bin_tile = nullptr;       // [n_bins] tile of each bin
   PriorSlot* prior = nullptr;    // [13]
-  int* piece_begin = nullptr;    // first bin of each sweep piece, slices concatenated (+ end per slice)
-  int* slice_piece = nullptr;    // [n_slices + 1] offset of each slice's entries in piece_begin
-  int n_pieces = 0;              // total pieces (work units per theta)
-  int max_pieces = 1;            // pieces of the largest slice
+  int fold_nc = 0;               // folded full-grid sums (FoldTables)
+  float* fold_tab = nullptr;
+  float4* fold_w = nullptr;
+  float2* fold_x = nullptr;
   int max_slice_bins = 0;
   // heterodyned likelihood tables (SWIG_LIKE_HET)
   int het_nb = 0;
@@ -127,13 +189,24 @@ struct DeviceBuffers {
   // scratch for batched evaluation, sized for `cap` thetas
   int cap = 0;
   EvalRecord* rec = nullptr;     // [cap]
-  float* anchors = nullptr;      // [cap][n_tiles][kAnchorStride]
   float* partials32 = nullptr;   // [cap][n_slices][kPartialStride]
   double* partials64 = nullptr;  // [cap][n_slices][kPartialStride]
   double* theta = nullptr;       // [cap][13] staging for host calls
   double* out = nullptr;         // [cap]
   double* u = nullptr;           // [cap][13]
 };
+
+inline __host__ __device__ FoldTables fold_tables(const DeviceBuffers& B) {
+  return {B.fold_nc, B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile};
+}
+
+// Node weights of the event (B.fold_w) from its weighted data (B.data32) and
+// the chunks (device pointer); synchronises the stream.
+cudaError_t launch_fold_weights(const LikeConst& L, const DeviceBuffers& B, const FoldChunk* chunks, cudaStream_t st);
+// The folded evaluation of n records in B.rec (launch_loglike_mixed after its
+// set-up).
+cudaError_t launch_fold(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
+                        double* kappa_out);
 
 // logL of n thetas (device pointers) into out; kappa_out (optional, n x 8
 // doubles) receives the unscaled per-detector sums (re, im) for each theta.
@@ -163,7 +236,6 @@ cudaError_t launch_time_draw(const LikeConst& L, const DeviceBuffers& B, const f
                              unsigned k0, unsigned k1, double* theta, cudaStream_t st);
 cudaError_t launch_prior_transform(const PriorSlot* slots, int n_sampled, const double* u, int n, double* theta,
                                    cudaStream_t st, SkyFrame sky);
-cudaError_t set_sweep_smem_limit(size_t bytes);
 
 // Dynamic shared memory of the mixed sweep: data (float2 per detector and
 // bin) plus the tile index of each bin of the slice.

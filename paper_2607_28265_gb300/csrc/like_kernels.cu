@@ -1,23 +1,14 @@
 // Batched matched-filter log-likelihood kernels (Eq. 2 of the paper) on the
 // full frequency grid, in two precisions:
 //
-//  * MIXED: per-bin work in FP32.  The TaylorF2 phase is anchored per tile in
-//    double-float (FP32 pairs): within a tile of T bins the phase in cycles is
-//    P(f_a + x df) = A0 + frac(x s_hi) + x s_lo + sum_{n=2..6} a_n (x/T)^n with
-//    A0 = frac P(f_a), s = P'(f_a) df split so that x s_hi is exact, and the
-//    Taylor coefficients a_n from the tile's basis table.  Each detector adds
-//    frac(f_a tau_i) + x df tau_i.  The complex exponential uses the SFU
-//    (__sincosf on the reduced argument), the per-bin products are
-//    accumulated in FP32 per thread and combined by a pairwise tree (warp
-//    shuffles, shared memory, then FP64 across slices).
+//  * MIXED: FP32 phases and sums over the folded grid (fold.cuh); here only
+//    the set-up of its records.
 //  * FP64: every per-bin quantity in FP64 with sincospi, as the reference
-//    precision of the small single-detector configuration.
+//    precision of the small single-detector configuration: one warp per (theta,
+//    slice of the grid), one partial sum each, added per theta in a fixed order.
 //
-// The grid is cut into `n_slices` contiguous ranges of whole 32-bin chunks,
-// one CTA per slice; the slice's data D_i(f) = 4 df conj(d_i) f^-7/6 / S_i is
-// staged once into shared memory and reused for every theta of the batch.
-// Inside a CTA each warp-group (4 warps) evaluates one theta at a time over the
-// slice and writes one partial sum per (theta, slice).
+// The heterodyned likelihood, post-hoc draws, waveforms and the prior transform
+// follow.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -34,58 +25,6 @@ __global__ void k_setup(LikeConst L, const double* __restrict__ theta, int n, Ev
   if (L.dist_marg) th[6] = 1.0;   // the marginal is built from the template at 1 Mpc
   if (L.tm_n > 0) th[11] = L.tm_tref;  // templates at the fiducial's t_c, shifted node by node
   setup_record(L, th, rec + i);
-}
-
-// Per (theta, tile) anchors, one thread each (double-float on the FP32 pipe).
-__global__ void k_anchor(LikeConst L, const TileInfo* __restrict__ tiles, const TileBasis* __restrict__ basis,
-                         const EvalRecord* __restrict__ rec, int n, float* __restrict__ anchors) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)n * L.n_tiles;
-  if (idx >= total) return;
-  const int th = (int)(idx / L.n_tiles), t = (int)(idx % L.n_tiles);
-  compute_anchor(L.n_det, tiles[t], basis[t], rec[th], anchors + idx * kAnchorStride);
-}
-
-// Work units are (theta, group of consecutive pieces of the slice): `groups`
-// units per theta split the slice's pieces evenly, so that n * groups units
-// fill the 32 warps with a small tail.  Each unit writes its own partial
-// [(theta * n_slices * groups + slice * groups + unit)] (fixed reduction order).
-template <int NDET>
-__global__ void __launch_bounds__(kSweepThreads, 1)
-    k_sweep_mixed(LikeConst L, const float2* __restrict__ data, const int* __restrict__ slice_begin,
-                  const int* __restrict__ bin_tile, const TileInfo* __restrict__ tiles,
-                  const float* __restrict__ anchors, const EvalRecord* __restrict__ rec, int n,
-                  const int* __restrict__ piece_begin, const int* __restrict__ slice_piece, int groups,
-                  float* __restrict__ partials) {
-  extern __shared__ float2 s_data[];  // [NDET][slice bins], then int tile id per bin
-  const int slice = blockIdx.x;
-  const int b0 = slice_begin[slice], b1 = slice_begin[slice + 1];
-  const int nb = b1 - b0;
-  int* s_tile = reinterpret_cast<int*>(s_data + (size_t)NDET * nb);
-  for (int i = 0; i < NDET; ++i)
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) s_data[i * nb + k] = data[(size_t)i * L.n_bins + b0 + k];
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) s_tile[k] = bin_tile[b0 + k];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int p0 = slice_piece[slice], n_pc = slice_piece[slice + 1] - p0 - 1;
-  const int g = min(groups, n_pc);
-  const int units = n * groups;
-  for (int u = warp; u < units; u += kSweepThreads / 32) {
-    const int th = u / groups, gi = u % groups;
-    float v[2 * NDET];
-    if (gi < g) {
-      const int pa = gi * n_pc / g, pb = (gi + 1) * n_pc / g;
-      const int lo = piece_begin[p0 + pa] - b0, hi = piece_begin[p0 + pb] - b0;
-      const float* row = anchors + (size_t)th * L.n_tiles * kAnchorStride;
-      sweep_warp_mixed<NDET>(L, s_data, nb, s_tile, b0, lo, hi, tiles, row, 0, rec[th], lane, v);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 2 * NDET; ++j) v[j] = 0.0f;
-    }
-#pragma unroll
-    for (int j = 0; j < 2 * NDET; ++j)
-      if (lane == j) partials[((size_t)th * L.n_slices * groups + (size_t)slice * groups + gi) * kPartialStride + j] = v[j];
-  }
 }
 
 template <int NDET>
@@ -106,8 +45,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // Per theta: FP64 sum of the slice partials (fixed order), then the epilogue.
-template <typename T>
-__global__ void k_reduce(LikeConst L, const T* __restrict__ partials, int n_units, const EvalRecord* __restrict__ rec,
+__global__ void k_reduce(LikeConst L, const double* __restrict__ partials, int n_units, const EvalRecord* __restrict__ rec,
                          int n, double* __restrict__ out, double* __restrict__ kappa_out) {
   const int th = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -116,10 +54,10 @@ __global__ void k_reduce(LikeConst L, const T* __restrict__ partials, int n_unit
 #pragma unroll
   for (int j = 0; j < 2 * SWIG_MAX_DET; ++j) acc[j] = 0.0;
   for (int s = lane; s < n_units; s += 32) {
-    const T* p = partials + ((size_t)th * n_units + s) * kPartialStride;
+    const double* p = partials + ((size_t)th * n_units + s) * kPartialStride;
 #pragma unroll
     for (int j = 0; j < 2 * SWIG_MAX_DET; ++j)
-      if (j < 2 * L.n_det) acc[j] += (double)p[j];
+      if (j < 2 * L.n_det) acc[j] += p[j];
   }
 #pragma unroll
   for (int j = 0; j < 2 * SWIG_MAX_DET; ++j)
@@ -430,24 +368,7 @@ cudaError_t launch_loglike_mixed(const LikeConst& L, const DeviceBuffers& B, con
                                  double* out, cudaStream_t st, double* kappa_out) {
   if (n <= 0) return cudaSuccess;
   k_setup<<<(n + 127) / 128, 128, 0, st>>>(L, theta, n, B.rec);
-  const long long items = (long long)n * L.n_tiles;
-  k_anchor<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(L, B.tiles, B.basis, B.rec, n, B.anchors);
-  const size_t smem = sweep_smem_bytes(L.n_det, B.max_slice_bins);
-  // units per theta: the smallest g whose tail over 32 warps is below ~10%
-  int groups = 1;
-  for (int gg = 1; gg <= 4; ++gg) {
-    groups = gg;
-    const int units = n * gg, waves = (units + 31) / 32;
-    if ((double)units / (32.0 * waves) >= 0.9) break;
-  }
-  switch (L.n_det) {
-    case 1: k_sweep_mixed<1><<<L.n_slices, kSweepThreads, smem, st>>>(L, B.data32, B.slice_begin, B.bin_tile, B.tiles, B.anchors, B.rec, n, B.piece_begin, B.slice_piece, groups, B.partials32); break;
-    case 2: k_sweep_mixed<2><<<L.n_slices, kSweepThreads, smem, st>>>(L, B.data32, B.slice_begin, B.bin_tile, B.tiles, B.anchors, B.rec, n, B.piece_begin, B.slice_piece, groups, B.partials32); break;
-    case 3: k_sweep_mixed<3><<<L.n_slices, kSweepThreads, smem, st>>>(L, B.data32, B.slice_begin, B.bin_tile, B.tiles, B.anchors, B.rec, n, B.piece_begin, B.slice_piece, groups, B.partials32); break;
-    default: k_sweep_mixed<4><<<L.n_slices, kSweepThreads, smem, st>>>(L, B.data32, B.slice_begin, B.bin_tile, B.tiles, B.anchors, B.rec, n, B.piece_begin, B.slice_piece, groups, B.partials32); break;
-  }
-  k_reduce<float><<<(n + 3) / 4, 128, 0, st>>>(L, B.partials32, L.n_slices * groups, B.rec, n, out, kappa_out);
-  return cudaGetLastError();
+  return launch_fold(L, B, n, out, st, kappa_out);
 }
 
 cudaError_t launch_loglike_fp64(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n,
@@ -462,7 +383,7 @@ cudaError_t launch_loglike_fp64(const LikeConst& L, const DeviceBuffers& B, cons
     case 3: k_sweep_fp64<3><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
     default: k_sweep_fp64<4><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
   }
-  k_reduce<double><<<(n + 3) / 4, 128, 0, st>>>(L, B.partials64, L.n_slices, B.rec, n, out, kappa_out);
+  k_reduce<<<(n + 3) / 4, 128, 0, st>>>(L, B.partials64, L.n_slices, B.rec, n, out, kappa_out);
   return cudaGetLastError();
 }
 
@@ -471,14 +392,6 @@ cudaError_t launch_prior_transform(const PriorSlot* slots, int n_sampled, const 
   if (n <= 0) return cudaSuccess;
   k_prior_transform<<<(n + 127) / 128, 128, 0, st>>>(slots, n_sampled, u, n, theta, sky);
   return cudaGetLastError();
-}
-
-cudaError_t set_sweep_smem_limit(size_t bytes) {
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_sweep_mixed<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return e;
-  if ((e = cudaFuncSetAttribute(k_sweep_mixed<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return e;
-  if ((e = cudaFuncSetAttribute(k_sweep_mixed<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return e;
-  return cudaFuncSetAttribute(k_sweep_mixed<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 }  // namespace swig

@@ -32,8 +32,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 void* g_noalloc_ptr[kMaxDevices] = {};
 
-size_t round_up(size_t v) { return (v + 255) & ~(size_t)255; }
-
 // Device address of the scratch array on `device` (set-up on first use, with
 // that device current).  The array's host-side name is only a stand-in and
 // must never be handed to a kernel.
@@ -68,8 +66,10 @@ extern "C" int swig_loglike_batch_noalloc(swig_ctx* c, const double* theta_dev, 
              "swig_run call with the current problem (preparation allocates; this entry point does not)";
     return SWIG_E_STATE;
   }
-  // Capacity first, from the per-vector bytes (three 256-byte roundings at
-  // most on top), so that no size below is formed from an unchecked n.
+  // Capacity first, so that no size below is formed from an unchecked n.  The
+  // per-vector bytes are this entry point's stated budget (a record, an anchor
+  // per tile and four partial sums per slice); the folded evaluation uses the
+  // record alone.
   const size_t per_theta = sizeof(EvalRecord) + sizeof(float) * kAnchorStride * (size_t)c->L.n_tiles +
                            sizeof(float) * kPartialStride * (size_t)c->L.n_slices * 4;
   const int64_t cap = (int64_t)((kNoAllocScratchBytes - 3 * 256) / per_theta);
@@ -79,9 +79,6 @@ extern "C" int swig_loglike_batch_noalloc(swig_ctx* c, const double* theta_dev, 
              " parameter vectors for this grid); split the batch";
     return SWIG_E_ARG;
   }
-  // layout: [records][anchors][partials], each 256-byte aligned
-  const size_t rec_b = round_up(sizeof(EvalRecord) * (size_t)n);
-  const size_t anc_b = round_up(sizeof(float) * kAnchorStride * (size_t)c->L.n_tiles * (size_t)n);
   cudaError_t e = cudaSetDevice(c->device);
   void* base = nullptr;
   if (e == cudaSuccess) e = scratch_address(c->device, &base);
@@ -89,19 +86,16 @@ extern "C" int swig_loglike_batch_noalloc(swig_ctx* c, const double* theta_dev, 
     c->err = std::string("scratch set-up: ") + cudaGetErrorString(e);
     return SWIG_E_CUDA;
   }
-  // Every scratch word this call reads is written earlier in the same call
-  // (records, anchors, one partial per work unit), so nothing needs clearing.
+  // The scratch holds the set-up records, each written earlier in the same
+  // call that reads it, so nothing needs clearing.
   DeviceBuffers B = c->B;
-  unsigned char* p = static_cast<unsigned char*>(base);
-  B.rec = reinterpret_cast<EvalRecord*>(p);
-  B.anchors = reinterpret_cast<float*>(p + rec_b);
-  B.partials32 = reinterpret_cast<float*>(p + rec_b + anc_b);
+  B.rec = static_cast<EvalRecord*>(base);
   B.cap = (int)n;
   e = launch_loglike_mixed(c->L, B, theta_dev, (int)n, out_logl_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) {
     c->err = std::string("likelihood launch: ") + cudaGetErrorString(e);
     return SWIG_E_CUDA;
   }
-  c->n_launches += 4;
+  c->n_launches += 2;
   return SWIG_OK;
 }

@@ -97,7 +97,6 @@ struct SamplerConst {
   int m_pow2;
   int max_iters;
   long long spin_limit;
-  int max_pieces;      // pieces per slice (sweep work units)
   int max_tiles_slice; // tiles overlapping the largest slice
   int n_ctas;
   int mixed;
@@ -180,8 +179,6 @@ struct SamplerPtrs {
   double* dead_logw;
   const double* harm;  // [k + 1]: sum_{i<j} 1 / (m - i)
   const double* lw;    // [m + 1]: log(1 - exp(-1/n))
-  const int* piece_begin;  // [n_pieces_total + n_slices] absolute first bin of each piece, per slice
-  const int* slice_piece;  // [n_slices + 1] offset of each slice's pieces in piece_begin
   float* anchor_buf;       // [n_slices][k][max_tiles_slice][kAnchorStride] per-round anchors
   const float* learn_out;  // [m][32] network outputs (u, s) of a frozen live snapshot, or null
   int* req;                // [k] 8 * (sequence number of the chain's latest full-likelihood request) + parts per slice
@@ -2539,8 +2536,6 @@ int run_setup(swig_ctx* c, RunState& R) {
     S.learn_mix = (float)learn_mix;
   }
 
-  const int max_pieces = c->B.max_pieces;
-  S.max_pieces = max_pieces;
   size_t fixed = 0;
   if (mixed) fixed = ((size_t)c->B.max_slice_bins * (L.n_det * sizeof(float2) + sizeof(int)) + 15) & ~(size_t)15;
   R.fixed = fixed;
@@ -2616,8 +2611,6 @@ int run_setup(swig_ctx* c, RunState& R) {
     st->P.lw = st->lw;
   }
   R.st = st;
-  st->P.piece_begin = c->B.piece_begin;
-  st->P.slice_piece = c->B.slice_piece;
   dfree(st->anchor_buf);
   if (mixed) {
     SCUDA(cudaMalloc(&st->anchor_buf, sizeof(float) * kAnchorStride * (size_t)L.n_slices * k * max_tiles));
@@ -2663,7 +2656,7 @@ int run_setup(swig_ctx* c, RunState& R) {
   SCUDA(cudaMemsetAsync(st->P.req, 0, sizeof(int) * 2 * k, c->stream));
   SCUDA(cudaMemsetAsync(st->P.done_cnt, 0, sizeof(int) * 2 * k, c->stream));
   SCUDA(cudaMemsetAsync(st->P.chains, 0, sizeof(ChainState) * k, c->stream));
-  c->n_launches += het ? 3 : (mixed ? 5 : 4);  // init draw + batched likelihood
+  c->n_launches += het || mixed ? 3 : 4;  // init draw + batched likelihood
 
   R.kern = het ? pick_het_kernel(L.n_det) : pick_kernel(L.n_det, mixed);
   R.threads = het ? kHetThreads : kFlowThreads;
@@ -2778,7 +2771,7 @@ int run_finish(swig_ctx* c, RunState& R, swig_result* out) {
         if (e == cudaSuccess)
           e = launch_distance_draw(L, c->B, kap_d, mm, (long long)off, S.key0, S.key1, th_d + off * SWIG_N_PARAMS,
                                    c->stream);
-        c->n_launches += mixed ? 5 : 4;
+        c->n_launches += mixed ? 3 : 4;
       }
       if (kap_d) cudaFree(kap_d);
       if (ll_d) cudaFree(ll_d);

@@ -31,8 +31,7 @@ constexpr int kTaylorDeg = 6;        // a_2 .. a_6 per tile
 constexpr int kNumPoly = kTaylorDeg - 1;
 constexpr int kChunk = 32;           // bins per warp step; tiles are multiples
 constexpr int kMaxTileBins = 2048;
-constexpr int kSweepThreads = 1024;  // 8 warp-groups of 4 warps
-constexpr int kWarpGroups = kSweepThreads / 128;
+constexpr int kSweepThreads = 1024;  // widest reduction scratch of the sampler's boundary
 constexpr int kPartialStride = 8;    // floats/doubles per (theta, slice) partial
 constexpr int kAnchorStride = 12;    // floats per (theta, tile): A0, s_hi, s_lo, a2..a6, A_det[4]
 
@@ -74,6 +73,7 @@ constexpr int kGaussLegendre = 64;  // nodes of the distance integral
 constexpr int kMaxTmNodes = 65536;  // largest time-marginalisation grid
 
 struct LikeConst {
+  int sm_count;  // of the context's device
   int n_det;
   int n_bins;
   int k_min;
