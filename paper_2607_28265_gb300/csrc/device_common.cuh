@@ -151,30 +151,38 @@ __host__ __device__ inline void taylorf2_tidal_coeffs(const MassTerms& t, double
   c[B_P73] = t.A * a12 * r7;
 }
 
-__host__ __device__ inline void taylorf2_basis_coeffs_from(const MassTerms& t, double chi1, double chi2,
-                                                           double lam1, double lam2, double* c) {
-  const double eta = t.eta, eta2 = eta * eta, eta3 = eta2 * eta;
-  const double pi2 = kPi * kPi;
-  const double a0 = 1.0;
+// The mass-only coefficients: powers of f up to the logarithm, and above it.
+__host__ __device__ inline void taylorf2_low_coeffs(const MassTerms& t, double* c) {
+  const double eta = t.eta;
   const double a2 = 3715.0 / 756.0 + 55.0 / 9.0 * eta;
   const double a5 = kPi * (38645.0 / 756.0 - 65.0 / 9.0 * eta);
   const double a5log = 3.0 * a5;
+  const double ir2 = t.ir * t.ir, ir3 = ir2 * t.ir, ir5 = ir3 * ir2;
+  const double third = 1.0 / 3.0;
+  const double ln_vlso = -0.89587973461402746;  // -ln(6)/2
+  c[B_M53] = t.A * ir5;
+  c[B_M1] = t.A * a2 * ir3;
+  c[B_LOG] = t.A * a5log * third;
+  c[B_ONE] = t.A * (a5 + a5log * (t.lpm * third - ln_vlso)) - 0.125;
+}
+__host__ __device__ inline void taylorf2_high_coeffs(const MassTerms& t, double* c) {
+  const double eta = t.eta, eta2 = eta * eta, eta3 = eta2 * eta;
+  const double pi2 = kPi * kPi;
   const double a6 = 11583231236531.0 / 4694215680.0 - 640.0 / 3.0 * pi2 - 6848.0 / 21.0 * kEulerGamma +
                     (-15737765635.0 / 3048192.0 + 2255.0 / 12.0 * pi2) * eta + 76055.0 / 1728.0 * eta2 -
                     127825.0 / 1296.0 * eta3;
   const double a6log = -6848.0 / 21.0;
   const double a7 = kPi * (77096675.0 / 254016.0 + 378515.0 / 1512.0 * eta - 74045.0 / 756.0 * eta2);
-  const double ir2 = t.ir * t.ir, ir3 = ir2 * t.ir, ir5 = ir3 * ir2;
-  const double r2 = t.r * t.r;
-  const double third = 1.0 / 3.0;
-  const double ln4 = 1.3862943611198906188, ln_vlso = -0.89587973461402746;  // ln 4, -ln(6)/2
-  c[B_M53] = t.A * a0 * ir5;
-  c[B_M1] = t.A * a2 * ir3;
-  c[B_LOG] = t.A * a5log * third;
+  const double third = 1.0 / 3.0, ln4 = 1.3862943611198906188;
   c[B_P13] = t.A * t.r * (a6 + a6log * (ln4 + t.lpm * third));
   c[B_P13LOG] = t.A * t.r * a6log * third;
-  c[B_P23] = t.A * a7 * r2;
-  c[B_ONE] = t.A * (a5 + a5log * (t.lpm * third - ln_vlso)) - 0.125;
+  c[B_P23] = t.A * a7 * (t.r * t.r);
+}
+
+__host__ __device__ inline void taylorf2_basis_coeffs_from(const MassTerms& t, double chi1, double chi2,
+                                                           double lam1, double lam2, double* c) {
+  taylorf2_low_coeffs(t, c);
+  taylorf2_high_coeffs(t, c);
   taylorf2_spin_coeffs(t, chi1, chi2, c);
   taylorf2_tidal_coeffs(t, lam1, lam2, c);
 }
@@ -187,7 +195,24 @@ __host__ __device__ inline void taylorf2_basis_coeffs(double mc, double q, doubl
 // sqrt(5/24) pi^(-2/3) (G Mc / c^3)^(5/6) c / (1 Mpc): Newtonian SPA amplitude
 // times d_L[Mpc].
 __host__ __device__ inline double amplitude_per_mpc(double mc) {
-  return sqrt(5.0 / 24.0) * exp(-2.0 / 3.0 * log(kPi)) * exp(5.0 / 6.0 * log(mc * kMtsunS)) * kCSI / kMpcM;
+  constexpr double kSqrtPi = 0.45643546458763845 * 0.46619407703541166;  // sqrt(5/24) pi^(-2/3)
+  return kSqrtPi * (kCSI / kMpcM) * exp(5.0 / 6.0 * log(mc * kMtsunS));
+}
+
+// Antenna patterns from the sines and cosines of the source's longitude
+// (RA - GMST) (sl, cl), declination (sd, cd) and 2 psi (s2, c2): with u = e D e -
+// n D n and v = 2 e D n on the unit vectors e (east) and n (north), F+ = c2 u -
+// s2 v and Fx = -(s2 u + c2 v) in antenna_fp_fx's polarisation basis.
+__device__ inline void antenna_from_sc(const double* d, double sl, double cl, double sd, double cd, double s2,
+                                       double c2, double* fp, double* fx) {
+  const double nx = -sd * cl, ny = -sd * sl;
+  const double ex = cl * d[1] - sl * d[0], ey = cl * d[3] - sl * d[1], ez = cl * d[4] - sl * d[2];  // e D
+  const double dx = nx * d[0] + ny * d[1] + cd * d[2], dy = nx * d[1] + ny * d[3] + cd * d[4],
+               dz = nx * d[2] + ny * d[4] + cd * d[5];  // n D
+  const double u = (cl * ey - sl * ex) - (nx * dx + ny * dy + cd * dz);
+  const double v = 2.0 * (nx * ex + ny * ey + cd * ez);
+  *fp = c2 * u - s2 * v;
+  *fx = -(s2 * u + c2 * v);
 }
 
 // Antenna patterns of detector tensor D (xx xy xz yy yz zz) for a source at

@@ -17,14 +17,137 @@
 
 namespace swig {
 
-__global__ void k_setup(LikeConst L, const double* __restrict__ theta, int n, EvalRecord* __restrict__ rec) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// Set-up records (FP64), 32 parameter vectors per block, one per lane, one
+// piece of the record per warp: a warp's FP64 instruction takes 64 cycles of
+// its scheduler however many lanes it serves, so a record's pieces run side by
+// side on the SM's four schedulers and the vectors ride along in the lanes.
+// What bounds it is the longest chain, the logarithm, exponential and
+// divisions of the mass terms.  (One thread per record: 30 us for any batch.)
+constexpr int kSetupWarps = 8;
+
+__global__ void __launch_bounds__(32 * kSetupWarps)
+    k_setup(LikeConst L, const double* __restrict__ theta, int n, EvalRecord* __restrict__ rec) {
+  __shared__ double s_th[SWIG_N_PARAMS][33];
+  __shared__ double s_m[8][32];      // MassTerms, in EvalRecord::mterm's order
+  __shared__ double s_sc[8][32];     // sines and cosines of RA - GMST, Dec, 2 psi, phi_c
+  __shared__ double s_ci[32], s_amp[32], s_hh[SWIG_MAX_DET][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * 32, i = i0 + lane;
+  // a dependent kernel may start; it waits for this grid's end before it
+  // reads a record (griddepcontrol.wait)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int e = threadIdx.x; e < 32 * SWIG_N_PARAMS; e += blockDim.x) {
+    const int v = e / SWIG_N_PARAMS, j = e - v * SWIG_N_PARAMS;
+    double x = i0 + v < n ? theta[(size_t)i0 * SWIG_N_PARAMS + e] : 1.0;
+    if (j == 6 && L.dist_marg) x = 1.0;      // the marginal is built from the template at 1 Mpc
+    if (j == 11 && L.tm_n > 0) x = L.tm_tref;  // templates at the fiducial's t_c, shifted node by node
+    s_th[j][v] = x;
+  }
+  __syncthreads();
   double th[SWIG_N_PARAMS];
-  for (int j = 0; j < SWIG_N_PARAMS; ++j) th[j] = theta[(size_t)SWIG_N_PARAMS * i + j];
-  if (L.dist_marg) th[6] = 1.0;   // the marginal is built from the template at 1 Mpc
-  if (L.tm_n > 0) th[11] = L.tm_tref;  // templates at the fiducial's t_c, shifted node by node
-  setup_record(L, th, rec + i);
+#pragma unroll
+  for (int j = 0; j < SWIG_N_PARAMS; ++j) th[j] = s_th[j][lane];
+  const bool valid = theta_valid(th);
+  switch (warp) {
+    case 0:
+      if (valid) {
+        const MassTerms t = taylorf2_mass_terms(th[0], th[1]);
+        const double m[8] = {t.eta, t.dm, t.m1, t.m2, t.A, t.r, t.ir, t.lpm};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s_m[k][lane] = m[k];
+      }
+      break;
+    case 1: s_amp[lane] = valid ? amplitude_per_mpc(th[0]) / th[6] : 0.0; break;
+    case 2: sincos(th[9] - L.gmst, &s_sc[0][lane], &s_sc[1][lane]); break;
+    case 3: sincos(th[10], &s_sc[2][lane], &s_sc[3][lane]); break;
+    case 4: sincos(2.0 * th[8], &s_sc[4][lane], &s_sc[5][lane]); break;
+    case 5: s_ci[lane] = cos(th[7]); break;
+    case 6:
+      if (L.phase_marg)
+        s_sc[6][lane] = 0.0, s_sc[7][lane] = 1.0;
+      else
+        sincos(th[12], &s_sc[6][lane], &s_sc[7][lane]);
+      break;
+    default: break;
+  }
+  __syncthreads();
+  EvalRecord* r = rec + i;
+  if (warp < 4) {  // a share of the phase coefficients
+    if (i < n) {
+      double c[NBASIS];
+#pragma unroll
+      for (int j = 0; j < NBASIS; ++j) c[j] = 0.0;
+      MassTerms t;
+      t.eta = s_m[0][lane], t.dm = s_m[1][lane], t.m1 = s_m[2][lane], t.m2 = s_m[3][lane];
+      t.A = s_m[4][lane], t.r = s_m[5][lane], t.ir = s_m[6][lane], t.lpm = s_m[7][lane];
+      auto put = [&](int j) {
+        const double v = valid ? c[j] : 0.0;
+        const dfl d = df_from_double(v);
+        r->c[j] = v;
+        r->c_hi[j] = d.hi;
+        r->c_lo[j] = d.lo;
+      };
+      if (warp == 0) {
+        taylorf2_low_coeffs(t, c);
+        put(B_M53), put(B_M1), put(B_LOG), put(B_ONE);
+      } else if (warp == 1) {
+        taylorf2_high_coeffs(t, c);
+        put(B_P13), put(B_P13LOG), put(B_P23);
+      } else if (warp == 2) {
+        taylorf2_spin_coeffs(t, th[2], th[3], c);
+        put(B_M23), put(B_M13);
+      } else {
+        taylorf2_tidal_coeffs(t, th[4], th[5], c);
+        put(B_P53), put(B_P73);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (valid) r->mterm[k] = s_m[k][lane];
+      }
+    }
+  } else {  // projection and time shift of one detector
+    const int d = warp - 4;
+    double pre = 0.0, pim = 0.0, gd = 0.0, tau = 0.0, term = 0.0;
+    const double amp = s_amp[lane];
+    if (d < L.n_det) {
+      const double sl = s_sc[0][lane], cl = s_sc[1][lane], sd = s_sc[2][lane], cd = s_sc[3][lane];
+      double fp, fx;
+      antenna_from_sc(L.dten[d], sl, cl, sd, cd, s_sc[4][lane], s_sc[5][lane], &fp, &fx);
+      const double ci = s_ci[lane], sph = s_sc[6][lane], cph = s_sc[7][lane];
+      const double re0 = fp * (0.5 * (1.0 + ci * ci)), im0 = -fx * ci;
+      pre = re0 * cph - im0 * sph;
+      pim = re0 * sph + im0 * cph;
+      gd = -(cd * (cl * L.vertex[d][0] + sl * L.vertex[d][1]) + sd * L.vertex[d][2]) * (1.0 / kCSI);
+      tau = th[11] + gd;
+      const double cre = amp * pre, cim = amp * pim;
+      term = (cre * cre + cim * cim) * L.K[d];
+    }
+    s_hh[d][lane] = term;
+    if (i < n) {
+      const dfl tv = df_from_double(tau);
+      r->pre[d] = pre;
+      r->pim[d] = pim;
+      r->cre[d] = amp * pre;
+      r->cim[d] = amp * pim;
+      r->gdel[d] = gd;
+      r->tau[d] = tau;
+      r->tau_hi[d] = tv.hi;
+      r->tau_lo[d] = tv.lo;
+    }
+  }
+  __syncthreads();
+  if (warp == 0 && i < n) {
+    double hh = 0.0;
+#pragma unroll
+    for (int d = 0; d < SWIG_MAX_DET; ++d) hh += s_hh[d][lane];
+    r->hh = hh;
+    r->amp = s_amp[lane];
+    r->valid = valid ? 1 : 0;
+  }
+}
+
+// k_setup of n vectors.
+static void launch_setup(const LikeConst& L, const double* theta, int n, EvalRecord* rec, cudaStream_t st) {
+  k_setup<<<(n + 31) / 32, 32 * kSetupWarps, 0, st>>>(L, theta, n, rec);
 }
 
 template <int NDET>
@@ -299,7 +422,7 @@ cudaError_t launch_het_tm(const LikeConst& L, const DeviceBuffers& B, int n, dou
 cudaError_t launch_loglike_het(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n, double* out,
                                cudaStream_t st, double* kappa_out, double* vv_out, float* ell) {
   if (n <= 0) return cudaSuccess;
-  k_setup<<<(n + 127) / 128, 128, 0, st>>>(L, theta, n, B.rec);
+  launch_setup(L, theta, n, B.rec, st);
   if (L.tm_n > 0) {
     switch (L.n_det) {
       case 1: return launch_het_tm<1>(L, B, n, out, st, kappa_out, vv_out, ell);
@@ -345,7 +468,7 @@ __global__ void k_waveform(LikeConst L, const EvalRecord* __restrict__ rec, doub
 
 cudaError_t launch_waveform(const LikeConst& L, const double* theta_dev, EvalRecord* rec_dev, double2* out,
                             cudaStream_t st) {
-  k_setup<<<1, 32, 0, st>>>(L, theta_dev, 1, rec_dev);
+  launch_setup(L, theta_dev, 1, rec_dev, st);
   dim3 grid((L.n_bins + 255) / 256, L.n_det);
   k_waveform<<<grid, 256, 0, st>>>(L, rec_dev, out);
   return cudaGetLastError();
@@ -367,14 +490,14 @@ __global__ void k_prior_transform(const PriorSlot* __restrict__ slots, int n_sam
 cudaError_t launch_loglike_mixed(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n,
                                  double* out, cudaStream_t st, double* kappa_out) {
   if (n <= 0) return cudaSuccess;
-  k_setup<<<(n + 127) / 128, 128, 0, st>>>(L, theta, n, B.rec);
+  launch_setup(L, theta, n, B.rec, st);
   return launch_fold(L, B, n, out, st, kappa_out);
 }
 
 cudaError_t launch_loglike_fp64(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n,
                                 double* out, cudaStream_t st, double* kappa_out) {
   if (n <= 0) return cudaSuccess;
-  k_setup<<<(n + 127) / 128, 128, 0, st>>>(L, theta, n, B.rec);
+  launch_setup(L, theta, n, B.rec, st);
   const int gy = (n + 7) / 8 < 64 ? (n + 7) / 8 : 64;
   dim3 grid(L.n_slices, gy);
   switch (L.n_det) {
