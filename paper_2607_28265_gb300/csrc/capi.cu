@@ -352,10 +352,10 @@ void fold_plan(const swig_ctx* c, int n_det, std::vector<FoldChunk>& chunks, std
     fits.push_back(best);
     k += ck.nbins;
   }
-  const size_t nc = chunks.size();
-  tab.assign(FR_ROWS * nc, 0.0f);
+  const size_t nc = chunks.size(), ld = fold_ld((int)nc);
+  tab.assign(FR_ROWS * ld, 0.0f);
   for (size_t q = 0; q < nc; ++q) {
-    auto put = [&](int row, double v) { tab[(size_t)row * nc + q] = (float)v; };
+    auto put = [&](int row, double v) { tab[(size_t)row * ld + q] = (float)v; };
     auto put2 = [&](int row, int row_lo, double v) {
       float a, b;
       split_df(v, &a, &b);
@@ -376,7 +376,7 @@ void fold_plan(const swig_ctx* c, int n_det, std::vector<FoldChunk>& chunks, std
     put2(FR_H_HI, FR_H_LO, h);
     put2(FR_SM_HI, FR_SM_LO, chunks[q].slope_h);
     put(FR_LIM, chunks[q].kind ? 1e30 : om_dev);
-    put(FR_KIND, chunks[q].kind);
+    std::memcpy(&tab[FR_KIND * ld + q], &chunks[q].kind, sizeof(int));
   }
 }
 
@@ -954,9 +954,11 @@ int ensure_scratch(swig_ctx* c, int n) {
   free_scratch(B);
   const int cap = std::max(n, 256);
   CUDA_TRY(c, cudaMalloc(&B.rec, sizeof(EvalRecord) * cap));
-  const size_t units = (size_t)c->L.n_slices * 4;  // up to 4 work units per (theta, slice)
-  CUDA_TRY(c, cudaMalloc(&B.partials32, sizeof(float) * kPartialStride * units * cap));
-  CUDA_TRY(c, cudaMalloc(&B.partials64, sizeof(double) * kPartialStride * units * cap));
+  // partial sums of the FP64 batch (4096 at a time) and of the dataflow
+  // sampler's request slots (at most 4096): up to 4 per (theta, slice)
+  const size_t units = (size_t)c->L.n_slices * 4 * std::min(cap, 4096);
+  CUDA_TRY(c, cudaMalloc(&B.partials32, sizeof(float) * kPartialStride * units));
+  CUDA_TRY(c, cudaMalloc(&B.partials64, sizeof(double) * kPartialStride * units));
   CUDA_TRY(c, cudaMalloc(&B.theta, sizeof(double) * SWIG_N_PARAMS * cap));
   CUDA_TRY(c, cudaMalloc(&B.out, sizeof(double) * cap));
   CUDA_TRY(c, cudaMalloc(&B.u, sizeof(double) * SWIG_N_PARAMS * cap));
@@ -1188,8 +1190,14 @@ int prepare(swig_ctx* c) {
   return SWIG_OK;
 }
 
+// Parameter vectors evaluated per launch: the mixed and heterodyned paths keep
+// a record each (0.6 KB), FP64 also a partial sum per slice.
+static int batch_chunk(const swig_ctx* c) {
+  return c->prepared_like == SWIG_LIKE_FULL && c->prepared_precision == SWIG_PREC_FP64 ? 4096 : 16384;
+}
+
 int loglike_device(swig_ctx* c, const double* theta_dev, int64_t n, double* out_dev, cudaStream_t st) {
-  const int chunk = 4096;
+  const int chunk = batch_chunk(c);
   for (int64_t off = 0; off < n; off += chunk) {
     const int m = (int)std::min<int64_t>(chunk, n - off);
     int rc = ensure_scratch(c, m);
@@ -1402,7 +1410,7 @@ int swig_loglike_batch(swig_ctx* c, const double* theta, int64_t n, double* out_
   if (n < 0 || n > (1 << 20) || !theta || !out_logl) return fail(c, SWIG_E_ARG, "need 0 <= n <= 2^20 and non-null buffers");
   int rc = prepare(c);
   if (rc) return rc;
-  const int chunk = 4096;
+  const int chunk = batch_chunk(c);
   for (int64_t off = 0; off < n; off += chunk) {
     const int m = (int)std::min<int64_t>(chunk, n - off);
     if ((rc = ensure_scratch(c, m))) return rc;

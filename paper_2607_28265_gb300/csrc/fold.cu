@@ -155,40 +155,109 @@ cudaError_t launch_fold_weights(const LikeConst& L, const DeviceBuffers& B, cons
 }
 
 // ---------------------------------------------------------------------------
-// Batched evaluation: a CTA of 16 warps per parameter vector (grid-stride).
+// Batched evaluation.  A team of T warps (T a power of two up to 16, a CTA
+// holds 16 / T teams) takes one parameter vector at a time: anchors of a panel
+// of chunks into shared memory, a warp per chunk over its nodes, the warps'
+// sums and the FP64 epilogue on the team's first warp.  An evaluation is a
+// chain of latencies (table loads, the double-float sums, the epilogue's FP64),
+// so a team waits more than it works: small batches take T = 16 for the
+// shortest chain, large ones one warp per vector and as many vectors in flight
+// as there are warps (32 per SM), without block barriers.
 // ---------------------------------------------------------------------------
-template <int NDET>
-__global__ void __launch_bounds__(32 * kFoldWarps, 2)
-    k_fold(LikeConst L, FoldTables F, const EvalRecord* __restrict__ rec, int n, double* __restrict__ out,
+constexpr int kFoldSlots = 512;  // anchors in shared memory, all teams together
+
+// Dynamic shared memory: anchors, abscissae and, RES, the weights and table.
+inline __host__ __device__ size_t fold_fixed_bytes() {
+  return sizeof(float) * kFoldSlots * kFoldAnchor + sizeof(float2) * 32 * kFoldKinds;
+}
+inline size_t fold_resident_bytes(int nc, int n_det) {
+  return (size_t)nc * n_det * 32 * sizeof(float4) + sizeof(float) * FR_ROWS * fold_ld(nc);
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__device__ __forceinline__ void team_sync(int team, int T) {
+  if (T == 1)
+    __syncwarp();
+  else
+    named_barrier(1 + team, 32 * T);
+}
+
+template <int NDET, bool RES>
+__global__ void __launch_bounds__(32 * kFoldWarps, 1)
+    k_fold(LikeConst L, FoldTables F, const EvalRecord* __restrict__ rec, int n, int T, double* __restrict__ out,
            double* __restrict__ kappa_out) {
-  __shared__ __align__(16) float s_an[kFoldPanel * kFoldAnchor];
-  __shared__ FoldIn s_in;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ FoldIn s_in[kFoldWarps];
   __shared__ float s_sum[2 * NDET][kFoldWarps];
   __shared__ double s_dir[2 * NDET][kFoldWarps];
-  __shared__ int s_bad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int th = blockIdx.x; th < n; th += gridDim.x) {
+  __shared__ int s_bad[kFoldWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / T, tw = warp - team * T, tid = 32 * tw + lane;  // within the team
+  const int teams = kFoldWarps / T, panel = min(128, kFoldSlots / teams);
+  float* s_anchor = reinterpret_cast<float*>(smem);
+  float2* s_x = reinterpret_cast<float2*>(s_anchor + kFoldSlots * kFoldAnchor);
+  const float4* w = F.w;
+  const float* tab = F.tab;
+  const int ld = F.ld;
+  if (RES) {
+    float4* s_w = reinterpret_cast<float4*>(s_x + 32 * kFoldKinds);
+    float4* s_t = s_w + F.nc * NDET * 32;
+    const float4* g_t = reinterpret_cast<const float4*>(F.tab);
+    for (int k = threadIdx.x; k < FR_ROWS * ld / 4; k += blockDim.x) cp_async16(s_t + k, g_t + k);
+    for (int k = threadIdx.x; k < F.nc * NDET * 32; k += blockDim.x) cp_async16(s_w + k, F.w + k);
+    w = s_w;
+    tab = reinterpret_cast<const float*>(s_t);
+  }
+  for (int k = threadIdx.x; k < 32 * kFoldKinds; k += blockDim.x) s_x[k] = F.x[k];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  // the set-up kernel's records, while this one's start overlapped its end
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  float* an = s_anchor + team * panel * kFoldAnchor;
+  const float2 x0 = s_x[lane];
+  for (int th = blockIdx.x * teams + team; th < n; th += gridDim.x * teams) {
     const EvalRecord& r = rec[th];
-    __syncthreads();  // the previous vector's shared memory has been read
-    if (tid < (int)(sizeof(FoldIn) / sizeof(float))) reinterpret_cast<float*>(&s_in)[tid] = fold_in_word(r, tid);
-    if (tid == 0) s_bad = 0;
-    const bool valid = r.valid != 0;  // block-uniform
-    __syncthreads();
+    team_sync(team, T);  // the previous vector's shared memory has been read
+    if (tid < (int)(sizeof(FoldIn) / sizeof(float)))
+      reinterpret_cast<float*>(&s_in[team])[tid] = fold_in_word(r, tid);
+    if (tid == 0) s_bad[team] = 0;
+    const bool valid = r.valid != 0;  // team-uniform
+    team_sync(team, T);
     FoldAcc<NDET> acc;
     acc.clear();
     if (valid)
-      for (int base = 0; base < F.nc; base += kFoldPanel) {
-        const int np = min(kFoldPanel, F.nc - base);
-        const int npw = (np + 31) & ~31;  // a warp's lanes share one quarter
-        for (int it = tid; it < 4 * npw; it += blockDim.x) {
-          const int sub = it / npw, q = it - sub * npw;
-          if (q < np && !fold_anchor<NDET>(F, s_in, sub, base + q, s_an + q * kFoldAnchor)) s_bad = 1;
+      for (int base = 0; base < F.nc; base += panel) {
+        const int np = min(panel, F.nc - base);
+        // two nodes' data in turn, one in flight while the other is summed
+        // (the first during the anchors)
+        FoldNode<NDET> v0, v1;
+        const float4* wq = w + (base + tw) * NDET * 32 + lane;
+        auto kind = [&](int q) { return __float_as_int(tab[FR_KIND * ld + base + q]); };
+        if (tw < np) fold_load<NDET>(wq, kind(tw), x0, s_x, lane, v0);
+        // quarter sub of 32 chunks per warp and turn
+        const int np32 = (np + 31) >> 5;
+        for (int it = tw, sub = 0, blk = tw; it < 4 * np32; it += T, blk += T) {
+          while (blk >= np32) blk -= np32, ++sub;
+          const int q = 32 * blk + lane;
+          if (q < np && !fold_anchor<NDET>(tab, ld, s_in[team], sub, base + q, an + q * kFoldAnchor)) s_bad[team] = 1;
         }
-        __syncthreads();
-        if (tid < np && !fold_in_band<NDET>(F, s_an + tid * kFoldAnchor, base + tid)) s_bad = 1;
-        for (int q = warp; q < np; q += kFoldWarps)
-          fold_chunk<NDET>(F, s_an + q * kFoldAnchor, base + q, lane, acc);
-        if (base + kFoldPanel < F.nc) __syncthreads();
+        team_sync(team, T);
+        for (int q = tid; q < np; q += 32 * T)
+          if (!fold_in_band<NDET>(tab, ld, an + q * kFoldAnchor, base + q)) s_bad[team] = 1;
+        const float* aq = an + tw * kFoldAnchor;
+        for (int q = tw; q < np; q += 2 * T, wq += 2 * T * NDET * 32, aq += 2 * T * kFoldAnchor) {
+          if (q + T < np) fold_load<NDET>(wq + T * NDET * 32, kind(q + T), x0, s_x, lane, v1);
+          fold_chunk<NDET>(aq, v0, acc);
+          if (q + T < np) {
+            if (q + 2 * T < np) fold_load<NDET>(wq + 2 * T * NDET * 32, kind(q + 2 * T), x0, s_x, lane, v0);
+            fold_chunk<NDET>(aq + T * kFoldAnchor, v1, acc);
+          }
+        }
+        team_sync(team, T);
       }
 #pragma unroll
     for (int i = 0; i < NDET; ++i) {
@@ -204,36 +273,29 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 2)
         s_sum[2 * i + 1][warp] = im;
       }
     }
-    __syncthreads();
-    const bool bad = valid && s_bad;  // block-uniform
+    team_sync(team, T);
+    const bool bad = valid && s_bad[team];  // team-uniform
     if (bad) {
       double v[2 * NDET];
-      fold_direct<NDET>(L, F, r, warp, kFoldWarps, lane, s_an + warp * kAnchorStride, v);
+      fold_direct<NDET>(L, F, r, tw, T, lane, an + tw * kAnchorStride, v);
       if (lane == 0)
 #pragma unroll
         for (int j = 0; j < 2 * NDET; ++j) s_dir[j][warp] = v[j];
-      __syncthreads();
+      team_sync(team, T);
     }
-    if (warp == 0) {
-      // the warps' sums in FP64 by a fixed tree, component j on lane j
+    if (tw == 0) {
+      // the warps' sums in warp order (double-float), component j on lane j
       double kapc = 0.0;
-#pragma unroll
-      for (int j = 0; j < 2 * NDET; ++j) {
-        double v;
+      if (lane < 2 * NDET) {
         if (bad) {
-          v = lane < kFoldWarps ? s_dir[j][lane] : 0.0;
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          for (int w = 0; w < T; ++w) kapc += s_dir[lane][warp + w];
         } else {
-          dfl t = {lane < kFoldWarps ? s_sum[j][lane] : 0.0f, 0.0f};
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1)
-            t = df_add(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
-          v = (double)t.hi + (double)t.lo;
+          dfl t = {0.0f, 0.0f};
+          for (int w = 0; w < T; ++w) t = df_add(t, dfl{s_sum[lane][warp + w], 0.0f});
+          kapc = (double)t.hi + (double)t.lo;
         }
-        v = __shfl_sync(0xffffffffu, v, 0);
-        if (lane == j) kapc = v;
       }
+      __syncwarp();
       const double ll = loglike_epilogue_warp<NDET>(L, r, kapc, lane);
       if (lane == 0) out[th] = ll;
       if (kappa_out && lane < 2 * SWIG_MAX_DET) kappa_out[(size_t)th * 2 * SWIG_MAX_DET + lane] = kapc;
@@ -243,12 +305,37 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 2)
 
 namespace {
 
+template <int NDET, bool RES>
+cudaError_t fold_launch_as(const LikeConst& L, const FoldTables& F, const EvalRecord* rec, int n, double* out,
+                           cudaStream_t st, double* kappa_out, size_t smem) {
+  cudaError_t e = cudaFuncSetAttribute(k_fold<NDET, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // the widest team that leaves no vector waiting for a second turn
+  const int ctas = L.sm_count;
+  int T = kFoldWarps;
+  while (T > 1 && (long long)n * T > (long long)ctas * kFoldWarps) T /= 2;
+  const int teams = kFoldWarps / T, need = (n + teams - 1) / teams;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(need < ctas ? need : ctas);
+  cfg.blockDim = dim3(32 * kFoldWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_fold<NDET, RES>, L, F, rec, n, T, out, kappa_out);
+}
+
 template <int NDET>
 cudaError_t fold_launch(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
                         double* kappa_out) {
-  const int grid = n < 2 * L.sm_count ? n : 2 * L.sm_count;
-  k_fold<NDET><<<grid, 32 * kFoldWarps, 0, st>>>(L, fold_tables(B), B.rec, n, out, kappa_out);
-  return cudaGetLastError();
+  const FoldTables F = fold_tables(B);
+  const size_t fixed = fold_fixed_bytes(), res = fixed + fold_resident_bytes(F.nc, NDET);
+  if (n > L.sm_count && res <= 220 * 1024)
+    return fold_launch_as<NDET, true>(L, F, B.rec, n, out, st, kappa_out, res);
+  return fold_launch_as<NDET, false>(L, F, B.rec, n, out, st, kappa_out, fixed);
 }
 
 }  // namespace

@@ -29,8 +29,7 @@
 
 namespace swig {
 
-constexpr int kFoldWarps = 16;     // warps of a CTA that evaluates one parameter vector
-constexpr int kFoldPanel = 128;    // chunks whose anchors are in shared memory at once
+constexpr int kFoldWarps = 16;     // warps of an evaluating CTA
 constexpr int kFoldAnchor = 16;    // floats per (evaluation, chunk) anchor
 
 // What an evaluation reads of its record: coefficients and time shifts in
@@ -88,10 +87,10 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
 // anchor is the eleven-term double-float sums; four lanes of different warps
 // share it (a lane per chunk took 2.2x as long alone).
 template <int NDET>
-__device__ __forceinline__ bool fold_anchor(const FoldTables& F, const FoldIn& r, int sub, int q, float* out) {
-  const float* T = F.tab + q;
-  const int nc = F.nc;
-  auto row = [&](int k) { return __ldg(T + (size_t)k * nc); };
+__device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int ld, const FoldIn& r, int sub, int q,
+                                            float* out) {
+  const float* T = tab + q;
+  auto row = [&](int k) { return T[k * ld]; };
   if (sub == 0) {
     dfl A = {0.0f, 0.0f};
 #pragma unroll
@@ -134,7 +133,7 @@ __device__ __forceinline__ bool fold_anchor(const FoldTables& F, const FoldIn& r
 // (kernels.h FR_LIM): |slope| + sum_n n a^(n-1) |a_n| in cycles, a the half
 // axis of the Bernstein ellipse of the interpolation bound.
 template <int NDET>
-__device__ __forceinline__ bool fold_in_band(const FoldTables& F, const float* an, int q) {
+__device__ __forceinline__ bool fold_in_band(const float* __restrict__ tab, int ld, const float* an, int q) {
   float b = 0.0f;
 #pragma unroll
   for (int i = 1; i < NDET; ++i) b = fmaxf(b, fabsf(an[5 + i]));
@@ -144,41 +143,52 @@ __device__ __forceinline__ bool fold_in_band(const FoldTables& F, const float* a
     g *= kFoldEllipse;
     om = fmaf((float)n * g, fabsf(an[7 + n]), om);
   }
-  return om <= __ldg(F.tab + (size_t)FR_LIM * F.nc + q);  // false for a NaN as well
+  return om <= tab[FR_LIM * ld + q];  // false for a NaN as well
 }
 
-// Accumulators of a lane: per detector the four real products of the complex
-// multiply-add, for the nodes +x and -x in the two halves of a pair.
+// Accumulators of a lane: per detector the real and imaginary sums, for the
+// nodes +x and -x in the two halves of a pair.
 template <int NDET>
 struct FoldAcc {
-  f2 rr[NDET], ri[NDET], ir[NDET], ii[NDET];
+  f2 re[NDET], im[NDET];
   __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int i = 0; i < NDET; ++i) rr[i] = ri[i] = ir[i] = ii[i] = 0ull;
+    for (int i = 0; i < NDET; ++i) re[i] = im[i] = 0ull;
   }
-  __device__ __forceinline__ void total(int i, float& re, float& im) const {
-    float a, b, c, d, e, f, g, h;
-    f2_split(rr[i], a, b);
-    f2_split(ri[i], c, d);
-    f2_split(ir[i], e, f);
-    f2_split(ii[i], g, h);
-    re = (a + b) + (c + d);
-    im = (e + f) - (g + h);
+  __device__ __forceinline__ void total(int i, float& r, float& m) const {
+    float a, b, c, d;
+    f2_split(re[i], a, b);
+    f2_split(im[i], c, d);
+    r = a + b;
+    m = c + d;
   }
 };
 
-// Chunk q of one evaluation by one warp, two nodes (+x, -x) per lane.  The
+// The lane's node weights and abscissa of a chunk.
+template <int NDET>
+struct FoldNode {
+  float4 w[NDET];
+  float2 x;
+};
+// w: the chunk's weights at this lane; kind: its node kind, x0 the lane's
+// Chebyshev abscissa and x the table of all kinds.
+template <int NDET>
+__device__ __forceinline__ void fold_load(const float4* __restrict__ w, int kind, float2 x0,
+                                          const float2* __restrict__ x, int lane, FoldNode<NDET>& v) {
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) v.w[i] = w[32 * i];
+  v.x = x0;
+  if (kind) v.x = x[32 * kind + lane];  // warp-uniform
+}
+
+// One chunk of one evaluation by one warp, two nodes (+x, -x) per lane.  The
 // phase is E(x) + O(x), even and odd Taylor parts: at the two nodes E + O and
 // E - O, so the polynomial is formed once for both; the slope's product with x
 // is carried in double-float and reduced to its fractional part.
 template <int NDET>
-__device__ __forceinline__ void fold_chunk(const FoldTables& F, const float* __restrict__ an, int q, int lane,
+__device__ __forceinline__ void fold_chunk(const float* __restrict__ an, const FoldNode<NDET>& v,
                                            FoldAcc<NDET>& acc) {
-  const float4* W = F.w + (size_t)q * NDET * 32 + lane;
-  float4 w[NDET];
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) w[i] = __ldg(W + 32 * i);
-  const float2 xv = __ldg(F.x + 32 * (int)__ldg(F.tab + (size_t)FR_KIND * F.nc + q) + lane);
+  const float2 xv = v.x;
   const float4 A = *reinterpret_cast<const float4*>(an), B = *reinterpret_cast<const float4*>(an + 4);
   const float4 C = *reinterpret_cast<const float4*>(an + 8), D = *reinterpret_cast<const float4*>(an + 12);
   const float x = xv.x, x2 = x * x;
@@ -204,11 +214,9 @@ __device__ __forceinline__ void fold_chunk(const FoldTables& F, const float* __r
     __sincosf(pa, &sa, &ca);
     __sincosf(pb, &sb, &cb);
     const f2 c2 = f2_make(ca, cb), s2 = f2_make(sa, sb);
-    const f2 wr = f2_make(w[i].x, w[i].y), wi = f2_make(w[i].z, w[i].w);
-    acc.rr[i] = f2_fma(wr, c2, acc.rr[i]);
-    acc.ri[i] = f2_fma(wi, s2, acc.ri[i]);
-    acc.ir[i] = f2_fma(wi, c2, acc.ir[i]);
-    acc.ii[i] = f2_fma(wr, s2, acc.ii[i]);
+    const f2 wr = f2_make(v.w[i].x, v.w[i].y), wi = f2_make(v.w[i].z, v.w[i].w);
+    acc.re[i] = f2_fma(wr, c2, f2_fma(wi, s2, acc.re[i]));
+    acc.im[i] = f2_fma(wi, c2, f2_fma(f2_mul(wr, none), s2, acc.im[i]));
   }
 }
 

@@ -88,13 +88,13 @@ static_assert(kHetAncExact < kHetAncStride, "chunk anchor layout");
 inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) + 2 * 32 * 4; }
 
 // Folded full-grid sums (fold.cuh): the grid in chunks of kFoldNodes nodes.
-// Rows of the [FR_ROWS][chunks] table: at the chunk's centre f_c, with h the
+// Rows of the [FR_ROWS][ld] table (a column per chunk): at the chunk's centre f_c, with h the
 // half width [Hz] that scales the node abscissae to |x| <= 1, the basis values
 // and first derivatives times h (double-float; the constant basis function,
 // last, has no derivatives), derivatives of orders 2..kFoldDeg times h^n / n!
 // (float), the order-9 remainder bound max |phi_j^(9)| h^9 / 9!, f_c, h and the
 // reference slope times h (double-float), the bandwidth the weights serve
-// [cycles] and the node kind.
+// [cycles] and the node kind (an int's bits).
 constexpr int kFoldNodes = 64;
 constexpr int kFoldDeg = 8;
 constexpr int kFoldSlopes = NBASIS - 1;
@@ -139,9 +139,10 @@ struct FoldChunk {
 
 struct FoldTables {
   int nc;             // chunks
-  const float* tab;   // [FR_ROWS][nc]
+  int ld;             // row length of tab: nc rounded up to 4
+  const float* tab;   // [FR_ROWS][ld]
   const float4* w;    // [nc][n_det][32] node weights (+x re, -x re, +x im, -x im)
-  const float2* x;    // [kFoldKinds][32] abscissae (hi, lo)
+  const float2* x;    // [kFoldKinds][32] the lanes' node abscissae (hi, lo)
   // bin by bin (fold_direct)
   const float2* data;
   const TileInfo* tiles;
@@ -196,8 +197,9 @@ struct DeviceBuffers {
   double* u = nullptr;           // [cap][13]
 };
 
+inline __host__ __device__ int fold_ld(int nc) { return (nc + 3) & ~3; }
 inline __host__ __device__ FoldTables fold_tables(const DeviceBuffers& B) {
-  return {B.fold_nc, B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile};
+  return {B.fold_nc, fold_ld(B.fold_nc), B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile};
 }
 
 // Node weights of the event (B.fold_w) from its weighted data (B.data32) and

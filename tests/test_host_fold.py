@@ -17,7 +17,7 @@ D1 = 2 * NB
 POLY = D1 + 2 * SLOPES
 BND = POLY + (DEG - 1) * SLOPES
 FC = BND + SLOPES
-H, SM, LIM, KIND, ROWS = FC + 2, FC + 4, FC + 6, FC + 7, FC + 8
+H, SM, LIM, ROWS = FC + 2, FC + 4, FC + 6, FC + 8
 BNS = [(1.5, 2.5), (0.5, 1.0), (-0.05, 0.05), (-0.05, 0.05), (0.0, 5000.0), (0.0, 5000.0)]
 H1_4S = [(1.1, 1.3), (0.5, 1.0), (0.0, 0.0), (0.0, 0.0), (0.0, 0.0), (0.0, 0.0)]
 WIDE = [(0.87, 3.0), (0.125, 1.0), (-0.1, 0.1), (-0.1, 0.1), (0.0, 5000.0), (0.0, 5000.0)]
