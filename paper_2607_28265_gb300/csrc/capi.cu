@@ -425,6 +425,7 @@ void free_problem(DeviceBuffers& B) {
   dfree(B.het_coef);
   dfree(B.het_coefB);
   dfree(B.het_fid);
+  dfree(B.het_ew);
   dfree(B.het_tm_g);
   dfree(B.het_tm_w);
   dfree(B.het_nu_wt);
@@ -717,6 +718,29 @@ std::vector<float2> nufft_stage_twiddles(const std::vector<float2>& tw, int M) {
   return tws;
 }
 
+// Edge weights of the heterodyned contraction by chunks of 32 edges (31 bins):
+// per chunk, detector and lane l (edge 31 q + l, bin 31 q + l) the edge's hat
+// weight g_ie (every edge in one chunk: lane 31 only at the grid's last edge),
+// half the bin's B0 and, with detector 0, f_e - f_a; zeros past the end.
+std::vector<float4> het_edge_weights(const std::vector<float2>& g, const std::vector<float2>& coefB,
+                                     const std::vector<float>& dfe, int nb, int nc, int n_det) {
+  std::vector<float4> ew((size_t)nc * n_det * 32, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+  for (int q = 0; q < nc; ++q)
+    for (int i = 0; i < n_det; ++i)
+      for (int l = 0; l < 32; ++l) {
+        const int e = 31 * q + l;
+        if (e > nb) continue;
+        float4& w = ew[((size_t)q * n_det + i) * 32 + l];
+        if (l < 31 || e == nb) {
+          w.x = g[(size_t)i * (nb + 1) + e].x;
+          w.y = g[(size_t)i * (nb + 1) + e].y;
+        }
+        if (l < 31 && e < nb) w.z = 0.5f * coefB[(size_t)i * nb + e].x;
+        if (i == 0) w.w = dfe[(size_t)q * kHetChunkEdges + l];
+      }
+  return ew;
+}
+
 // Gather pieces of the time pass's non-uniform FFT: each grid point's
 // entries (ptr[l] .. ptr[l + 1], consecutive edges from edge[l]) in runs of
 // at most kNufftPiece, piece = (first entry, entries, first edge, 0), and the
@@ -859,8 +883,8 @@ int prepare_het(swig_ctx* c) {
   CUDA_TRY(c, cudaMemcpy(B.het_coefB, coefB.data(), sizeof(float2) * coefB.size(), cudaMemcpyHostToDevice));
   c->h2d_bytes += sizeof(float) * (eb.size() + ef.size() + inv_w.size()) + sizeof(float4) * coef.size() +
                   sizeof(float2) * coefB.size();
+  std::vector<float2> g, w;
   if (L.tm_n > 0) {
-    std::vector<float2> g, w;
     L.tm_M = 0;
     L.tm_pieces = L.tm_points = 0;
     std::vector<int> ptr, edge;
@@ -905,6 +929,17 @@ int prepare_het(swig_ctx* c) {
     CUDA_TRY(c, cudaMemcpy(B.het_tm_g, g.data(), sizeof(float2) * g.size(), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMemcpy(B.het_tm_w, w.data(), sizeof(float2) * w.size(), cudaMemcpyHostToDevice));
     c->h2d_bytes += sizeof(float2) * (g.size() + w.size());
+  } else {
+    het_tm_tables(a01, f, idx, nb, n_det, 0.0, g, w);
+  }
+  const std::vector<float4> ew = het_edge_weights(g, coefB, dfe, nb, nc, n_det);
+  CUDA_TRY(c, cudaMalloc(&B.het_ew, sizeof(float4) * ew.size()));
+  CUDA_TRY(c, cudaMemcpy(B.het_ew, ew.data(), sizeof(float4) * ew.size(), cudaMemcpyHostToDevice));
+  c->h2d_bytes += sizeof(float4) * ew.size();
+  for (int i = 0; i < n_det; ++i) {
+    NSum b0;
+    for (int b = 0; b < nb; ++b) b0.add((double)coefB[(size_t)i * nb + b].x);
+    L.het_b0[i] = b0.value();
   }
   B.het_nb = nb;
   return SWIG_OK;

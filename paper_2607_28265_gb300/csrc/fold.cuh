@@ -25,6 +25,7 @@
 // (one far from the prior box) is summed bin by bin instead (fold_direct).
 #pragma once
 
+#include "packed.cuh"
 #include "sweep.cuh"
 
 namespace swig {
@@ -46,33 +47,6 @@ static_assert(offsetof(EvalRecord, c_lo) == offsetof(EvalRecord, c_hi) + sizeof(
 __device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
   return w < 2 * NBASIS ? reinterpret_cast<const float*>(&r.c_hi)[w]
                         : reinterpret_cast<const float*>(&r.tau_hi)[w - 2 * NBASIS];
-}
-
-// Two FP32 operations per instruction (the packed forms of the Blackwell FP32
-// pipe); a pair is held in one 64-bit register.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 f2_make(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_split(f2 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-  f2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-  f2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-  f2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 
 // One quarter (sub 0 .. 3) of the anchor of chunk q for the evaluation `r`,

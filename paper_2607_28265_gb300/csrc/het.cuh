@@ -24,6 +24,7 @@
 #pragma once
 
 #include "device_common.cuh"
+#include "packed.cuh"
 
 namespace swig {
 
@@ -47,6 +48,9 @@ struct HetTables {
   int n_chunks;
   const float* chunk;  // [HC_ROWS][n_chunks]
   const float* dfe;    // [n_chunks][32]
+  // edge weights of the contraction (het_edge_weights in capi.cu): per chunk,
+  // detector and lane (Re g_ie, Im g_ie, B0_ib / 2, f_e - f_a with detector 0)
+  const float4* ew;    // [n_chunks][n_det][32]
 };
 
 __host__ __device__ inline HetTables het_tables(const DeviceBuffers& B) {
@@ -68,6 +72,7 @@ __host__ __device__ inline HetTables het_tables(const DeviceBuffers& B) {
   H.n_chunks = B.het_nc;
   H.chunk = B.het_chunk;
   H.dfe = B.het_dfe;
+  H.ew = B.het_ew;
   return H;
 }
 
@@ -92,6 +97,22 @@ __device__ inline void het_prepare(const LikeConst& L, const HetTables& H, const
     p.rho_re[i] = (float)((r.cre[i] * f0.cre[i] + r.cim[i] * f0.cim[i]) * iden);
     p.rho_im[i] = (float)((r.cim[i] * f0.cre[i] - r.cre[i] * f0.cim[i]) * iden);
   }
+}
+
+// het_prepare by a warp, one constant per lane.
+template <int NDET>
+__device__ __forceinline__ void het_prepare_warp(const LikeConst& L, const HetTables& H, const EvalRecord& r,
+                                                 HetPrep<NDET>& p, int lane) {
+  const EvalRecord& f0 = *H.fid;
+  if (lane < NBASIS) p.dc[lane] = df_from_double(r.c[lane] - f0.c[lane]);
+  if (lane >= 16 && lane < 16 + NDET) {
+    const int i = lane - 16;
+    p.dtau[i] = df_from_double(r.tau[i] - f0.tau[i]);
+    const double iden = L.het_fid_iden[i];
+    p.rho_re[i] = (float)((r.cre[i] * f0.cre[i] + r.cim[i] * f0.cim[i]) * iden);
+    p.rho_im[i] = (float)((r.cim[i] * f0.cre[i] - r.cre[i] * f0.cim[i]) * iden);
+  }
+  __syncwarp();
 }
 
 // Anchor of chunk q for one evaluation (one thread per chunk; rows of the
@@ -357,6 +378,298 @@ __device__ inline void het_chunks_warp(const HetTables& H, const HetPrep<NDET>& 
     }
   }
   cp_async_wait<0>();
+}
+
+// ---------------------------------------------------------------------------
+// Contraction by edges.  r_i(e) = rho_i u_i(e) with |u| = 1, so with the hat
+// weights g_ie of the header
+//   Z_i = rho_i sum_e g_ie u_i(e),
+//   <h|h>_i = |rho_i|^2 sum_b B0_ib (1 + Re u_i(e_b) u_i*(e_b+1)) / 2
+// (|r| is the same at both ends of a bin, so the B1 term vanishes): one phasor,
+// one complex multiply-add and one term of the bin's phase difference per edge
+// and detector, on 16 bytes of weights instead of 24 of summary data.  A warp
+// takes a chunk of 32 edges for N evaluations at once (N = 2: packed FP32, the
+// weights loaded once for all).
+// ---------------------------------------------------------------------------
+template <int NDET, int N>
+struct HetAcc {
+  using O = PkOps<N>;
+  typename O::T zr[NDET], zi[NDET], hh[NDET];  // sum g u; sum (B0 / 2) (1 - Re u u*')
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) zr[i] = zi[i] = hh[i] = O::all(0.0f);
+  }
+};
+
+// Phase differences of one edge from the double-float sum over the basis
+// (chunks whose Taylor form does not serve the evaluation).
+template <int NDET>
+__device__ __noinline__ void het_exact_phase(const HetTables& H, const HetPrep<NDET>& p, int e, float* out) {
+  const size_t ne = (size_t)H.n_bins + 1;
+  dfl dp = {0.0f, 0.0f};
+  for (int j = 0; j < NBASIS; ++j)
+    dp = df_add(dp, df_mul(p.dc[j], dfl{__ldg(H.edge_basis + 2 * j * ne + e),
+                                        __ldg(H.edge_basis + (2 * j + 1) * ne + e)}));
+  const dfl fe = {__ldg(H.edge_f + e), __ldg(H.edge_f + ne + e)};
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) out[i] = df_frac(df_add(dp, df_mul(fe, p.dtau[i])));
+}
+
+// What the anchors of N evaluations read (interleaved, evaluation k at [..][k]):
+// coefficient differences in double-float and their magnitudes, and the delay
+// differences.
+template <int NDET, int N>
+struct __align__(8) HetIn {
+  float dc_hi[NBASIS][N], dc_lo[NBASIS][N], dc_abs[NBASIS][N];
+  float dt_hi[NDET][N], dt_lo[NDET][N];
+};
+// Evaluation k's share, one value per lane (after het_prepare_warp).
+template <int NDET, int N>
+__device__ __forceinline__ void het_in_set(HetIn<NDET, N>& in, int k, const HetPrep<NDET>& p, int lane) {
+  if (lane < NBASIS) {
+    in.dc_hi[lane][k] = p.dc[lane].hi;
+    in.dc_lo[lane][k] = p.dc[lane].lo;
+    in.dc_abs[lane][k] = fabsf(p.dc[lane].hi);
+  }
+  if (lane < NDET) {
+    in.dt_hi[lane][k] = p.dtau[lane].hi;
+    in.dt_lo[lane][k] = p.dtau[lane].lo;
+  }
+}
+
+// One quarter (sub 0 .. 3) of the anchors of chunk q for N evaluations, value m
+// of evaluation k to out[N m + k]: sub 0 the phases frac(dP(f_a) + f_a dtau_i),
+// sub 1 a_1, 1 / S and the exact flag, sub 2 and 3 the Taylor terms (het_anchor
+// has them all for one evaluation on one thread).
+template <int NDET, int N>
+__device__ __forceinline__ void het_anchor_part(const HetTables& H, const HetIn<NDET, N>& in, int sub, int q,
+                                                float* out) {
+  using O = PkOps<N>;
+  using T = typename O::T;
+  const int nc = H.n_chunks;
+  const float* tab = H.chunk + q;
+  auto row = [&](int r) { return O::all(__ldg(tab + r * nc)); };
+  auto put = [&](int m, T v) { *reinterpret_cast<T*>(out + N * m) = v; };
+  auto dc = [&](int j) { return DflN<N>{O::load(in.dc_hi[j]), O::load(in.dc_lo[j])}; };
+  if (sub == 0) {
+    DflN<N> A = {O::all(0.0f), O::all(0.0f)};
+#pragma unroll
+    for (int j = 0; j < NBASIS; ++j)
+      A = dfn_add<N>(A, dfn_mul<N>(dc(j), DflN<N>{row(HC_VAL_HI + j), row(HC_VAL_LO + j)}));
+    const DflN<N> fa = {row(HC_FA_HI), row(HC_FA_LO)};
+#pragma unroll
+    for (int i = 0; i < NDET; ++i)
+      put(kHetAncPhase + i,
+          dfn_frac<N>(dfn_add<N>(A, dfn_mul<N>(fa, DflN<N>{O::load(in.dt_hi[i]), O::load(in.dt_lo[i])}))));
+  } else if (sub == 1) {
+    DflN<N> S = {O::all(0.0f), O::all(0.0f)};
+    T R = O::all(0.0f);
+#pragma unroll
+    for (int j = 0; j < NBASIS; ++j) {
+      S = dfn_add<N>(S, dfn_mul<N>(dc(j), DflN<N>{row(HC_D1_HI + j), row(HC_D1_LO + j)}));
+      R = O::fma(O::load(in.dc_abs[j]), row(HC_BND + j), R);
+    }
+    put(0, O::add(S.hi, S.lo));
+    put(kHetAncInvS, row(HC_INV_S));
+    float r[N];
+    O::get(R, r);
+#pragma unroll
+    for (int k = 0; k < N; ++k) out[N * kHetAncExact + k] = r[k] > kHetTaylorEps ? 1.0f : 0.0f;
+  } else {
+    constexpr int kHalf = (kHetPoly + 1) / 2;  // orders 2 .. kHalf + 1, and above
+    T a[kHalf];
+#pragma unroll
+    for (int m = 0; m < kHalf; ++m) a[m] = O::all(0.0f);
+    const int m0 = sub == 2 ? 0 : kHalf;
+#pragma unroll
+    for (int j = 0; j < NBASIS; ++j) {
+      const T c = O::load(in.dc_hi[j]);
+#pragma unroll
+      for (int m = 0; m < kHalf; ++m)
+        if (m0 + m < kHetPoly) a[m] = O::fma(c, row(HC_POLY + (m0 + m) * NBASIS + j), a[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < kHalf; ++m)
+      if (m0 + m < kHetPoly) put(1 + m0 + m, a[m]);
+  }
+}
+
+// Anchors of np chunks from q0 on for `sets` groups of N evaluations by the
+// warps first, first + stride, ... of a CTA: quarter by quarter, 32 chunks per
+// warp and turn.  Group g's anchors at s_an + (g panel + q) N kHetAncStride.
+template <int NDET, int N>
+__device__ __forceinline__ void het_anchors(const HetTables& H, const HetIn<NDET, N>* in, int sets, int q0, int np,
+                                            int panel, float* s_an, int first, int stride, int lane) {
+  const int nb = (np + 31) >> 5, per = sets * nb;  // warp turns of a quarter
+  for (int sub = 0, t = first; sub < 4;) {
+    if (t >= per) {
+      t -= per;
+      ++sub;
+      continue;
+    }
+    const int g = t / nb, q = 32 * (t - g * nb) + lane;
+    if (q < np)
+      het_anchor_part<NDET, N>(H, in[g], sub, q0 + q, s_an + (size_t)(g * panel + q) * N * kHetAncStride);
+    t += stride;
+  }
+}
+
+// Chunk q of N evaluations.  an: kHetAncStride values per evaluation, value m
+// of evaluation k at an[N m + k]; in: their inputs; p[k]: its constants (exact chunks only); w: the chunk's weights
+// at this lane.  TM: Z is not formed, y[e] = sum_i rho_i g_ie u_i(e) is stored.
+template <int NDET, int N, bool TM = false>
+__device__ __forceinline__ void het_edges(const HetTables& H, const float* __restrict__ an,
+                                          const HetIn<NDET, N>& in, const HetPrep<NDET>* const* p, int q, int lane,
+                                          const float4* w, HetAcc<NDET, N>& acc, float2* y = nullptr) {
+  using O = PkOps<N>;
+  using T = typename O::T;
+  const float d = w[0].w;
+  T ph[NDET];
+  bool exact = false;
+#pragma unroll
+  for (int k = 0; k < N; ++k) exact = exact || an[N * kHetAncExact + k] != 0.0f;
+  {
+    const T d2 = O::all(d), x = O::mul(d2, O::load(an + N * kHetAncInvS));
+    T v = O::load(an + N * kHetPoly);
+#pragma unroll
+    for (int n = kHetPoly - 1; n >= 0; --n) v = O::fma(v, x, O::load(an + N * n));
+    v = O::mul(v, x);
+#pragma unroll
+    for (int i = 0; i < NDET; ++i)
+      ph[i] = O::add(O::load(an + N * (kHetAncPhase + i)), O::fma(d2, O::load(in.dt_hi[i]), v));
+  }
+  if (exact) {  // warp-uniform, rare
+    float f[NDET][N];
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) O::get(ph[i], f[i]);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (an[N * kHetAncExact + k] != 0.0f) {
+        float g[NDET];
+        het_exact_phase<NDET>(H, *p[k], min(31 * q + lane, H.n_bins), g);
+#pragma unroll
+        for (int i = 0; i < NDET; ++i) f[i][k] = g[i];
+      }
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) ph[i] = O::set(f[i]);
+  }
+  float yr = 0.0f, yi = 0.0f;
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) {
+    const T m = O::all(12582912.0f), nm = O::all(-12582912.0f), mone = O::all(-1.0f);
+    const T r = O::mul(O::fma(O::add(O::add(ph[i], m), nm), mone, ph[i]), O::all(6.283185307179586f));
+    float a[N], c[N], s[N];
+    O::get(r, a);
+#pragma unroll
+    for (int k = 0; k < N; ++k) __sincosf(a[k], &s[k], &c[k]);  // u = c - i s
+    const T co = O::set(c), si = O::set(s);
+    float cn[N], sn[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      cn[k] = __shfl_down_sync(0xffffffffu, c[k], 1);
+      sn[k] = __shfl_down_sync(0xffffffffu, s[k], 1);
+    }
+    const T gr = O::all(w[i].x), gi = O::all(w[i].y);
+    if (TM) {
+      const float zr = w[i].x * c[0] + w[i].y * s[0], zi = w[i].y * c[0] - w[i].x * s[0];
+      yr += p[0]->rho_re[i] * zr - p[0]->rho_im[i] * zi;
+      yi += p[0]->rho_re[i] * zi + p[0]->rho_im[i] * zr;
+    } else {
+      acc.zr[i] = O::fma(gr, co, O::fma(gi, si, acc.zr[i]));
+      acc.zi[i] = O::fma(gi, co, O::fma(O::all(-w[i].x), si, acc.zi[i]));
+    }
+    // 1 - (c c' + s s'), zero-weighted where the lane has no bin
+    const T dd = O::fma(O::fma(si, O::set(sn), O::mul(co, O::set(cn))), mone, O::all(1.0f));
+    acc.hh[i] = O::fma(O::all(w[i].z), dd, acc.hh[i]);
+  }
+  if (TM) {
+    const int e = 31 * q + lane;
+    if (e <= H.n_bins && (lane < 31 || e == H.n_bins)) y[e] = make_float2(yr, yi);
+  }
+}
+
+// The results of one evaluation from its sums (T_i = sum g u, D_i = sum (B0 /
+// 2) (1 - Re u u*'), FP64): Z_i and <h|h>_i of detector i, and the cache of
+// projection-only evaluations, kap = (Z_i / C_i) / inv_scale_i and vv = <h|h>_i
+// / |C_i|^2 A1^2, in which rho_i drops out.
+__device__ __forceinline__ void het_detector(const LikeConst& L, const EvalRecord& fid, const EvalRecord& r, int i,
+                                             double tr, double ti, double dsum, double* Z, double* hh, double* kap2,
+                                             double* vv) {
+  const double c0r = fid.cre[i], c0i = fid.cim[i], iden = L.het_fid_iden[i];
+  // (T / C0): kap before the data scale
+  const double kr = (tr * c0r + ti * c0i) * iden, ki = (ti * c0r - tr * c0i) * iden;
+  const double cr = r.cre[i], ci = r.cim[i];
+  Z[0] = cr * kr - ci * ki;
+  Z[1] = cr * ki + ci * kr;
+  const double b = (L.het_b0[i] - dsum) * iden;
+  *hh = (cr * cr + ci * ci) * b;
+  kap2[0] = kr / L.inv_scale[i];
+  kap2[1] = ki / L.inv_scale[i];
+  *vv = b * (L.amp1 * L.amp1);
+}
+
+// The edge products y_e of one evaluation (time marginalisation) by a whole
+// CTA: anchors of a panel of chunks in s_an, then the chunks q = warp, warp +
+// n_warps, ... of every panel.  The caller's prep and in are visible after the
+// first barrier here; y after the caller's next one.
+template <int NDET>
+__device__ inline void het_products(const HetTables& H, const HetPrep<NDET>& prep, const HetIn<NDET, 1>& in,
+                                    float* s_an, int panel, int warp, int n_warps, int lane, HetAcc<NDET, 1>& acc,
+                                    float2* y) {
+  const HetPrep<NDET>* pp[1] = {&prep};
+  for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
+    const int np = min(panel, H.n_chunks - q0);
+    __syncthreads();
+    het_anchors<NDET, 1>(H, &in, 1, q0, np, panel, s_an, warp, n_warps, lane);
+    __syncthreads();
+    for (int q = warp; q < np; q += n_warps) {
+      float4 w[NDET];
+#pragma unroll
+      for (int i = 0; i < NDET; ++i) w[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
+      het_edges<NDET, 1, true>(H, s_an + q * kHetAncStride, in, pp, q0 + q, lane, w, acc, y);
+    }
+  }
+}
+
+// Vector k's sums over the warps in warp order (double-float, rounded once to
+// FP64): lane 3 i + kind (Re T, Im T, D) of detector i; part[warp][i][K kind +
+// vector].
+template <int NDET, int K>
+__device__ __forceinline__ double het_part_sum(const float (*part)[NDET][3 * K], int n_warps, int k, int lane) {
+  double v = 0.0;
+  if (lane < 3 * NDET) {
+    const int i = lane / 3, kind = lane - 3 * i;
+    dfl t = {0.0f, 0.0f};
+    for (int w = 0; w < n_warps; ++w) t = df_add(t, dfl{part[w][i][K * kind + k], 0.0f});
+    v = (double)t.hi + (double)t.lo;
+  }
+  __syncwarp();
+  return v;
+}
+
+// Network Z and <h|h> from those sums, one detector per lane, added in
+// detector order (every lane); kap: component j of the cache on lane j, vv:
+// detector i's on lane i.
+template <int NDET>
+__device__ __forceinline__ void het_network(const LikeConst& L, const EvalRecord& fid, const EvalRecord& r, double v,
+                                            int lane, double& Zr, double& Zi, double& HH, double& kap, double& vv) {
+  const unsigned full = 0xffffffffu;
+  const int d = lane < NDET ? lane : 0;
+  const double tr = __shfl_sync(full, v, 3 * d), ti = __shfl_sync(full, v, 3 * d + 1);
+  const double ds = __shfl_sync(full, v, 3 * d + 2);
+  double Z[2], hh, k2[2], vi;
+  het_detector(L, fid, r, d, tr, ti, ds, Z, &hh, k2, &vi);
+  Zr = Zi = HH = 0.0;
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) {
+    Zr += __shfl_sync(full, Z[0], i);
+    Zi += __shfl_sync(full, Z[1], i);
+    HH += __shfl_sync(full, hh, i);
+  }
+  const double k0 = __shfl_sync(full, k2[0], lane < 2 * NDET ? lane >> 1 : 0);
+  const double k1 = __shfl_sync(full, k2[1], lane < 2 * NDET ? lane >> 1 : 0);
+  kap = lane < 2 * NDET ? ((lane & 1) ? k1 : k0) : 0.0;
+  vv = lane < NDET ? vi : 0.0;
 }
 
 // Warp-sum of the lane sums (all lanes receive them).
@@ -684,44 +997,6 @@ __device__ inline void het_cache(const LikeConst& L, const EvalRecord& r, int i,
     kap2[0] = kap2[1] = 0.0;
     *vv = 0.0;
   }
-}
-
-// One warp evaluates the heterodyned logL of record r (all lanes return it);
-// optionally the per-detector cache of het_cache (lane 0 writes it).
-template <int NDET>
-__device__ inline double het_loglike_warp(const LikeConst& L, const HetTables& H, const EvalRecord& r, int lane,
-                                          double* kap_out = nullptr, double* vv_out = nullptr) {
-  if (!r.valid) {
-    if (lane == 0 && kap_out)
-      for (int j = 0; j < 2 * SWIG_MAX_DET; ++j) kap_out[j] = 0.0;
-    if (lane == 0 && vv_out)
-      for (int i = 0; i < SWIG_MAX_DET; ++i) vv_out[i] = 0.0;
-    return -INFINITY;
-  }
-  HetPrep<NDET> p;
-  het_prepare<NDET>(L, H, r, p);
-  float zr[NDET], zi[NDET], hh[NDET];
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) zr[i] = zi[i] = hh[i] = 0.0f;
-  const int nc = het_chunks(H.n_bins);
-  for (int q = 0; q < nc; ++q) het_chunk<NDET>(H, p, 31 * q, lane, zr, zi, hh);
-  het_warp_reduce<NDET>(zr, zi, hh);
-  double Z_re = 0.0, Z_im = 0.0, HH = 0.0;
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-    Z_re += (double)zr[i];
-    Z_im += (double)zi[i];
-    HH += (double)hh[i];
-  }
-  if (lane == 0 && kap_out && vv_out) {
-    for (int i = 0; i < SWIG_MAX_DET; ++i) {
-      kap_out[2 * i] = kap_out[2 * i + 1] = 0.0;
-      vv_out[i] = 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) het_cache(L, r, i, zr[i], zi[i], hh[i], kap_out + 2 * i, vv_out + i);
-  }
-  return het_epilogue(L, Z_re, Z_im, HH);
 }
 
 }  // namespace swig

@@ -177,6 +177,7 @@ struct DeviceBuffers {
   float* het_chunk = nullptr;       // [HC_ROWS][het_nc] chunk anchor tables
   float* het_dfe = nullptr;         // [het_nc][32] f_e - f_a of each chunk's edges
   EvalRecord* het_fid = nullptr;    // fiducial record
+  float4* het_ew = nullptr;         // [het_nc][n_det][32] edge weights (HetTables::ew)
   // time marginalisation on the heterodyned bins (t_c marginalised)
   float2* het_tm_g = nullptr;       // [n_det][N_b + 1] edge weights: Z_i = sum_e g_ie r_i(e)
   float2* het_tm_w = nullptr;       // [N_b + 1] exp(-2 pi i f_e dt), the step between grid nodes
@@ -196,6 +197,28 @@ struct DeviceBuffers {
   double* out = nullptr;         // [cap]
   double* u = nullptr;           // [cap][13]
 };
+
+// Shared memory of a time-marginalised evaluation: het_tm_smem_bytes with the
+// anchors of a panel of chunks over the time pass's grid, or appended where the
+// grid is smaller.
+struct HetTmLayout {
+  size_t bytes;
+  int anc_off, panel;
+};
+inline HetTmLayout het_tm_layout(const LikeConst& L, const DeviceBuffers& B) {
+  HetTmLayout lay;
+  lay.panel = B.het_nc < 128 ? B.het_nc : 128;
+  const size_t anc = (size_t)lay.panel * kHetAncStride * sizeof(float);
+  const size_t ys = (((size_t)B.het_nb + 1) * 2 * sizeof(float) + 15) / 16 * 16;
+  lay.bytes = (het_tm_smem_bytes(B.het_nb, L.tm_M, L.tm_M > 0 ? L.tm_pieces : 0) + 15) / 16 * 16;
+  if ((size_t)L.tm_M * 2 * sizeof(float) >= anc) {
+    lay.anc_off = (int)ys;
+  } else {
+    lay.anc_off = (int)lay.bytes;
+    lay.bytes += anc;
+  }
+  return lay;
+}
 
 inline __host__ __device__ int fold_ld(int nc) { return (nc + 3) & ~3; }
 inline __host__ __device__ FoldTables fold_tables(const DeviceBuffers& B) {

@@ -330,33 +330,104 @@ cudaError_t launch_distance_draw(const LikeConst& L, const DeviceBuffers& B, con
 }
 
 // ---------------------------------------------------------------------------
-// Heterodyned likelihood, one warp per theta.
+// Heterodyned likelihood: up to eight parameter vectors per CTA, so that a
+// chunk's weights are read once for all of them and two share each packed FP32
+// instruction.  Anchors of a panel of chunks (a thread per pair, chunk and
+// quarter), then a warp per chunk over the vectors' pairs; the warps' sums and the FP64
+// epilogue a warp per vector.  (A warp per vector walking all chunks with an
+// eleven-term double-float sum per edge took 266 us for 1000 vectors on 5000
+// bins, 15 % of the issue slots.)
 // ---------------------------------------------------------------------------
+constexpr int kHetBatch = 8;
+constexpr int kHetWarps = kHetTmThreads / 32;
+constexpr int kHetPanel = 256;  // chunks anchored at once
+
 template <int NDET>
-__global__ void k_het(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, double* __restrict__ out,
-                      double* __restrict__ kappa_out, double* __restrict__ vv_out) {
-  const int th = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (th >= n) return;
-  const double v = het_loglike_warp<NDET>(L, H, rec[th], lane,
-                                          kappa_out ? kappa_out + (size_t)th * 2 * SWIG_MAX_DET : nullptr,
-                                          vv_out ? vv_out + (size_t)th * SWIG_MAX_DET : nullptr);
-  if (lane == 0) out[th] = v;
+__global__ void __launch_bounds__(kHetTmThreads, 1)
+    k_het(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, int per, double* __restrict__ out,
+          double* __restrict__ kappa_out, double* __restrict__ vv_out) {
+  extern __shared__ __align__(16) float s_an[];  // [pairs][kHetPanel][kHetAncStride][2]
+  __shared__ HetPrep<NDET> s_prep[kHetBatch];
+  __shared__ HetIn<NDET, 2> s_in[kHetBatch / 2];
+  __shared__ float s_part[kHetWarps][NDET][3 * kHetBatch];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int panel = min(kHetPanel, H.n_chunks);
+  for (int base = blockIdx.x * per; base < n; base += gridDim.x * per) {
+    const int m = min(per, n - base), pairs = (m + 1) / 2;
+    __syncthreads();
+    if (warp < 2 * pairs) {  // (an odd batch's last pair holds its vector twice)
+      het_prepare_warp<NDET>(L, H, rec[base + min(warp, m - 1)], s_prep[warp], lane);
+      het_in_set<NDET, 2>(s_in[warp >> 1], warp & 1, s_prep[warp], lane);
+    }
+    HetAcc<NDET, 2> acc[kHetBatch / 2];
+#pragma unroll
+    for (int p = 0; p < kHetBatch / 2; ++p) acc[p].clear();
+    for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
+      const int np = min(panel, H.n_chunks - q0);
+      __syncthreads();
+      het_anchors<NDET, 2>(H, s_in, pairs, q0, np, panel, s_an, warp, kHetWarps, lane);
+      __syncthreads();
+      for (int q = warp; q < np; q += kHetWarps) {
+        float4 w[NDET];
+#pragma unroll
+        for (int i = 0; i < NDET; ++i) w[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
+        if (q + kHetWarps < np && lane < 4 * NDET)  // the next chunk's lines
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(H.ew + ((size_t)(q0 + q + kHetWarps) * NDET) * 32 + 8 * lane));
+#pragma unroll
+        for (int p = 0; p < kHetBatch / 2; ++p)
+          if (p < pairs) {
+            const HetPrep<NDET>* pp[2] = {&s_prep[2 * p], &s_prep[2 * p + 1]};
+            het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * 2 * kHetAncStride, s_in[p], pp, q0 + q, lane, w,
+                               acc[p]);
+          }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) {
+      float a[32];  // value 8 kind + vector
+#pragma unroll
+      for (int p = 0; p < kHetBatch / 2; ++p) {
+        PkOps<2>::get(acc[p].zr[i], a + 2 * p);
+        PkOps<2>::get(acc[p].zi[i], a + kHetBatch + 2 * p);
+        PkOps<2>::get(acc[p].hh[i], a + 2 * kHetBatch + 2 * p);
+        a[3 * kHetBatch + 2 * p] = a[3 * kHetBatch + 2 * p + 1] = 0.0f;
+      }
+      const float v = warp_transpose_sum(a, lane);
+      if (lane < 3 * kHetBatch) s_part[warp][i][lane] = v;
+    }
+    __syncthreads();
+    if (warp < m) {
+      const EvalRecord& r = rec[base + warp];
+      const double v = het_part_sum<NDET, kHetBatch>(s_part, kHetWarps, warp, lane);
+      double Zr, Zi, HH, kap = 0.0, vv = 0.0;
+      het_network<NDET>(L, *H.fid, r, v, lane, Zr, Zi, HH, kap, vv);
+      const size_t th = base + warp;
+      const bool valid = r.valid != 0;
+      if (lane == 0) out[th] = valid ? het_epilogue(L, Zr, Zi, HH) : -INFINITY;
+      if (kappa_out && lane < 2 * SWIG_MAX_DET) kappa_out[th * 2 * SWIG_MAX_DET + lane] = valid ? kap : 0.0;
+      if (vv_out && lane < SWIG_MAX_DET) vv_out[th * SWIG_MAX_DET + lane] = valid ? vv : 0.0;
+    }
+  }
 }
 
 // Time-marginalised heterodyned likelihood, one CTA per theta (the thread
 // count and the chunk-to-warp assignment of the persistent sampler, so both
-// give the same sums): the warps contract the bins as above, storing the edge
+// give the same sums): the warps contract the chunks, storing the edge
 // products y_e in shared memory, then share the grid's 32-node chunks.
-// ell (optional) receives every node's log weight, [n][tm_n].
+// ell (optional) receives every node's log weight, [n][tm_n].  The anchors lie
+// where the time pass's grid follows (or after it, anc_off).
 template <int NDET>
 __global__ void __launch_bounds__(kHetTmThreads, 1)
-    k_het_tm(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, double* __restrict__ out,
-             double* __restrict__ kappa_out, double* __restrict__ vv_out, float* __restrict__ ell) {
+    k_het_tm(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, int anc_off, int panel,
+             double* __restrict__ out, double* __restrict__ kappa_out, double* __restrict__ vv_out,
+             float* __restrict__ ell) {
   extern __shared__ __align__(16) unsigned char smem[];
   float2* y = reinterpret_cast<float2*>(smem);
-  __shared__ float s_hh[kHetTmThreads / 32][NDET];
-  __shared__ float s_tm[kHetTmThreads / 32][2];
+  float* s_an = reinterpret_cast<float*>(smem + anc_off);
+  __shared__ HetPrep<NDET> s_prep;
+  __shared__ HetIn<NDET, 1> s_in;
+  __shared__ float s_hh[kHetWarps][NDET];
+  __shared__ float s_tm[kHetWarps][2];
   const int th = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   if (th >= n) return;
   const EvalRecord& r = rec[th];
@@ -374,18 +445,21 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
       for (int j = threadIdx.x; j < L.tm_n; j += blockDim.x) ell_th[j] = -INFINITY;
     return;
   }
-  HetPrep<NDET> p;
-  het_prepare<NDET>(L, H, r, p);
-  if (L.tm_M > 0) tm_load_twiddles(L, H, smem, H.n_bins);  // read after the __syncthreads below
-  float zr[NDET], zi[NDET], hh[NDET];
+  if (warp == 0) {
+    het_prepare_warp<NDET>(L, H, r, s_prep, lane);
+    het_in_set<NDET, 1>(s_in, 0, s_prep, lane);
+  }
+  if (L.tm_M > 0) tm_load_twiddles(L, H, smem, H.n_bins);  // read after the barriers below
+  HetAcc<NDET, 1> acc;
+  acc.clear();
+  het_products<NDET>(H, s_prep, s_in, s_an, panel, warp, n_warps, lane, acc, y);
 #pragma unroll
-  for (int i = 0; i < NDET; ++i) zr[i] = zi[i] = hh[i] = 0.0f;
-  const int nc = het_chunks(H.n_bins);
-  for (int q = warp; q < nc; q += n_warps) het_chunk<NDET, true>(H, p, 31 * q, lane, zr, zi, hh, y);
-  het_warp_reduce<NDET>(zr, zi, hh);
-  if (lane == 0)
+  for (int i = 0; i < NDET; ++i) {
+    float d = acc.hh[i];
 #pragma unroll
-    for (int i = 0; i < NDET; ++i) s_hh[warp][i] = hh[i];
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0) s_hh[warp][i] = d;
+  }
   __syncthreads();
   float wm, ws;
   if (L.tm_M > 0)
@@ -401,9 +475,9 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
   if (threadIdx.x == 0) {
     double HH = 0.0;
     for (int i = 0; i < NDET; ++i) {
-      double h = 0.0;
-      for (int w = 0; w < n_warps; ++w) h += (double)s_hh[w][i];
-      HH += h;
+      double d = 0.0;
+      for (int w = 0; w < n_warps; ++w) d += (double)s_hh[w][i];
+      HH += (r.cre[i] * r.cre[i] + r.cim[i] * r.cim[i]) * (L.het_b0[i] - d) * L.het_fid_iden[i];
     }
     out[th] = tm_finish(L, s_tm, n_warps, HH);
   }
@@ -412,10 +486,26 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
 template <int NDET>
 cudaError_t launch_het_tm(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
                           double* kappa_out, double* vv_out, float* ell) {
-  const size_t bytes = het_tm_smem_bytes(B.het_nb, L.tm_M, L.tm_M > 0 ? L.tm_pieces : 0);
-  cudaError_t e = cudaFuncSetAttribute(k_het_tm<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const HetTmLayout lay = het_tm_layout(L, B);
+  cudaError_t e = cudaFuncSetAttribute(k_het_tm<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes);
   if (e != cudaSuccess) return e;
-  k_het_tm<NDET><<<n, kHetTmThreads, bytes, st>>>(L, het_tables(B), B.rec, n, out, kappa_out, vv_out, ell);
+  k_het_tm<NDET><<<n, kHetTmThreads, lay.bytes, st>>>(L, het_tables(B), B.rec, n, lay.anc_off, lay.panel, out,
+                                                      kappa_out, vv_out, ell);
+  return cudaGetLastError();
+}
+
+template <int NDET>
+cudaError_t launch_het_plain(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
+                             double* kappa_out, double* vv_out) {
+  // as few vectors per CTA as fill the device once
+  int per = (n + L.sm_count - 1) / L.sm_count;
+  per = per < kHetBatch ? per : kHetBatch;
+  const int panel = B.het_nc < kHetPanel ? B.het_nc : kHetPanel, ctas = (n + per - 1) / per;
+  const size_t bytes = (size_t)((per + 1) / 2) * panel * 2 * kHetAncStride * sizeof(float);
+  const cudaError_t e = cudaFuncSetAttribute(k_het<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  k_het<NDET><<<ctas < L.sm_count ? ctas : L.sm_count, kHetTmThreads, bytes, st>>>(L, het_tables(B), B.rec, n, per, out,
+                                                                                  kappa_out, vv_out);
   return cudaGetLastError();
 }
 
@@ -431,15 +521,12 @@ cudaError_t launch_loglike_het(const LikeConst& L, const DeviceBuffers& B, const
       default: return launch_het_tm<4>(L, B, n, out, st, kappa_out, vv_out, ell);
     }
   }
-  const HetTables H = het_tables(B);
-  const unsigned grid = (unsigned)((n + 3) / 4);
   switch (L.n_det) {
-    case 1: k_het<1><<<grid, 128, 0, st>>>(L, H, B.rec, n, out, kappa_out, vv_out); break;
-    case 2: k_het<2><<<grid, 128, 0, st>>>(L, H, B.rec, n, out, kappa_out, vv_out); break;
-    case 3: k_het<3><<<grid, 128, 0, st>>>(L, H, B.rec, n, out, kappa_out, vv_out); break;
-    default: k_het<4><<<grid, 128, 0, st>>>(L, H, B.rec, n, out, kappa_out, vv_out); break;
+    case 1: return launch_het_plain<1>(L, B, n, out, st, kappa_out, vv_out);
+    case 2: return launch_het_plain<2>(L, B, n, out, st, kappa_out, vv_out);
+    case 3: return launch_het_plain<3>(L, B, n, out, st, kappa_out, vv_out);
+    default: return launch_het_plain<4>(L, B, n, out, st, kappa_out, vv_out);
   }
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

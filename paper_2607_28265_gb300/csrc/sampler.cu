@@ -2067,21 +2067,6 @@ __global__ void __launch_bounds__(kFlowThreads, 1)
 // boundaries) and the warps then share the time grid's 32-node chunks
 // (het.cuh tm_pass); there are no projection-only blocks in that mode.
 template <int NDET>
-__device__ __forceinline__ void het_prepare_warp(const LikeConst& L, const HetTables& H, const EvalRecord& r,
-                                                 HetPrep<NDET>& p, int lane) {
-  const EvalRecord& f0 = *H.fid;
-  if (lane < NBASIS) p.dc[lane] = df_from_double(r.c[lane] - f0.c[lane]);
-  if (lane >= 16 && lane < 16 + NDET) {
-    const int i = lane - 16;
-    p.dtau[i] = df_from_double(r.tau[i] - f0.tau[i]);
-    const double iden = L.het_fid_iden[i];
-    p.rho_re[i] = (float)((r.cre[i] * f0.cre[i] + r.cim[i] * f0.cim[i]) * iden);
-    p.rho_im[i] = (float)((r.cim[i] * f0.cre[i] - r.cre[i] * f0.cim[i]) * iden);
-  }
-  __syncwarp();
-}
-
-template <int NDET>
 __global__ void __launch_bounds__(kHetThreads, 1)
     k_ns_het(LikeConst L, SamplerConst S, DeviceBuffers B, SamplerPtrs P) {
   static_assert(sizeof(HetStage<NDET>) == (size_t)NDET * 32 * (16 + 8) + 2 * 32 * 4, "stage layout (kernels.h)");

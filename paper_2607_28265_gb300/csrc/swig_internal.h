@@ -115,6 +115,7 @@ struct LikeConst {
   int tm_pieces, tm_points;
   // heterodyned likelihood: 1 / |C0_i|^2 of the fiducial's projection factors
   double het_fid_iden[SWIG_MAX_DET];
+  double het_b0[SWIG_MAX_DET];  // sum of B0 over the bins (the fiducial's <h|h>_i)
 };
 
 }  // namespace swig
