@@ -1186,6 +1186,9 @@ int prepare(swig_ctx* c) {
     CUDA_TRY(c, cudaMemcpy(B.basis, basis.data(), sizeof(TileBasis) * basis.size(), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMalloc(&B.bin_tile, sizeof(int) * n));
     CUDA_TRY(c, cudaMemcpy(B.bin_tile, bin_tile.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    B.max_slice_tiles = 1;
+    for (int q = 0; q < n_slices; ++q)
+      B.max_slice_tiles = std::max(B.max_slice_tiles, bin_tile[slice_begin[q + 1] - 1] - bin_tile[slice_begin[q]] + 1);
     if (!c->cfg_set || c->cfg.likelihood == SWIG_LIKE_FULL) {
       const int rc = prepare_fold(c);
       if (rc) return rc;

@@ -1,0 +1,475 @@
+// The chain sampler: persistent nested-sampling kernel of the mixed-precision
+// full grid (folded sums) and of the heterodyned likelihood, with t_c sampled or
+// marginalised (chain.cuh has a chain's control).
+//
+// One cooperative launch runs up to max_iters iterations.  Between boundaries a
+// CTA takes one chain at a time and runs it to its end; the grid meets around
+// the boundaries alone.  Several events (a campaign) share a launch: the chains
+// of all are dealt to the CTAs as these come free, CTA e runs event e's boundary,
+// and the launch returns before any event starts new chains once one has left
+// the running state.  Which CTA runs a chain does not enter its arithmetic.
+#include <cuda_runtime.h>
+
+#include "chain.cuh"
+
+namespace swig {
+
+// Fixed shared memory: the chain, the event's constants, and the inputs and
+// sums of a round's evaluation.
+template <int NDET>
+struct ChainShared {
+  ChainWork w;
+  LikeConst L;
+  SamplerConst S;
+  float2 x[32 * kFoldKinds];  // folded: node abscissae
+  // folded: partial sums per candidate and group; bin by bin: per warp
+  float sum[kCand][kFoldGroups][2 * NDET];
+  double dir[kChainWarps][2 * NDET];
+  // heterodyned
+  HetPrep<NDET> prep[kCand];
+  HetIn<NDET, 2> in[kCand / 2];
+  HetIn<NDET, 1> in1;
+  float part[kChainWarps][NDET][3 * kCand];
+  float hh[kChainWarps][NDET];
+  float tm[kChainWarps][2];
+  unsigned long long prof[8], cta[4];
+  int task, event, exact;
+};
+
+size_t chain_fixed_bytes(int n_det) {
+  size_t b = 0;
+  switch (n_det) {
+    case 1: b = sizeof(ChainShared<1>); break;
+    case 2: b = sizeof(ChainShared<2>); break;
+    case 3: b = sizeof(ChainShared<3>); break;
+    default: b = sizeof(ChainShared<4>); break;
+  }
+  return (b + 15) & ~(size_t)15;
+}
+
+// Folded full-grid sums of the round's candidates: anchors of a panel of chunks
+// (quarter by quarter), then a (candidate, group of chunks) per warp and turn,
+// the chunks q = group, group + 4, ...; the group sums go to s.sum.
+template <int NDET>
+__device__ __forceinline__ void eval_fold(ChainShared<NDET>& s, const FoldTables& F, const float4* W, const float* tab,
+                                          float* s_an, int slots, int warp, int lane) {
+  ChainWork& w = s.w;
+  const int na = w.n_act, ld = F.ld;
+  int panel = slots / na & ~31;  // whole turns, and a multiple of the groups
+  if (slots / na >= F.nc) panel = F.nc;
+  FoldAcc<NDET> acc[2];
+  acc[0].clear();
+  acc[1].clear();
+  const float2 x0 = s.x[lane];
+  for (int base = 0; base < F.nc; base += panel) {
+    const int np = min(panel, F.nc - base), nb = (np + 31) >> 5, per = na * nb;
+    for (int it = warp; it < 4 * per; it += kChainWarps) {
+      const int sub = it / per, rem = it - sub * per, a = rem / nb, q = 32 * (rem - a * nb) + lane;
+      const int k = w.list[a];
+      if (q < np && !fold_anchor<NDET>(tab, ld, w.rec[k], sub, base + q, s_an + (a * panel + q) * kFoldAnchor))
+        w.bad[k] = 1;
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < na * np; it += kChainBlock) {
+      const int a = it / np, q = it - a * np;
+      if (!fold_in_band<NDET>(tab, ld, s_an + (a * panel + q) * kFoldAnchor, base + q)) w.bad[w.list[a]] = 1;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int u = warp + j * kChainWarps;
+      if (u < kFoldGroups * na) {
+        const int a = u >> 2, g = u & 3;
+        const float* an = s_an + (a * panel + g) * kFoldAnchor;
+        const float4* wq = W + (base + g) * NDET * 32 + lane;
+        auto kind = [&](int q) { return __float_as_int(tab[FR_KIND * ld + base + q]); };
+        FoldNode<NDET> v0, v1;
+        if (g < np) fold_load<NDET>(wq, kind(g), x0, s.x, lane, v0);
+        for (int q = g; q < np; q += 8, wq += 8 * NDET * 32, an += 8 * kFoldAnchor) {
+          if (q + 4 < np) fold_load<NDET>(wq + 4 * NDET * 32, kind(q + 4), x0, s.x, lane, v1);
+          fold_chunk<NDET>(an, v0, acc[j]);
+          if (q + 4 < np) {
+            if (q + 8 < np) fold_load<NDET>(wq + 8 * NDET * 32, kind(q + 8), x0, s.x, lane, v0);
+            fold_chunk<NDET>(an + 4 * kFoldAnchor, v1, acc[j]);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int u = warp + j * kChainWarps;
+    if (u < kFoldGroups * na) {
+#pragma unroll
+      for (int i = 0; i < NDET; ++i) {
+        float re, im;
+        acc[j].total(i, re, im);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          re += __shfl_xor_sync(0xffffffffu, re, o);
+          im += __shfl_xor_sync(0xffffffffu, im, o);
+        }
+        if (lane == 0) {
+          s.sum[w.list[u >> 2]][u & 3][2 * i] = re;
+          s.sum[w.list[u >> 2]][u & 3][2 * i + 1] = im;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int a = 0; a < na; ++a) {
+    const int k = w.list[a];
+    if (!w.bad[k]) continue;  // block-uniform, rare: bin by bin
+    double v[2 * NDET];
+    fold_direct<NDET>(s.L, F, w.rec[k], warp, kChainWarps, lane, s_an + warp * kAnchorStride, v);
+    if (lane == 0)
+#pragma unroll
+      for (int j = 0; j < 2 * NDET; ++j) s.dir[warp][j] = v[j];
+    __syncthreads();
+    if (threadIdx.x < 2 * NDET) {
+      double t = 0.0;
+      for (int q = 0; q < kChainWarps; ++q) t += s.dir[q][threadIdx.x];
+      w.kap[k][threadIdx.x] = t;
+    }
+    __syncthreads();
+  }
+}
+
+// logL of the round's candidates from their group sums, by warp 0: candidate
+// lane / 4, detector lane % 4.
+template <int NDET>
+__device__ __forceinline__ void finish_fold(ChainShared<NDET>& s, int lane) {
+  ChainWork& w = s.w;
+  const LikeConst& L = s.L;
+  const int k = lane >> 2, i = lane & 3;
+  const bool on = (w.act >> k) & 1u;
+  double kre = 0.0, kim = 0.0, tr = 0.0, ti = 0.0;
+  if (on) {
+    if (i < NDET) {
+      if (w.bad[k]) {
+        kre = w.kap[k][2 * i];
+        kim = w.kap[k][2 * i + 1];
+      } else {
+        dfl a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
+#pragma unroll
+        for (int g = 0; g < kFoldGroups; ++g) {
+          a = df_add(a, dfl{s.sum[k][g][2 * i], 0.0f});
+          b = df_add(b, dfl{s.sum[k][g][2 * i + 1], 0.0f});
+        }
+        kre = (double)a.hi + (double)a.lo;
+        kim = (double)b.hi + (double)b.lo;
+      }
+      const EvalRecord& r = w.rec[k];
+      const double a = kre * L.inv_scale[i], b = kim * L.inv_scale[i];
+      tr = r.cre[i] * a - r.cim[i] * b;
+      ti = r.cre[i] * b + r.cim[i] * a;
+    }
+    w.kap[k][2 * i] = kre;
+    w.kap[k][2 * i + 1] = kim;
+  }
+  const int l0 = lane & ~3;
+  double zr = __shfl_sync(0xffffffffu, tr, l0), zi = __shfl_sync(0xffffffffu, ti, l0);
+#pragma unroll
+  for (int d = 1; d < NDET; ++d) {
+    zr += __shfl_sync(0xffffffffu, tr, l0 + d);
+    zi += __shfl_sync(0xffffffffu, ti, l0 + d);
+  }
+  if (L.dist_marg) {  // a candidate after another, the quadrature across the warp
+    for (int a = 0; a < w.n_act; ++a) {
+      const int kk = w.list[a];
+      const double ll = distance_marg_logl_warp(L, __shfl_sync(0xffffffffu, zr, 4 * kk),
+                                                __shfl_sync(0xffffffffu, zi, 4 * kk), w.rec[kk].hh, lane);
+      if (lane == 0) w.ly[kk] = ll;
+    }
+  } else if (on && i == 0) {
+    const double base = -0.5 * w.rec[k].hh - 0.5 * L.DD;
+    double out = zr + base;
+    if (L.phase_marg) {
+      const double x = sqrt(zr * zr + zi * zi);
+      out = (L.fast_epilogue ? x + (double)log_i0e_f32((float)x) : log_bessel_i0(x)) + base;
+    }
+    w.ly[k] = out;
+  }
+  __syncwarp();
+}
+
+// Heterodyned sums of the round's candidates: pairs of candidates per packed
+// instruction, a warp per chunk over all pairs (see k_het); a warp per candidate
+// forms its result.
+template <int NDET>
+__device__ __forceinline__ void eval_het(ChainShared<NDET>& s, const HetTables& H, float* s_an, int bytes, int warp,
+                                         int lane) {
+  ChainWork& w = s.w;
+  const int na = w.n_act, pairs = (na + 1) / 2;
+  if (warp < 2 * pairs) {  // (an odd round's last pair holds its candidate twice)
+    het_prepare_warp<NDET>(s.L, H, w.rec[w.list[min(warp, na - 1)]], s.prep[warp], lane);
+    het_in_set<NDET, 2>(s.in[warp >> 1], warp & 1, s.prep[warp], lane);
+  }
+  const int fit = bytes / (pairs * 2 * kHetAncStride * (int)sizeof(float));
+  const int panel = fit >= H.n_chunks ? H.n_chunks : fit & ~31;
+  HetAcc<NDET, 2> acc[kCand / 2];
+#pragma unroll
+  for (int p = 0; p < kCand / 2; ++p) acc[p].clear();
+  for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
+    const int np = min(panel, H.n_chunks - q0);
+    __syncthreads();
+    het_anchors<NDET, 2>(H, s.in, pairs, q0, np, panel, s_an, warp, kChainWarps, lane);
+    __syncthreads();
+    for (int q = warp; q < np; q += kChainWarps) {
+      float4 v[NDET];
+#pragma unroll
+      for (int i = 0; i < NDET; ++i) v[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
+#pragma unroll
+      for (int p = 0; p < kCand / 2; ++p)
+        if (p < pairs) {
+          const HetPrep<NDET>* pp[2] = {&s.prep[2 * p], &s.prep[2 * p + 1]};
+          het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * 2 * kHetAncStride, s.in[p], pp, q0 + q, lane, v, acc[p]);
+        }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) {
+    float a[32];
+#pragma unroll
+    for (int p = 0; p < kCand / 2; ++p) {
+      PkOps<2>::get(acc[p].zr[i], a + 2 * p);
+      PkOps<2>::get(acc[p].zi[i], a + kCand + 2 * p);
+      PkOps<2>::get(acc[p].hh[i], a + 2 * kCand + 2 * p);
+      a[3 * kCand + 2 * p] = a[3 * kCand + 2 * p + 1] = 0.0f;
+    }
+    const float v = warp_transpose_sum(a, lane);
+    if (lane < 3 * kCand) s.part[warp][i][lane] = v;
+  }
+  __syncthreads();
+  if (warp < na) {
+    const int k = w.list[warp];
+    const double v = het_part_sum<NDET, kCand>(s.part, kChainWarps, warp, lane);
+    double Zr, Zi, HH, kap, vv;
+    het_network<NDET>(s.L, *H.fid, w.rec[k], v, lane, Zr, Zi, HH, kap, vv);
+    if (lane < 2 * SWIG_MAX_DET) w.kap[k][lane] = kap;
+    if (lane < SWIG_MAX_DET) w.vv[k][lane] = vv;
+    const double ll = het_epilogue(s.L, Zr, Zi, HH);
+    if (lane == 0) w.ly[k] = ll;
+  }
+}
+
+// Time-marginalised: a candidate after another, as k_het_tm.
+template <int NDET>
+__device__ __forceinline__ void eval_het_tm(ChainShared<NDET>& s, const HetTables& H, unsigned char* scratch,
+                                            const ChainLayout& lay, int warp, int lane) {
+  ChainWork& w = s.w;
+  const LikeConst& L = s.L;
+  float2* y = reinterpret_cast<float2*>(scratch);
+  for (int a = 0; a < w.n_act; ++a) {
+    const int k = w.list[a];
+    const EvalRecord& r = w.rec[k];
+    if (warp == 0) {
+      het_prepare_warp<NDET>(L, H, r, s.prep[0], lane);
+      het_in_set<NDET, 1>(s.in1, 0, s.prep[0], lane);
+    }
+    HetAcc<NDET, 1> acc;
+    acc.clear();
+    het_products<NDET>(H, s.prep[0], s.in1, reinterpret_cast<float*>(scratch + lay.anc_off), lay.panel, warp,
+                       kChainWarps, lane, acc, y);
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) {
+      float d = acc.hh[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if (lane == 0) s.hh[warp][i] = d;
+    }
+    __syncthreads();
+    float wm, ws;
+    if (L.tm_M > 0)
+      tm_pass_nufft(L, H, y, tm_nufft_grid(scratch, H.n_bins), tm_nufft_tw(scratch, H.n_bins, L.tm_M), warp,
+                    kChainWarps, lane, nullptr, wm, ws);
+    else
+      tm_pass(L, H, y, warp, kChainWarps, lane, nullptr, wm, ws);
+    if (lane == 0) {
+      s.tm[warp][0] = wm;
+      s.tm[warp][1] = ws;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double HH = 0.0;
+      for (int i = 0; i < NDET; ++i) {
+        double d = 0.0;
+        for (int q = 0; q < kChainWarps; ++q) d += (double)s.hh[q][i];
+        HH += (r.cre[i] * r.cre[i] + r.cim[i] * r.cim[i]) * (L.het_b0[i] - d) * L.het_fid_iden[i];
+      }
+      w.ly[k] = tm_finish(L, s.tm, kChainWarps, HH);
+      for (int j = 0; j < 2 * SWIG_MAX_DET; ++j) w.kap[k][j] = 0.0;
+      for (int i = 0; i < SWIG_MAX_DET; ++i) w.vv[k][i] = 0.0;
+    }
+    __syncthreads();
+  }
+}
+
+template <int NDET, int MODE>
+__global__ void __launch_bounds__(kChainBlock, 1)
+    k_ns_chain(const ChainEvent* __restrict__ ev, int n_ev, NSGlobal* gb, ChainLayout lay) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  ChainShared<NDET>& s = *reinterpret_cast<ChainShared<NDET>*>(smem);
+  unsigned char* scratch = smem + lay.scratch_off;
+  ChainWork& w = s.w;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int k_chains = ev[0].S.nrep;
+  const bool timer = blockIdx.x == 0 && tid == 0;
+  unsigned long long t0 = gtimer(), t1;
+  if (tid < 8) s.prof[tid] = 0;
+  if (tid < 4) s.cta[tid] = 0;
+  if (tid == 0) s.event = -1;
+  NSGlobal* g0 = ev[0].P.g;
+  for (;;) {
+    if (!grid_sync(gb, lay.n_ctas, lay.spin_limit)) return;
+    if (timer) {
+      t1 = gtimer();
+      g0->t_wait_sweep += t1 - t0;
+      t0 = t1;
+      g0->rounds += 1;
+    }
+    if ((int)blockIdx.x < n_ev) ns_boundary_check(ev[blockIdx.x].L, ev[blockIdx.x].S, ev[blockIdx.x].P, scratch);
+    if (!grid_sync(gb, lay.n_ctas, lay.spin_limit)) return;
+    bool all_run = true;
+    for (int e = 0; e < n_ev; ++e) all_run = all_run && *(volatile int*)&ev[e].P.g->status == ST_RUNNING;
+    if (!all_run) return;
+    if ((int)blockIdx.x < n_ev) ns_boundary_advance(ev[blockIdx.x].L, ev[blockIdx.x].S, ev[blockIdx.x].P, scratch);
+    if (timer) *(volatile int*)&gb->task = 0;
+    if (!grid_sync(gb, lay.n_ctas, lay.spin_limit)) return;
+    if (timer) {
+      t1 = gtimer();
+      g0->t_bound += t1 - t0;
+      t0 = t1;
+    }
+    for (;;) {
+      __syncthreads();
+      if (tid == 0) s.task = atomicAdd(&gb->task, 1);
+      __syncthreads();
+      const int task = s.task;
+      if (task >= n_ev * k_chains) break;
+      const int e = task / k_chains, c = task - e * k_chains;
+      const ChainEvent& E = ev[e];
+      if (s.event != e) {  // the event's constants and, resident, its weights and tables
+        __syncthreads();
+        const unsigned* src = reinterpret_cast<const unsigned*>(&E.L);
+        for (int q = tid; q < (int)(sizeof(LikeConst) / 4); q += kChainBlock) reinterpret_cast<unsigned*>(&s.L)[q] = src[q];
+        src = reinterpret_cast<const unsigned*>(&E.S);
+        for (int q = tid; q < (int)(sizeof(SamplerConst) / 4); q += kChainBlock)
+          reinterpret_cast<unsigned*>(&s.S)[q] = src[q];
+        if (MODE == CHAIN_FOLD) {
+          for (int q = tid; q < 32 * kFoldKinds; q += kChainBlock) s.x[q] = E.F.x[q];
+          if (lay.res_off > 0) {
+            float4* d = reinterpret_cast<float4*>(smem + lay.res_off);
+            const int nw = E.F.nc * NDET * 32, nt = FR_ROWS * E.F.ld / 4;
+            const float4* tab4 = reinterpret_cast<const float4*>(E.F.tab);
+            for (int q = tid; q < nw; q += kChainBlock) cp_async16(d + q, E.F.w + q);
+            for (int q = tid; q < nt; q += kChainBlock) cp_async16(d + nw + q, tab4 + q);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+          }
+        }
+        __syncthreads();
+        if (tid == 0) s.event = e;
+      }
+      if (MODE == CHAIN_HET_TM && E.L.tm_M > 0) tm_load_twiddles(s.L, E.H, scratch, E.H.n_bins);
+      const SamplerPtrs& P = E.P;
+      const float4* W = E.F.w;
+      const float* tab = E.F.tab;
+      if (MODE == CHAIN_FOLD && lay.res_off > 0) {
+        W = reinterpret_cast<const float4*>(smem + lay.res_off);
+        tab = reinterpret_cast<const float*>(W + E.F.nc * NDET * 32);
+      }
+      // written by CTA e at the boundary: read through L2, never a stale L1 line
+      const double logl_star = __ldcg(&P.g->logl_star);
+      const long long it = __ldcg(&P.g->iter);
+      if (warp == 0) {
+        warp_copy_cg(&w.ch, &P.chains[c], sizeof(ChainState), lane);
+        warp_copy_cg(&w.rx, &P.recx[c], sizeof(EvalRecord), lane);
+      }
+      unsigned long long* prof = c == 0 && e == 0 ? s.prof : nullptr;
+      bool have = false;
+      for (long long guard = 0; guard < (1ll << 24); ++guard) {
+        long long tc = 0;
+        if (warp == 0) {
+          tc = clock64();
+          if (MODE == CHAIN_FOLD && have) finish_fold<NDET>(s, lane);
+          chain_control<NDET, MODE != CHAIN_FOLD>(s.L, s.S, P, w, c, it, logl_star, have, lane, prof);
+          if (lane == 0) {
+            const long long t2 = clock64();
+            s.cta[2] += t2 - tc;
+            s.cta[3] += t2 - tc;
+            tc = t2;
+          }
+        }
+        __syncthreads();
+        if (w.status == ROUND_DONE) break;
+        chain_setup<NDET>(s.L, w, warp, lane);
+        if (prof && tid == 0) prof[4] += clock64() - tc;
+        if (MODE == CHAIN_FOLD)
+          eval_fold<NDET>(s, E.F, W, tab, reinterpret_cast<float*>(scratch),
+                          lay.scratch_bytes / (int)(kFoldAnchor * sizeof(float)), warp, lane);
+        else if (MODE == CHAIN_HET)
+          eval_het<NDET>(s, E.H, reinterpret_cast<float*>(scratch), lay.scratch_bytes, warp, lane);
+        else
+          eval_het_tm<NDET>(s, E.H, scratch, lay, warp, lane);
+        __syncthreads();
+        if (tid == 0) {
+          s.cta[0] += w.n_act;
+          s.cta[1] += clock64() - tc;
+        }
+        have = true;
+      }
+      if (warp == 0) warp_copy(&P.chains[c], &w.ch, sizeof(ChainState), lane);
+    }
+    if (tid == 0) {
+      if (ev[0].P.cta_prof) {
+        unsigned long long* cp = ev[0].P.cta_prof + 4 * (size_t)blockIdx.x;
+        for (int j = 0; j < 4; ++j) cp[j] += s.cta[j];
+      }
+      if (blockIdx.x == 0) {
+        g0->f_units += s.cta[0];
+        g0->f_unit_cyc += s.cta[1];
+        g0->f_idle_cyc += s.cta[2];
+      }
+      for (int j = 0; j < 4; ++j) s.cta[j] = 0;
+      // the CTA that ran the first event's first chain
+      if (s.prof[7]) {
+        atomicAdd(&g0->c_result, s.prof[0]);
+        atomicAdd(&g0->c_step, s.prof[1]);
+        atomicAdd(&g0->c_prop, s.prof[2]);
+        atomicAdd(&g0->c_free, s.prof[3]);
+        atomicAdd(&g0->c_setup, s.prof[4]);
+        atomicAdd(&g0->n_free, s.prof[5]);
+        atomicAdd(&g0->n_setup, s.prof[6]);
+        atomicAdd(&g0->n_step, s.prof[7]);
+        for (int j = 0; j < 8; ++j) s.prof[j] = 0;
+      }
+    }
+    if (timer) {
+      t1 = gtimer();
+      g0->t_ctrl += t1 - t0;
+      t0 = t1;
+    }
+  }
+}
+
+namespace {
+template <int NDET>
+void* chain_kernel_as(int mode) {
+  switch (mode) {
+    case CHAIN_FOLD: return (void*)k_ns_chain<NDET, CHAIN_FOLD>;
+    case CHAIN_HET: return (void*)k_ns_chain<NDET, CHAIN_HET>;
+    default: return (void*)k_ns_chain<NDET, CHAIN_HET_TM>;
+  }
+}
+}  // namespace
+
+void* chain_kernel(int n_det, int mode) {
+  switch (n_det) {
+    case 1: return chain_kernel_as<1>(mode);
+    case 2: return chain_kernel_as<2>(mode);
+    case 3: return chain_kernel_as<3>(mode);
+    default: return chain_kernel_as<4>(mode);
+  }
+}
+
+}  // namespace swig

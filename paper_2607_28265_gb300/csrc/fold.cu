@@ -170,15 +170,6 @@ constexpr int kFoldSlots = 512;  // anchors in shared memory, all teams together
 inline __host__ __device__ size_t fold_fixed_bytes() {
   return sizeof(float) * kFoldSlots * kFoldAnchor + sizeof(float2) * 32 * kFoldKinds;
 }
-inline size_t fold_resident_bytes(int nc, int n_det) {
-  return (size_t)nc * n_det * 32 * sizeof(float4) + sizeof(float) * FR_ROWS * fold_ld(nc);
-}
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-
 __device__ __forceinline__ void team_sync(int team, int T) {
   if (T == 1)
     __syncwarp();

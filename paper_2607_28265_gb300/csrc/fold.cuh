@@ -31,7 +31,7 @@
 namespace swig {
 
 constexpr int kFoldWarps = 16;     // warps of an evaluating CTA
-constexpr int kFoldAnchor = 16;    // floats per (evaluation, chunk) anchor
+constexpr int kFoldAnchor = kFoldAnchorFloats;
 
 // What an evaluation reads of its record: coefficients and time shifts in
 // double-float.
@@ -49,8 +49,8 @@ __device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
                         : reinterpret_cast<const float*>(&r.tau_hi)[w - 2 * NBASIS];
 }
 
-// One quarter (sub 0 .. 3) of the anchor of chunk q for the evaluation `r`,
-// written to out[kFoldAnchor]:
+// One quarter (sub 0 .. 3) of the anchor of chunk q for the evaluation `r` (a
+// FoldIn or an EvalRecord), written to out[kFoldAnchor]:
 //   sub 0: out[i] = frac(P(f_c) + f_c tau_i), double-float sums;
 //   sub 1: out[4], out[5] = the scaled slope h (P'(f_c) + tau_0 - s) as a
 //          double-float, out[5 + i] = h (tau_i - tau_0), i = 1 .. 3;
@@ -60,8 +60,8 @@ __device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
 // Returns false when the remainder is too large.  The serial part of an
 // anchor is the eleven-term double-float sums; four lanes of different warps
 // share it (a lane per chunk took 2.2x as long alone).
-template <int NDET>
-__device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int ld, const FoldIn& r, int sub, int q,
+template <int NDET, typename Rec>
+__device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int ld, const Rec& r, int sub, int q,
                                             float* out) {
   const float* T = tab + q;
   auto row = [&](int k) { return T[k * ld]; };
@@ -213,6 +213,12 @@ __device__ __noinline__ void fold_direct(const LikeConst& L, const FoldTables& F
 #pragma unroll
     for (int j = 0; j < 2 * NDET; ++j) out[j] += (double)v[j];
   }
+}
+
+// Asynchronous 16-byte copy, global to shared memory.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
 
 // Distance-marginalised logL (distance_marg_logl) by a whole warp: the 64

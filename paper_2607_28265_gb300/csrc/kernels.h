@@ -96,6 +96,7 @@ inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) 
 // reference slope times h (double-float), the bandwidth the weights serve
 // [cycles] and the node kind (an int's bits).
 constexpr int kFoldNodes = 64;
+constexpr int kFoldAnchorFloats = 16;  // per (evaluation, chunk)
 constexpr int kFoldDeg = 8;
 constexpr int kFoldSlopes = NBASIS - 1;
 enum FoldRow {
@@ -165,7 +166,8 @@ struct DeviceBuffers {
   float* fold_tab = nullptr;
   float4* fold_w = nullptr;
   float2* fold_x = nullptr;
-  int max_slice_bins = 0;
+  int max_slice_bins = 0;        // largest slice: bins, and (mixed) tiles that overlap it
+  int max_slice_tiles = 1;
   // heterodyned likelihood tables (SWIG_LIKE_HET)
   int het_nb = 0;
   float* het_edge_basis = nullptr;  // [2 * NBASIS][N_b + 1] (row per basis function, hi / lo)
@@ -223,6 +225,11 @@ inline HetTmLayout het_tm_layout(const LikeConst& L, const DeviceBuffers& B) {
 inline __host__ __device__ int fold_ld(int nc) { return (nc + 3) & ~3; }
 inline __host__ __device__ FoldTables fold_tables(const DeviceBuffers& B) {
   return {B.fold_nc, fold_ld(B.fold_nc), B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile};
+}
+
+// Bytes of the weights and table (weights first) in shared memory.
+inline __host__ __device__ size_t fold_resident_bytes(int nc, int n_det) {
+  return (size_t)nc * n_det * 32 * sizeof(float4) + sizeof(float) * FR_ROWS * fold_ld(nc);
 }
 
 // Node weights of the event (B.fold_w) from its weighted data (B.data32) and
