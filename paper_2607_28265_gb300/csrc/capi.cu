@@ -1131,6 +1131,7 @@ int prepare(swig_ctx* c) {
   weight_data(c, n_det, dre, dim, L.K, &dd_sum, dmax);
   for (int i = 0; i < n_det; ++i) {
     L.inv_scale[i] = prec == SWIG_PREC_MIXED ? (dmax[i] > 0.0 ? dmax[i] : 1.0) : 1.0;
+    L.rscale[i] = 1.0 / L.inv_scale[i];
     for (int r = 0; r < 3; ++r) L.vertex[i][r] = c->vertex[i][r];
     const double* x = c->xarm[i];
     const double* y = c->yarm[i];
@@ -1140,7 +1141,9 @@ int prepare(swig_ctx* c) {
     L.dten[i][3] = 0.5 * (x[1] * x[1] - y[1] * y[1]);
     L.dten[i][4] = 0.5 * (x[1] * x[2] - y[1] * y[2]);
     L.dten[i][5] = 0.5 * (x[2] * x[2] - y[2] * y[2]);
+    for (int q = 0; q < 6; ++q) L.dten_f[i][q] = (float)L.dten[i][q];
   }
+  L.gmst_f = (float)L.gmst;
   L.DD = dd_sum;
   {
     const double a1 = std::sqrt(5.0 / 24.0) * std::pow(kPi, -2.0 / 3.0) * std::pow(kMtsunS, 5.0 / 6.0) * kCSI / kMpcM;

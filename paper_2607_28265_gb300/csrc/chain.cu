@@ -15,130 +15,187 @@
 namespace swig {
 
 // Fixed shared memory: the chain, the event's constants, and the inputs and
-// sums of a round's evaluation.
+// sums of a round's evaluation (only what the mode uses, so that the folded
+// weights fit beside it).
+template <int NDET, int MODE>
+struct ChainEval;
 template <int NDET>
+struct ChainEval<NDET, CHAIN_FOLD> {
+  float2 x[32 * kFoldKinds];  // node abscissae
+  FoldPair in[kCand / 2];
+  FoldPair cur;               // the chain's current point
+  int base_ok;                // its partial sums are formed
+  float sum[kCand][kChainWarps][2 * NDET];  // per group
+  double tot[kCand][2 * NDET];
+  double dir[kChainWarps][2 * NDET];  // bin by bin, per warp
+};
+template <int NDET>
+struct ChainEval<NDET, CHAIN_HET> {
+  HetPrep<NDET> prep[kCand];
+  HetIn<NDET, 2> in[kCand / 2];
+  float part[kChainWarps][NDET][3 * kCand];  // per warp: value 8 kind + slot
+  double tot[NDET][3 * kCand];
+};
+template <int NDET>
+struct ChainEval<NDET, CHAIN_HET_TM> {
+  HetPrep<NDET> prep;
+  HetIn<NDET, 1> in;
+  float hh[kChainWarps][NDET];
+  float tm[kChainWarps][2];
+};
+template <int NDET, int MODE>
 struct ChainShared {
   ChainWork w;
   LikeConst L;
   SamplerConst S;
-  float2 x[32 * kFoldKinds];  // folded: node abscissae
-  // folded: partial sums per candidate and group; bin by bin: per warp
-  float sum[kCand][kFoldGroups][2 * NDET];
-  double dir[kChainWarps][2 * NDET];
-  // heterodyned
-  HetPrep<NDET> prep[kCand];
-  HetIn<NDET, 2> in[kCand / 2];
-  HetIn<NDET, 1> in1;
-  float part[kChainWarps][NDET][3 * kCand];
-  float hh[kChainWarps][NDET];
-  float tm[kChainWarps][2];
+  ChainEval<NDET, MODE> e;
   unsigned long long prof[8], cta[4];
-  int task, event, exact;
+  int task, event;
 };
 
-size_t chain_fixed_bytes(int n_det) {
-  size_t b = 0;
-  switch (n_det) {
-    case 1: b = sizeof(ChainShared<1>); break;
-    case 2: b = sizeof(ChainShared<2>); break;
-    case 3: b = sizeof(ChainShared<3>); break;
-    default: b = sizeof(ChainShared<4>); break;
-  }
+namespace {
+template <int NDET>
+size_t shared_bytes(int mode) {
+  return mode == CHAIN_FOLD  ? sizeof(ChainShared<NDET, CHAIN_FOLD>)
+         : mode == CHAIN_HET ? sizeof(ChainShared<NDET, CHAIN_HET>)
+                             : sizeof(ChainShared<NDET, CHAIN_HET_TM>);
+}
+}  // namespace
+
+size_t chain_fixed_bytes(int n_det, int mode) {
+  const size_t b = n_det == 1   ? shared_bytes<1>(mode)
+                   : n_det == 2 ? shared_bytes<2>(mode)
+                   : n_det == 3 ? shared_bytes<3>(mode)
+                                : shared_bytes<4>(mode);
   return (b + 15) & ~(size_t)15;
 }
 
-// Folded full-grid sums of the round's candidates: anchors of a panel of chunks
-// (quarter by quarter), then a (candidate, group of chunks) per warp and turn,
-// the chunks q = group, group + 4, ...; the group sums go to s.sum.
+// Folded full-grid sums of the round's candidates, two at a time: anchors of a
+// panel of chunks (packed over the pair, quarter by quarter), then a (pair, group
+// of chunks) per warp, the chunks q = group, group + G, ..., the weights loaded
+// once for both.  The groups' sums go to s.e.sum.  A block that leaves the masses
+// and tides alone takes the sums over their basis functions from base (the
+// current point's) and adds the spin terms only.
 template <int NDET>
-__device__ __forceinline__ void eval_fold(ChainShared<NDET>& s, const FoldTables& F, const float4* W, const float* tab,
-                                          float* s_an, int slots, int warp, int lane) {
+__device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, const FoldTables& F, const float4* W,
+                                         const float* tab, float* base, float* s_an, int slots, int warp, int lane) {
   ChainWork& w = s.w;
-  const int na = w.n_act, ld = F.ld;
+  const int na = w.n_act, pairs = (na + 1) / 2, ld = F.ld;
+  const int G = pairs <= 1 ? 16 : pairs == 2 ? 8 : kFoldGroups;
+  const bool use = base != nullptr && !(w.fl & (BF_INTR | BF_TIDE));  // uniform
+  if (threadIdx.x < pairs * 16) {
+    const int p = threadIdx.x >> 4, j = threadIdx.x & 15;
+    const EvalRecord& a = w.rec[w.list[2 * p]];
+    const EvalRecord& b = w.rec[w.list[min(2 * p + 1, na - 1)]];
+    fold_pair_set(s.e.in[p], j, a, b);
+  } else if (use && !s.e.base_ok && threadIdx.x >= 256 && threadIdx.x < 272) {
+    fold_pair_set(s.e.cur, threadIdx.x & 15, w.rx, w.rx);
+  }
+  __syncthreads();
+  if (use && !s.e.base_ok) {
+    const int nb = (F.nc + 31) >> 5;
+    for (int it = warp; it < 4 * nb; it += kChainWarps) {
+      const int q = 32 * (it % nb) + lane;
+      if (q < F.nc) fold_base(tab, ld, s.e.cur, it / nb, q, base, F.ld);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s.e.base_ok = 1;
+  }
   int panel = slots / na & ~31;  // whole turns, and a multiple of the groups
   if (slots / na >= F.nc) panel = F.nc;
   FoldAcc<NDET> acc[2];
   acc[0].clear();
   acc[1].clear();
-  const float2 x0 = s.x[lane];
-  for (int base = 0; base < F.nc; base += panel) {
-    const int np = min(panel, F.nc - base), nb = (np + 31) >> 5, per = na * nb;
-    for (int it = warp; it < 4 * per; it += kChainWarps) {
-      const int sub = it / per, rem = it - sub * per, a = rem / nb, q = 32 * (rem - a * nb) + lane;
-      const int k = w.list[a];
-      if (q < np && !fold_anchor<NDET>(tab, ld, w.rec[k], sub, base + q, s_an + (a * panel + q) * kFoldAnchor))
-        w.bad[k] = 1;
+  const float2 x0 = s.e.x[lane];
+  const int p = warp / G, g = warp - p * G;  // this warp's pair and group
+  for (int q0 = 0; q0 < F.nc; q0 += panel) {
+    const int np = min(panel, F.nc - q0), nb = (np + 31) >> 5, per = pairs * nb;
+    for (int it = warp, sub = 0, t = warp; it < 4 * per; it += kChainWarps, t += kChainWarps) {
+      while (t >= per) t -= per, ++sub;
+      const int a = t / nb, q = 32 * (t - a * nb) + lane;
+      if (q < np) {
+        const int k0 = 2 * a, k1 = min(2 * a + 1, na - 1);
+        const int bad = fold_anchor_pair<NDET>(tab, ld, s.e.in[a], use ? base : nullptr, sub, q0 + q, q,
+                                               s_an + (k0 * panel + q) * kFoldAnchor,
+                                               s_an + (k1 * panel + q) * kFoldAnchor);
+        if (bad & 1) w.bad[w.list[k0]] = 1;
+        if (bad & 2) w.bad[w.list[k1]] = 1;
+      }
     }
     __syncthreads();
     for (int it = threadIdx.x; it < na * np; it += kChainBlock) {
       const int a = it / np, q = it - a * np;
-      if (!fold_in_band<NDET>(tab, ld, s_an + (a * panel + q) * kFoldAnchor, base + q)) w.bad[w.list[a]] = 1;
+      if (!fold_in_band<NDET>(tab, ld, s_an + (a * panel + q) * kFoldAnchor, q, q0 + q)) w.bad[w.list[a]] = 1;
     }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int u = warp + j * kChainWarps;
-      if (u < kFoldGroups * na) {
-        const int a = u >> 2, g = u & 3;
-        const float* an = s_an + (a * panel + g) * kFoldAnchor;
-        const float4* wq = W + (base + g) * NDET * 32 + lane;
-        auto kind = [&](int q) { return __float_as_int(tab[FR_KIND * ld + base + q]); };
-        FoldNode<NDET> v0, v1;
-        if (g < np) fold_load<NDET>(wq, kind(g), x0, s.x, lane, v0);
-        for (int q = g; q < np; q += 8, wq += 8 * NDET * 32, an += 8 * kFoldAnchor) {
-          if (q + 4 < np) fold_load<NDET>(wq + 4 * NDET * 32, kind(q + 4), x0, s.x, lane, v1);
-          fold_chunk<NDET>(an, v0, acc[j]);
-          if (q + 4 < np) {
-            if (q + 8 < np) fold_load<NDET>(wq + 8 * NDET * 32, kind(q + 8), x0, s.x, lane, v0);
-            fold_chunk<NDET>(an + 4 * kFoldAnchor, v1, acc[j]);
-          }
-        }
+    if (p < pairs) {
+      const bool two = 2 * p + 1 < na;
+      const float* an0 = s_an + (2 * p * panel + g) * kFoldAnchor;
+      const float* an1 = an0 + panel * kFoldAnchor;
+      const float4* wq = W + (q0 + g) * NDET * 32 + lane;
+      auto kind = [&](int q) { return __float_as_int(tab[FR_KIND * ld + q0 + q]); };
+      for (int q = g; q < np; q += G, wq += G * NDET * 32, an0 += G * kFoldAnchor, an1 += G * kFoldAnchor) {
+        FoldNode<NDET> v;
+        fold_load<NDET>(wq, kind(q), x0, s.e.x, lane, v);
+        fold_chunk<NDET>(an0, q, v, acc[0]);
+        if (two) fold_chunk<NDET>(an1, q, v, acc[1]);
       }
     }
     __syncthreads();
   }
+  if (p < pairs)
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const int u = warp + j * kChainWarps;
-    if (u < kFoldGroups * na) {
+    for (int j = 0; j < 2; ++j)
+      if (2 * p + j < na) {
+        const int k = w.list[2 * p + j];
 #pragma unroll
-      for (int i = 0; i < NDET; ++i) {
-        float re, im;
-        acc[j].total(i, re, im);
+        for (int i = 0; i < NDET; ++i) {
+          float re, im;
+          acc[j].total(i, re, im);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          re += __shfl_xor_sync(0xffffffffu, re, o);
-          im += __shfl_xor_sync(0xffffffffu, im, o);
-        }
-        if (lane == 0) {
-          s.sum[w.list[u >> 2]][u & 3][2 * i] = re;
-          s.sum[w.list[u >> 2]][u & 3][2 * i + 1] = im;
+          for (int o = 16; o > 0; o >>= 1) {
+            re += __shfl_xor_sync(0xffffffffu, re, o);
+            im += __shfl_xor_sync(0xffffffffu, im, o);
+          }
+          if (lane == 0) {
+            s.e.sum[k][g][2 * i] = re;
+            s.e.sum[k][g][2 * i + 1] = im;
+          }
         }
       }
-    }
-  }
   __syncthreads();
+  {  // the groups' sums (double-float, four threads a value), rounded once to FP64
+    const int v = threadIdx.x >> 2, a = v / (2 * NDET), j = v - a * (2 * NDET), g0 = threadIdx.x & 3;
+    const int k = a < na ? w.list[a] : 0;
+    dfl t = {0.0f, 0.0f};
+    for (int r = g0; r < G; r += 4) t = df_add(t, dfl{s.e.sum[k][r][j], 0.0f});
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1)
+      t = df_add(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
+    if (a < na && g0 == 0) s.e.tot[k][j] = (double)t.hi + (double)t.lo;
+  }
   for (int a = 0; a < na; ++a) {
     const int k = w.list[a];
     if (!w.bad[k]) continue;  // block-uniform, rare: bin by bin
+    __syncthreads();
     double v[2 * NDET];
     fold_direct<NDET>(s.L, F, w.rec[k], warp, kChainWarps, lane, s_an + warp * kAnchorStride, v);
     if (lane == 0)
 #pragma unroll
-      for (int j = 0; j < 2 * NDET; ++j) s.dir[warp][j] = v[j];
+      for (int j = 0; j < 2 * NDET; ++j) s.e.dir[warp][j] = v[j];
     __syncthreads();
     if (threadIdx.x < 2 * NDET) {
       double t = 0.0;
-      for (int q = 0; q < kChainWarps; ++q) t += s.dir[q][threadIdx.x];
-      w.kap[k][threadIdx.x] = t;
+      for (int q = 0; q < kChainWarps; ++q) t += s.e.dir[q][threadIdx.x];
+      s.e.tot[k][threadIdx.x] = t;
     }
     __syncthreads();
   }
 }
 
-// logL of the round's candidates from their group sums, by warp 0: candidate
+// logL of the round's candidates from their sums, by warp 0: candidate
 // lane / 4, detector lane % 4.
 template <int NDET>
-__device__ __forceinline__ void finish_fold(ChainShared<NDET>& s, int lane) {
+__device__ __forceinline__ void finish_fold(ChainShared<NDET, CHAIN_FOLD>& s, int lane) {
   ChainWork& w = s.w;
   const LikeConst& L = s.L;
   const int k = lane >> 2, i = lane & 3;
@@ -146,19 +203,8 @@ __device__ __forceinline__ void finish_fold(ChainShared<NDET>& s, int lane) {
   double kre = 0.0, kim = 0.0, tr = 0.0, ti = 0.0;
   if (on) {
     if (i < NDET) {
-      if (w.bad[k]) {
-        kre = w.kap[k][2 * i];
-        kim = w.kap[k][2 * i + 1];
-      } else {
-        dfl a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
-#pragma unroll
-        for (int g = 0; g < kFoldGroups; ++g) {
-          a = df_add(a, dfl{s.sum[k][g][2 * i], 0.0f});
-          b = df_add(b, dfl{s.sum[k][g][2 * i + 1], 0.0f});
-        }
-        kre = (double)a.hi + (double)a.lo;
-        kim = (double)b.hi + (double)b.lo;
-      }
+      kre = s.e.tot[k][2 * i];
+      kim = s.e.tot[k][2 * i + 1];
       const EvalRecord& r = w.rec[k];
       const double a = kre * L.inv_scale[i], b = kim * L.inv_scale[i];
       tr = r.cre[i] * a - r.cim[i] * b;
@@ -197,15 +243,15 @@ __device__ __forceinline__ void finish_fold(ChainShared<NDET>& s, int lane) {
 // instruction, a warp per chunk over all pairs (see k_het); a warp per candidate
 // forms its result.
 template <int NDET>
-__device__ __forceinline__ void eval_het(ChainShared<NDET>& s, const HetTables& H, float* s_an, int bytes, int warp,
-                                         int lane) {
+__device__ __forceinline__ void eval_het(ChainShared<NDET, CHAIN_HET>& s, const HetTables& H, const float* tab,
+                                         float* s_an, int bytes, int warp, int lane) {
   ChainWork& w = s.w;
   const int na = w.n_act, pairs = (na + 1) / 2;
   if (warp < 2 * pairs) {  // (an odd round's last pair holds its candidate twice)
-    het_prepare_warp<NDET>(s.L, H, w.rec[w.list[min(warp, na - 1)]], s.prep[warp], lane);
-    het_in_set<NDET, 2>(s.in[warp >> 1], warp & 1, s.prep[warp], lane);
+    het_prepare_warp<NDET>(s.L, H, w.rec[w.list[min(warp, na - 1)]], s.e.prep[warp], lane);
+    het_in_set<NDET, 2>(s.e.in[warp >> 1], warp & 1, s.e.prep[warp], lane);
   }
-  const int fit = bytes / (pairs * 2 * kHetAncStride * (int)sizeof(float));
+  const int fit = bytes / (pairs * kHetAncPair * (int)sizeof(float));
   const int panel = fit >= H.n_chunks ? H.n_chunks : fit & ~31;
   HetAcc<NDET, 2> acc[kCand / 2];
 #pragma unroll
@@ -213,7 +259,7 @@ __device__ __forceinline__ void eval_het(ChainShared<NDET>& s, const HetTables& 
   for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
     const int np = min(panel, H.n_chunks - q0);
     __syncthreads();
-    het_anchors<NDET, 2>(H, s.in, pairs, q0, np, panel, s_an, warp, kChainWarps, lane);
+    het_anchors<NDET, 2>(H, tab, s.e.in, pairs, q0, np, panel, s_an, warp, kChainWarps, lane);
     __syncthreads();
     for (int q = warp; q < np; q += kChainWarps) {
       float4 v[NDET];
@@ -222,8 +268,8 @@ __device__ __forceinline__ void eval_het(ChainShared<NDET>& s, const HetTables& 
 #pragma unroll
       for (int p = 0; p < kCand / 2; ++p)
         if (p < pairs) {
-          const HetPrep<NDET>* pp[2] = {&s.prep[2 * p], &s.prep[2 * p + 1]};
-          het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * 2 * kHetAncStride, s.in[p], pp, q0 + q, lane, v, acc[p]);
+          const HetPrep<NDET>* pp[2] = {&s.e.prep[2 * p], &s.e.prep[2 * p + 1]};
+          het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * kHetAncPair, s.e.in[p], pp, q0 + q, lane, v, acc[p]);
         }
     }
   }
@@ -238,24 +284,55 @@ __device__ __forceinline__ void eval_het(ChainShared<NDET>& s, const HetTables& 
       a[3 * kCand + 2 * p] = a[3 * kCand + 2 * p + 1] = 0.0f;
     }
     const float v = warp_transpose_sum(a, lane);
-    if (lane < 3 * kCand) s.part[warp][i][lane] = v;
+    if (lane < 3 * kCand) s.e.part[warp][i][lane] = v;
   }
   __syncthreads();
-  if (warp < na) {
-    const int k = w.list[warp];
-    const double v = het_part_sum<NDET, kCand>(s.part, kChainWarps, warp, lane);
-    double Zr, Zi, HH, kap, vv;
-    het_network<NDET>(s.L, *H.fid, w.rec[k], v, lane, Zr, Zi, HH, kap, vv);
-    if (lane < 2 * SWIG_MAX_DET) w.kap[k][lane] = kap;
-    if (lane < SWIG_MAX_DET) w.vv[k][lane] = vv;
-    const double ll = het_epilogue(s.L, Zr, Zi, HH);
-    if (lane == 0) w.ly[k] = ll;
+  if (threadIdx.x < 4 * 3 * kCand * NDET) {  // (whole warps)
+    // the warps' sums (double-float, four threads a value), rounded once to FP64
+    const int v = threadIdx.x >> 2, i = v / (3 * kCand), j = v - i * (3 * kCand), g0 = threadIdx.x & 3;
+    dfl t = {0.0f, 0.0f};
+#pragma unroll
+    for (int r = 0; r < kChainWarps; r += 4) t = df_add(t, dfl{s.e.part[r + g0][i][j], 0.0f});
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1)
+      t = df_add(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
+    if (g0 == 0) s.e.tot[i][j] = (double)t.hi + (double)t.lo;
   }
+}
+
+// logL and caches of the round's candidates, by warp 0: slot lane / 4, detector
+// lane % 4 (het_detector with the reciprocal of the data scale).
+template <int NDET>
+__device__ __forceinline__ void finish_het(ChainShared<NDET, CHAIN_HET>& s, const HetTables& H, int lane) {
+  ChainWork& w = s.w;
+  const LikeConst& L = s.L;
+  const int a = lane >> 2, i = lane & 3;
+  const bool on = a < w.n_act;
+  const int k = on ? w.list[a] : 0;
+  double Z[2] = {0.0, 0.0}, hh = 0.0, k2[2] = {0.0, 0.0}, vv = 0.0;
+  if (on && i < NDET)
+    het_detector(L, *H.fid, w.rec[k], i, s.e.tot[i][a], s.e.tot[i][kCand + a], s.e.tot[i][2 * kCand + a], Z, &hh, k2,
+                 &vv);
+  if (on) {
+    w.kap[k][2 * i] = k2[0];
+    w.kap[k][2 * i + 1] = k2[1];
+    w.vv[k][i] = vv;
+  }
+  const int l0 = lane & ~3;
+  double Zr = 0.0, Zi = 0.0, HH = 0.0;
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) {
+    Zr += __shfl_sync(0xffffffffu, Z[0], l0 + d);
+    Zi += __shfl_sync(0xffffffffu, Z[1], l0 + d);
+    HH += __shfl_sync(0xffffffffu, hh, l0 + d);
+  }
+  if (on && i == 0) w.ly[k] = het_epilogue(L, Zr, Zi, HH);
+  __syncwarp();
 }
 
 // Time-marginalised: a candidate after another, as k_het_tm.
 template <int NDET>
-__device__ __forceinline__ void eval_het_tm(ChainShared<NDET>& s, const HetTables& H, unsigned char* scratch,
+__device__ __forceinline__ void eval_het_tm(ChainShared<NDET, CHAIN_HET_TM>& s, const HetTables& H, unsigned char* scratch,
                                             const ChainLayout& lay, int warp, int lane) {
   ChainWork& w = s.w;
   const LikeConst& L = s.L;
@@ -264,19 +341,19 @@ __device__ __forceinline__ void eval_het_tm(ChainShared<NDET>& s, const HetTable
     const int k = w.list[a];
     const EvalRecord& r = w.rec[k];
     if (warp == 0) {
-      het_prepare_warp<NDET>(L, H, r, s.prep[0], lane);
-      het_in_set<NDET, 1>(s.in1, 0, s.prep[0], lane);
+      het_prepare_warp<NDET>(L, H, r, s.e.prep, lane);
+      het_in_set<NDET, 1>(s.e.in, 0, s.e.prep, lane);
     }
     HetAcc<NDET, 1> acc;
     acc.clear();
-    het_products<NDET>(H, s.prep[0], s.in1, reinterpret_cast<float*>(scratch + lay.anc_off), lay.panel, warp,
+    het_products<NDET>(H, s.e.prep, s.e.in, reinterpret_cast<float*>(scratch + lay.anc_off), lay.panel, warp,
                        kChainWarps, lane, acc, y);
 #pragma unroll
     for (int i = 0; i < NDET; ++i) {
       float d = acc.hh[i];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if (lane == 0) s.hh[warp][i] = d;
+      if (lane == 0) s.e.hh[warp][i] = d;
     }
     __syncthreads();
     float wm, ws;
@@ -286,18 +363,18 @@ __device__ __forceinline__ void eval_het_tm(ChainShared<NDET>& s, const HetTable
     else
       tm_pass(L, H, y, warp, kChainWarps, lane, nullptr, wm, ws);
     if (lane == 0) {
-      s.tm[warp][0] = wm;
-      s.tm[warp][1] = ws;
+      s.e.tm[warp][0] = wm;
+      s.e.tm[warp][1] = ws;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       double HH = 0.0;
       for (int i = 0; i < NDET; ++i) {
         double d = 0.0;
-        for (int q = 0; q < kChainWarps; ++q) d += (double)s.hh[q][i];
+        for (int q = 0; q < kChainWarps; ++q) d += (double)s.e.hh[q][i];
         HH += (r.cre[i] * r.cre[i] + r.cim[i] * r.cim[i]) * (L.het_b0[i] - d) * L.het_fid_iden[i];
       }
-      w.ly[k] = tm_finish(L, s.tm, kChainWarps, HH);
+      w.ly[k] = tm_finish(L, s.e.tm, kChainWarps, HH);
       for (int j = 0; j < 2 * SWIG_MAX_DET; ++j) w.kap[k][j] = 0.0;
       for (int i = 0; i < SWIG_MAX_DET; ++i) w.vv[k][i] = 0.0;
     }
@@ -309,7 +386,7 @@ template <int NDET, int MODE>
 __global__ void __launch_bounds__(kChainBlock, 1)
     k_ns_chain(const ChainEvent* __restrict__ ev, int n_ev, NSGlobal* gb, ChainLayout lay) {
   extern __shared__ __align__(16) unsigned char smem[];
-  ChainShared<NDET>& s = *reinterpret_cast<ChainShared<NDET>*>(smem);
+  ChainShared<NDET, MODE>& s = *reinterpret_cast<ChainShared<NDET, MODE>*>(smem);
   unsigned char* scratch = smem + lay.scratch_off;
   ChainWork& w = s.w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -356,8 +433,8 @@ __global__ void __launch_bounds__(kChainBlock, 1)
         src = reinterpret_cast<const unsigned*>(&E.S);
         for (int q = tid; q < (int)(sizeof(SamplerConst) / 4); q += kChainBlock)
           reinterpret_cast<unsigned*>(&s.S)[q] = src[q];
-        if (MODE == CHAIN_FOLD) {
-          for (int q = tid; q < 32 * kFoldKinds; q += kChainBlock) s.x[q] = E.F.x[q];
+        if constexpr (MODE == CHAIN_FOLD) {
+          for (int q = tid; q < 32 * kFoldKinds; q += kChainBlock) s.e.x[q] = E.F.x[q];
           if (lay.res_off > 0) {
             float4* d = reinterpret_cast<float4*>(smem + lay.res_off);
             const int nw = E.F.nc * NDET * 32, nt = FR_ROWS * E.F.ld / 4;
@@ -367,17 +444,26 @@ __global__ void __launch_bounds__(kChainBlock, 1)
             asm volatile("cp.async.wait_all;" ::: "memory");
           }
         }
+        if constexpr (MODE == CHAIN_HET)
+          if (lay.res_off > 0) {
+            float* d = reinterpret_cast<float*>(smem + lay.res_off);
+            for (int q = tid; q < HC_ROWS * E.H.n_chunks; q += kChainBlock) cp_async<4>(d + q, E.H.chunk + q);
+            cp_async_commit();
+            cp_async_wait<0>();
+          }
         __syncthreads();
         if (tid == 0) s.event = e;
       }
       if (MODE == CHAIN_HET_TM && E.L.tm_M > 0) tm_load_twiddles(s.L, E.H, scratch, E.H.n_bins);
       const SamplerPtrs& P = E.P;
+      float* base = lay.base_off > 0 ? reinterpret_cast<float*>(smem + lay.base_off) : nullptr;
       const float4* W = E.F.w;
-      const float* tab = E.F.tab;
+      const float* tab = MODE == CHAIN_FOLD ? E.F.tab : E.H.chunk;
       if (MODE == CHAIN_FOLD && lay.res_off > 0) {
         W = reinterpret_cast<const float4*>(smem + lay.res_off);
         tab = reinterpret_cast<const float*>(W + E.F.nc * NDET * 32);
       }
+      if (MODE == CHAIN_HET && lay.res_off > 0) tab = reinterpret_cast<const float*>(smem + lay.res_off);
       // written by CTA e at the boundary: read through L2, never a stale L1 line
       const double logl_star = __ldcg(&P.g->logl_star);
       const long long it = __ldcg(&P.g->iter);
@@ -387,12 +473,19 @@ __global__ void __launch_bounds__(kChainBlock, 1)
       }
       unsigned long long* prof = c == 0 && e == 0 ? s.prof : nullptr;
       bool have = false;
+      if constexpr (MODE == CHAIN_FOLD)
+        if (tid == 0) s.e.base_ok = 0;
       for (long long guard = 0; guard < (1ll << 24); ++guard) {
         long long tc = 0;
         if (warp == 0) {
           tc = clock64();
-          if (MODE == CHAIN_FOLD && have) finish_fold<NDET>(s, lane);
+          if constexpr (MODE == CHAIN_FOLD)
+            if (have) finish_fold<NDET>(s, lane);
+          if constexpr (MODE == CHAIN_HET)
+            if (have) finish_het<NDET>(s, E.H, lane);
           chain_control<NDET, MODE != CHAIN_FOLD>(s.L, s.S, P, w, c, it, logl_star, have, lane, prof);
+          if constexpr (MODE == CHAIN_FOLD)
+            if (lane == 0 && w.status == ROUND_EVAL && (w.fl & (BF_INTR | BF_TIDE))) s.e.base_ok = 0;
           if (lane == 0) {
             const long long t2 = clock64();
             s.cta[2] += t2 - tc;
@@ -404,11 +497,11 @@ __global__ void __launch_bounds__(kChainBlock, 1)
         if (w.status == ROUND_DONE) break;
         chain_setup<NDET>(s.L, w, warp, lane);
         if (prof && tid == 0) prof[4] += clock64() - tc;
-        if (MODE == CHAIN_FOLD)
-          eval_fold<NDET>(s, E.F, W, tab, reinterpret_cast<float*>(scratch),
+        if constexpr (MODE == CHAIN_FOLD)
+          eval_fold<NDET>(s, E.F, W, tab, base, reinterpret_cast<float*>(scratch),
                           lay.scratch_bytes / (int)(kFoldAnchor * sizeof(float)), warp, lane);
-        else if (MODE == CHAIN_HET)
-          eval_het<NDET>(s, E.H, reinterpret_cast<float*>(scratch), lay.scratch_bytes, warp, lane);
+        else if constexpr (MODE == CHAIN_HET)
+          eval_het<NDET>(s, E.H, tab, reinterpret_cast<float*>(scratch), lay.scratch_bytes, warp, lane);
         else
           eval_het_tm<NDET>(s, E.H, scratch, lay, warp, lane);
         __syncthreads();

@@ -30,7 +30,7 @@ namespace swig {
 
 constexpr int kCand = 8;          // candidates per round at most
 constexpr int kChainWarps = kChainBlock / 32;
-constexpr int kFoldGroups = 4;    // partial sums per candidate (chunk q to group q mod 4)
+constexpr int kFoldGroups = 4;    // groups of chunks (partial sums) of a full round's pairs
 static_assert(kChainBlock == kHetTmThreads, "the sampler and the batched time-marginalised kernel share sum orders");
 
 // What the control keeps of a chain between its rounds, and a round's
@@ -55,6 +55,16 @@ struct ChainWork {
 };
 
 enum { ROUND_EVAL = 0, ROUND_DONE = 1 };
+
+// Sign and unit-interval tests on the bits: an FP64 comparison costs the
+// scheduler 64 cycles.
+__device__ __forceinline__ bool fp64_negative(double v) {  // v < 0 (not -0); v is no NaN
+  return __double_as_longlong(v) < 0 && (__double_as_longlong(v) << 1) != 0;
+}
+__device__ __forceinline__ bool fp64_in_unit(double v) {  // 0 <= v <= 1, false for a NaN
+  const long long b = __double_as_longlong(v);
+  return (b >= 0 && b <= 0x3FF0000000000000ll) || (b << 1) == 0;
+}
 
 // Apply the results of the pending candidates in the step's order.  ok: the
 // candidates whose logL exceeds logL* (bits).  Returns the accepted candidate
@@ -102,7 +112,7 @@ __device__ __forceinline__ int chain_consume(const SamplerConst& S, ChainState& 
         }
       }
       const double t = w.t[k];
-      if (t < 0.0)
+      if (fp64_negative(t))
         ch.lo = t;
       else
         ch.hi = t;
@@ -204,7 +214,7 @@ __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWor
     for (int k = 0; k < n; ++k) {
       const double tk = lo + (hi - lo) * __shfl_sync(0xffffffffu, u, k);
       if (lane == k) t = tk;
-      if (tk < 0.0)
+      if (fp64_negative(tk))
         lo = tk;
       else
         hi = tk;
@@ -223,7 +233,7 @@ __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWor
     if (on) {
       const double v = ch.x[j] + t * ch.dir[j];
       w.y[lane][j] = v;
-      if (!(v >= 0.0 && v <= 1.0)) inside = false;
+      if (!fp64_in_unit(v)) inside = false;
       // the sky angles go through FP64: the delays need them to ~1e-10
       if (inside)
         w.th[lane][slot] = (S.sky.on && (slot == 9 || slot == 10)) ? prior_slot_inverse(S.prior[slot], v)

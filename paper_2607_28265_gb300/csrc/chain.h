@@ -25,13 +25,14 @@ enum ChainMode { CHAIN_FOLD = 0, CHAIN_HET = 1, CHAIN_HET_TM = 2 };
 struct ChainLayout {
   int scratch_off, scratch_bytes;
   int res_off;            // 0: weights and tables are read from global memory
+  int base_off;           // folded: partial sums of the current point (0: none)
   int anc_off, panel;     // time marginalisation: HetTmLayout's, from scratch_off
   int n_ctas;
   long long spin_limit;
 };
 
 // Bytes before the scratch.
-size_t chain_fixed_bytes(int n_det);
+size_t chain_fixed_bytes(int n_det, int mode);
 void* chain_kernel(int n_det, int mode);
 constexpr int kChainBlock = 512;
 constexpr size_t kChainSmemMax = 224 * 1024;

@@ -396,7 +396,7 @@ __device__ inline void setup_projection_f32(const LikeConst& L, const double* th
       continue;
     }
     float d[6];
-    for (int q = 0; q < 6; ++q) d[q] = (float)L.dten[i][q];
+    for (int q = 0; q < 6; ++q) d[q] = L.dten_f[i][q];
     auto form = [&d](const float* a, const float* b) {
       return a[0] * (d[0] * b[0] + d[1] * b[1] + d[2] * b[2]) + a[1] * (d[1] * b[0] + d[3] * b[1] + d[4] * b[2]) +
              a[2] * (d[2] * b[0] + d[4] * b[1] + d[5] * b[2]);
@@ -444,7 +444,7 @@ __device__ inline void setup_projection_det(const LikeConst& L, const double* th
     float sph = 0.0f, cph = 1.0f;
     if (!L.phase_marg) sincosf((float)th[12], &sph, &cph);
     float d[6];
-    for (int q = 0; q < 6; ++q) d[q] = (float)L.dten[i][q];
+    for (int q = 0; q < 6; ++q) d[q] = L.dten_f[i][q];
     auto form = [&d](const float* a, const float* b) {
       return a[0] * (d[0] * b[0] + d[1] * b[1] + d[2] * b[2]) + a[1] * (d[1] * b[0] + d[3] * b[1] + d[4] * b[2]) +
              a[2] * (d[2] * b[0] + d[4] * b[1] + d[5] * b[2]);

@@ -234,18 +234,18 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
         for (int it = tw, sub = 0, blk = tw; it < 4 * np32; it += T, blk += T) {
           while (blk >= np32) blk -= np32, ++sub;
           const int q = 32 * blk + lane;
-          if (q < np && !fold_anchor<NDET>(tab, ld, s_in[team], sub, base + q, an + q * kFoldAnchor)) s_bad[team] = 1;
+          if (q < np && !fold_anchor<NDET>(tab, ld, s_in[team], sub, base + q, q, an + q * kFoldAnchor)) s_bad[team] = 1;
         }
         team_sync(team, T);
         for (int q = tid; q < np; q += 32 * T)
-          if (!fold_in_band<NDET>(tab, ld, an + q * kFoldAnchor, base + q)) s_bad[team] = 1;
+          if (!fold_in_band<NDET>(tab, ld, an + q * kFoldAnchor, q, base + q)) s_bad[team] = 1;
         const float* aq = an + tw * kFoldAnchor;
         for (int q = tw; q < np; q += 2 * T, wq += 2 * T * NDET * 32, aq += 2 * T * kFoldAnchor) {
           if (q + T < np) fold_load<NDET>(wq + T * NDET * 32, kind(q + T), x0, s_x, lane, v1);
-          fold_chunk<NDET>(aq, v0, acc);
+          fold_chunk<NDET>(aq, q, v0, acc);
           if (q + T < np) {
             if (q + 2 * T < np) fold_load<NDET>(wq + 2 * T * NDET * 32, kind(q + 2 * T), x0, s_x, lane, v0);
-            fold_chunk<NDET>(aq + T * kFoldAnchor, v1, acc);
+            fold_chunk<NDET>(aq + T * kFoldAnchor, q + T, v1, acc);
           }
         }
         team_sync(team, T);

@@ -49,8 +49,15 @@ __device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
                         : reinterpret_cast<const float*>(&r.tau_hi)[w - 2 * NBASIS];
 }
 
+// An anchor's sixteen values lie in four 16-byte blocks whose order turns with
+// the chunk, so that the lanes' stores (a chunk each, 64 bytes apart) meet 8
+// banks instead of 2.
+__device__ __forceinline__ int fold_block(int q, int b) { return 4 * (b ^ ((q >> 1) & 3)); }
+__device__ __forceinline__ int fold_at(int q, int m) { return fold_block(q, m >> 2) + (m & 3); }
+
 // One quarter (sub 0 .. 3) of the anchor of chunk q for the evaluation `r` (a
-// FoldIn or an EvalRecord), written to out[kFoldAnchor]:
+// FoldIn or an EvalRecord), written to out[kFoldAnchor], value m at fold_at(sw, m)
+// (sw: the chunk's place in its panel):
 //   sub 0: out[i] = frac(P(f_c) + f_c tau_i), double-float sums;
 //   sub 1: out[4], out[5] = the scaled slope h (P'(f_c) + tau_0 - s) as a
 //          double-float, out[5 + i] = h (tau_i - tau_0), i = 1 .. 3;
@@ -62,7 +69,7 @@ __device__ __forceinline__ float fold_in_word(const EvalRecord& r, int w) {
 // share it (a lane per chunk took 2.2x as long alone).
 template <int NDET, typename Rec>
 __device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int ld, const Rec& r, int sub, int q,
-                                            float* out) {
+                                            int sw, float* out) {
   const float* T = tab + q;
   auto row = [&](int k) { return T[k * ld]; };
   if (sub == 0) {
@@ -72,18 +79,18 @@ __device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int l
       A = df_add(A, df_mul(dfl{r.c_hi[j], r.c_lo[j]}, dfl{row(FR_VAL_HI + j), row(FR_VAL_LO + j)}));
     const dfl fc = {row(FR_FC_HI), row(FR_FC_LO)};
 #pragma unroll
-    for (int i = 0; i < NDET; ++i) out[i] = df_frac(df_add(A, df_mul(fc, dfl{r.tau_hi[i], r.tau_lo[i]})));
+    for (int i = 0; i < NDET; ++i) out[fold_at(sw, i)] = df_frac(df_add(A, df_mul(fc, dfl{r.tau_hi[i], r.tau_lo[i]})));
   } else if (sub == 1) {
     const dfl h = {row(FR_H_HI), row(FR_H_LO)};
     dfl S = df_add(df_mul(h, dfl{r.tau_hi[0], r.tau_lo[0]}), dfl{-row(FR_SM_HI), -row(FR_SM_LO)});
 #pragma unroll
     for (int j = 0; j < kFoldSlopes; ++j)
       S = df_add(S, df_mul(dfl{r.c_hi[j], r.c_lo[j]}, dfl{row(FR_D1_HI + j), row(FR_D1_LO + j)}));
-    out[4] = S.hi;
-    out[5] = S.lo;
+    out[fold_at(sw, 4)] = S.hi;
+    out[fold_at(sw, 5)] = S.lo;
 #pragma unroll
     for (int i = 1; i < NDET; ++i)
-      out[5 + i] = h.hi * ((r.tau_hi[i] - r.tau_hi[0]) + (r.tau_lo[i] - r.tau_lo[0]));
+      out[fold_at(sw, 5 + i)] = h.hi * ((r.tau_hi[i] - r.tau_hi[0]) + (r.tau_lo[i] - r.tau_lo[0]));
   } else {
     const int n0 = sub == 2 ? 2 : 3, nn = sub == 2 ? 4 : 3;
     float a[4] = {0.0f, 0.0f, 0.0f, 0.0f}, R = 0.0f;
@@ -97,25 +104,160 @@ __device__ __forceinline__ bool fold_anchor(const float* __restrict__ tab, int l
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m)
-      if (m < nn) out[7 + n0 + 2 * m] = a[m];
+      if (m < nn) out[fold_at(sw, 7 + n0 + 2 * m)] = a[m];
     return R <= kFoldTaylorEps;  // false for a NaN as well
   }
   return true;
+}
+
+// Two evaluations' inputs interleaved: (hi a, hi b, lo a, lo b) per coefficient
+// and time shift.
+struct FoldPair {
+  float4 c[NBASIS], tau[SWIG_MAX_DET];
+};
+// Word j (0 .. 14) of a pair's inputs from their records (16 threads).
+__device__ __forceinline__ void fold_pair_set(FoldPair& in, int j, const EvalRecord& a, const EvalRecord& b) {
+  if (j < NBASIS)
+    in.c[j] = make_float4(a.c_hi[j], b.c_hi[j], a.c_lo[j], b.c_lo[j]);
+  else if (j < NBASIS + SWIG_MAX_DET)
+    in.tau[j - NBASIS] = make_float4(a.tau_hi[j - NBASIS], b.tau_hi[j - NBASIS], a.tau_lo[j - NBASIS], b.tau_lo[j - NBASIS]);
+}
+__device__ __forceinline__ DflN<2> fold_dfl2(const float4& v) { return {f2_make(v.x, v.y), f2_make(v.z, v.w)}; }
+// The basis functions of the spin terms come last in every sum, so that the
+// sums over the others can be kept while only spins, sky or t_c move.
+__device__ constexpr int kFoldRest[NBASIS - 2] = {B_M53, B_M1, B_LOG, B_P13, B_P13LOG, B_P23, B_P53, B_P73, B_ONE};
+__device__ constexpr int kFoldSpin[2] = {B_M23, B_M13};
+
+// One quarter of the anchors of chunk q for two evaluations (fold_anchor on
+// packed pairs), to oa and ob.  base: the sums over kFoldRest of a point with
+// the same masses and tides (rows: value hi, lo, slope hi, lo, a_2 .. a_8), or
+// null.  Returns the evaluations (bits) whose Taylor remainder is too large.
+template <int NDET>
+__device__ __forceinline__ int fold_anchor_pair(const float* __restrict__ tab, int ld, const FoldPair& in,
+                                                const float* __restrict__ base, int sub, int q, int sw, float* oa,
+                                                float* ob) {
+  using O = PkOps<2>;
+  const float* T = tab + q;
+  auto row = [&](int k) { return O::all(T[k * ld]); };
+  auto put = [&](int m, f2 v) { f2_split(v, oa[fold_at(sw, m)], ob[fold_at(sw, m)]); };
+  auto pre = [&](int k) { return O::all(base[k * ld + q]); };
+  if (sub == 0) {
+    DflN<2> A = {O::all(0.0f), O::all(0.0f)};
+    auto add = [&](int j) {
+      A = dfn_add<2>(A, dfn_mul<2>(fold_dfl2(in.c[j]), DflN<2>{row(FR_VAL_HI + j), row(FR_VAL_LO + j)}));
+    };
+    if (base) {
+      A = {pre(0), pre(1)};
+    } else {
+#pragma unroll
+      for (int r = 0; r < NBASIS - 2; ++r) add(kFoldRest[r]);
+    }
+    add(kFoldSpin[0]);
+    add(kFoldSpin[1]);
+    const DflN<2> fc = {row(FR_FC_HI), row(FR_FC_LO)};
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) put(i, dfn_frac<2>(dfn_add<2>(A, dfn_mul<2>(fc, fold_dfl2(in.tau[i])))));
+  } else if (sub == 1) {
+    DflN<2> S = {O::all(0.0f), O::all(0.0f)};
+    auto add = [&](int j) {
+      S = dfn_add<2>(S, dfn_mul<2>(fold_dfl2(in.c[j]), DflN<2>{row(FR_D1_HI + j), row(FR_D1_LO + j)}));
+    };
+    if (base) {
+      S = {pre(2), pre(3)};
+    } else {
+#pragma unroll
+      for (int r = 0; r < NBASIS - 3; ++r) add(kFoldRest[r]);  // (the constant has no slope)
+    }
+    add(kFoldSpin[0]);
+    add(kFoldSpin[1]);
+    const DflN<2> h = {row(FR_H_HI), row(FR_H_LO)};
+    S = dfn_add<2>(S, dfn_add<2>(dfn_mul<2>(h, fold_dfl2(in.tau[0])), DflN<2>{O::all(-T[FR_SM_HI * ld]), O::all(-T[FR_SM_LO * ld])}));
+    put(4, S.hi);
+    put(5, S.lo);
+    const DflN<2> t0 = fold_dfl2(in.tau[0]);
+#pragma unroll
+    for (int i = 1; i < NDET; ++i) {
+      const DflN<2> ti = fold_dfl2(in.tau[i]);
+      put(5 + i, O::mul(h.hi, O::add(pk_sub<2>(ti.hi, t0.hi), pk_sub<2>(ti.lo, t0.lo))));
+    }
+  } else {
+    const int n0 = sub == 2 ? 2 : 3, nn = sub == 2 ? 4 : 3;
+    f2 a[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) a[m] = base && m < nn ? pre(2 + n0 + 2 * m) : O::all(0.0f);
+    auto add = [&](int j) {
+      const f2 c = f2_make(in.c[j].x, in.c[j].y);
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (m < nn) a[m] = O::fma(c, row(FR_POLY + (n0 + 2 * m - 2) * kFoldSlopes + j), a[m]);
+    };
+    if (!base) {
+#pragma unroll
+      for (int r = 0; r < NBASIS - 3; ++r) add(kFoldRest[r]);
+    }
+    add(kFoldSpin[0]);
+    add(kFoldSpin[1]);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (m < nn) put(7 + n0 + 2 * m, a[m]);
+    if (sub == 3) {
+      float ra = 0.0f, rb = 0.0f;
+#pragma unroll
+      for (int j = 0; j < kFoldSlopes; ++j) {
+        const float b = T[(FR_BND + j) * ld];
+        ra = fmaf(fabsf(in.c[j].x), b, ra);
+        rb = fmaf(fabsf(in.c[j].y), b, rb);
+      }
+      return (ra <= kFoldTaylorEps ? 0 : 1) | (rb <= kFoldTaylorEps ? 0 : 2);
+    }
+  }
+  return 0;
+}
+
+// The same quarter's sums over kFoldRest of one point (both halves of `in`) into
+// base (kFoldBaseRows rows of ldb).
+__device__ __forceinline__ void fold_base(const float* __restrict__ tab, int ld, const FoldPair& in, int sub, int q,
+                                          float* base, int ldb) {
+  const float* T = tab + q;
+  auto put = [&](int k, float v) { base[k * ldb + q] = v; };
+  if (sub < 2) {
+    DflN<1> A = {0.0f, 0.0f};
+    const int n = sub == 0 ? NBASIS - 2 : NBASIS - 3;
+    for (int r = 0; r < n; ++r) {
+      const int j = kFoldRest[r];
+      const int hi = sub == 0 ? FR_VAL_HI + j : FR_D1_HI + j, lo = sub == 0 ? FR_VAL_LO + j : FR_D1_LO + j;
+      A = dfn_add<1>(A, dfn_mul<1>(DflN<1>{in.c[j].x, in.c[j].z}, DflN<1>{T[hi * ld], T[lo * ld]}));
+    }
+    put(2 * sub, A.hi);
+    put(2 * sub + 1, A.lo);
+  } else {
+    const int n0 = sub == 2 ? 2 : 3, nn = sub == 2 ? 4 : 3;
+    float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int r = 0; r < NBASIS - 3; ++r) {
+      const int j = kFoldRest[r];
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (m < nn) a[m] = fmaf(in.c[j].x, T[(FR_POLY + (n0 + 2 * m - 2) * kFoldSlopes + j) * ld], a[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (m < nn) put(2 + n0 + 2 * m, a[m]);
+  }
 }
 
 // Whether the finished anchor of chunk q keeps below the chunk's bandwidth
 // (kernels.h FR_LIM): |slope| + sum_n n a^(n-1) |a_n| in cycles, a the half
 // axis of the Bernstein ellipse of the interpolation bound.
 template <int NDET>
-__device__ __forceinline__ bool fold_in_band(const float* __restrict__ tab, int ld, const float* an, int q) {
+__device__ __forceinline__ bool fold_in_band(const float* __restrict__ tab, int ld, const float* an, int sw, int q) {
   float b = 0.0f;
 #pragma unroll
-  for (int i = 1; i < NDET; ++i) b = fmaxf(b, fabsf(an[5 + i]));
-  float om = fabsf(an[4]) + b, g = 1.0f;
+  for (int i = 1; i < NDET; ++i) b = fmaxf(b, fabsf(an[fold_at(sw, 5 + i)]));
+  float om = fabsf(an[fold_at(sw, 4)]) + b, g = 1.0f;
 #pragma unroll
   for (int n = 2; n <= kFoldDeg; ++n) {
     g *= kFoldEllipse;
-    om = fmaf((float)n * g, fabsf(an[7 + n]), om);
+    om = fmaf((float)n * g, fabsf(an[fold_at(sw, 7 + n)]), om);
   }
   return om <= tab[FR_LIM * ld + q];  // false for a NaN as well
 }
@@ -160,11 +302,13 @@ __device__ __forceinline__ void fold_load(const float4* __restrict__ w, int kind
 // E - O, so the polynomial is formed once for both; the slope's product with x
 // is carried in double-float and reduced to its fractional part.
 template <int NDET>
-__device__ __forceinline__ void fold_chunk(const float* __restrict__ an, const FoldNode<NDET>& v,
+__device__ __forceinline__ void fold_chunk(const float* __restrict__ an, int sw, const FoldNode<NDET>& v,
                                            FoldAcc<NDET>& acc) {
   const float2 xv = v.x;
-  const float4 A = *reinterpret_cast<const float4*>(an), B = *reinterpret_cast<const float4*>(an + 4);
-  const float4 C = *reinterpret_cast<const float4*>(an + 8), D = *reinterpret_cast<const float4*>(an + 12);
+  const float4 A = *reinterpret_cast<const float4*>(an + fold_block(sw, 0));
+  const float4 B = *reinterpret_cast<const float4*>(an + fold_block(sw, 1));
+  const float4 C = *reinterpret_cast<const float4*>(an + fold_block(sw, 2));
+  const float4 D = *reinterpret_cast<const float4*>(an + fold_block(sw, 3));
   const float x = xv.x, x2 = x * x;
   // C = (b_3, a_2, a_3, a_4), D = (a_5, a_6, a_7, a_8)
   const float ev = x2 * fmaf(x2, fmaf(x2, fmaf(x2, D.w, D.y), C.w), C.y);

@@ -442,13 +442,12 @@ __device__ __forceinline__ void het_in_set(HetIn<NDET, N>& in, int k, const HetP
 // sub 1 a_1, 1 / S and the exact flag, sub 2 and 3 the Taylor terms (het_anchor
 // has them all for one evaluation on one thread).
 template <int NDET, int N>
-__device__ __forceinline__ void het_anchor_part(const HetTables& H, const HetIn<NDET, N>& in, int sub, int q,
-                                                float* out) {
+__device__ __forceinline__ void het_anchor_part(const float* __restrict__ chunk, int nc, const HetIn<NDET, N>& in,
+                                                int sub, int q, float* out) {
   using O = PkOps<N>;
   using T = typename O::T;
-  const int nc = H.n_chunks;
-  const float* tab = H.chunk + q;
-  auto row = [&](int r) { return O::all(__ldg(tab + r * nc)); };
+  const float* tab = chunk + q;
+  auto row = [&](int r) { return O::all(tab[r * nc]); };
   auto put = [&](int m, T v) { *reinterpret_cast<T*>(out + N * m) = v; };
   auto dc = [&](int j) { return DflN<N>{O::load(in.dc_hi[j]), O::load(in.dc_lo[j])}; };
   if (sub == 0) {
@@ -496,9 +495,10 @@ __device__ __forceinline__ void het_anchor_part(const HetTables& H, const HetIn<
 
 // Anchors of np chunks from q0 on for `sets` groups of N evaluations by the
 // warps first, first + stride, ... of a CTA: quarter by quarter, 32 chunks per
-// warp and turn.  Group g's anchors at s_an + (g panel + q) N kHetAncStride.
+// warp and turn.  chunk: H.chunk or its copy in shared memory.  Group g's anchors at s_an + (g panel + q)
+// kHetAncPair (N = 2) or kHetAncOne.
 template <int NDET, int N>
-__device__ __forceinline__ void het_anchors(const HetTables& H, const HetIn<NDET, N>* in, int sets, int q0, int np,
+__device__ __forceinline__ void het_anchors(const HetTables& H, const float* chunk, const HetIn<NDET, N>* in, int sets, int q0, int np,
                                             int panel, float* s_an, int first, int stride, int lane) {
   const int nb = (np + 31) >> 5, per = sets * nb;  // warp turns of a quarter
   for (int sub = 0, t = first; sub < 4;) {
@@ -509,7 +509,7 @@ __device__ __forceinline__ void het_anchors(const HetTables& H, const HetIn<NDET
     }
     const int g = t / nb, q = 32 * (t - g * nb) + lane;
     if (q < np)
-      het_anchor_part<NDET, N>(H, in[g], sub, q0 + q, s_an + (size_t)(g * panel + q) * N * kHetAncStride);
+      het_anchor_part<NDET, N>(chunk, H.n_chunks, in[g], sub, q0 + q, s_an + (size_t)(g * panel + q) * (N == 2 ? kHetAncPair : kHetAncOne));
     t += stride;
   }
 }
@@ -603,8 +603,8 @@ __device__ __forceinline__ void het_detector(const LikeConst& L, const EvalRecor
   Z[1] = cr * ki + ci * kr;
   const double b = (L.het_b0[i] - dsum) * iden;
   *hh = (cr * cr + ci * ci) * b;
-  kap2[0] = kr / L.inv_scale[i];
-  kap2[1] = ki / L.inv_scale[i];
+  kap2[0] = kr * L.rscale[i];
+  kap2[1] = ki * L.rscale[i];
   *vv = b * (L.amp1 * L.amp1);
 }
 
@@ -620,13 +620,13 @@ __device__ inline void het_products(const HetTables& H, const HetPrep<NDET>& pre
   for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
     const int np = min(panel, H.n_chunks - q0);
     __syncthreads();
-    het_anchors<NDET, 1>(H, &in, 1, q0, np, panel, s_an, warp, n_warps, lane);
+    het_anchors<NDET, 1>(H, H.chunk, &in, 1, q0, np, panel, s_an, warp, n_warps, lane);
     __syncthreads();
     for (int q = warp; q < np; q += n_warps) {
       float4 w[NDET];
 #pragma unroll
       for (int i = 0; i < NDET; ++i) w[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
-      het_edges<NDET, 1, true>(H, s_an + q * kHetAncStride, in, pp, q0 + q, lane, w, acc, y);
+      het_edges<NDET, 1, true>(H, s_an + q * kHetAncOne, in, pp, q0 + q, lane, w, acc, y);
     }
   }
 }

@@ -83,6 +83,10 @@ constexpr int kHetAncPhase = kHetPoly + 1;
 constexpr int kHetAncInvS = kHetAncPhase + SWIG_MAX_DET;
 constexpr int kHetAncExact = kHetAncInvS + 1;
 static_assert(kHetAncExact < kHetAncStride, "chunk anchor layout");
+// Floats from one chunk's anchor to the next: two evaluations interleaved, and
+// one, padded so that the lanes' stores (a chunk each) meet all banks.
+constexpr int kHetAncPair = 2 * kHetAncStride + 2;
+constexpr int kHetAncOne = kHetAncStride + 1;
 // Per-warp shared-memory stage of one chunk's table data (summary data, bin
 // widths, edge offsets), filled by cp.async one chunk ahead: bytes per stage.
 inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) + 2 * 32 * 4; }
@@ -97,6 +101,7 @@ inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) 
 // [cycles] and the node kind (an int's bits).
 constexpr int kFoldNodes = 64;
 constexpr int kFoldAnchorFloats = 16;  // per (evaluation, chunk)
+constexpr int kFoldBaseRows = 11;      // rows [ld] of a point's partial sums (fold.cuh fold_base)
 constexpr int kFoldDeg = 8;
 constexpr int kFoldSlopes = NBASIS - 1;
 enum FoldRow {
@@ -210,7 +215,7 @@ struct HetTmLayout {
 inline HetTmLayout het_tm_layout(const LikeConst& L, const DeviceBuffers& B) {
   HetTmLayout lay;
   lay.panel = B.het_nc < 128 ? B.het_nc : 128;
-  const size_t anc = (size_t)lay.panel * kHetAncStride * sizeof(float);
+  const size_t anc = (size_t)lay.panel * kHetAncOne * sizeof(float);
   const size_t ys = (((size_t)B.het_nb + 1) * 2 * sizeof(float) + 15) / 16 * 16;
   lay.bytes = (het_tm_smem_bytes(B.het_nb, L.tm_M, L.tm_M > 0 ? L.tm_pieces : 0) + 15) / 16 * 16;
   if ((size_t)L.tm_M * 2 * sizeof(float) >= anc) {

@@ -346,7 +346,7 @@ template <int NDET>
 __global__ void __launch_bounds__(kHetTmThreads, 1)
     k_het(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, int per, double* __restrict__ out,
           double* __restrict__ kappa_out, double* __restrict__ vv_out) {
-  extern __shared__ __align__(16) float s_an[];  // [pairs][kHetPanel][kHetAncStride][2]
+  extern __shared__ __align__(16) float s_an[];  // [pairs][panel][kHetAncPair]
   __shared__ HetPrep<NDET> s_prep[kHetBatch];
   __shared__ HetIn<NDET, 2> s_in[kHetBatch / 2];
   __shared__ float s_part[kHetWarps][NDET][3 * kHetBatch];
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
       const int np = min(panel, H.n_chunks - q0);
       __syncthreads();
-      het_anchors<NDET, 2>(H, s_in, pairs, q0, np, panel, s_an, warp, kHetWarps, lane);
+      het_anchors<NDET, 2>(H, H.chunk, s_in, pairs, q0, np, panel, s_an, warp, kHetWarps, lane);
       __syncthreads();
       for (int q = warp; q < np; q += kHetWarps) {
         float4 w[NDET];
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
         for (int p = 0; p < kHetBatch / 2; ++p)
           if (p < pairs) {
             const HetPrep<NDET>* pp[2] = {&s_prep[2 * p], &s_prep[2 * p + 1]};
-            het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * 2 * kHetAncStride, s_in[p], pp, q0 + q, lane, w,
+            het_edges<NDET, 2>(H, s_an + ((size_t)p * panel + q) * kHetAncPair, s_in[p], pp, q0 + q, lane, w,
                                acc[p]);
           }
       }
@@ -501,7 +501,7 @@ cudaError_t launch_het_plain(const LikeConst& L, const DeviceBuffers& B, int n, 
   int per = (n + L.sm_count - 1) / L.sm_count;
   per = per < kHetBatch ? per : kHetBatch;
   const int panel = B.het_nc < kHetPanel ? B.het_nc : kHetPanel, ctas = (n + per - 1) / per;
-  const size_t bytes = (size_t)((per + 1) / 2) * panel * 2 * kHetAncStride * sizeof(float);
+  const size_t bytes = (size_t)((per + 1) / 2) * panel * kHetAncPair * sizeof(float);
   const cudaError_t e = cudaFuncSetAttribute(k_het<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   k_het<NDET><<<ctas < L.sm_count ? ctas : L.sm_count, kHetTmThreads, bytes, st>>>(L, het_tables(B), B.rec, n, per, out,

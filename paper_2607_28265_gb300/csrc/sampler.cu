@@ -916,11 +916,13 @@ int run_setup(swig_ctx* c, RunState& R) {
   // the partial buffers hold 4 per slice and theta)
   S.flow_parts = c->cfg.flow_parts > 0 ? c->cfg.flow_parts : SWIG_FLOW_PARTS;
   // chain sampler: candidates per round (chain.cuh).  Four rungs per end and
-  // four draws unless a smaller launch shape is asked for; with t_c marginalised
+  // two draws unless a smaller launch shape is asked for (first iterations of the
+  // 128 s run, ms: (rungs, draws) = (4, 2) 16.0, (4, 3) 16.4, (4, 4) 16.7, (4, 8)
+  // 18.3, (3, 3) 17.8, (2, 4) 19.8; heterodyned 45.8, 46.9, 47.5, 52.9, 49.8, 55.8); with t_c marginalised
   // an evaluation costs as much as a round's latency: one at a time
   const int shape = c->cfg.flow_parts;
   S.spec_out = L.tm_n > 0 ? 1 : shape >= 3 ? 1 : shape == 2 ? 2 : 4;
-  S.spec_shr = L.tm_n > 0 ? 1 : shape >= 4 ? 1 : shape >= 2 ? 2 : 4;
+  S.spec_shr = L.tm_n > 0 ? 1 : shape >= 4 ? 1 : 2;
   S.one_end = c->cfg.stepout_one_end ? 1 : 0;
   // learned proposal: retrain every learn_interval iterations (one launch each)
   R.learned = c->cfg.proposal == SWIG_PROPOSAL_LEARNED;
@@ -943,13 +945,13 @@ int run_setup(swig_ctx* c, RunState& R) {
     R.mode = mixed ? CHAIN_FOLD : L.tm_n > 0 ? CHAIN_HET_TM : CHAIN_HET;
     ChainLayout& y = R.lay;
     std::memset(&y, 0, sizeof(y));
-    y.scratch_off = (int)chain_fixed_bytes(L.n_det);
+    y.scratch_off = (int)chain_fixed_bytes(L.n_det, R.mode);
     size_t scratch = sort_bytes;
     if (R.mode == CHAIN_FOLD) {
       // anchors of eight candidates over every chunk, at least of 64 chunks
       scratch = std::max(scratch, sizeof(float) * kFoldAnchorFloats * 8 * (size_t)std::min(c->B.fold_nc, 128));
     } else if (R.mode == CHAIN_HET) {
-      scratch = std::max(scratch, sizeof(float) * kHetAncStride * 8 * (size_t)std::max(32, std::min(c->B.het_nc, 256)));
+      scratch = std::max(scratch, sizeof(float) * kHetAncPair * 4 * (size_t)std::max(32, std::min(c->B.het_nc, 256)));
     } else {
       const HetTmLayout lay = het_tm_layout(L, c->B);
       y.anc_off = lay.anc_off;
@@ -959,7 +961,19 @@ int run_setup(swig_ctx* c, RunState& R) {
     y.scratch_bytes = (int)((scratch + 15) & ~(size_t)15);
     R.smem = (size_t)y.scratch_off + y.scratch_bytes;
     if (R.mode == CHAIN_FOLD) {
+      const size_t base = sizeof(float) * kFoldBaseRows * fold_ld(c->B.fold_nc);
+      if (R.smem + base <= kChainSmemMax) {
+        y.base_off = (int)R.smem;
+        R.smem += base;
+      }
       const size_t res = fold_resident_bytes(c->B.fold_nc, L.n_det);
+      if (R.smem + res <= kChainSmemMax) {
+        y.res_off = (int)R.smem;
+        R.smem += res;
+      }
+    }
+    if (R.mode == CHAIN_HET) {
+      const size_t res = sizeof(float) * HC_ROWS * (size_t)c->B.het_nc;
       if (R.smem + res <= kChainSmemMax) {
         y.res_off = (int)R.smem;
         R.smem += res;
@@ -1363,13 +1377,18 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
   // shared memory: the largest scratch; weights and tables resident if every
   // event's fit beside it
   ChainLayout lay = R[i0].lay;
-  size_t res = 0;
+  size_t res = 0, base = 0;
   for (int i = i0; i < i1; ++i) {
     lay.scratch_bytes = std::max(lay.scratch_bytes, R[i].lay.scratch_bytes);
     res = std::max(res, fold_resident_bytes(ctxs[i]->B.fold_nc, n_det));
+    base = std::max(base, sizeof(float) * kFoldBaseRows * fold_ld(ctxs[i]->B.fold_nc));
   }
   size_t smem = (size_t)lay.scratch_off + lay.scratch_bytes;
-  lay.res_off = 0;
+  lay.res_off = lay.base_off = 0;
+  if (smem + base <= kChainSmemMax) {
+    lay.base_off = (int)smem;
+    smem += base;
+  }
   if (smem + res <= kChainSmemMax) {
     lay.res_off = (int)smem;
     smem += res;

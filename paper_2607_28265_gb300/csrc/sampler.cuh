@@ -128,7 +128,8 @@ struct SamplerPtrs {
 // Draws built on Philox-4x32-10 (device_common.cuh).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double u01_from(uint4 r) {  // 53-bit uniform in [0, 1)
-  return ((double)(r.x >> 5) * 67108864.0 + (double)(r.y >> 6)) * (1.0 / 9007199254740992.0);
+  const unsigned long long m = ((unsigned long long)(r.x >> 5) << 26) | (r.y >> 6);
+  return (double)m * (1.0 / 9007199254740992.0);
 }
 
 __device__ __forceinline__ double chain_uniform(const SamplerConst& S, ChainState& ch, int c, long long it) {
@@ -207,7 +208,7 @@ __device__ inline double free_loglike_mixed(const LikeConst& L, const double* th
   if (!(mc > 0.0f && dl > 0.0f)) return -INFINITY;
   const float rel = exp2f(0.8333333333f * log2f(mc)) / dl;  // Mc^(5/6) / d_L
   float sl, cl, sd, cd, sp, cp;
-  sincosf(ra - (float)L.gmst, &sl, &cl);
+  sincosf(ra - L.gmst_f, &sl, &cl);
   sincosf(dec, &sd, &cd);
   sincosf(psi, &sp, &cp);
   const float east[3] = {-sl, cl, 0.0f};
@@ -224,7 +225,7 @@ __device__ inline double free_loglike_mixed(const LikeConst& L, const double* th
   float zr = 0.0f, zi = 0.0f, hh = 0.0f;
   for (int i = 0; i < L.n_det; ++i) {
     float d[6];
-    for (int q = 0; q < 6; ++q) d[q] = (float)L.dten[i][q];
+    for (int q = 0; q < 6; ++q) d[q] = L.dten_f[i][q];
     auto form = [&d](const float* a, const float* b) {
       return a[0] * (d[0] * b[0] + d[1] * b[1] + d[2] * b[2]) + a[1] * (d[1] * b[0] + d[3] * b[1] + d[4] * b[2]) +
              a[2] * (d[2] * b[0] + d[4] * b[1] + d[5] * b[2]);
