@@ -32,22 +32,20 @@ constexpr int kMlpOffB2 = kMlpOffW2 + kMlpH * kMlpH;
 constexpr int kMlpOffW3 = kMlpOffB2 + kMlpH;
 constexpr int kMlpOffB3 = kMlpOffW3 + kMlpH * kMlpOut;
 constexpr int kMlpParams = kMlpOffB3 + kMlpOut;  // 76,058
-constexpr int kMlpMaxSplit = 8;                  // split-K partial buffers
+constexpr int kMlpMaxSplit = 8;                  // parts of the rows in the weight gradients
 
 struct Mlp {
-  int cap = 0;  // rows (live points) the buffers hold
+  int cap = 0;  // rows (live points) the buffers hold, each padded to 16 rows
   float* params = nullptr;
   float* adam_m = nullptr;
   float* adam_v = nullptr;
   float* grad = nullptr;
-  int* step = nullptr;  // Adam step counter
+  int step = 0;         // Adam steps taken
   __nv_bfloat16* w1b = nullptr;  // [16][256], rows 13..15 zero
   __nv_bfloat16* w2b = nullptr;  // [256][256]
   __nv_bfloat16* w3b = nullptr;  // [256][32], columns 26..31 zero
   __nv_bfloat16* xb = nullptr;   // [cap][16] standardised inputs
-  float* z1 = nullptr;           // [cap][256]
-  __nv_bfloat16* h1b = nullptr;
-  float* z2 = nullptr;
+  __nv_bfloat16* h1b = nullptr;  // [cap][256]
   __nv_bfloat16* h2b = nullptr;
   float* out = nullptr;           // [cap][32]
   float* dout = nullptr;          // [cap][32]
@@ -60,20 +58,20 @@ struct Mlp {
   float* tls = nullptr;           // [cap][13]
   int* nbr = nullptr;             // [cap][26] neighbour indices
   double* stats = nullptr;        // mean[13], sd[13]
+  double* live = nullptr;         // [cap][d] live points of a call on host buffers
+  double* xs = nullptr;           // [cap][d] standardised coordinates
+  float* xf = nullptr;            // [d][cap] the same in FP32
   double* row_loss = nullptr;     // [cap]
   double* loss = nullptr;         // [1]
-  float* part = nullptr;          // [kMlpMaxSplit][256][256] split-K partials
-  cudaGraphExec_t graph = nullptr;  // one training step for (graph_rows, graph_d)
-  int graph_rows = 0, graph_d = 0, graph_nodes = 0;
-  float graph_lr = 0.0f;
+  int sms = 0;                    // SMs of the device
 };
 
 cudaError_t mlp_alloc(Mlp& M, int cap);
 void mlp_free(Mlp& M);
 // Philox-4x32-10 initial weights N(0, 1/fan_in), biases 0; resets Adam.
 cudaError_t mlp_init(Mlp& M, uint64_t seed, cudaStream_t st, long long* launches);
-// Copy FP32 parameters (device pointer) into the master weights; resets Adam.
-cudaError_t mlp_load(Mlp& M, const float* params_dev, cudaStream_t st, long long* launches);
+// Copy FP32 parameters (host) into the master weights; resets Adam.
+cudaError_t mlp_load(Mlp& M, const float* params, cudaStream_t st, long long* launches);
 // Standardised inputs and training targets of n live points (device, n x d doubles).
 cudaError_t mlp_targets(Mlp& M, const double* live_u, int n, int d, int k, cudaStream_t st, long long* launches);
 // Standardised inputs given directly (device, n x 13 floats).
@@ -82,9 +80,7 @@ cudaError_t mlp_inputs(Mlp& M, const float* x_std, int n, cudaStream_t st, long 
 cudaError_t mlp_forward(Mlp& M, int n, cudaStream_t st, long long* launches);
 // Forward, loss and parameter gradient into M.grad (loss in M.loss).
 cudaError_t mlp_loss_grad(Mlp& M, int n, int d, cudaStream_t st, long long* launches);
-// One Adam step on M.grad (step counter on the device).
-cudaError_t mlp_adam(Mlp& M, float lr, cudaStream_t st, long long* launches);
-// `steps` training steps (loss_grad + adam) replayed from a captured graph.
+// `steps` training steps (gradient and Adam), two kernels each.
 cudaError_t mlp_train(Mlp& M, int n, int d, int steps, float lr, cudaStream_t st, long long* launches);
 
 }  // namespace swig
