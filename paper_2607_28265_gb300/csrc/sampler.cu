@@ -1428,8 +1428,10 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
     }
     NSGlobal g0;
     std::memset(&g0, 0, sizeof(g0));
-    if (e == cudaSuccess) e = cudaMemcpy(gb, &g0, sizeof(g0), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(evd, hd.data(), sizeof(ChainEvent) * hd.size(), cudaMemcpyHostToDevice);
+    // on the launch's stream, which does not wait for the default stream's copies
+    if (e == cudaSuccess) e = cudaMemcpyAsync(gb, &g0, sizeof(g0), cudaMemcpyHostToDevice, c0->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(evd, hd.data(), sizeof(ChainEvent) * hd.size(), cudaMemcpyHostToDevice, c0->stream);
     int n_ev = (int)hd.size();
     void* args[] = {(void*)&evd, (void*)&n_ev, (void*)&gb, (void*)&lay};
     if (e == cudaSuccess) e = cudaEventRecord(ev0, c0->stream);
