@@ -12,8 +12,8 @@
 //
 // Measured (one GB300, first iterations of the 128 s three-detector run, nlive
 // 1000, nrep 100): 4 iterations 145 ms with one candidate at a time across all
-// SMs (a request to every SM's slice of the grid, control on one warp), 18.7 ms
-// here; heterodyned, 8 iterations 133 -> 47.9 ms.  1.3 candidates are evaluated
+// SMs (a request to every SM's slice of the grid, control on one warp), 12.9 ms
+// here; heterodyned, 8 iterations 133 -> 38.3 ms.  1.3 candidates are evaluated
 // per candidate used; with fewer per round the latencies dominate.
 //
 // A round costs its latency once: the set-up's FP64 chains (64 cycles an
@@ -29,6 +29,7 @@
 namespace swig {
 
 constexpr int kCand = 8;          // candidates per round at most
+constexpr int kFreeRungs = 8;     // rungs per end of a projection-only step, and its draws at a time
 constexpr int kChainWarps = kChainBlock / 32;
 constexpr int kFoldGroups = 4;    // groups of chunks (partial sums) of a full round's pairs
 static_assert(kChainBlock == kHetTmThreads, "the sampler and the batched time-marginalised kernel share sum orders");
@@ -48,13 +49,17 @@ struct ChainWork {
   double sc[4][kCand];       // sines and cosines of RA - GMST and Dec
   unsigned inside, act;      // candidate bits: in the unit cube; to be evaluated
   int list[kCand], n_act;    // the latter's numbers
-  int n_cand, n_left;        // candidates; stepping out: of them on the left
+  int n_cand, n_left;        // candidates; stepping out: of them on the left,
+  int n_rung;                // ... on both ends (the others are draws ahead)
+  double lo, hi;             // the bracket that those draws assume
   int fl;                    // record pieces that the block moves
   int status;
   int bad[kCand];            // folded sums: outside the band, summed bin by bin
+  double fth[2 * kFreeRungs][SWIG_N_PARAMS];  // projection-only steps: a lane's theta
 };
 
 enum { ROUND_EVAL = 0, ROUND_DONE = 1 };
+constexpr int kGuess0 = 96;  // of 128: the share of right guesses that a chain starts from
 
 // Sign and unit-interval tests on the bits: an FP64 comparison costs the
 // scheduler 64 cycles.
@@ -66,65 +71,108 @@ __device__ __forceinline__ bool fp64_in_unit(double v) {  // 0 <= v <= 1, false 
   return (b >= 0 && b <= 0x3FF0000000000000ll) || (b << 1) == 0;
 }
 
+// What the rungs of one end say: n of them (candidates first ..), `room` more
+// expansions allowed.  moved: expansions; evals: points that the step looked at;
+// shut: the end stays; left: it left the unit cube.
+struct EndResult {
+  int moved, evals;
+  bool shut, left;
+};
+__device__ __forceinline__ EndResult end_result(unsigned inside, unsigned ok, int first, int n, int room) {
+  const unsigned in = inside >> first, go = in & (ok >> first);
+  EndResult e;
+  e.moved = min(__ffs(~go) - 1, n);
+  const bool more = e.moved < n;  // a rung that was not taken: the end
+  e.left = more && !((in >> e.moved) & 1u);
+  e.evals = e.moved + (more && !e.left);
+  e.shut = more || e.moved >= room;
+  return e;
+}
+
+// theta_valid on the bits.  (A component of 2^1000 or more, whose sum may
+// overflow, takes the sum.)
+__device__ __forceinline__ bool chain_theta_valid(const double* th) {
+  bool big = false;
+#pragma unroll
+  for (int j = 0; j < SWIG_N_PARAMS; ++j) big = big || (__double2hiint(th[j]) & 0x7fffffff) >= (1023 + 1000) << 20;
+  if (big) return theta_valid(th);
+  const long long mc = __double_as_longlong(th[0]), q = __double_as_longlong(th[1]), dl = __double_as_longlong(th[6]);
+  return mc > 0 && q > 0 && q <= 0x3FF0000000000000ll && dl > 0;
+}
+
 // Apply the results of the pending candidates in the step's order.  ok: the
 // candidates whose logL exceeds logL* (bits).  Returns the accepted candidate
-// or -1.  Lane-uniform.
-__device__ __forceinline__ int chain_consume(const SamplerConst& S, ChainState& ch, const ChainWork& w, unsigned ok,
-                                             bool full) {
-  const int n = w.n_cand, nl = w.n_left;
+// or -1.  All lanes compute; lane 0 writes the state.
+__device__ __forceinline__ int chain_consume(const SamplerConst& S, ChainWork& w, unsigned ok, int lane) {
+  ChainState& ch = w.ch;
+  const int n = w.n_cand, nl = w.n_left, nr = w.n_rung;
   const unsigned inside = w.inside;
-  int evals = 0, hit = -1;
-  if (ch.phase == PH_OUT) {
-    for (int k = 0; k < nl && (ch.side & 1); ++k) {
-      if ((inside >> k) & 1u) {
-        ++evals;
-        if ((ok >> k) & 1u) {
-          ch.lo -= 1.0;
-          if (++ch.n_out >= kMaxStepOut) ch.side &= ~1;
-          continue;
-        }
-      }
-      ch.side &= ~1;
+  double lo = ch.lo, hi = ch.hi;
+  int evals = 0, hit = -1, k = 0, phase = ch.phase, n_shrink = ch.n_shrink;
+  if (phase == PH_OUT) {
+    int side = ch.side, closed = ch.closed, out = ch.n_out, outr = ch.n_out_r, score = ch.score;
+    if (nl > 0) {
+      const EndResult e = end_result(inside, ok, 0, nl, kMaxStepOut - out);
+      evals += e.evals;
+      out += e.moved;
+      if (e.moved > 0) lo = e.moved < nl ? w.t[e.moved] : w.t[nl - 1] - 1.0;
+      if (e.shut) side &= ~1;
+      if (e.left) closed |= 1;
     }
-    for (int k = nl; k < n && (ch.side & 2); ++k) {
-      if ((inside >> k) & 1u) {
-        ++evals;
-        if ((ok >> k) & 1u) {
-          ch.hi += 1.0;
-          if (++ch.n_out_r >= kMaxStepOut) ch.side &= ~2;
-          continue;
-        }
-      }
-      ch.side &= ~2;
+    if (nr > nl) {
+      const EndResult e = end_result(inside, ok, nl, nr - nl, kMaxStepOut - outr);
+      evals += e.evals;
+      outr += e.moved;
+      if (e.moved > 0) hi = e.moved < nr - nl ? w.t[nl + e.moved] : w.t[nr - 1] + 1.0;
+      if (e.shut) side &= ~2;
+      if (e.left) closed |= 2;
     }
-    if (ch.side == 0) {
-      ch.phase = PH_SHRINK;
-      ch.n_shrink = 0;
+    k = n;
+    if (side == 0) {
+      phase = PH_SHRINK;
+      n_shrink = 0;
+      score += 16 * (closed == 3) - ((kGuess0 + score) >> 3);
+      closed = 0;
+      // the draws ahead stand if the bracket became the one they assume
+      if (__double_as_longlong(lo) == __double_as_longlong(w.lo) &&
+          __double_as_longlong(hi) == __double_as_longlong(w.hi))
+        k = nr;
     }
-  } else {
-    for (int k = 0; k < n; ++k) {
-      ++ch.ctr;  // its uniform
-      if ((inside >> k) & 1u) {
-        ++evals;
-        if ((ok >> k) & 1u) {
-          hit = k;
-          break;
-        }
-      }
-      const double t = w.t[k];
-      if (fp64_negative(t))
-        ch.lo = t;
-      else
-        ch.hi = t;
-      if (++ch.n_shrink >= kMaxShrink) {
-        ++ch.n_caps;
-        finish_step(S, ch);
+    __syncwarp();
+    if (lane == 0) ch.side = side, ch.closed = closed, ch.n_out = out, ch.n_out_r = outr, ch.score = score;
+  }
+  bool capped = false;
+  unsigned ctr = ch.ctr;
+  for (; k < n; ++k) {
+    ++ctr;  // its uniform
+    if ((inside >> k) & 1u) {
+      ++evals;
+      if ((ok >> k) & 1u) {
+        hit = k;
         break;
       }
     }
+    const double t = w.t[k];
+    if (fp64_negative(t))
+      lo = t;
+    else
+      hi = t;
+    if (++n_shrink >= kMaxShrink) {
+      capped = true;
+      break;
+    }
   }
-  ch.n_evals += evals;
-  if (full) ch.n_full += evals;
+  __syncwarp();
+  if (lane == 0) {
+    ch.lo = lo, ch.hi = hi, ch.phase = phase, ch.n_shrink = n_shrink, ch.ctr = ctr;
+    ch.n_evals += evals;
+    ch.n_full += evals;
+    if (capped) {
+      ++ch.n_caps;
+      finish_step(S, ch);
+    }
+  }
+  __syncwarp();
   return hit;
 }
 
@@ -156,6 +204,10 @@ __device__ __forceinline__ void chain_start_step(const SamplerConst& S, ChainSta
     learned = true;
   }
   if (!learned) {
+    const float* Lb = chol + (size_t)b * kMaxDim * kMaxDim;
+    float row[kMaxDim];  // (CTA 0 writes L_b: through L2)
+#pragma unroll
+    for (int q = 0; q < kMaxDim; ++q) row[q] = q < nb && q <= lane && lane < nb ? __ldcg(&Lb[lane * kMaxDim + q]) : 0.0f;
     // z_r, r < nb, one Philox block each at consecutive counters
     float z = 0.0f;
     if (lane < nb) {
@@ -165,12 +217,13 @@ __device__ __forceinline__ void chain_start_step(const SamplerConst& S, ChainSta
       z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
     }
     ctr += (unsigned)nb;
-    const float* Lb = chol + (size_t)b * kMaxDim * kMaxDim;
     float v = 0.0f;
-    for (int q = 0; q < nb; ++q) {
-      const float zq = __shfl_sync(0xffffffffu, z, q);
-      if (lane < nb && q <= lane) v = fmaf(__ldcg(&Lb[lane * kMaxDim + q]), zq, v);  // CTA 0 writes L_b
-    }
+#pragma unroll
+    for (int q = 0; q < kMaxDim; ++q)
+      if (q < nb) {
+        const float zq = __shfl_sync(0xffffffffu, z, q);
+        if (lane < nb && q <= lane) v = fmaf(row[q], zq, v);
+      }
     const float vd = __shfl_sync(0xffffffffu, v, lane < S.ndim ? S.block_rank[lane] : 0);
     if (inb) dir = (double)vd;
   }
@@ -190,28 +243,25 @@ __device__ __forceinline__ void chain_start_step(const SamplerConst& S, ChainSta
 
 // The round's candidates: bracket coordinates, points and theta, one candidate
 // per lane, written to w.  All lanes.
+//
+// While most steps come to the cube's boundary on both ends (75 % in a run's
+// first iterations, 22 % late), a round that steps out also takes the first
+// draws of the shrinkage, from the bracket that this would leave: both ends at
+// the last rung inside.  A right guess saves the step a round; a wrong one costs
+// two candidates.  Taken where the guess held for half of the chain's last eight
+// steps or so (late, with either this guess or that neither end moves, the
+// candidates cost more than the rounds: 250 iterations 1.28 -> 1.43 s).
 __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWork& w, int c, long long it, int lane) {
   ChainState& ch = w.ch;
   const int b = ch.block, nb = S.block_size[b];
-  int n, nl = 0;
-  double t = 0.0;
-  if (ch.phase == PH_OUT) {
-    const bool l = ch.side & 1, r = (ch.side & 2) && !(S.one_end && l);
-    // an end alone may use both ends' rungs
-    const int d = l && r ? S.spec_out : min(2 * S.spec_out, kCand);
-    nl = l ? min(d, kMaxStepOut - ch.n_out) : 0;
-    n = nl + (r ? min(d, kMaxStepOut - ch.n_out_r) : 0);
-    // rung by rung, as the step moves its end (each addition rounds)
-    const int m = lane < nl ? lane : lane - nl;
-    t = lane < nl ? ch.lo : ch.hi;
-    for (int i = 1; i < max(nl, n - nl); ++i)
-      if (i <= m) t += lane < nl ? -1.0 : 1.0;
-  } else {
-    n = min(S.spec_shr, kMaxShrink - ch.n_shrink);
-    const double u = u01_from(philox4x32_10(make_uint4(ch.ctr + (unsigned)lane, (unsigned)c, (unsigned)it, 0u), S.key0,
-                                            S.key1));
-    double lo = ch.lo, hi = ch.hi;
-    for (int k = 0; k < n; ++k) {
+  const auto at = [&](int j, double t) { return ch.x[j] + t * ch.dir[j]; };
+  // draws first .. first + n - 1 (lanes) of a bracket, each after the ones
+  // before it were rejected
+  const auto draws = [&](double lo, double hi, int first, int n) {
+    const double u = u01_from(philox4x32_10(make_uint4(ch.ctr + (unsigned)(lane - first), (unsigned)c, (unsigned)it, 0u),
+                                            S.key0, S.key1));
+    double t = 0.0;
+    for (int k = first; k < first + n; ++k) {
       const double tk = lo + (hi - lo) * __shfl_sync(0xffffffffu, u, k);
       if (lane == k) t = tk;
       if (fp64_negative(tk))
@@ -219,6 +269,53 @@ __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWor
       else
         hi = tk;
     }
+    return t;
+  };
+  int n, nl = 0, nr = 0;
+  double t = 0.0;
+  if (ch.phase == PH_OUT) {
+    const bool l = ch.side & 1, r = (ch.side & 2) && !(S.one_end && l);
+    // an end alone may use both ends' rungs; rungs 0 .. 7 on lanes 0 .. 7
+    // (left) and 8 .. 15 (right)
+    const int d = l && r ? S.spec_out : min(2 * S.spec_out, kCand);
+    const int dl = l ? min(d, kMaxStepOut - ch.n_out) : 0, dr = r ? min(d, kMaxStepOut - ch.n_out_r) : 0;
+    const bool right = lane & 8;
+    const int m = lane & 7;
+    // rung by rung, as the step moves its end (each addition rounds)
+    t = right ? ch.hi : ch.lo;
+    for (int i = 1; i < max(dl, dr); ++i)
+      if (i <= m) t += right ? 1.0 : -1.0;
+    bool in = lane < 16 && m < (right ? dr : dl);
+    if (in)
+      for (int q = 0; q < nb; ++q)
+        if (!fp64_in_unit(at(S.block_dims[b][q], t))) in = false;
+    const unsigned ins = __ballot_sync(0xffffffffu, in);
+    // rungs inside the cube in a row; the next one closes the end unseen
+    const int cl = __ffs(~(ins & 0xffu)) - 1, cr = __ffs(~((ins >> 8) & 0xffu)) - 1;
+    nl = min(cl + 1, dl);
+    nr = nl + min(cr + 1, dr);
+    const double lo = l ? __shfl_sync(0xffffffffu, t, min(cl, 7)) : ch.lo;
+    const double hi = r ? __shfl_sync(0xffffffffu, t, 8 + min(cr, 7)) : ch.hi;
+    // (a guess needs the rungs that leave the cube, on every open end)
+    const bool ahead = S.spec_mix > 0 && kGuess0 + ch.score >= 64 && r == ((ch.side & 2) != 0) &&
+                       (!l || cl < dl) && (!r || cr < dr);
+    int nd = 0;
+    if (ahead) {
+      nd = S.spec_mix;
+      if (nd > 1) nd += (min(cl, dl) + min(cr, dr) + nd) & 1;  // candidates go in pairs
+      nd = min(nd, kCand - nr);
+    }
+    n = nr + nd;
+    t = __shfl_sync(0xffffffffu, t, lane < nl ? lane : lane < nr ? 8 + lane - nl : 0);
+    const double td = draws(lo, hi, nr, nd);
+    if (lane >= nr) t = td;
+    if (lane == 0) {
+      w.lo = lo;
+      w.hi = hi;
+    }
+  } else {
+    n = min(S.spec_shr, kMaxShrink - ch.n_shrink);
+    t = draws(ch.lo, ch.hi, 0, n);
   }
   const bool on = lane < n;
   bool inside = on;
@@ -231,7 +328,7 @@ __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWor
   for (int r = 0; r < nb; ++r) {
     const int j = S.block_dims[b][r], slot = S.slot_of_dim[j];
     if (on) {
-      const double v = ch.x[j] + t * ch.dir[j];
+      const double v = at(j, t);
       w.y[lane][j] = v;
       if (!fp64_in_unit(v)) inside = false;
       // the sky angles go through FP64: the delays need them to ~1e-10
@@ -246,30 +343,137 @@ __device__ __forceinline__ void chain_candidates(const SamplerConst& S, ChainWor
   if (lane == 0) {
     w.n_cand = n;
     w.n_left = nl;
+    w.n_rung = nr;
     w.inside = m;
   }
   __syncwarp();
 }
 
-// Accept candidate k: point, theta, logL and, from a full evaluation, the
-// per-detector sums and the record.  All lanes.
-__device__ __forceinline__ void chain_accept(const SamplerConst& S, ChainWork& w, int k, bool full, int lane) {
+// Accept candidate k: point, theta, logL, per-detector sums and the record.
+// All lanes.
+__device__ __forceinline__ void chain_accept(const SamplerConst& S, ChainWork& w, int k, int lane) {
   ChainState& ch = w.ch;
   const int b = ch.block;
   if (lane < S.ndim && ((S.block_mask[b] >> lane) & 1u)) ch.x[lane] = w.y[k][lane];
   if (lane < SWIG_N_PARAMS) ch.th[lane] = w.th[k][lane];
-  if (full) {
-    if (lane < 2 * SWIG_MAX_DET) ch.kap[lane] = w.kap[k][lane];
-    if (lane < SWIG_MAX_DET) ch.vv[lane] = w.vv[k][lane];
-    warp_copy(&w.rx, &w.rec[k], sizeof(EvalRecord), lane);
-  }
+  if (lane < 2 * SWIG_MAX_DET) ch.kap[lane] = w.kap[k][lane];
+  if (lane < SWIG_MAX_DET) ch.vv[lane] = w.vv[k][lane];
+  warp_copy(&w.rx, &w.rec[k], sizeof(EvalRecord), lane);
   __syncwarp();
   if (lane == 0) {
     ch.lx = w.ly[k];
-    ch.proj_dirty = full ? 0 : 1;
+    ch.proj_dirty = 0;
     finish_step(S, ch);
   }
   __syncwarp();
+}
+
+// A whole slice step of a projection-only block, whose logL follows from the
+// current point's sums: a candidate per lane, up to kFreeRungs rungs of each end
+// (left on lanes 0 .. 7, right on 8 .. 15) or as many draws at a time, the
+// decisions by ballots.  Points, draws and counts are those of one candidate
+// after another.  Returns the points evaluated.
+template <bool HET>
+__device__ __forceinline__ int chain_free_step(const LikeConst& L, const SamplerConst& S, ChainWork& w, int c,
+                                               long long it, double logl_star, int lane) {
+  ChainState& ch = w.ch;
+  const int b = ch.block, nb = S.block_size[b];
+  const int row = lane & (2 * kFreeRungs - 1);
+  double* th = w.fth[row];
+  if (lane < 2 * kFreeRungs) {
+#pragma unroll
+    for (int s = 0; s < SWIG_N_PARAMS; ++s) th[s] = ch.th[s];
+  }
+  // logL at bracket coordinate t of the lanes that are on (bits: inside, above logL*)
+  double ly = 0.0;
+  const auto look = [&](double t, bool on, unsigned& inside, unsigned& ok) {
+    bool in = on;
+    if (on)
+      for (int r = 0; r < nb; ++r) {
+        const int j = S.block_dims[b][r], slot = S.slot_of_dim[j];
+        const double v = ch.x[j] + t * ch.dir[j];
+        if (!fp64_in_unit(v)) in = false;
+        if (in) th[slot] = prior_slot_inverse_f32(S.prior[slot], v);
+      }
+    inside = __ballot_sync(0xffffffffu, in);
+    if (in) ly = free_loglike_mixed(L, th, ch.kap, HET ? ch.vv : nullptr);
+    ok = __ballot_sync(0xffffffffu, in && ly > logl_star);
+    __syncwarp();
+  };
+  double lo = ch.lo, hi = ch.hi;
+  int evals = 0, seen = 0, side = 3, out = 0, outr = 0;
+  unsigned inside, ok;
+  while (side) {
+    const int dl = side & 1 ? min(kFreeRungs, kMaxStepOut - out) : 0;
+    const int dr = side & 2 ? min(kFreeRungs, kMaxStepOut - outr) : 0;
+    const bool right = lane >= kFreeRungs;
+    const int m = lane & (kFreeRungs - 1);
+    double t = right ? hi : lo;  // rung by rung (each addition rounds)
+    for (int i = 1; i < kFreeRungs; ++i)
+      if (i <= m) t += right ? 1.0 : -1.0;
+    look(t, lane < 2 * kFreeRungs && m < (right ? dr : dl), inside, ok);
+    seen += __popc(inside);
+    if (dl > 0) {
+      const EndResult e = end_result(inside & ((1u << kFreeRungs) - 1u), ok, 0, dl, kMaxStepOut - out);
+      evals += e.evals;
+      out += e.moved;
+      const double tn = __shfl_sync(0xffffffffu, t, min(e.moved, kFreeRungs - 1));
+      lo = e.moved < kFreeRungs ? tn : tn - 1.0;
+      if (e.shut) side &= ~1;
+    }
+    if (dr > 0) {
+      const EndResult e = end_result(inside, ok, kFreeRungs, dr, kMaxStepOut - outr);
+      evals += e.evals;
+      outr += e.moved;
+      const double tn = __shfl_sync(0xffffffffu, t, kFreeRungs + min(e.moved, kFreeRungs - 1));
+      hi = e.moved < kFreeRungs ? tn : tn + 1.0;
+      if (e.shut) side &= ~2;
+    }
+  }
+  unsigned ctr = ch.ctr;
+  int n_shrink = 0, hit = -1;
+  double t = 0.0;
+  while (hit < 0 && n_shrink < kMaxShrink) {
+    const int n = min(kFreeRungs, kMaxShrink - n_shrink);
+    const double u = u01_from(philox4x32_10(make_uint4(ctr + (unsigned)lane, (unsigned)c, (unsigned)it, 0u), S.key0,
+                                            S.key1));
+    for (int k = 0; k < n; ++k) {  // each draw after the ones before it were rejected
+      const double tk = lo + (hi - lo) * __shfl_sync(0xffffffffu, u, k);
+      if (lane == k) t = tk;
+      if (fp64_negative(tk))
+        lo = tk;
+      else
+        hi = tk;
+    }
+    look(t, lane < n, inside, ok);
+    seen += __popc(inside);
+    hit = __ffs(ok) - 1;
+    const int used = hit >= 0 ? hit + 1 : n;
+    evals += __popc(inside & ((1u << used) - 1u));
+    ctr += (unsigned)used;
+    n_shrink += used;
+  }
+  __syncwarp();
+  if (hit >= 0) {
+    if (lane == hit) {
+      for (int r = 0; r < nb; ++r) {
+        const int j = S.block_dims[b][r], slot = S.slot_of_dim[j];
+        ch.x[j] = ch.x[j] + t * ch.dir[j];
+        ch.th[slot] = th[slot];
+      }
+      ch.lx = ly;
+      ch.proj_dirty = 1;
+    }
+  }
+  __syncwarp();
+  if (lane == 0) {
+    ch.ctr = ctr;
+    ch.n_evals += evals;
+    if (hit < 0) ++ch.n_caps;
+    finish_step(S, ch);
+  }
+  __syncwarp();
+  return seen;
 }
 
 // Warp 0 between two evaluations: apply the results (have: a round is pending,
@@ -288,16 +492,13 @@ __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerC
       tk = t2;
     }
   };
-  auto apply = [&](bool full) {
+  auto apply = [&] {
     const bool in = lane < w.n_cand && ((w.inside >> lane) & 1u);
     const unsigned ok = __ballot_sync(0xffffffffu, in && w.ly[lane < kCand ? lane : 0] > logl_star);
-    int hit = -1;
-    if (lane == 0) hit = chain_consume(S, ch, w, ok, full);
-    hit = __shfl_sync(0xffffffffu, hit, 0);
-    __syncwarp();
-    if (hit >= 0) chain_accept(S, w, hit, full, lane);
+    const int hit = chain_consume(S, w, ok, lane);
+    if (hit >= 0) chain_accept(S, w, hit, lane);
   };
-  if (have) apply(true);
+  if (have) apply();
   lap(0);
   for (int guard = 0; guard < 1 << 20; ++guard) {
     if (ch.done) break;
@@ -306,29 +507,28 @@ __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerC
       if (prof && lane == 0) prof[7] += 1;
       lap(1);
     }
-    chain_candidates(S, w, c, it, lane);
-    lap(2);
-    const unsigned inside = w.inside;
-    if (inside == 0u) {
-      apply(!S.block_free[ch.block]);
+    if (S.block_free[ch.block]) {
+      const int seen = chain_free_step<HET>(L, S, w, c, it, logl_star, lane);
+      if (prof && lane == 0) prof[5] += seen;
+      lap(3);
       continue;
     }
-    if (S.block_free[ch.block]) {
-      if ((inside >> lane) & 1u) w.ly[lane] = free_loglike_mixed(L, w.th[lane], ch.kap, HET ? ch.vv : nullptr);
-      __syncwarp();
-      if (prof && lane == 0) prof[5] += __popc(inside);
-      apply(false);
-      lap(3);
+    chain_candidates(S, w, c, it, lane);
+    const unsigned inside = w.inside;
+    if (inside == 0u) {
+      lap(2);
+      apply();
       continue;
     }
     bool valid = false;
     if ((inside >> lane) & 1u) {
-      valid = theta_valid(w.th[lane]);
+      valid = chain_theta_valid(w.th[lane]);
       if (!valid) w.ly[lane] = -INFINITY;
     }
     const unsigned act = __ballot_sync(0xffffffffu, valid);
     if (act == 0u) {
-      apply(true);
+      lap(2);
+      apply();
       continue;
     }
     if (valid) {
@@ -343,6 +543,7 @@ __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerC
       if (prof) prof[6] += __popc(inside);
     }
     __syncwarp();
+    lap(2);
     return;
   }
   if (lane == 0) w.status = ROUND_DONE;

@@ -923,6 +923,7 @@ int run_setup(swig_ctx* c, RunState& R) {
   const int shape = c->cfg.flow_parts;
   S.spec_out = L.tm_n > 0 ? 1 : shape >= 3 ? 1 : shape == 2 ? 2 : 4;
   S.spec_shr = L.tm_n > 0 ? 1 : shape >= 4 ? 1 : 2;
+  S.spec_mix = L.tm_n > 0 ? 0 : S.spec_shr;
   S.one_end = c->cfg.stepout_one_end ? 1 : 0;
   // learned proposal: retrain every learn_interval iterations (one launch each)
   R.learned = c->cfg.proposal == SWIG_PROPOSAL_LEARNED;

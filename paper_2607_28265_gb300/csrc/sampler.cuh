@@ -57,7 +57,7 @@ struct SamplerConst {
   int claim_off;  // FP64 sampler: byte offset of the claim words in dynamic shared memory
   // chain sampler (chain.cuh), the launch shape: rungs per bracket end and
   // shrinkage draws evaluated at a time; one end of a bracket after the other
-  int spec_out, spec_shr, one_end;
+  int spec_out, spec_shr, spec_mix, one_end;
 };
 
 struct ChainState {
@@ -73,6 +73,8 @@ struct ChainState {
   long long n_evals, n_full;
   int side;     // PH_OUT: bit 0 the left end still stepping out, bit 1 the right end
   int n_out_r;  // PH_OUT: expansions of the right end
+  int closed;   // ... ends that left the unit cube (bits)
+  int score;    // chain sampler: how often its guess held lately (chain.cuh)
 };
 
 struct NSGlobal {
