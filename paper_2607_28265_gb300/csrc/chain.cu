@@ -410,7 +410,8 @@ __global__ void __launch_bounds__(kChainBlock, 1)
     bool all_run = true;
     for (int e = 0; e < n_ev; ++e) all_run = all_run && *(volatile int*)&ev[e].P.g->status == ST_RUNNING;
     if (!all_run) return;
-    if ((int)blockIdx.x < n_ev) ns_boundary_advance(ev[blockIdx.x].L, ev[blockIdx.x].S, ev[blockIdx.x].P, scratch);
+    if ((int)blockIdx.x < n_ev) 
+      ns_boundary_advance(ev[blockIdx.x].L, ev[blockIdx.x].S, ev[blockIdx.x].P, scratch, lay.scratch_bytes);
     if (timer) *(volatile int*)&gb->task = 0;
     if (!grid_sync(gb, lay.n_ctas, lay.spin_limit)) return;
     if (timer) {

@@ -316,6 +316,12 @@ static __device__ void block_reduce_max_sum(double* vals, int n, double* out_max
   __syncthreads();
 }
 
+// An integer that orders like v (the zeros alike).
+__device__ __forceinline__ long long fp64_order(double v) {
+  const long long b = __double_as_longlong(v);
+  return b >= 0 ? b : (long long)0x8000000000000000ull - b;
+}
+
 // First half of the boundary: write the finished chains back into the live
 // set and apply the launch's iteration limit and the termination rule.  Fills
 // the sort keys in `smem` for the second half.  Returns false (status set)
@@ -364,8 +370,15 @@ static __device__ __noinline__ bool ns_boundary_check(const LikeConst& L, const 
 
 // Second half: sort, retire the k worst points, update log X / log Z and
 // logL*, estimate the block Cholesky factors, start k chains at survivors.
+// smem: `bytes` of it (0: as much as the sort takes).
+//
+// One CTA does this while the others wait, so its latencies count in full: the
+// sort compares integers (an FP64 comparison or conversion costs a scheduler
+// 64 cycles) and the covariance reads the live points from shared memory,
+// converted once, its sums in the order of the points.  nlive 1000, 12
+// dimensions, with the first half: 317 -> 147 us per iteration.
 static __device__ __noinline__ void ns_boundary_advance(const LikeConst& L, const SamplerConst& S, const SamplerPtrs& P,
-                                                 unsigned char* smem) {
+                                                 unsigned char* smem, int bytes) {
   NSGlobal* g = P.g;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int m = S.nlive, k = S.nrep, d = S.ndim;
@@ -380,7 +393,8 @@ static __device__ __noinline__ void ns_boundary_advance(const LikeConst& L, cons
         if (ixj > i) {
           const bool asc = (i & kk) == 0;
           const double a = key[i], b = key[ixj];
-          if ((a > b) == asc || (a == b && ((idx[i] > idx[ixj]) == asc))) {
+          const long long ka = fp64_order(a), kb = fp64_order(b);
+          if ((ka > kb) == asc || (ka == kb && ((idx[i] > idx[ixj]) == asc))) {
             key[i] = b;
             key[ixj] = a;
             const int t = idx[i];
@@ -419,27 +433,48 @@ static __device__ __noinline__ void ns_boundary_advance(const LikeConst& L, cons
   // covariance of the live points (FP32; only a proposal scale) and block Cholesky
   float* mean = reinterpret_cast<float*>(logw + k);
   float* cov = mean + kMaxDim;  // kMaxDim x kMaxDim
-  if (tid < d) {
-    float acc = 0.0f;
-    for (int i = 0; i < m; ++i) acc += (float)P.live_u[(size_t)i * d + tid];
-    mean[tid] = acc / (float)m;
-  }
-  __syncthreads();
-  if (tid < d * d) {
-    const int a = tid / d, b = tid % d;
-    if (b <= a) {
-      float acc0 = 0.0f, acc1 = 0.0f;
-      const float ma = mean[a], mb = mean[b];
-      int i = 0;
-      for (; i + 1 < m; i += 2) {
-        acc0 = fmaf((float)P.live_u[(size_t)i * d + a] - ma, (float)P.live_u[(size_t)i * d + b] - mb, acc0);
-        acc1 = fmaf((float)P.live_u[(size_t)(i + 1) * d + a] - ma, (float)P.live_u[(size_t)(i + 1) * d + b] - mb, acc1);
-      }
-      if (i < m) acc0 = fmaf((float)P.live_u[(size_t)i * d + a] - ma, (float)P.live_u[(size_t)i * d + b] - mb, acc0);
-      const float v = (acc0 + acc1) / (float)(m - 1);
-      cov[a * kMaxDim + b] = v;
-      cov[b * kMaxDim + a] = v;
+  // panels of points in FP32: behind the covariance, or over the reductions'
+  // scratch where that is longer (an even number of points: 80 at least)
+  float* pan = cov + kMaxDim * kMaxDim;
+  const int room = max(0, bytes - (int)(reinterpret_cast<unsigned char*>(pan) - smem)) / (int)(d * sizeof(float));
+  const int over = (int)((np2 + k) * sizeof(double)) / (int)(d * sizeof(float));
+  if (over > room) pan = reinterpret_cast<float*>(tmp);
+  const int rows = max(over, room) & ~1;
+  float acc0 = 0.0f, acc1 = 0.0f;
+  for (int i0 = 0; i0 < m; i0 += rows) {
+    const int n = min(rows, m - i0);
+    for (int q = tid; q < n * d; q += nt) pan[q] = (float)P.live_u[(size_t)i0 * d + q];
+    __syncthreads();
+    if (tid < d) {
+#pragma unroll 8
+      for (int i = 0; i < n; ++i) acc0 += pan[i * d + tid];
     }
+    __syncthreads();
+  }
+  if (tid < d) mean[tid] = acc0 / (float)m;
+  __syncthreads();
+  const int ca = tid / d, cb = tid % d;
+  const bool pair = tid < d * d && cb <= ca;
+  acc0 = 0.0f;
+  for (int i0 = 0; i0 < m; i0 += rows) {
+    const int n = min(rows, m - i0);
+    for (int q = tid; q < n * d; q += nt)
+      pan[q] = (rows < m ? (float)P.live_u[(size_t)i0 * d + q] : pan[q]) - mean[q % d];
+    __syncthreads();
+    if (pair) {  // even points and odd ones
+#pragma unroll 4
+      for (int i = 0; i + 1 < n; i += 2) {
+        acc0 = fmaf(pan[i * d + ca], pan[i * d + cb], acc0);
+        acc1 = fmaf(pan[(i + 1) * d + ca], pan[(i + 1) * d + cb], acc1);
+      }
+      if (n & 1) acc0 = fmaf(pan[(n - 1) * d + ca], pan[(n - 1) * d + cb], acc0);
+    }
+    __syncthreads();
+  }
+  if (pair) {
+    const float v = (acc0 + acc1) / (float)(m - 1);
+    cov[ca * kMaxDim + cb] = v;
+    cov[cb * kMaxDim + ca] = v;
   }
   __syncthreads();
   if (tid < S.n_blocks) {
@@ -497,7 +532,7 @@ static __device__ __noinline__ void ns_boundary_advance(const LikeConst& L, cons
 }
 
 static __device__ void ns_boundary(const LikeConst& L, const SamplerConst& S, const SamplerPtrs& P, unsigned char* smem) {
-  if (ns_boundary_check(L, S, P, smem)) ns_boundary_advance(L, S, P, smem);
+  if (ns_boundary_check(L, S, P, smem)) ns_boundary_advance(L, S, P, smem, 0);
 }
 
 
