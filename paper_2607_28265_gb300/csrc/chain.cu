@@ -31,7 +31,10 @@ struct ChainEval<NDET, CHAIN_FOLD> {
 };
 template <int NDET>
 struct ChainEval<NDET, CHAIN_HET> {
-  HetPrep<NDET> prep[kCand];
+  double fc[NBASIS], ft[SWIG_MAX_DET];  // the fiducial's coefficients and delays
+  HetPrep<NDET> prep[kCand], cur_prep;
+  HetIn<NDET, 1> cur;         // the chain's current point
+  int base_ok;                // its partial sums are formed
   HetIn<NDET, 2> in[kCand / 2];
   float part[kChainWarps][NDET][3 * kCand];  // per warp: value 8 kind + slot
   double tot[NDET][3 * kCand];
@@ -81,7 +84,7 @@ __device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, cons
                                          const float* tab, float* base, float* s_an, int slots, int warp, int lane) {
   ChainWork& w = s.w;
   const int na = w.n_act, pairs = (na + 1) / 2, ld = F.ld;
-  const int G = pairs <= 1 ? 16 : pairs == 2 ? 8 : kFoldGroups;
+  const int G = kChainWarps / pairs;
   const bool use = base != nullptr && !(w.fl & (BF_INTR | BF_TIDE));  // uniform
   if (threadIdx.x < pairs * 16) {
     const int p = threadIdx.x >> 4, j = threadIdx.x & 15;
@@ -244,12 +247,25 @@ __device__ __forceinline__ void finish_fold(ChainShared<NDET, CHAIN_FOLD>& s, in
 // forms its result.
 template <int NDET>
 __device__ __forceinline__ void eval_het(ChainShared<NDET, CHAIN_HET>& s, const HetTables& H, const float* tab,
-                                         float* s_an, int bytes, int warp, int lane) {
+                                         float* base, float* s_an, int bytes, int warp, int lane) {
   ChainWork& w = s.w;
   const int na = w.n_act, pairs = (na + 1) / 2;
+  const bool use = base != nullptr && !(w.fl & (BF_INTR | BF_TIDE)), form = use && !s.e.base_ok;  // uniform
   if (warp < 2 * pairs) {  // (an odd round's last pair holds its candidate twice)
-    het_prepare_warp<NDET>(s.L, H, w.rec[w.list[min(warp, na - 1)]], s.e.prep[warp], lane);
+    het_differences<NDET>(s.e.fc, s.e.ft, w.rec[w.list[min(warp, na - 1)]], s.e.prep[warp], lane);
     het_in_set<NDET, 2>(s.e.in[warp >> 1], warp & 1, s.e.prep[warp], lane);
+  } else if (form && warp == kChainWarps - 1) {
+    het_differences<NDET>(s.e.fc, s.e.ft, w.rx, s.e.cur_prep, lane);
+    het_in_set<NDET, 1>(s.e.cur, 0, s.e.cur_prep, lane);
+  }
+  if (form) {
+    __syncthreads();
+    const int nb = (H.n_chunks + 31) >> 5;
+    for (int t = warp; t < 4 * nb; t += kChainWarps) {
+      const int q = 32 * (t % nb) + lane;
+      if (q < H.n_chunks) het_anchor_part<NDET, 1, -1>(tab, H.n_chunks, s.e.cur, t / nb, q, nullptr, base + q);
+    }
+    if (threadIdx.x == 0) s.e.base_ok = 1;
   }
   const int fit = bytes / (pairs * kHetAncPair * (int)sizeof(float));
   const int panel = fit >= H.n_chunks ? H.n_chunks : fit & ~31;
@@ -259,12 +275,25 @@ __device__ __forceinline__ void eval_het(ChainShared<NDET, CHAIN_HET>& s, const 
   for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
     const int np = min(panel, H.n_chunks - q0);
     __syncthreads();
-    het_anchors<NDET, 2>(H, tab, s.e.in, pairs, q0, np, panel, s_an, warp, kChainWarps, lane);
+    // the first chunk's weights, then always the next one's: in flight meanwhile
+    float4 nx[NDET];
+    const float4* ew = H.ew + (size_t)q0 * NDET * 32 + lane;
+    if (warp < np)
+#pragma unroll
+      for (int i = 0; i < NDET; ++i) nx[i] = __ldg(ew + (warp * NDET + i) * 32);
+    if (use)
+      het_anchors<NDET, 2, 1>(H, tab, s.e.in, pairs, q0, np, panel, base, s_an, warp, kChainWarps, lane);
+    else
+      het_anchors<NDET, 2>(H, tab, s.e.in, pairs, q0, np, panel, base, s_an, warp, kChainWarps, lane);
     __syncthreads();
     for (int q = warp; q < np; q += kChainWarps) {
       float4 v[NDET];
+      const int qn = min(q + kChainWarps, np - 1);
 #pragma unroll
-      for (int i = 0; i < NDET; ++i) v[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
+      for (int i = 0; i < NDET; ++i) {
+        v[i] = nx[i];
+        nx[i] = __ldg(ew + (qn * NDET + i) * 32);
+      }
 #pragma unroll
       for (int p = 0; p < kCand / 2; ++p)
         if (p < pairs) {
@@ -445,6 +474,10 @@ __global__ void __launch_bounds__(kChainBlock, 1)
             asm volatile("cp.async.wait_all;" ::: "memory");
           }
         }
+        if constexpr (MODE == CHAIN_HET) {
+          if (tid < NBASIS) s.e.fc[tid] = E.H.fid->c[tid];
+          if (tid < SWIG_MAX_DET) s.e.ft[tid] = E.H.fid->tau[tid];
+        }
         if constexpr (MODE == CHAIN_HET)
           if (lay.res_off > 0) {
             float* d = reinterpret_cast<float*>(smem + lay.res_off);
@@ -474,7 +507,7 @@ __global__ void __launch_bounds__(kChainBlock, 1)
       }
       unsigned long long* prof = c == 0 && e == 0 ? s.prof : nullptr;
       bool have = false;
-      if constexpr (MODE == CHAIN_FOLD)
+      if constexpr (MODE != CHAIN_HET_TM)
         if (tid == 0) s.e.base_ok = 0;
       for (long long guard = 0; guard < (1ll << 24); ++guard) {
         long long tc = 0;
@@ -485,7 +518,7 @@ __global__ void __launch_bounds__(kChainBlock, 1)
           if constexpr (MODE == CHAIN_HET)
             if (have) finish_het<NDET>(s, E.H, lane);
           chain_control<NDET, MODE != CHAIN_FOLD>(s.L, s.S, P, w, c, it, logl_star, have, lane, prof);
-          if constexpr (MODE == CHAIN_FOLD)
+          if constexpr (MODE != CHAIN_HET_TM)
             if (lane == 0 && w.status == ROUND_EVAL && (w.fl & (BF_INTR | BF_TIDE))) s.e.base_ok = 0;
           if (lane == 0) {
             const long long t2 = clock64();
@@ -502,7 +535,7 @@ __global__ void __launch_bounds__(kChainBlock, 1)
           eval_fold<NDET>(s, E.F, W, tab, base, reinterpret_cast<float*>(scratch),
                           lay.scratch_bytes / (int)(kFoldAnchor * sizeof(float)), warp, lane);
         else if constexpr (MODE == CHAIN_HET)
-          eval_het<NDET>(s, E.H, tab, reinterpret_cast<float*>(scratch), lay.scratch_bytes, warp, lane);
+          eval_het<NDET>(s, E.H, tab, base, reinterpret_cast<float*>(scratch), lay.scratch_bytes, warp, lane);
         else
           eval_het_tm<NDET>(s, E.H, scratch, lay, warp, lane);
         __syncthreads();

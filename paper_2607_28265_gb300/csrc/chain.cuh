@@ -31,7 +31,6 @@ namespace swig {
 constexpr int kCand = 8;          // candidates per round at most
 constexpr int kFreeRungs = 8;     // rungs per end of a projection-only step, and its draws at a time
 constexpr int kChainWarps = kChainBlock / 32;
-constexpr int kFoldGroups = 4;    // groups of chunks (partial sums) of a full round's pairs
 static_assert(kChainBlock == kHetTmThreads, "the sampler and the batched time-marginalised kernel share sum orders");
 
 // What the control keeps of a chain between its rounds, and a round's

@@ -99,20 +99,30 @@ __device__ inline void het_prepare(const LikeConst& L, const HetTables& H, const
   }
 }
 
+// The differences by a warp, one per lane, against the fiducial's c and tau.
+template <int NDET>
+__device__ __forceinline__ void het_differences(const double* f0c, const double* f0tau, const EvalRecord& r,
+                                                HetPrep<NDET>& p, int lane) {
+  const bool c = lane < NBASIS, t = lane >= 16 && lane < 16 + NDET;
+  const double x = c ? r.c[lane] - f0c[lane] : t ? r.tau[lane - 16] - f0tau[lane - 16] : 0.0;
+  const dfl d = df_from_double(x);
+  if (c) p.dc[lane] = d;
+  if (t) p.dtau[lane - 16] = d;
+  __syncwarp();
+}
+
 // het_prepare by a warp, one constant per lane.
 template <int NDET>
 __device__ __forceinline__ void het_prepare_warp(const LikeConst& L, const HetTables& H, const EvalRecord& r,
                                                  HetPrep<NDET>& p, int lane) {
   const EvalRecord& f0 = *H.fid;
-  if (lane < NBASIS) p.dc[lane] = df_from_double(r.c[lane] - f0.c[lane]);
-  if (lane >= 16 && lane < 16 + NDET) {
-    const int i = lane - 16;
-    p.dtau[i] = df_from_double(r.tau[i] - f0.tau[i]);
+  if (lane < NDET) {
+    const int i = lane;
     const double iden = L.het_fid_iden[i];
     p.rho_re[i] = (float)((r.cre[i] * f0.cre[i] + r.cim[i] * f0.cim[i]) * iden);
     p.rho_im[i] = (float)((r.cim[i] * f0.cre[i] - r.cre[i] * f0.cim[i]) * iden);
   }
-  __syncwarp();
+  het_differences<NDET>(f0.c, f0.tau, r, p, lane);
 }
 
 // Anchor of chunk q for one evaluation (one thread per chunk; rows of the
@@ -437,79 +447,113 @@ __device__ __forceinline__ void het_in_set(HetIn<NDET, N>& in, int k, const HetP
   }
 }
 
+// The basis functions that only the spins move: the other sums (rows of
+// kHetBaseRows values per chunk: A, a_1 in double-float, the bound, a_2 ..)
+// stand while masses and tides do.
+__device__ __forceinline__ constexpr bool het_moved(int j) { return j == B_M23 || j == B_M13; }
+enum { HB_A = 0, HB_S = 2, HB_R = 4, HB_POLY = 5 };
+static_assert(HB_POLY + kHetPoly == kHetBaseRows, "base rows");
+
 // One quarter (sub 0 .. 3) of the anchors of chunk q for N evaluations, value m
 // of evaluation k to out[N m + k]: sub 0 the phases frac(dP(f_a) + f_a dtau_i),
 // sub 1 a_1, 1 / S and the exact flag, sub 2 and 3 the Taylor terms (het_anchor
-// has them all for one evaluation on one thread).
-template <int NDET, int N>
+// has them all for one evaluation on one thread).  WITH 1: from the base rows
+// (stride nc) and the moved functions; -1: the base rows themselves (N = 1),
+// at out[m nc].
+template <int NDET, int N, int WITH = 0>
 __device__ __forceinline__ void het_anchor_part(const float* __restrict__ chunk, int nc, const HetIn<NDET, N>& in,
-                                                int sub, int q, float* out) {
+                                                int sub, int q, const float* base, float* out) {
   using O = PkOps<N>;
   using T = typename O::T;
   const float* tab = chunk + q;
   auto row = [&](int r) { return O::all(tab[r * nc]); };
+  auto from = [&](int m) { return O::all(WITH == 1 ? base[m * nc + q] : 0.0f); };
   auto put = [&](int m, T v) { *reinterpret_cast<T*>(out + N * m) = v; };
   auto dc = [&](int j) { return DflN<N>{O::load(in.dc_hi[j]), O::load(in.dc_lo[j])}; };
+  auto takes = [](int j) { return WITH == 0 || het_moved(j) == (WITH == 1); };
   if (sub == 0) {
-    DflN<N> A = {O::all(0.0f), O::all(0.0f)};
+    DflN<N> A = {from(HB_A), from(HB_A + 1)};
 #pragma unroll
     for (int j = 0; j < NBASIS; ++j)
-      A = dfn_add<N>(A, dfn_mul<N>(dc(j), DflN<N>{row(HC_VAL_HI + j), row(HC_VAL_LO + j)}));
-    const DflN<N> fa = {row(HC_FA_HI), row(HC_FA_LO)};
+      if (takes(j)) A = dfn_add<N>(A, dfn_mul<N>(dc(j), DflN<N>{row(HC_VAL_HI + j), row(HC_VAL_LO + j)}));
+    if constexpr (WITH < 0) {
+      out[HB_A * nc] = A.hi;
+      out[(HB_A + 1) * nc] = A.lo;
+    } else {
+      const DflN<N> fa = {row(HC_FA_HI), row(HC_FA_LO)};
 #pragma unroll
-    for (int i = 0; i < NDET; ++i)
-      put(kHetAncPhase + i,
-          dfn_frac<N>(dfn_add<N>(A, dfn_mul<N>(fa, DflN<N>{O::load(in.dt_hi[i]), O::load(in.dt_lo[i])}))));
-  } else if (sub == 1) {
-    DflN<N> S = {O::all(0.0f), O::all(0.0f)};
-    T R = O::all(0.0f);
-#pragma unroll
-    for (int j = 0; j < NBASIS; ++j) {
-      S = dfn_add<N>(S, dfn_mul<N>(dc(j), DflN<N>{row(HC_D1_HI + j), row(HC_D1_LO + j)}));
-      R = O::fma(O::load(in.dc_abs[j]), row(HC_BND + j), R);
+      for (int i = 0; i < NDET; ++i)
+        put(kHetAncPhase + i,
+            dfn_frac<N>(dfn_add<N>(A, dfn_mul<N>(fa, DflN<N>{O::load(in.dt_hi[i]), O::load(in.dt_lo[i])}))));
     }
-    put(0, O::add(S.hi, S.lo));
-    put(kHetAncInvS, row(HC_INV_S));
-    float r[N];
-    O::get(R, r);
+  } else if (sub == 1) {
+    DflN<N> S = {from(HB_S), from(HB_S + 1)};
+    T R = from(HB_R);
 #pragma unroll
-    for (int k = 0; k < N; ++k) out[N * kHetAncExact + k] = r[k] > kHetTaylorEps ? 1.0f : 0.0f;
+    for (int j = 0; j < NBASIS; ++j)
+      if (takes(j)) {
+        S = dfn_add<N>(S, dfn_mul<N>(dc(j), DflN<N>{row(HC_D1_HI + j), row(HC_D1_LO + j)}));
+        R = O::fma(O::load(in.dc_abs[j]), row(HC_BND + j), R);
+      }
+    if constexpr (WITH < 0) {
+      out[HB_S * nc] = S.hi;
+      out[(HB_S + 1) * nc] = S.lo;
+      out[HB_R * nc] = R;
+    } else {
+      put(0, O::add(S.hi, S.lo));
+      put(kHetAncInvS, row(HC_INV_S));
+      float r[N];
+      O::get(R, r);
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[N * kHetAncExact + k] = r[k] > kHetTaylorEps ? 1.0f : 0.0f;
+    }
   } else {
     constexpr int kHalf = (kHetPoly + 1) / 2;  // orders 2 .. kHalf + 1, and above
     T a[kHalf];
-#pragma unroll
-    for (int m = 0; m < kHalf; ++m) a[m] = O::all(0.0f);
     const int m0 = sub == 2 ? 0 : kHalf;
 #pragma unroll
-    for (int j = 0; j < NBASIS; ++j) {
-      const T c = O::load(in.dc_hi[j]);
+    for (int m = 0; m < kHalf; ++m) a[m] = m0 + m < kHetPoly ? from(HB_POLY + m0 + m) : O::all(0.0f);
 #pragma unroll
-      for (int m = 0; m < kHalf; ++m)
-        if (m0 + m < kHetPoly) a[m] = O::fma(c, row(HC_POLY + (m0 + m) * NBASIS + j), a[m]);
-    }
+    for (int j = 0; j < NBASIS; ++j)
+      if (takes(j)) {
+        const T c = O::load(in.dc_hi[j]);
+#pragma unroll
+        for (int m = 0; m < kHalf; ++m)
+          if (m0 + m < kHetPoly) a[m] = O::fma(c, row(HC_POLY + (m0 + m) * NBASIS + j), a[m]);
+      }
 #pragma unroll
     for (int m = 0; m < kHalf; ++m)
-      if (m0 + m < kHetPoly) put(1 + m0 + m, a[m]);
+      if (m0 + m < kHetPoly) {
+        if constexpr (WITH < 0)
+          out[(HB_POLY + m0 + m) * nc] = a[m];
+        else
+          put(1 + m0 + m, a[m]);
+      }
   }
 }
 
 // Anchors of np chunks from q0 on for `sets` groups of N evaluations by the
-// warps first, first + stride, ... of a CTA: quarter by quarter, 32 chunks per
-// warp and turn.  chunk: H.chunk or its copy in shared memory.  Group g's anchors at s_an + (g panel + q)
-// kHetAncPair (N = 2) or kHetAncOne.
-template <int NDET, int N>
-__device__ __forceinline__ void het_anchors(const HetTables& H, const float* chunk, const HetIn<NDET, N>* in, int sets, int q0, int np,
-                                            int panel, float* s_an, int first, int stride, int lane) {
-  const int nb = (np + 31) >> 5, per = sets * nb;  // warp turns of a quarter
+// warps first, first + stride, ... of a CTA: quarter by quarter, 32 chunks (of
+// all groups, one after the other) per warp and turn.  chunk: H.chunk or its
+// copy in shared memory.  Group g's anchors at s_an + (g panel + q) kHetAncPair
+// (N = 2) or kHetAncOne.
+template <int NDET, int N, int WITH = 0>
+__device__ __forceinline__ void het_anchors(const HetTables& H, const float* chunk, const HetIn<NDET, N>* in, int sets,
+                                            int q0, int np, int panel, const float* base, float* s_an, int first,
+                                            int stride, int lane) {
+  const int all = sets * np, per = (all + 31) >> 5;  // warp turns of a quarter
   for (int sub = 0, t = first; sub < 4;) {
     if (t >= per) {
       t -= per;
       ++sub;
       continue;
     }
-    const int g = t / nb, q = 32 * (t - g * nb) + lane;
-    if (q < np)
-      het_anchor_part<NDET, N>(chunk, H.n_chunks, in[g], sub, q0 + q, s_an + (size_t)(g * panel + q) * (N == 2 ? kHetAncPair : kHetAncOne));
+    const int v = 32 * t + lane;
+    if (v < all) {
+      const int g = v / np, q = v - g * np;
+      het_anchor_part<NDET, N, WITH>(chunk, H.n_chunks, in[g], sub, q0 + q, base,
+                                     s_an + (size_t)(g * panel + q) * (N == 2 ? kHetAncPair : kHetAncOne));
+    }
     t += stride;
   }
 }
@@ -620,7 +664,7 @@ __device__ inline void het_products(const HetTables& H, const HetPrep<NDET>& pre
   for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
     const int np = min(panel, H.n_chunks - q0);
     __syncthreads();
-    het_anchors<NDET, 1>(H, H.chunk, &in, 1, q0, np, panel, s_an, warp, n_warps, lane);
+    het_anchors<NDET, 1>(H, H.chunk, &in, 1, q0, np, panel, nullptr, s_an, warp, n_warps, lane);
     __syncthreads();
     for (int q = warp; q < np; q += n_warps) {
       float4 w[NDET];

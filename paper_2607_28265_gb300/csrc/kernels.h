@@ -87,6 +87,8 @@ static_assert(kHetAncExact < kHetAncStride, "chunk anchor layout");
 // one, padded so that the lanes' stores (a chunk each) meet all banks.
 constexpr int kHetAncPair = 2 * kHetAncStride + 2;
 constexpr int kHetAncOne = kHetAncStride + 1;
+// Partial sums of a chain's current point per chunk (het.cuh).
+constexpr int kHetBaseRows = 5 + kHetPoly;
 // Per-warp shared-memory stage of one chunk's table data (summary data, bin
 // widths, edge offsets), filled by cp.async one chunk ahead: bytes per stage.
 inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) + 2 * 32 * 4; }

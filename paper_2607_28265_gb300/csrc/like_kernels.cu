@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     const int m = min(per, n - base), pairs = (m + 1) / 2;
     __syncthreads();
     if (warp < 2 * pairs) {  // (an odd batch's last pair holds its vector twice)
-      het_prepare_warp<NDET>(L, H, rec[base + min(warp, m - 1)], s_prep[warp], lane);
+      het_differences<NDET>(H.fid->c, H.fid->tau, rec[base + min(warp, m - 1)], s_prep[warp], lane);
       het_in_set<NDET, 2>(s_in[warp >> 1], warp & 1, s_prep[warp], lane);
     }
     HetAcc<NDET, 2> acc[kHetBatch / 2];
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
       const int np = min(panel, H.n_chunks - q0);
       __syncthreads();
-      het_anchors<NDET, 2>(H, H.chunk, s_in, pairs, q0, np, panel, s_an, warp, kHetWarps, lane);
+      het_anchors<NDET, 2>(H, H.chunk, s_in, pairs, q0, np, panel, nullptr, s_an, warp, kHetWarps, lane);
       __syncthreads();
       for (int q = warp; q < np; q += kHetWarps) {
         float4 w[NDET];

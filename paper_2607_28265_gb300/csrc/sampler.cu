@@ -974,6 +974,11 @@ int run_setup(swig_ctx* c, RunState& R) {
       }
     }
     if (R.mode == CHAIN_HET) {
+      const size_t base = sizeof(float) * kHetBaseRows * ((size_t)c->B.het_nc + 3 & ~(size_t)3);
+      if (R.smem + base <= kChainSmemMax) {
+        y.base_off = (int)R.smem;
+        R.smem += base;
+      }
       const size_t res = sizeof(float) * HC_ROWS * (size_t)c->B.het_nc;
       if (R.smem + res <= kChainSmemMax) {
         y.res_off = (int)R.smem;
