@@ -344,14 +344,23 @@ constexpr int kHetPanel = 256;  // chunks anchored at once
 
 template <int NDET>
 __global__ void __launch_bounds__(kHetTmThreads, 1)
-    k_het(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, int per, double* __restrict__ out,
-          double* __restrict__ kappa_out, double* __restrict__ vv_out) {
-  extern __shared__ __align__(16) float s_an[];  // [pairs][panel][kHetAncPair]
+    k_het(LikeConst L, HetTables H, const EvalRecord* __restrict__ rec, int n, int per, int tab_off,
+          double* __restrict__ out, double* __restrict__ kappa_out, double* __restrict__ vv_out) {
+  extern __shared__ __align__(16) float s_an[];  // [pairs][panel][kHetAncPair], the chunk table
   __shared__ HetPrep<NDET> s_prep[kHetBatch];
   __shared__ HetIn<NDET, 2> s_in[kHetBatch / 2];
   __shared__ float s_part[kHetWarps][NDET][3 * kHetBatch];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int panel = min(kHetPanel, H.n_chunks);
+  const float* tab = H.chunk;
+  if (tab_off > 0) {
+    for (int q = threadIdx.x; q < HC_ROWS * H.n_chunks; q += kHetTmThreads) cp_async<4>(s_an + tab_off + q, H.chunk + q);
+    cp_async_commit();
+    tab = s_an + tab_off;
+  }
+  // the set-up kernel's records, while this one's start overlapped its end
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  cp_async_wait<0>();
   for (int base = blockIdx.x * per; base < n; base += gridDim.x * per) {
     const int m = min(per, n - base), pairs = (m + 1) / 2;
     __syncthreads();
@@ -365,14 +374,22 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     for (int q0 = 0; q0 < H.n_chunks; q0 += panel) {
       const int np = min(panel, H.n_chunks - q0);
       __syncthreads();
-      het_anchors<NDET, 2>(H, H.chunk, s_in, pairs, q0, np, panel, nullptr, s_an, warp, kHetWarps, lane);
+      // the first chunk's weights, then always the next one's: in flight meanwhile
+      float4 nx[NDET];
+      const float4* ew = H.ew + (size_t)q0 * NDET * 32 + lane;
+      if (warp < np)
+#pragma unroll
+        for (int i = 0; i < NDET; ++i) nx[i] = __ldg(ew + (warp * NDET + i) * 32);
+      het_anchors<NDET, 2>(H, tab, s_in, pairs, q0, np, panel, nullptr, s_an, warp, kHetWarps, lane);
       __syncthreads();
       for (int q = warp; q < np; q += kHetWarps) {
         float4 w[NDET];
+        const int qn = min(q + kHetWarps, np - 1);
 #pragma unroll
-        for (int i = 0; i < NDET; ++i) w[i] = __ldg(H.ew + ((size_t)(q0 + q) * NDET + i) * 32 + lane);
-        if (q + kHetWarps < np && lane < 4 * NDET)  // the next chunk's lines
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(H.ew + ((size_t)(q0 + q + kHetWarps) * NDET) * 32 + 8 * lane));
+        for (int i = 0; i < NDET; ++i) {
+          w[i] = nx[i];
+          nx[i] = __ldg(ew + (qn * NDET + i) * 32);
+        }
 #pragma unroll
         for (int p = 0; p < kHetBatch / 2; ++p)
           if (p < pairs) {
@@ -431,6 +448,9 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
   const int th = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   if (th >= n) return;
   const EvalRecord& r = rec[th];
+  if (L.tm_M > 0) tm_load_twiddles(L, H, smem, H.n_bins);  // read after the barriers below
+  // the set-up kernel's records, while this one's start overlapped its end
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) {
     // no projection-only reuse under time marginalisation: the caches are zero
     if (kappa_out)
@@ -449,7 +469,6 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     het_prepare_warp<NDET>(L, H, r, s_prep, lane);
     het_in_set<NDET, 1>(s_in, 0, s_prep, lane);
   }
-  if (L.tm_M > 0) tm_load_twiddles(L, H, smem, H.n_bins);  // read after the barriers below
   HetAcc<NDET, 1> acc;
   acc.clear();
   het_products<NDET>(H, s_prep, s_in, s_an, panel, warp, n_warps, lane, acc, y);
@@ -483,15 +502,30 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
   }
 }
 
+// A heterodyned kernel whose start overlaps the set-up kernel before it on st.
+template <typename... P, typename... A>
+cudaError_t launch_after_setup(void (*kern)(P...), int grid, size_t bytes, cudaStream_t st, A... args) {
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kHetTmThreads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <int NDET>
 cudaError_t launch_het_tm(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
                           double* kappa_out, double* vv_out, float* ell) {
   const HetTmLayout lay = het_tm_layout(L, B);
-  cudaError_t e = cudaFuncSetAttribute(k_het_tm<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes);
-  if (e != cudaSuccess) return e;
-  k_het_tm<NDET><<<n, kHetTmThreads, lay.bytes, st>>>(L, het_tables(B), B.rec, n, lay.anc_off, lay.panel, out,
-                                                      kappa_out, vv_out, ell);
-  return cudaGetLastError();
+  return launch_after_setup(k_het_tm<NDET>, n, lay.bytes, st, L, het_tables(B), (const EvalRecord*)B.rec, n,
+                            lay.anc_off, lay.panel, out, kappa_out, vv_out, ell);
 }
 
 template <int NDET>
@@ -501,12 +535,12 @@ cudaError_t launch_het_plain(const LikeConst& L, const DeviceBuffers& B, int n, 
   int per = (n + L.sm_count - 1) / L.sm_count;
   per = per < kHetBatch ? per : kHetBatch;
   const int panel = B.het_nc < kHetPanel ? B.het_nc : kHetPanel, ctas = (n + per - 1) / per;
-  const size_t bytes = (size_t)((per + 1) / 2) * panel * kHetAncPair * sizeof(float);
-  const cudaError_t e = cudaFuncSetAttribute(k_het<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  k_het<NDET><<<ctas < L.sm_count ? ctas : L.sm_count, kHetTmThreads, bytes, st>>>(L, het_tables(B), B.rec, n, per, out,
-                                                                                  kappa_out, vv_out);
-  return cudaGetLastError();
+  size_t bytes = (size_t)((per + 1) / 2) * panel * kHetAncPair * sizeof(float);
+  const size_t tab = sizeof(float) * HC_ROWS * (size_t)B.het_nc;
+  const int tab_off = bytes + tab <= 200 * 1024 ? (int)(bytes / sizeof(float)) : 0;
+  if (tab_off) bytes += tab;
+  return launch_after_setup(k_het<NDET>, ctas < L.sm_count ? ctas : L.sm_count, bytes, st, L, het_tables(B),
+                            (const EvalRecord*)B.rec, n, per, tab_off, out, kappa_out, vv_out);
 }
 
 cudaError_t launch_loglike_het(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n, double* out,
