@@ -915,6 +915,12 @@ int prepare_het(swig_ctx* c) {
         CUDA_TRY(c, cudaMemcpy(B.het_nu_point, point.data(), sizeof(int4) * point.size(), cudaMemcpyHostToDevice));
       }
       c->h2d_bytes += sizeof(int4) * (piece.size() + point.size());
+      // their weights, entry i of 32 pieces in a row: the lanes take a piece each
+      std::vector<float> wrow((piece.size() + 31) / 32 * 32 * kNufftPiece, 0.0f);
+      for (size_t p = 0; p < piece.size(); ++p)
+        for (int i = 0; i < piece[p].y; ++i)
+          wrow[(p / 32 * kNufftPiece + i) * 32 + p % 32] = wt[(size_t)piece[p].x + i];
+      wt.swap(wrow);
       CUDA_TRY(c, cudaMalloc(&B.het_nu_wt, sizeof(float) * std::max<size_t>(1, wt.size())));
       CUDA_TRY(c, cudaMalloc(&B.het_nu_corr, sizeof(float) * corr.size()));
       tw = nufft_stage_twiddles(tw, L.tm_M);

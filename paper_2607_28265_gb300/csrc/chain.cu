@@ -396,14 +396,11 @@ __device__ __forceinline__ void eval_het_tm(ChainShared<NDET, CHAIN_HET_TM>& s, 
       s.e.tm[warp][1] = ws;
     }
     __syncthreads();
+    if (warp == 0) {
+      const double ll = tm_finish<NDET>(L, r, s.e.hh, s.e.tm, kChainWarps, lane);
+      if (lane == 0) w.ly[k] = ll;
+    }
     if (threadIdx.x == 0) {
-      double HH = 0.0;
-      for (int i = 0; i < NDET; ++i) {
-        double d = 0.0;
-        for (int q = 0; q < kChainWarps; ++q) d += (double)s.e.hh[q][i];
-        HH += (r.cre[i] * r.cre[i] + r.cim[i] * r.cim[i]) * (L.het_b0[i] - d) * L.het_fid_iden[i];
-      }
-      w.ly[k] = tm_finish(L, s.e.tm, kChainWarps, HH);
       for (int j = 0; j < 2 * SWIG_MAX_DET; ++j) w.kap[k][j] = 0.0;
       for (int i = 0; i < SWIG_MAX_DET; ++i) w.vv[k][i] = 0.0;
     }

@@ -898,9 +898,11 @@ __device__ inline void nufft_gather(const LikeConst& L, const HetTables& H, cons
     for (int u = 1; u < kPre; ++u)
       if (r == u) d = dp[u];
     if (r >= kPre) d = __ldg(&H.nu_piece[p]);
+    // entry i of 32 pieces in a row
+    const float* wt = H.nu_wt + (size_t)(p >> 5) * kNufftPiece * 32 + (p & 31);
     float w[kNufftPiece];
 #pragma unroll
-    for (int i = 0; i < kNufftPiece; ++i) w[i] = i < d.y ? __ldg(&H.nu_wt[d.x + i]) : 0.0f;
+    for (int i = 0; i < kNufftPiece; ++i) w[i] = i < d.y ? __ldg(wt + 32 * i) : 0.0f;
     float br = 0.0f, bi = 0.0f;
 #pragma unroll
     for (int i = 0; i < kNufftPiece; ++i)
@@ -974,19 +976,31 @@ __device__ inline void tm_pass_nufft(const LikeConst& L, const HetTables& H, con
   }
   float m = -INFINITY, s = 0.0f;
   const int nq = (L.tm_n + kTmNodes - 1) / kTmNodes;
-  for (int q = warp; q < nq; q += n_warps) {
-    const int j = q * kTmNodes + lane;
-    if (j < L.tm_n) {
-      const int mi = j - L.tm_j0;
-      const float2 z = g[mi < 0 ? mi + M : mi];
-      const float cr = H.nu_corr[j];
-      const float l = tm_node_logw(L, z.x * cr, z.y * cr);
-      if (ell) ell[j] = l;
-      if (l > m) {
-        s = s * __expf(m - l) + 1.0f;
-        m = l;
-      } else {
-        s += __expf(l - m);
+  // four nodes per lane at a time, taken up in order
+  constexpr int kAhead = 4;
+  for (int q0 = warp; q0 < nq; q0 += kAhead * n_warps) {
+    float l[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int j = (q0 + u * n_warps) * kTmNodes + lane;
+      if (j < L.tm_n) {
+        const int mi = j - L.tm_j0;
+        const float2 z = g[mi < 0 ? mi + M : mi];
+        const float cr = __ldg(H.nu_corr + j);
+        l[u] = tm_node_logw(L, z.x * cr, z.y * cr);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int j = (q0 + u * n_warps) * kTmNodes + lane;
+      if (j < L.tm_n) {
+        if (ell) ell[j] = l[u];
+        if (l[u] > m) {
+          s = s * __expf(m - l[u]) + 1.0f;
+          m = l[u];
+        } else {
+          s += __expf(l[u] - m);
+        }
       }
     }
   }
@@ -1015,15 +1029,35 @@ __device__ __forceinline__ void tm_load_twiddles(const LikeConst& L, const HetTa
   for (int k = threadIdx.x; k < L.tm_M; k += blockDim.x) tw[k] = __ldg(&H.nu_tw[k]);
 }
 
-// Time-marginalised logL from the warps' (max, sum) pairs (warp order) and
-// the network <h|h>: log((1/N_t) sum_j exp(l_j)) - <h|h>/2 - <d|d>/2.
-__device__ inline double tm_finish(const LikeConst& L, const float (*wms)[2], int n_warps, double HH) {
+// Time-marginalised logL of record r from the warps' (max, sum) pairs and
+// detector sums D, both added in warp order: log((1/N_t) sum_j exp(l_j)) -
+// <h|h>/2 - <d|d>/2.  By a warp: a warp's pair, a detector, a logarithm per lane
+// (on one thread the FP64 chains took 39,000 cycles of an evaluation's 100,000).
+template <int NDET>
+__device__ inline double tm_finish(const LikeConst& L, const EvalRecord& r, const float (*hh)[NDET],
+                                   const float (*wms)[2], int n_warps, int lane) {
+  const unsigned full = 0xffffffffu;
+  double d = 0.0, a = 0.0, iden = 0.0;
+  if (lane < NDET) {
+    for (int w = 0; w < n_warps; ++w) d += (double)hh[w][lane];
+    a = (r.cre[lane] * r.cre[lane] + r.cim[lane] * r.cim[lane]) * (L.het_b0[lane] - d);
+    iden = L.het_fid_iden[lane];
+  }
+  double HH = 0.0;
+#pragma unroll
+  for (int i = 0; i < NDET; ++i) HH += __shfl_sync(full, a, i) * __shfl_sync(full, iden, i);
   float M = -INFINITY;
   for (int w = 0; w < n_warps; ++w) M = fmaxf(M, wms[w][0]);
+  const bool on = lane < n_warps && wms[lane][0] > -INFINITY;
+  const double e = on ? exp((double)wms[lane][0] - (double)M) : 0.0, ws = on ? (double)wms[lane][1] : 0.0;
+  const unsigned some = __ballot_sync(full, on);
   double S = 0.0;
-  for (int w = 0; w < n_warps; ++w)
-    if (wms[w][0] > -INFINITY) S += (double)wms[w][1] * exp((double)wms[w][0] - (double)M);
-  return (double)M + log(S) - log((double)L.tm_n) - 0.5 * HH - 0.5 * L.DD;
+  for (int w = 0; w < n_warps; ++w) {
+    const double ew = __shfl_sync(full, e, w), sw = __shfl_sync(full, ws, w);
+    if ((some >> w) & 1u) S += sw * ew;
+  }
+  const double lg = log(lane == 0 ? S : (double)L.tm_n);
+  return (double)M + __shfl_sync(full, lg, 0) - __shfl_sync(full, lg, 1) - 0.5 * HH - 0.5 * L.DD;
 }
 
 // Per-detector sums cached for projection-only evaluations: (Z_i / C_i) /

@@ -192,7 +192,7 @@ struct DeviceBuffers {
   float2* het_tm_w = nullptr;       // [N_b + 1] exp(-2 pi i f_e dt), the step between grid nodes
   // ... by non-uniform FFT (L.tm_M > 0): kernel weight of every (grid point,
   // edge) entry in grid-point order, deconvolution 1 / Phi per node, twiddles
-  float* het_nu_wt = nullptr;       // [entries]
+  float* het_nu_wt = nullptr;       // [pieces / 32][kNufftPiece][32]
   float* het_nu_corr = nullptr;     // [N_t]
   float2* het_nu_tw = nullptr;      // [M] stage-major twiddles: span h at h - 1 + p, exp(2 pi i p / (2 h))
   int4* het_nu_piece = nullptr;     // [pieces] (first entry, entries, first edge, 0)

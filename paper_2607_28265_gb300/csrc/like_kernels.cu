@@ -491,14 +491,9 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
     s_tm[warp][1] = ws;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double HH = 0.0;
-    for (int i = 0; i < NDET; ++i) {
-      double d = 0.0;
-      for (int w = 0; w < n_warps; ++w) d += (double)s_hh[w][i];
-      HH += (r.cre[i] * r.cre[i] + r.cim[i] * r.cim[i]) * (L.het_b0[i] - d) * L.het_fid_iden[i];
-    }
-    out[th] = tm_finish(L, s_tm, n_warps, HH);
+  if (warp == 0) {
+    const double ll = tm_finish<NDET>(L, r, s_hh, s_tm, n_warps, lane);
+    if (lane == 0) out[th] = ll;
   }
 }
 
