@@ -88,17 +88,6 @@ __device__ __forceinline__ EndResult end_result(unsigned inside, unsigned ok, in
   return e;
 }
 
-// theta_valid on the bits.  (A component of 2^1000 or more, whose sum may
-// overflow, takes the sum.)
-__device__ __forceinline__ bool chain_theta_valid(const double* th) {
-  bool big = false;
-#pragma unroll
-  for (int j = 0; j < SWIG_N_PARAMS; ++j) big = big || (__double2hiint(th[j]) & 0x7fffffff) >= (1023 + 1000) << 20;
-  if (big) return theta_valid(th);
-  const long long mc = __double_as_longlong(th[0]), q = __double_as_longlong(th[1]), dl = __double_as_longlong(th[6]);
-  return mc > 0 && q > 0 && q <= 0x3FF0000000000000ll && dl > 0;
-}
-
 // Apply the results of the pending candidates in the step's order.  ok: the
 // candidates whose logL exceeds logL* (bits).  Returns the accepted candidate
 // or -1.  All lanes compute; lane 0 writes the state.
@@ -521,7 +510,7 @@ __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerC
     }
     bool valid = false;
     if ((inside >> lane) & 1u) {
-      valid = chain_theta_valid(w.th[lane]);
+      valid = theta_valid_bits(w.th[lane]);
       if (!valid) w.ly[lane] = -INFINITY;
     }
     const unsigned act = __ballot_sync(0xffffffffu, valid);

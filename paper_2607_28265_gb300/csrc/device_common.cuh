@@ -106,14 +106,17 @@ struct MassTerms {
   double eta, dm, m1, m2, A, r, ir, lpm;
 };
 
-__host__ __device__ inline MassTerms taylorf2_mass_terms(double mc, double q) {
-  MassTerms t;
-  const double opq = 1.0 + q;
-  const double inv_opq = 1.0 / opq, inv_q = 1.0 / q;
+// Those that follow from the mass ratio alone.
+__host__ __device__ inline void taylorf2_ratio_terms(double q, MassTerms& t) {
+  const double opq = 1.0 + q, inv_opq = 1.0 / opq;
   t.m1 = inv_opq;
   t.m2 = q * inv_opq;
   t.dm = (1.0 - q) * inv_opq;                 // (m1 - m2) / M
   t.eta = t.m1 * t.m2;                        // q / (1 + q)^2
+}
+// The others.
+__host__ __device__ inline void taylorf2_scale_terms(double mc, double q, MassTerms& t) {
+  const double opq = 1.0 + q, inv_q = 1.0 / q;
   const double inv_eta = opq * opq * inv_q;   // 1 / eta
   t.A = (3.0 / (256.0 * kPi)) * inv_eta;      // 3 / (128 eta) in cycles
   // ln(pi M) = ln(pi T_sun Mc) - (3/5) ln eta = ln((pi T_sun Mc)^5 / eta^3) / 5
@@ -122,6 +125,11 @@ __host__ __device__ inline MassTerms taylorf2_mass_terms(double mc, double q) {
   t.lpm = 0.2 * log(x2 * x2 * x * (inv_eta * inv_eta * inv_eta));
   t.r = exp(t.lpm * (1.0 / 3.0));
   t.ir = 1.0 / t.r;
+}
+__host__ __device__ inline MassTerms taylorf2_mass_terms(double mc, double q) {
+  MassTerms t;
+  taylorf2_ratio_terms(q, t);
+  taylorf2_scale_terms(mc, q, t);
   return t;
 }
 
@@ -286,6 +294,17 @@ __device__ inline bool theta_valid(const double* th) {
   double s = 0.0;
   for (int j = 0; j < SWIG_N_PARAMS; ++j) s += th[j];
   return (th[0] > 0.0) && (th[1] > 0.0) && (th[1] <= 1.0) && (th[6] > 0.0) && isfinite(s);
+}
+
+// theta_valid on the bits: FP64 additions and comparisons cost 64 cycles each.  (A component of 2^1000 or more, whose sum may
+// overflow, takes the sum.)
+__device__ __forceinline__ bool theta_valid_bits(const double* th) {
+  bool big = false;
+#pragma unroll
+  for (int j = 0; j < SWIG_N_PARAMS; ++j) big = big || (__double2hiint(th[j]) & 0x7fffffff) >= (1023 + 1000) << 20;
+  if (big) return theta_valid(th);
+  const long long mc = __double_as_longlong(th[0]), q = __double_as_longlong(th[1]), dl = __double_as_longlong(th[6]);
+  return mc > 0 && q > 0 && q <= 0x3FF0000000000000ll && dl > 0;
 }
 
 // split = false leaves c_hi / c_lo to the caller (a warp splits the
