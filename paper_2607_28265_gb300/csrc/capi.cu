@@ -395,7 +395,6 @@ std::vector<float2> fold_abscissae() {
 
 void free_scratch(DeviceBuffers& B) {
   dfree(B.rec);
-  dfree(B.partials32);
   dfree(B.partials64);
   dfree(B.theta);
   dfree(B.out);
@@ -418,15 +417,10 @@ void free_problem(DeviceBuffers& B) {
   dfree(B.prior);
   dfree(B.het_edge_basis);
   dfree(B.het_edge_f);
-  dfree(B.het_inv_width);
   dfree(B.het_chunk);
-  dfree(B.het_dfe);
   B.het_nc = 0;
-  dfree(B.het_coef);
-  dfree(B.het_coefB);
   dfree(B.het_fid);
   dfree(B.het_ew);
-  dfree(B.het_tm_g);
   dfree(B.het_tm_w);
   dfree(B.het_nu_wt);
   dfree(B.het_nu_corr);
@@ -511,17 +505,22 @@ void weight_data(const swig_ctx* c, int n_det, std::vector<double>& dre, std::ve
   dre.assign((size_t)n_det * n, 0.0);
   dim.assign((size_t)n_det * n, 0.0);
   NSum dsum;
+  std::vector<double> p76(n), p73(n);  // the powers of f, once for all detectors
+  for (int64_t k = 0; k < n; ++k) {
+    const double f = (double)(c->k_min + k) * c->df;
+    p76[k] = std::pow(f, -7.0 / 6.0);
+    p73[k] = std::pow(f, -7.0 / 3.0);
+  }
   for (int i = 0; i < n_det; ++i) {
     NSum Ks;
     dmax[i] = 0.0;
     for (int64_t k = 0; k < n; ++k) {
-      const double f = (double)(c->k_min + k) * c->df;
       const double w = 4.0 * c->df / c->psd[i][k];
       const double re = c->data[i][2 * k], im = c->data[i][2 * k + 1];
-      const double a = w * std::pow(f, -7.0 / 6.0);
+      const double a = w * p76[k];
       dre[i * n + k] = a * re;
       dim[i * n + k] = -a * im;
-      Ks.add(w * std::pow(f, -7.0 / 3.0));
+      Ks.add(w * p73[k]);
       dsum.add(w * (re * re + im * im));
       dmax[i] = std::max(dmax[i], std::hypot(re, im) * a);
     }
@@ -847,8 +846,6 @@ int prepare_het(swig_ctx* c) {
   std::vector<float2> coefB;
   std::vector<double> a01;  // FP64 (A0.re, A0.im, A1.re, A1.im) for the edge weights
   het_summary(f, idx, nb, n_det, c->df, c->data, c->psd, h0, coef, coefB, a01);
-  std::vector<float> inv_w(nb);
-  for (int b = 0; b < nb; ++b) inv_w[b] = (float)(1.0 / (f[idx[b + 1]] - f[idx[b]]));
   std::vector<float> eb((size_t)(nb + 1) * 2 * NBASIS), ef((size_t)(nb + 1) * 2);
   // transposed (row per basis function and hi/lo part) so that a warp reads
   // 32 consecutive edges of a row
@@ -865,24 +862,15 @@ int prepare_het(swig_ctx* c) {
   std::vector<float> ct, dfe;
   const int nc = het_chunk_tables(f, idx, nb, ct, dfe);
   CUDA_TRY(c, cudaMalloc(&B.het_chunk, sizeof(float) * ct.size()));
-  CUDA_TRY(c, cudaMalloc(&B.het_dfe, sizeof(float) * dfe.size()));
   CUDA_TRY(c, cudaMemcpy(B.het_chunk, ct.data(), sizeof(float) * ct.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(B.het_dfe, dfe.data(), sizeof(float) * dfe.size(), cudaMemcpyHostToDevice));
-  c->h2d_bytes += sizeof(float) * (ct.size() + dfe.size());
+  c->h2d_bytes += sizeof(float) * ct.size();
   B.het_nc = nc;
   for (int i = 0; i < n_det; ++i) L.het_fid_iden[i] = 1.0 / (fid.cre[i] * fid.cre[i] + fid.cim[i] * fid.cim[i]);
   CUDA_TRY(c, cudaMalloc(&B.het_edge_basis, sizeof(float) * eb.size()));
   CUDA_TRY(c, cudaMalloc(&B.het_edge_f, sizeof(float) * ef.size()));
-  CUDA_TRY(c, cudaMalloc(&B.het_inv_width, sizeof(float) * inv_w.size()));
-  CUDA_TRY(c, cudaMalloc(&B.het_coef, sizeof(float4) * coef.size()));
-  CUDA_TRY(c, cudaMalloc(&B.het_coefB, sizeof(float2) * coefB.size()));
   CUDA_TRY(c, cudaMemcpy(B.het_edge_basis, eb.data(), sizeof(float) * eb.size(), cudaMemcpyHostToDevice));
   CUDA_TRY(c, cudaMemcpy(B.het_edge_f, ef.data(), sizeof(float) * ef.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(B.het_inv_width, inv_w.data(), sizeof(float) * inv_w.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(B.het_coef, coef.data(), sizeof(float4) * coef.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(B.het_coefB, coefB.data(), sizeof(float2) * coefB.size(), cudaMemcpyHostToDevice));
-  c->h2d_bytes += sizeof(float) * (eb.size() + ef.size() + inv_w.size()) + sizeof(float4) * coef.size() +
-                  sizeof(float2) * coefB.size();
+  c->h2d_bytes += sizeof(float) * (eb.size() + ef.size());
   std::vector<float2> g, w;
   if (L.tm_n > 0) {
     L.tm_M = 0;
@@ -930,11 +918,9 @@ int prepare_het(swig_ctx* c) {
       CUDA_TRY(c, cudaMemcpy(B.het_nu_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice));
       c->h2d_bytes += sizeof(float) * (wt.size() + corr.size()) + sizeof(float2) * tw.size();
     }
-    CUDA_TRY(c, cudaMalloc(&B.het_tm_g, sizeof(float2) * g.size()));
     CUDA_TRY(c, cudaMalloc(&B.het_tm_w, sizeof(float2) * w.size()));
-    CUDA_TRY(c, cudaMemcpy(B.het_tm_g, g.data(), sizeof(float2) * g.size(), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMemcpy(B.het_tm_w, w.data(), sizeof(float2) * w.size(), cudaMemcpyHostToDevice));
-    c->h2d_bytes += sizeof(float2) * (g.size() + w.size());
+    c->h2d_bytes += sizeof(float2) * w.size();
   } else {
     het_tm_tables(a01, f, idx, nb, n_det, 0.0, g, w);
   }
@@ -998,7 +984,6 @@ int ensure_scratch(swig_ctx* c, int n) {
   // partial sums of the FP64 batch (4096 at a time) and of the dataflow
   // sampler's request slots (at most 4096): up to 4 per (theta, slice)
   const size_t units = (size_t)c->L.n_slices * 4 * std::min(cap, 4096);
-  CUDA_TRY(c, cudaMalloc(&B.partials32, sizeof(float) * kPartialStride * units));
   CUDA_TRY(c, cudaMalloc(&B.partials64, sizeof(double) * kPartialStride * units));
   CUDA_TRY(c, cudaMalloc(&B.theta, sizeof(double) * SWIG_N_PARAMS * cap));
   CUDA_TRY(c, cudaMalloc(&B.out, sizeof(double) * cap));

@@ -32,11 +32,7 @@ struct HetTables {
   int n_bins;                 // N_b
   const float* edge_basis;    // [2 * NBASIS][N_b + 1] phi_j(f_e): row 2j hi parts, row 2j+1 lo parts
   const float* edge_f;        // [2][N_b + 1] f_e: hi parts, lo parts
-  const float* inv_width;     // [N_b] 1 / (e_{b+1} - e_b)
-  const float4* coef;         // [n_det][N_b] (A0.re, A0.im, A1.re, A1.im)
-  const float2* coefB;        // [n_det][N_b] (B0, B1)
   const EvalRecord* fid;      // fiducial record
-  const float2* tm_g;         // [n_det][N_b + 1] time marginalisation: edge weights g_ie
   const float2* tm_w;         // [N_b + 1] exp(-2 pi i f_e dt), one grid step
   // non-uniform FFT form of the time pass (see het_nufft_tables)
   const float* nu_wt;
@@ -47,7 +43,6 @@ struct HetTables {
   // chunk anchors (kernels.h HetChunkRow)
   int n_chunks;
   const float* chunk;  // [HC_ROWS][n_chunks]
-  const float* dfe;    // [n_chunks][32]
   // edge weights of the contraction (het_edge_weights in capi.cu): per chunk,
   // detector and lane (Re g_ie, Im g_ie, B0_ib / 2, f_e - f_a with detector 0)
   const float4* ew;    // [n_chunks][n_det][32]
@@ -58,11 +53,7 @@ __host__ __device__ inline HetTables het_tables(const DeviceBuffers& B) {
   H.n_bins = B.het_nb;
   H.edge_basis = B.het_edge_basis;
   H.edge_f = B.het_edge_f;
-  H.inv_width = B.het_inv_width;
-  H.coef = B.het_coef;
-  H.coefB = B.het_coefB;
   H.fid = B.het_fid;
-  H.tm_g = B.het_tm_g;
   H.tm_w = B.het_tm_w;
   H.nu_wt = B.het_nu_wt;
   H.nu_corr = B.het_nu_corr;
@@ -71,7 +62,6 @@ __host__ __device__ inline HetTables het_tables(const DeviceBuffers& B) {
   H.nu_point = B.het_nu_point;
   H.n_chunks = B.het_nc;
   H.chunk = B.het_chunk;
-  H.dfe = B.het_dfe;
   H.ew = B.het_ew;
   return H;
 }
@@ -85,20 +75,6 @@ struct HetPrep {
   float rho_re[NDET], rho_im[NDET];
 };
 
-template <int NDET>
-__device__ inline void het_prepare(const LikeConst& L, const HetTables& H, const EvalRecord& r, HetPrep<NDET>& p) {
-  const EvalRecord& f0 = *H.fid;
-#pragma unroll
-  for (int j = 0; j < NBASIS; ++j) p.dc[j] = df_from_double(r.c[j] - f0.c[j]);
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-    p.dtau[i] = df_from_double(r.tau[i] - f0.tau[i]);
-    const double iden = L.het_fid_iden[i];
-    p.rho_re[i] = (float)((r.cre[i] * f0.cre[i] + r.cim[i] * f0.cim[i]) * iden);
-    p.rho_im[i] = (float)((r.cim[i] * f0.cre[i] - r.cre[i] * f0.cim[i]) * iden);
-  }
-}
-
 // The differences by a warp, one per lane, against the fiducial's c and tau.
 template <int NDET>
 __device__ __forceinline__ void het_differences(const double* f0c, const double* f0tau, const EvalRecord& r,
@@ -111,7 +87,7 @@ __device__ __forceinline__ void het_differences(const double* f0c, const double*
   __syncwarp();
 }
 
-// het_prepare by a warp, one constant per lane.
+// The constants by a warp, one per lane.
 template <int NDET>
 __device__ __forceinline__ void het_prepare_warp(const LikeConst& L, const HetTables& H, const EvalRecord& r,
                                                  HetPrep<NDET>& p, int lane) {
@@ -125,169 +101,6 @@ __device__ __forceinline__ void het_prepare_warp(const LikeConst& L, const HetTa
   het_differences<NDET>(f0.c, f0.tau, r, p, lane);
 }
 
-// Anchor of chunk q for one evaluation (one thread per chunk; rows of the
-// chunk table are read coalesced across threads): the phase difference
-// dP(f) = sum_j (c_j - c0_j) phi_j(f) at the chunk's first edge f_a in
-// double-float, its scaled derivatives a_1 (double-float sum, stored FP32)
-// and a_2..a_10 (FP32), per detector frac(dP(f_a) + f_a dtau_i), and whether
-// this evaluation's Taylor remainder bound sum_j |c_j - c0_j| HC_BND_j
-// exceeds kHetTaylorEps (then the chunk is taken edge by edge).
-template <int NDET>
-__device__ inline void het_anchor(const HetTables& H, const HetPrep<NDET>& p, int q, float* out) {
-  const int nc = H.n_chunks;
-  const float* T = H.chunk + q;
-  auto row = [&](int r) { return __ldg(T + (size_t)r * nc); };
-  dfl A = {0.0f, 0.0f}, S = {0.0f, 0.0f};
-  float a[kHetPoly], R = 0.0f;
-#pragma unroll
-  for (int n = 0; n < kHetPoly; ++n) a[n] = 0.0f;
-#pragma unroll
-  for (int j = 0; j < NBASIS; ++j) {
-    const dfl c = p.dc[j];
-    R = fmaf(fabsf(c.hi), row(HC_BND + j), R);
-    A = df_add(A, df_mul(c, dfl{row(HC_VAL_HI + j), row(HC_VAL_LO + j)}));
-    S = df_add(S, df_mul(c, dfl{row(HC_D1_HI + j), row(HC_D1_LO + j)}));
-#pragma unroll
-    for (int n = 0; n < kHetPoly; ++n) a[n] = fmaf(c.hi, row(HC_POLY + n * NBASIS + j), a[n]);
-  }
-  out[0] = S.hi + S.lo;
-#pragma unroll
-  for (int n = 0; n < kHetPoly; ++n) out[1 + n] = a[n];
-  const dfl fa = {row(HC_FA_HI), row(HC_FA_LO)};
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) out[kHetAncPhase + i] = df_frac(df_add(A, df_mul(fa, p.dtau[i])));
-  out[kHetAncInvS] = row(HC_INV_S);
-  out[kHetAncExact] = R > kHetTaylorEps ? 1.0f : 0.0f;
-}
-
-// Bins [base, base + 31) of the contraction, accumulated into the lane's
-// per-detector sums: lane l holds edge base + l, bin base + l uses edges l and
-// l + 1 (the next edge by a shuffle).  All 32 lanes must call it together.
-// With TM the lanes also store the network edge products y_e of the time
-// marginalisation (each edge once: lanes 0..30, and the last edge).
-template <int NDET, bool TM = false>
-__device__ inline void het_chunk(const HetTables& H, const HetPrep<NDET>& p, int base, int lane, float* zr, float* zi,
-                                 float* hh, float2* y = nullptr) {
-  const float twopi = 6.283185307179586f;
-  const int e = base + lane;
-  float er[NDET], ei[NDET];
-  if (e <= H.n_bins) {
-    const size_t ne = (size_t)H.n_bins + 1;  // edges; lanes read consecutive edges of each row
-    dfl dp = {0.0f, 0.0f};
-#pragma unroll
-    for (int j = 0; j < NBASIS; ++j)
-      dp = df_add(dp, df_mul(p.dc[j], dfl{H.edge_basis[2 * j * ne + e], H.edge_basis[(2 * j + 1) * ne + e]}));
-    const dfl fe = {H.edge_f[e], H.edge_f[ne + e]};
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) {
-      const float ph = df_frac(df_add(dp, df_mul(fe, p.dtau[i])));
-      float s, co;
-      __sincosf(twopi * ph, &s, &co);  // exp(-2 pi i ph) = co - i s
-      er[i] = p.rho_re[i] * co + p.rho_im[i] * s;
-      ei[i] = p.rho_im[i] * co - p.rho_re[i] * s;
-    }
-    if (TM && (lane < 31 || e == H.n_bins)) {
-      float yr = 0.0f, yi = 0.0f;
-#pragma unroll
-      for (int i = 0; i < NDET; ++i) {
-        const float2 g = H.tm_g[(size_t)i * ne + e];
-        yr += g.x * er[i] - g.y * ei[i];
-        yi += g.x * ei[i] + g.y * er[i];
-      }
-      y[e] = make_float2(yr, yi);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) er[i] = ei[i] = 0.0f;
-  }
-  const int b = base + lane;
-  const bool has_bin = lane < 31 && b < H.n_bins;
-  const float iw = has_bin ? H.inv_width[b] : 0.0f;
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-    const float nr = __shfl_down_sync(0xffffffffu, er[i], 1);
-    const float ni = __shfl_down_sync(0xffffffffu, ei[i], 1);
-    if (has_bin) {
-      const float r0r = 0.5f * (er[i] + nr), r0i = 0.5f * (ei[i] + ni);
-      const float r1r = (nr - er[i]) * iw, r1i = (ni - ei[i]) * iw;
-      const float4 a = H.coef[(size_t)i * H.n_bins + b];
-      const float2 bb = H.coefB[(size_t)i * H.n_bins + b];
-      zr[i] += a.x * r0r - a.y * r0i + a.z * r1r - a.w * r1i;
-      zi[i] += a.x * r0i + a.y * r0r + a.z * r1i + a.w * r1r;
-      hh[i] += bb.x * (r0r * r0r + r0i * r0i) + 2.0f * bb.y * (r0r * r1r + r0i * r1i);
-    }
-  }
-}
-
-// Per-lane table data of one chunk step: edge offset, bin width and summary
-// data of the lane's bin.
-template <int NDET>
-struct HetBinData {
-  float d, iw;
-  float4 a[NDET];
-  float2 bb[NDET];
-};
-
-// het_chunk with the phase from chunk q's anchor `anc` (het_anchor) and the
-// lane's table data t (het_read_stage): lane l holds edge 31 q + l at
-// x = (f_e - f_a) / S, dP = sum_n a_n x^n (degree 10, FP32 Horner),
-// phase_i = frac(anchor_i + dP + (f_e - f_a) dtau_i).
-template <int NDET, bool TM = false>
-__device__ inline void het_chunk_anc(const HetTables& H, const HetPrep<NDET>& p, const float* anc, int q, int lane,
-                                     const HetBinData<NDET>& t, float* zr, float* zi, float* hh,
-                                     float2* y = nullptr) {
-  const float twopi = 6.283185307179586f;
-  const int base = 31 * q, e = base + lane;
-  float er[NDET], ei[NDET];
-  if (e <= H.n_bins) {
-    const float x = t.d * anc[kHetAncInvS];
-    float v = anc[kHetPoly];
-#pragma unroll
-    for (int n = kHetPoly - 1; n >= 0; --n) v = fmaf(v, x, anc[n]);
-    v *= x;
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) {
-      float ph = anc[kHetAncPhase + i] + fmaf(t.d, p.dtau[i].hi, v);
-      ph -= round_nearest(ph);
-      float s, co;
-      __sincosf(twopi * ph, &s, &co);  // exp(-2 pi i ph) = co - i s
-      er[i] = p.rho_re[i] * co + p.rho_im[i] * s;
-      ei[i] = p.rho_im[i] * co - p.rho_re[i] * s;
-    }
-    if (TM && (lane < 31 || e == H.n_bins)) {
-      float yr = 0.0f, yi = 0.0f;
-      const size_t ne = (size_t)H.n_bins + 1;
-#pragma unroll
-      for (int i = 0; i < NDET; ++i) {
-        const float2 g = H.tm_g[(size_t)i * ne + e];
-        yr += g.x * er[i] - g.y * ei[i];
-        yi += g.x * ei[i] + g.y * er[i];
-      }
-      y[e] = make_float2(yr, yi);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) er[i] = ei[i] = 0.0f;
-  }
-  const bool has_bin = lane < 31 && base + lane < H.n_bins;
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-    const float nr = __shfl_down_sync(0xffffffffu, er[i], 1);
-    const float ni = __shfl_down_sync(0xffffffffu, ei[i], 1);
-    if (has_bin) {
-      const float r0r = 0.5f * (er[i] + nr), r0i = 0.5f * (ei[i] + ni);
-      const float r1r = (nr - er[i]) * t.iw, r1i = (ni - ei[i]) * t.iw;
-      const float4 a = t.a[i];
-      const float2 bb = t.bb[i];
-      zr[i] += a.x * r0r - a.y * r0i + a.z * r1r - a.w * r1i;
-      zi[i] += a.x * r0i + a.y * r0r + a.z * r1i + a.w * r1r;
-      hh[i] += bb.x * (r0r * r0r + r0i * r0i) + 2.0f * bb.y * (r0r * r1r + r0i * r1i);
-    }
-  }
-}
-
-// Asynchronous global -> shared copies (cp.async, sm_80 and later): the
-// lane's own table entries of a chunk, waited for one chunk later.
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
 }
@@ -298,97 +111,6 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// Layout of one stage (kernels.h het_stage_bytes): a[NDET][32] (float4),
-// bb[NDET][32] (float2), iw[32], d[32].
-template <int NDET>
-struct HetStage {
-  float4 a[NDET][32];
-  float2 bb[NDET][32];
-  float iw[32];
-  float d[32];
-};
-
-// Lane l copies the entries of its bin 31 q + l and edge 31 q + l (the
-// entries it reads itself, so no cross-lane ordering is needed).
-template <int NDET>
-__device__ __forceinline__ void het_stage_chunk(const HetTables& H, int q, int lane, HetStage<NDET>* st) {
-  const int b = 31 * q + lane;
-  if (lane < 31 && b < H.n_bins) {
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) {
-      cp_async<16>(&st->a[i][lane], H.coef + (size_t)i * H.n_bins + b);
-      cp_async<8>(&st->bb[i][lane], H.coefB + (size_t)i * H.n_bins + b);
-    }
-    cp_async<4>(&st->iw[lane], H.inv_width + b);
-  }
-  if (b <= H.n_bins) cp_async<4>(&st->d[lane], H.dfe + (size_t)q * kHetChunkEdges + lane);
-}
-
-template <int NDET>
-__device__ __forceinline__ void het_read_stage(const HetTables& H, int q, int lane, const HetStage<NDET>* st,
-                                               HetBinData<NDET>& t) {
-  const int b = 31 * q + lane;
-  const bool has_bin = lane < 31 && b < H.n_bins;
-  t.d = b <= H.n_bins ? st->d[lane] : 0.0f;
-  t.iw = has_bin ? st->iw[lane] : 0.0f;
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-    t.a[i] = has_bin ? st->a[i][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    t.bb[i] = has_bin ? st->bb[i][lane] : make_float2(0.0f, 0.0f);
-  }
-}
-
-// The chunks q = first, first + stride, ... of one evaluation by one warp:
-// anchored chunks (het_chunk_anc) read their table data from the warp's two
-// shared-memory stages (`stage`, 2 x het_stage_bytes), filled by cp.async one
-// chunk ahead, or straight from global memory when there is no room for the
-// stages (stage == nullptr); exact chunks go edge by edge (het_chunk).
-template <int NDET, bool TM = false>
-__device__ inline void het_chunks_warp(const HetTables& H, const HetPrep<NDET>& p, const float* s_anc, int first,
-                                       int stride, int lane, unsigned char* stage, float* zr, float* zi, float* hh,
-                                       float2* y = nullptr) {
-  const int nc = H.n_chunks;
-  if (stage == nullptr) {
-    for (int q = first; q < nc; q += stride) {
-      const float* an = s_anc + q * kHetAncStride;
-      if (an[kHetAncExact] != 0.0f) {
-        het_chunk<NDET, TM>(H, p, 31 * q, lane, zr, zi, hh, y);
-        continue;
-      }
-      const int b = 31 * q + lane;
-      const bool has_bin = lane < 31 && b < H.n_bins;
-      HetBinData<NDET> t;
-      t.d = b <= H.n_bins ? __ldg(H.dfe + (size_t)q * kHetChunkEdges + lane) : 0.0f;
-      t.iw = has_bin ? __ldg(H.inv_width + b) : 0.0f;
-#pragma unroll
-      for (int i = 0; i < NDET; ++i) {
-        t.a[i] = has_bin ? __ldg(H.coef + (size_t)i * H.n_bins + b) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        t.bb[i] = has_bin ? __ldg(H.coefB + (size_t)i * H.n_bins + b) : make_float2(0.0f, 0.0f);
-      }
-      het_chunk_anc<NDET, TM>(H, p, an, q, lane, t, zr, zi, hh, y);
-    }
-    return;
-  }
-  HetStage<NDET>* st = reinterpret_cast<HetStage<NDET>*>(stage);
-  if (first < nc) het_stage_chunk<NDET>(H, first, lane, st);
-  cp_async_commit();
-  int buf = 0;
-  for (int q = first; q < nc; q += stride, buf ^= 1) {
-    if (q + stride < nc) het_stage_chunk<NDET>(H, q + stride, lane, st + (buf ^ 1));
-    cp_async_commit();
-    cp_async_wait<1>();  // this lane's copies of chunk q have landed
-    const float* an = s_anc + q * kHetAncStride;
-    if (an[kHetAncExact] != 0.0f) {
-      het_chunk<NDET, TM>(H, p, 31 * q, lane, zr, zi, hh, y);
-    } else {
-      HetBinData<NDET> t;
-      het_read_stage<NDET>(H, q, lane, st + buf, t);
-      het_chunk_anc<NDET, TM>(H, p, an, q, lane, t, zr, zi, hh, y);
-    }
-  }
-  cp_async_wait<0>();
-}
 
 // ---------------------------------------------------------------------------
 // Contraction by edges.  r_i(e) = rho_i u_i(e) with |u| = 1, so with the hat
@@ -456,8 +178,7 @@ static_assert(HB_POLY + kHetPoly == kHetBaseRows, "base rows");
 
 // One quarter (sub 0 .. 3) of the anchors of chunk q for N evaluations, value m
 // of evaluation k to out[N m + k]: sub 0 the phases frac(dP(f_a) + f_a dtau_i),
-// sub 1 a_1, 1 / S and the exact flag, sub 2 and 3 the Taylor terms (het_anchor
-// has them all for one evaluation on one thread).  WITH 1: from the base rows
+// sub 1 a_1, 1 / S and the exact flag, sub 2 and 3 the Taylor terms.  WITH 1: from the base rows
 // (stride nc) and the moved functions; -1: the base rows themselves (N = 1),
 // at out[m nc].
 template <int NDET, int N, int WITH = 0>
@@ -714,19 +435,6 @@ __device__ __forceinline__ void het_network(const LikeConst& L, const EvalRecord
   const double k1 = __shfl_sync(full, k2[1], lane < 2 * NDET ? lane >> 1 : 0);
   kap = lane < 2 * NDET ? ((lane & 1) ? k1 : k0) : 0.0;
   vv = lane < NDET ? vi : 0.0;
-}
-
-// Warp-sum of the lane sums (all lanes receive them).
-template <int NDET>
-__device__ inline void het_warp_reduce(float* zr, float* zi, float* hh) {
-#pragma unroll
-  for (int i = 0; i < NDET; ++i)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      zr[i] += __shfl_xor_sync(0xffffffffu, zr[i], o);
-      zi[i] += __shfl_xor_sync(0xffffffffu, zi[i], o);
-      hh[i] += __shfl_xor_sync(0xffffffffu, hh[i], o);
-    }
 }
 
 // FP64 epilogue: plain Re Z or phase-marginalised log I0(|Z|), minus
@@ -1058,23 +766,6 @@ __device__ inline double tm_finish(const LikeConst& L, const EvalRecord& r, cons
   }
   const double lg = log(lane == 0 ? S : (double)L.tm_n);
   return (double)M + __shfl_sync(full, lg, 0) - __shfl_sync(full, lg, 1) - 0.5 * HH - 0.5 * L.DD;
-}
-
-// Per-detector sums cached for projection-only evaluations: (Z_i / C_i) /
-// inv_scale_i as the chain's kappa, and <h|h>_i / |C_i|^2 times A1^2 (the
-// heterodyned Z_i is linear and <h|h>_i quadratic in C_i).
-__device__ inline void het_cache(const LikeConst& L, const EvalRecord& r, int i, double zr, double zi, double hh,
-                                 double* kap2, double* vv) {
-  const double cr = r.cre[i], ci = r.cim[i], c2 = cr * cr + ci * ci;
-  if (c2 > 0.0) {
-    const double ic2 = 1.0 / c2, k = ic2 / L.inv_scale[i];
-    kap2[0] = (zr * cr + zi * ci) * k;
-    kap2[1] = (zi * cr - zr * ci) * k;
-    *vv = hh * ic2 * (L.amp1 * L.amp1);
-  } else {
-    kap2[0] = kap2[1] = 0.0;
-    *vv = 0.0;
-  }
 }
 
 }  // namespace swig

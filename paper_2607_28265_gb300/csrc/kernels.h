@@ -89,9 +89,6 @@ constexpr int kHetAncPair = 2 * kHetAncStride + 2;
 constexpr int kHetAncOne = kHetAncStride + 1;
 // Partial sums of a chain's current point per chunk (het.cuh).
 constexpr int kHetBaseRows = 5 + kHetPoly;
-// Per-warp shared-memory stage of one chunk's table data (summary data, bin
-// widths, edge offsets), filled by cp.async one chunk ahead: bytes per stage.
-inline size_t het_stage_bytes(int n_det) { return (size_t)n_det * 32 * (16 + 8) + 2 * 32 * 4; }
 
 // Folded full-grid sums (fold.cuh): the grid in chunks of kFoldNodes nodes.
 // Rows of the [FR_ROWS][ld] table (a column per chunk): at the chunk's centre f_c, with h the
@@ -179,16 +176,11 @@ struct DeviceBuffers {
   int het_nb = 0;
   float* het_edge_basis = nullptr;  // [2 * NBASIS][N_b + 1] (row per basis function, hi / lo)
   float* het_edge_f = nullptr;      // [2][N_b + 1] (hi row, lo row)
-  float* het_inv_width = nullptr;   // [N_b]
-  float4* het_coef = nullptr;       // [n_det][N_b]
-  float2* het_coefB = nullptr;      // [n_det][N_b]
   int het_nc = 0;                   // chunks of kHetChunkEdges edges
   float* het_chunk = nullptr;       // [HC_ROWS][het_nc] chunk anchor tables
-  float* het_dfe = nullptr;         // [het_nc][32] f_e - f_a of each chunk's edges
   EvalRecord* het_fid = nullptr;    // fiducial record
   float4* het_ew = nullptr;         // [het_nc][n_det][32] edge weights (HetTables::ew)
   // time marginalisation on the heterodyned bins (t_c marginalised)
-  float2* het_tm_g = nullptr;       // [n_det][N_b + 1] edge weights: Z_i = sum_e g_ie r_i(e)
   float2* het_tm_w = nullptr;       // [N_b + 1] exp(-2 pi i f_e dt), the step between grid nodes
   // ... by non-uniform FFT (L.tm_M > 0): kernel weight of every (grid point,
   // edge) entry in grid-point order, deconvolution 1 / Phi per node, twiddles
@@ -200,7 +192,6 @@ struct DeviceBuffers {
   // scratch for batched evaluation, sized for `cap` thetas
   int cap = 0;
   EvalRecord* rec = nullptr;     // [cap]
-  float* partials32 = nullptr;   // [cap][n_slices][kPartialStride]
   double* partials64 = nullptr;  // [cap][n_slices][kPartialStride]
   double* theta = nullptr;       // [cap][13] staging for host calls
   double* out = nullptr;         // [cap]
@@ -260,9 +251,9 @@ cudaError_t launch_waveform(const LikeConst& L, const double* theta_dev, EvalRec
 // and their kappa sums from the preceding likelihood launch); writes theta[6].
 cudaError_t launch_distance_draw(const LikeConst& L, const DeviceBuffers& B, const double* kappa, int n,
                                  long long first, unsigned k0, unsigned k1, double* theta, cudaStream_t st);
-// Heterodyned logL of n thetas (device pointers), one warp per theta.
+// Heterodyned logL of n thetas (device pointers), up to eight per CTA.
 // kappa_out (n x 8) / vv_out (n x 4), optional: the per-detector cache of
-// projection-only evaluations (het.cuh het_cache).
+// projection-only evaluations (het.cuh het_detector).
 // With t_c marginalised (L.tm_n > 0) one CTA of kHetTmThreads per theta
 // instead, and ell (optional, n x tm_n) receives each node's log weight.
 cudaError_t launch_loglike_het(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n, double* out,

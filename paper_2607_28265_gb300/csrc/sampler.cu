@@ -1,9 +1,7 @@
 // Persistent Slice-within-Gibbs nested sampler (Sec. 2.2, 2.3, 3.2 of the paper).
 //
 // One cooperative launch runs up to `max_iters` nested-sampling iterations on
-// the device.  Every CTA owns one slice of the frequency grid (its data staged
-// once in shared memory).  The grid meets at a barrier only around the
-// iteration boundary:
+// the device.  The grid meets at a barrier only around the iteration boundary:
 //
 //   boundary  (CTA 0, once per NS iteration): write the k finished chains back
 //             into the live set, sort the live log-likelihoods, test the
@@ -13,7 +11,10 @@
 //             logL* to the lowest survivor, estimate the live covariance and
 //             its per-block Cholesky factors, and start k chains at survivors.
 //
-// Within the iteration everything runs as a dataflow (k_ns_flow):
+// Within the iteration the mixed-precision and heterodyned runs have a CTA
+// advance a chain (chain.cuh).  The FP64 run is a dataflow here (k_ns_flow):
+// every CTA owns one slice of the frequency grid (its data staged once in shared
+// memory), and
 //
 //   control   (warp 0 of the chain's home CTA): advance the chain's hit-and-run
 //             slice state machine (Neal 2003 stepping-out and shrinkage along a
@@ -30,8 +31,7 @@
 //             CTA has counted itself done.
 //
 // Every spin-wait is bounded; on expiry the kernel records SWIG_E_TIMEOUT and
-// every CTA returns at its next barrier.  The heterodyned likelihood has its
-// own persistent kernel (k_ns_het, one CTA per chain).
+// every CTA returns at its next barrier.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -858,9 +858,7 @@ int run_setup(swig_ctx* c, RunState& R) {
   S.dlogz = c->cfg.dlogz;
   S.key0 = (unsigned)(c->cfg.seed & 0xFFFFFFFFu);
   S.key1 = (unsigned)(c->cfg.seed >> 32);
-  S.mixed = mixed ? 1 : 0;
   S.n_ctas = het || mixed ? chain_ctas : L.n_slices;
-  S.het = het ? 1 : 0;
   S.spin_limit = c->wait_limit;
   if ((rc = make_sky_frame(c, &S.sky))) return rc;
   int nd = 0;

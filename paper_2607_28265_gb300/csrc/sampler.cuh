@@ -44,9 +44,7 @@ struct SamplerConst {
   int max_iters;
   long long spin_limit;
   int n_ctas;
-  int mixed;
   int flow_parts;   // parts per slice (dataflow kernel): fixed summation partition
-  int het;          // heterodyned likelihood (projection-only evaluations use ChainState::vv)
   SkyFrame sky;     // detector-frame sky parameterisation (slots 9, 10), or off
   int learn_on;     // learned directions available (SWIG_PROPOSAL_LEARNED)
   float learn_mix;  // probability of a learned direction per slice step
