@@ -42,6 +42,7 @@ struct swig_ctx {
   int prepared_like = SWIG_LIKE_FULL;
   swig::LikeConst L = {};
   swig::DeviceBuffers B;
+  double* pinned = nullptr;  // vectors, then results of a small batch (mapped host memory)
   swig::SamplerState* sampler = nullptr;
   swig::Mlp* mlp = nullptr;
   long long wait_limit = 10000000;  // spins of a bounded device wait (~100 ns each)
