@@ -1200,8 +1200,14 @@ int prepare(swig_ctx* c) {
       ftab[3 * k + 1] = std::cbrt(f);
       ftab[3 * k + 2] = std::log(f);
     }
-    CUDA_TRY(c, cudaMalloc(&B.ftab, sizeof(double) * ftab.size()));
-    CUDA_TRY(c, cudaMemcpy(B.ftab, ftab.data(), sizeof(double) * ftab.size(), cudaMemcpyHostToDevice));
+    double* base = nullptr;
+    CUDA_TRY(c, cudaMalloc(&B.ftab, sizeof(double) * NBASIS * n));
+    CUDA_TRY(c, cudaMalloc(&base, sizeof(double) * ftab.size()));
+    cudaError_t e = cudaMemcpyAsync(base, ftab.data(), sizeof(double) * ftab.size(), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = launch_fp64_basis(L, base, B.ftab, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    cudaFree(base);
+    CUDA_TRY(c, e);
     L.n_tiles = 0;
   }
   // prior slots (defaults when no prior was set: every slot sampled uniform on [0,1])

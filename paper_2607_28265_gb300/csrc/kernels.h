@@ -160,7 +160,7 @@ struct DeviceBuffers {
   // problem data
   float2* data32 = nullptr;      // [n_det][n_bins] scaled D_i (MIXED)
   double2* data64 = nullptr;     // [n_det][n_bins] D_i (FP64)
-  double* ftab = nullptr;        // [n_bins][3] f^-1/3, f^1/3, ln f (FP64)
+  double* ftab = nullptr;        // [NBASIS][n_bins] basis functions, f in row B_ONE (FP64)
   TileInfo* tiles = nullptr;     // [n_tiles]
   TileBasis* basis = nullptr;    // [n_tiles]
   int* slice_begin = nullptr;    // [n_slices + 1] first bin of each slice
@@ -230,6 +230,9 @@ inline __host__ __device__ size_t fold_resident_bytes(int nc, int n_det) {
   return (size_t)nc * n_det * 32 * sizeof(float4) + sizeof(float) * FR_ROWS * fold_ld(nc);
 }
 
+// FP64 path: the basis functions at every bin, tab [NBASIS][n_bins] (f in row
+// B_ONE), from base [n_bins][3] (f^-1/3, f^1/3, ln f).
+cudaError_t launch_fp64_basis(const LikeConst& L, const double* base, double* tab, cudaStream_t st);
 // Node weights of the event (B.fold_w) from its weighted data (B.data32) and
 // the chunks (device pointer); synchronises the stream.
 cudaError_t launch_fold_weights(const LikeConst& L, const DeviceBuffers& B, const FoldChunk* chunks, cudaStream_t st);

@@ -161,6 +161,25 @@ __global__ void __launch_bounds__(32 * kSetupWarps)
   }
 }
 
+// A kernel whose start overlaps the one before it on st (it waits for that one's
+// end before it reads its results).
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, size_t bytes, cudaStream_t st, A... args) {
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // k_setup of n vectors.
 static void launch_setup(const LikeConst& L, const double* theta, int n, EvalRecord* rec, cudaStream_t st) {
   k_setup<<<dim3((n + 31) / 32, 2), 32 * kSetupWarps, 0, st>>>(L, theta, n, rec);
@@ -174,18 +193,44 @@ __global__ void __launch_bounds__(256)
   const int slice = blockIdx.x;
   const int b0 = slice_begin[slice], b1 = slice_begin[slice + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int th = blockIdx.y * 8 + warp; th < n; th += gridDim.y * 8) {
-    double v[2 * NDET];
-    sweep_warp_fp64<NDET>(L, data, ftab, b0, b1, rec[th], lane, v);
-#pragma unroll
-    for (int j = 0; j < 2 * NDET; ++j)
-      if (lane == j) partials[((size_t)th * L.n_slices + slice) * kPartialStride + j] = v[j];
+    sweep_warp_fp64<NDET>(L, data, ftab, b0, b1, rec[th], lane,
+                          partials + ((size_t)th * L.n_slices + slice) * kPartialStride);
   }
+}
+
+// The basis functions at every bin (rows of n values; f in row B_ONE) from
+// f^-1/3, f^1/3 and ln f.
+__global__ void k_fp64_basis(const double* __restrict__ base, long long k_min, double df, int n, double* __restrict__ tab) {
+  const int bin = blockIdx.x * blockDim.x + threadIdx.x;
+  if (bin >= n) return;
+  const double um = base[3 * (size_t)bin], up = base[3 * (size_t)bin + 1], lf = base[3 * (size_t)bin + 2];
+  const double u2 = um * um, p2 = up * up;
+  auto put = [&](int j, double v) { tab[(size_t)j * n + bin] = v; };
+  put(B_M53, u2 * u2 * um);
+  put(B_M1, u2 * um);
+  put(B_M23, u2);
+  put(B_M13, um);
+  put(B_LOG, lf);
+  put(B_P13, up);
+  put(B_P13LOG, up * lf);
+  put(B_P23, p2);
+  put(B_P53, p2 * p2 * up);
+  put(B_P73, p2 * p2 * up * p2);
+  put(B_ONE, (double)(k_min + bin) * df);
+}
+
+cudaError_t launch_fp64_basis(const LikeConst& L, const double* base, double* tab, cudaStream_t st) {
+  k_fp64_basis<<<(L.n_bins + 255) / 256, 256, 0, st>>>(base, L.k_min, L.df, L.n_bins, tab);
+  return cudaGetLastError();
 }
 
 // Per theta: FP64 sum of the slice partials (fixed order), then the epilogue.
 __global__ void k_reduce(LikeConst L, const double* __restrict__ partials, int n_units, const EvalRecord* __restrict__ rec,
                          int n, double* __restrict__ out, double* __restrict__ kappa_out) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int th = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (th >= n) return;
@@ -200,8 +245,9 @@ __global__ void k_reduce(LikeConst L, const double* __restrict__ partials, int n
   }
 #pragma unroll
   for (int j = 0; j < 2 * SWIG_MAX_DET; ++j)
+    if (j < 2 * L.n_det)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+      for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
   if (lane == 0) {
     double kre[SWIG_MAX_DET], kim[SWIG_MAX_DET];
     for (int i = 0; i < SWIG_MAX_DET; ++i) {
@@ -513,29 +559,11 @@ __global__ void __launch_bounds__(kHetTmThreads, 1)
   }
 }
 
-// A heterodyned kernel whose start overlaps the set-up kernel before it on st.
-template <typename... P, typename... A>
-cudaError_t launch_after_setup(void (*kern)(P...), int grid, size_t bytes, cudaStream_t st, A... args) {
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kHetTmThreads);
-  cfg.dynamicSmemBytes = bytes;
-  cfg.stream = st;
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 template <int NDET>
 cudaError_t launch_het_tm(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
                           double* kappa_out, double* vv_out, float* ell) {
   const HetTmLayout lay = het_tm_layout(L, B);
-  return launch_after_setup(k_het_tm<NDET>, n, lay.bytes, st, L, het_tables(B), (const EvalRecord*)B.rec, n,
+  return launch_after(k_het_tm<NDET>, dim3(n), kHetTmThreads, lay.bytes, st, L, het_tables(B), (const EvalRecord*)B.rec, n,
                             lay.anc_off, lay.panel, out, kappa_out, vv_out, ell);
 }
 
@@ -550,7 +578,7 @@ cudaError_t launch_het_plain(const LikeConst& L, const DeviceBuffers& B, int n, 
   const size_t tab = sizeof(float) * HC_ROWS * (size_t)B.het_nc;
   const int tab_off = bytes + tab <= 200 * 1024 ? (int)(bytes / sizeof(float)) : 0;
   if (tab_off) bytes += tab;
-  return launch_after_setup(k_het<NDET>, ctas < L.sm_count ? ctas : L.sm_count, bytes, st, L, het_tables(B),
+  return launch_after(k_het<NDET>, dim3(ctas < L.sm_count ? ctas : L.sm_count), kHetTmThreads, bytes, st, L, het_tables(B),
                             (const EvalRecord*)B.rec, n, per, tab_off, out, kappa_out, vv_out);
 }
 
@@ -632,14 +660,14 @@ cudaError_t launch_loglike_fp64(const LikeConst& L, const DeviceBuffers& B, cons
   launch_setup(L, theta, n, B.rec, st);
   const int gy = (n + 7) / 8 < 64 ? (n + 7) / 8 : 64;
   dim3 grid(L.n_slices, gy);
-  switch (L.n_det) {
-    case 1: k_sweep_fp64<1><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
-    case 2: k_sweep_fp64<2><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
-    case 3: k_sweep_fp64<3><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
-    default: k_sweep_fp64<4><<<grid, 256, 0, st>>>(L, B.data64, B.ftab, B.slice_begin, B.rec, n, B.partials64); break;
-  }
-  k_reduce<<<(n + 3) / 4, 128, 0, st>>>(L, B.partials64, L.n_slices, B.rec, n, out, kappa_out);
-  return cudaGetLastError();
+  const auto sweep = L.n_det == 1 ? k_sweep_fp64<1> : L.n_det == 2 ? k_sweep_fp64<2> : L.n_det == 3 ? k_sweep_fp64<3>
+                                                                                               : k_sweep_fp64<4>;
+  cudaError_t e = launch_after(sweep, grid, 256, 0, st, L, (const double2*)B.data64, (const double*)B.ftab,
+                               (const int*)B.slice_begin, (const EvalRecord*)B.rec, n, B.partials64);
+  if (e == cudaSuccess)
+    e = launch_after(k_reduce, dim3((n + 3) / 4), 128, 0, st, L, (const double*)B.partials64, L.n_slices,
+                     (const EvalRecord*)B.rec, n, out, kappa_out);
+  return e;
 }
 
 cudaError_t launch_prior_transform(const PriorSlot* slots, int n_sampled, const double* u, int n, double* theta,

@@ -628,11 +628,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1)
         {
           const int lo = (int)(((long long)nb * part) / G), hi = (int)(((long long)nb * (part + 1)) / G);
           const size_t pidx = (((size_t)cc * L.n_slices + slice) * G + part) * kPartialStride;
-          double v[2 * NDET];
-          sweep_warp_fp64<NDET>(L, B.data64, B.ftab, b0 + lo, b0 + hi, *rec, lane, v);
-#pragma unroll
-          for (int j = 0; j < 2 * NDET; ++j)
-            if (lane == j) B.partials64[pidx + j] = v[j];
+          sweep_warp_fp64<NDET>(L, B.data64, B.ftab, b0 + lo, b0 + hi, *rec, lane, B.partials64 + pidx);
         }
         __syncwarp();
         if (lane == 0) red_release_add(&P.done_cnt[cc], 1);

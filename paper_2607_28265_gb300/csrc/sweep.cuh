@@ -167,43 +167,65 @@ __device__ __forceinline__ void sweep_warp_mixed(const LikeConst& L, const float
   }
 }
 
-// FP64 per-bin evaluation over [b0, b1) by one warp (global-memory data).
+// Warp sums of V values per lane (a power of two): the upper lanes of a pair
+// take over half of the values at each level, so V = 2 costs 6 additions for the
+// 10 of one value after the other.  Returns the sum of value `which`, the same on
+// the 32 / V lanes that share it.
+template <int V>
+__device__ __forceinline__ double warp_sums(double* a, int lane, int& which) {
+  which = 0;
+  int o = 16;
+#pragma unroll
+  for (int h = V / 2; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+    which += up ? h : 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double send = up ? a[k] : a[k + h], keep = up ? a[k + h] : a[k];
+      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+  return a[0];
+}
+
+// FP64 per-bin evaluation over [b0, b1) by one warp (global-memory data): the
+// sums 2 i (real part) and 2 i + 1 of detector i to out[..].
+// FP64 instructions bound it (64 cycles of a scheduler each): the phase is one
+// multiply-add per basis function on their tabulated values (ftab, row j of
+// n_bins values; f itself in row B_ONE), the argument's reduction is left to
+// sincospi, the sums share their reduction.  4 s grid, one detector, 100
+// vectors with set-up and reduction: 68.6 -> 53.3 us (powers formed per bin, every
+// sum reduced by itself, a reduction before sincospi's own).
 template <int NDET>
 __device__ __forceinline__ void sweep_warp_fp64(const LikeConst& L, const double2* data, const double* ftab, int b0,
                                                 int b1, const EvalRecord& r, int lane, double* out) {
-  double acc_re[NDET], acc_im[NDET];
+  constexpr int V = NDET == 1 ? 2 : NDET == 2 ? 4 : 8;
+  double acc[V];
 #pragma unroll
-  for (int i = 0; i < NDET; ++i) acc_re[i] = acc_im[i] = 0.0;
+  for (int j = 0; j < V; ++j) acc[j] = 0.0;
   for (int bin = b0 + lane; bin < b1; bin += 32) {
-    const double f = (double)(L.k_min + bin) * L.df;
-    const double um = ftab[3 * (size_t)bin];      // f^-1/3
-    const double up = ftab[3 * (size_t)bin + 1];  // f^1/3
-    const double lf = ftab[3 * (size_t)bin + 2];  // ln f
-    const double u2 = um * um, p2 = up * up;
-    double P = r.c[B_ONE] + r.c[B_LOG] * lf;
-    P += um * (r.c[B_M13] + um * (r.c[B_M23] + um * (r.c[B_M1] + u2 * r.c[B_M53])));
-    P += up * (r.c[B_P13] + r.c[B_P13LOG] * lf) + p2 * r.c[B_P23] + p2 * p2 * up * (r.c[B_P53] + p2 * r.c[B_P73]);
+    double phi[NBASIS];
+#pragma unroll
+    for (int j = 0; j < NBASIS; ++j) phi[j] = __ldg(ftab + (size_t)j * L.n_bins + bin);
+    const double f = phi[B_ONE];
+    double P = r.c[B_ONE];
+#pragma unroll
+    for (int j = NBASIS - 1; j >= 0; --j)
+      if (j != B_ONE) P = fma(r.c[j], phi[j], P);
 #pragma unroll
     for (int i = 0; i < NDET; ++i) {
-      double ph = fma(f, r.tau[i], P);
-      ph -= rint(ph);
       double s, co;
-      sincospi(2.0 * ph, &s, &co);
+      sincospi(2.0 * fma(f, r.tau[i], P), &s, &co);
       const double2 dv = data[(size_t)i * L.n_bins + bin];
-      acc_re[i] += dv.x * co + dv.y * s;
-      acc_im[i] += dv.y * co - dv.x * s;
+      acc[2 * i] += dv.x * co + dv.y * s;
+      acc[2 * i + 1] += dv.y * co - dv.x * s;
     }
   }
-#pragma unroll
-  for (int i = 0; i < NDET; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      acc_re[i] += __shfl_xor_sync(0xffffffffu, acc_re[i], o);
-      acc_im[i] += __shfl_xor_sync(0xffffffffu, acc_im[i], o);
-    }
-    out[2 * i] = acc_re[i];
-    out[2 * i + 1] = acc_im[i];
-  }
+  int which;
+  const double v = warp_sums<V>(acc, lane, which);
+  if ((lane & (32 / V - 1)) == 0 && which < 2 * NDET) out[which] = v;
 }
 
 }  // namespace swig
