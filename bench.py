@@ -47,11 +47,9 @@ import swig_inputs as si  # noqa: E402
 
 SFU_OPS_PER_CLK_SM = 16   # sin/cos results per clock per SM (sm_100-class SFU), used if the probe fails
 SFU_OPS_PER_BIN_DET = 2   # one sine and one cosine per bin and detector
-# DRAM bytes (read + write) per logL evaluation inside k_ns_flow (512
-# threads), from one ncu capture of a 2-iteration launch of the 128 s workload
-# (10.03 MB + 0.31 MB over 107,944 evaluations; profiles/
-# k_ns_flow_cfg2_hlv_128s_2iter.md), scaled to a full launch by its evaluations.
-TRAFFIC_B_PER_EVAL = (10.032128e6 + 0.309504e6) / 107944
+# The folded full grid evaluates node sums, not bins: 64 nodes per chunk and
+# detector, 78 chunks for the 128 s grid (20-2048 Hz).
+NODES_128S = 64 * 78
 METRIC = "logL evals/s (128 s 3-det BNS) and wall-s/posterior, plain vs learned+mixed"
 
 # workload name -> (event, sampler options, description)
@@ -282,9 +280,7 @@ def run_campaign(args, rank, world):
     if rank != 0:
         return None
     n_post = len(wls) * args.steps
-    bindet = sum(r.n_sweep_evals * 3 * wl.n_bins for res, _ in out for r, wl in zip(res, wls))
     peak, peak_source = measure_sfu_peak()
-    achieved = SFU_OPS_PER_BIN_DET * bindet / (total_ms * 1e-3) / 1e12
     line = {
         "metric": METRIC, "value": full_all / (total_ms_max * 1e-3), "unit": "logL evals/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": total_ms_max / args.steps,
@@ -298,9 +294,10 @@ def run_campaign(args, rank, world):
         "e2e": {"value": e2e_all / (e2e_ms_max * 1e-3), "unit": "logL evals/s", "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": int(d2h), "ms_per_step": e2e_ms_max},
         "gpu_launches": launches,
-        "roofline": {"kernel": "k_ns_multi (campaign persistent kernel)", "bound": "alu", "achieved": achieved,
-                     "peak": peak, "unit": "SFU Top/s", "frac": achieved / peak, "traffic": None,
-                     "work_per_launch": "2 SFU ops x bin-detector evaluations of the four events",
+        "roofline": {"kernel": "k_ns_chain (persistent SwiG kernel, a CTA per chain, several events)",
+                     "bound": "latency", "achieved": None,
+                     "peak": peak, "unit": "SFU Top/s", "frac": None, "traffic": None,
+                     "work_per_launch": "node sums of the four events' folded grids (not counted)",
                      "timing": "CUDA events around each batch (the batch's persistent launches and host steps)",
                      "peak_source": peak_source},
         "clocks": clocks.summary(),
@@ -432,11 +429,17 @@ def run_gpu(args, rank, world):
     clk = clocks.summary()
     sm_mhz_max = 2070.0
     peak = peak_sfu  # SFU Top/s, measured on this GPU by peak_probe.cu
-    achieved = SFU_OPS_PER_BIN_DET * bindet / (pers_ms * 1e-3) / 1e12 if pers_ms > 0 else 0.0
-    n_bins_eval = spec.get("het_bins", 0) + 1 if het else wl.n_bins
-    kernel = "k_ns_het (persistent SwiG kernel, heterodyned)" if het else "k_ns_flow (persistent SwiG kernel, dataflow)"
-    traffic = (TRAFFIC_B_PER_EVAL * total_evals / max(1, pers_launch)
-               if TRAFFIC_B_PER_EVAL is not None and args.workload == "cfg2" else None)
+    fp64 = spec["precision"] == "fp64"
+    # phasors per evaluation and detector: bin edges, nodes of the folded 128 s
+    # grid (other folded grids: not counted), or bins
+    n_bins_eval = spec.get("het_bins", 0) + 1 if het else wl.n_bins if fp64 else (
+        NODES_128S if args.workload.startswith(("cfg2", "cfg5")) else None)
+    achieved = (SFU_OPS_PER_BIN_DET * bindet * (n_bins_eval / wl.n_bins if not het and not fp64 else 1.0)
+                / (pers_ms * 1e-3) / 1e12 if pers_ms > 0 and n_bins_eval else None)
+    kernel = ("k_ns_chain (persistent SwiG kernel, a CTA per chain, heterodyned)" if het else
+              "k_ns_flow (persistent SwiG kernel, FP64 dataflow)" if fp64 else
+              "k_ns_chain (persistent SwiG kernel, a CTA per chain, folded full grid)")
+    traffic = None
     line = {
         "metric": METRIC,
         # full-grid (or heterodyned) evaluations: those that run the sweep, the
@@ -470,11 +473,12 @@ def run_gpu(args, rank, world):
             "achieved": achieved,
             "peak": peak,
             "unit": "SFU Top/s",
-            "frac": achieved / peak if peak else None,
+            "frac": achieved / peak if peak and achieved is not None else None,
             "traffic": traffic,
-            "traffic_unit": "bytes per launch (ncu, 2-iteration capture scaled by evaluations)",
-            "work_per_launch": (f"2 SFU ops x bin-detector evaluations (full evaluations x {len(wl.detectors)} x "
-                                f"{n_bins_eval} {'bin edges' if het else 'bins'})"),
+            "traffic_unit": "bytes per launch",
+            "work_per_launch": (f"2 SFU ops x phasors (full evaluations x {len(wl.detectors)} x "
+                                f"{n_bins_eval} {'bin edges' if het else 'bins' if fp64 else 'nodes'}); the latency "
+                                "of a chain's rounds bounds it, not this rate"),
             "launches": int(pers_launch),
             "avg_launch_ms": pers_ms / max(1, pers_launch),
             "peak_source": peak_source,
@@ -482,7 +486,7 @@ def run_gpu(args, rank, world):
         "clocks": clk,
     }
     if n_tm:
-        line["roofline"]["kernel"] = ("k_ns_het (persistent SwiG kernel, heterodyned, t_c marginalised: bin pass "
+        line["roofline"]["kernel"] = ("k_ns_chain (persistent SwiG kernel, heterodyned, t_c marginalised: edge pass "
                                       "plus the non-uniform FFT time pass)")
     if args.cpu_baseline and world == 1:
         line["cpu_baseline"] = cpu_baseline(args.workload, seconds=args.cpu_seconds,

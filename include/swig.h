@@ -109,12 +109,14 @@ typedef struct swig_sampler_cfg {
    * see Sec. 3.2 on fast and slow blocks).  A verification switch: the cached
    * and uncached samplers must agree in distribution.  0 = the cache. */
   int cache_off;
-  /* Launch shape of the full-grid mixed-precision sampler (0 selects the
-   * default in brackets; swig_autotune picks them per problem): slice parts,
-   * the number of sweep units each CTA's share of a proposal is split into,
-   * 1..4 [1]; stepout_one_end 1 steps a slice bracket out one end at a time
-   * instead of both ends in flight [0].  Both leave the evaluations and
-   * results the same up to the grouping of the per-part FP32 sums. */
+  /* Launch shape of the persistent samplers (0 selects the default in
+   * brackets; swig_autotune picks them per problem): flow_parts 1..4 [1] is
+   * how many points of a slice step are evaluated at a time (1: four rungs per
+   * bracket end and two draws, 2: two rungs, 3: one, 4: one and one draw; FP64:
+   * the sweep units that each CTA's share of a proposal is split into);
+   * stepout_one_end 1 steps a slice bracket out one end after the other
+   * instead of both at once [0].  Both leave the evaluations and results the
+   * same up to the grouping of the FP32 sums. */
   int flow_parts;
   int stepout_one_end;
 } swig_sampler_cfg;
@@ -276,9 +278,8 @@ int swig_autotune(swig_ctx* ctx, int iters, double* out, int n);
  * context keeps its samples.  Events that can share a launch (full grid, mixed
  * precision, covariance proposal, same detector count, chains and device) and
  * whose grids are within 1.5x of each other (the events of a launch advance
- * their iterations in step) run up to 4 at a time in one persistent launch: their slices of the
- * grid share each CTA's shared memory and their chains share the control and
- * sweep warps, which keeps the GPU busy while one event's chains wait.  Per
+ * their iterations in step) run up to 4 at a time in one persistent
+ * launch, whose CTAs take the chains of all events one after another.  Per
  * event the arithmetic and its order are those of swig_run, so the results
  * are the same; an event's persistent-kernel time in the profile is the
  * shared launch time.  Other events run one after another.  A context may
@@ -301,14 +302,13 @@ int swig_set_wait_limit(swig_ctx* ctx, long long spins);
  * set-up, out[17..19] the counts of the last three; out[20] milliseconds of
  * learned-proposal training (targets, Adam steps, output rows; CUDA events)
  * and out[21] the number of retrainings; out[22..24] for the first CTA's
- * sweep warps: (chain, slice) units evaluated, clock cycles spent in them and
- * cycles spent polling for work.  Then, for each CTA s of the last run's
+ * evaluations: units done, clock cycles spent in them and cycles in which they
+ * waited for the control.  Then, for each CTA s of the last run's
  * persistent kernel (single-event sampler), out[25 + 4 s .. 25 + 4 s + 3]:
- * its sweep warps' units, their cycles in units and polling, and its control
- * warp's cycles advancing chains.  In the heterodyned sampler a unit is one
- * contraction of a chain's proposal by the whole CTA (bin pass, time pass,
- * reductions), and the polling cycles are those the contracting warps wait
- * for the control warp (control and epilogue).  Writes min(n, 25 + 4 x CTAs)
+ * its units, their cycles, the waiting cycles and its control warp's cycles
+ * advancing chains.  A unit is one evaluation of a chain's candidate by the
+ * whole CTA; in the FP64 sampler one (chain, slice) sweep by a warp, the cycles
+ * waited those spent polling for work.  Writes min(n, 25 + 4 x CTAs)
  * values. */
 int swig_get_profile(swig_ctx* ctx, double* out, int n);
 /* Use `stream` (a cudaStream_t on the context's device, owned by the caller)
