@@ -54,7 +54,8 @@ struct ChainWork {
   int fl;                    // record pieces that the block moves
   int status;
   int bad[kCand];            // folded sums: outside the band, summed bin by bin
-  double fth[2 * kFreeRungs][SWIG_N_PARAMS];  // projection-only steps: a lane's theta
+  // projection-only steps: a lane's theta, the current point's sums
+  float fth[2 * kFreeRungs][SWIG_N_PARAMS], fkap[2 * SWIG_MAX_DET], fvv[SWIG_MAX_DET];
 };
 
 enum { ROUND_EVAL = 0, ROUND_DONE = 1 };
@@ -367,10 +368,23 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
   ChainState& ch = w.ch;
   const int b = ch.block, nb = S.block_size[b];
   const int row = lane & (2 * kFreeRungs - 1);
-  double* th = w.fth[row];
-  if (lane < 2 * kFreeRungs) {
+  float* th = w.fth[row];
+  {
+    // rounded once, a value per lane
+    const double x = lane < SWIG_N_PARAMS                        ? ch.th[lane]
+                     : lane < SWIG_N_PARAMS + 2 * SWIG_MAX_DET   ? ch.kap[lane - SWIG_N_PARAMS]
+                     : lane < SWIG_N_PARAMS + 3 * SWIG_MAX_DET   ? ch.vv[lane - SWIG_N_PARAMS - 2 * SWIG_MAX_DET]
+                                                                 : 0.0;
+    const float f = (float)x;
+    if (lane >= SWIG_N_PARAMS && lane < SWIG_N_PARAMS + 2 * SWIG_MAX_DET) w.fkap[lane - SWIG_N_PARAMS] = f;
+    if (lane >= SWIG_N_PARAMS + 2 * SWIG_MAX_DET && lane < SWIG_N_PARAMS + 3 * SWIG_MAX_DET)
+      w.fvv[lane - SWIG_N_PARAMS - 2 * SWIG_MAX_DET] = f;
 #pragma unroll
-    for (int s = 0; s < SWIG_N_PARAMS; ++s) th[s] = ch.th[s];
+    for (int s = 0; s < SWIG_N_PARAMS; ++s) {
+      const float v = __shfl_sync(0xffffffffu, f, s);
+      if (lane < 2 * kFreeRungs) th[s] = v;
+    }
+    __syncwarp();
   }
   // logL at bracket coordinate t of the lanes that are on (bits: inside, above logL*)
   double ly = 0.0;
@@ -381,10 +395,10 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
         const int j = S.block_dims[b][r], slot = S.slot_of_dim[j];
         const double v = ch.x[j] + t * ch.dir[j];
         if (!fp64_in_unit(v)) in = false;
-        if (in) th[slot] = prior_slot_inverse_f32(S.prior[slot], v);
+        if (in) th[slot] = (float)prior_slot_inverse_f32(S.prior[slot], v);
       }
     inside = __ballot_sync(0xffffffffu, in);
-    if (in) ly = free_loglike_mixed(L, th, ch.kap, HET ? ch.vv : nullptr);
+    if (in) ly = free_loglike_f32(L, th, w.fkap, HET ? w.fvv : nullptr);
     ok = __ballot_sync(0xffffffffu, in && ly > logl_star);
     __syncwarp();
   };
@@ -446,8 +460,9 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
     if (lane == hit) {
       for (int r = 0; r < nb; ++r) {
         const int j = S.block_dims[b][r], slot = S.slot_of_dim[j];
-        ch.x[j] = ch.x[j] + t * ch.dir[j];
-        ch.th[slot] = th[slot];
+        const double v = ch.x[j] + t * ch.dir[j];
+        ch.x[j] = v;
+        ch.th[slot] = prior_slot_inverse_f32(S.prior[slot], v);
       }
       ch.lx = ly;
       ch.proj_dirty = 1;

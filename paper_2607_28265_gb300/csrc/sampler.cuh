@@ -201,10 +201,11 @@ __device__ inline float log_i0_f32(float x) {
 // kap: per-detector sums cached at the chain's current point (full grid:
 // kappa_i; heterodyned: (Z_i / C_i) / inv_scale_i); vv (heterodyned only):
 // <h|h>_i / |C_i|^2 times A1^2, replacing the constant K_i A1^2 of the full grid.
-__device__ inline double free_loglike_mixed(const LikeConst& L, const double* th, const double* kap,
-                                            const double* vv = nullptr) {
-  const float mc = (float)th[0], dl = (float)th[6], iota = (float)th[7], psi = (float)th[8];
-  const float ra = (float)th[9], dec = (float)th[10], phic = (float)th[12];
+// th, kap and vv rounded to FP32 by the caller (a conversion takes a scheduler
+// 64 cycles).
+__device__ inline double free_loglike_f32(const LikeConst& L, const float* th, const float* kap, const float* vv) {
+  const float mc = th[0], dl = th[6], iota = th[7], psi = th[8];
+  const float ra = th[9], dec = th[10], phic = th[12];
   if (!(mc > 0.0f && dl > 0.0f)) return -INFINITY;
   const float rel = exp2f(0.8333333333f * log2f(mc)) / dl;  // Mc^(5/6) / d_L
   float sl, cl, sd, cd, sp, cp;
@@ -233,10 +234,10 @@ __device__ inline double free_loglike_mixed(const LikeConst& L, const double* th
     const float fp = form(X, X) - form(Y, Y), fx = 2.0f * form(X, Y);
     const float re0 = rel * fp * plus, im0 = rel * fx * cross;
     const float cre = re0 * cph - im0 * sph, cim = re0 * sph + im0 * cph;
-    const float a = (float)kap[2 * i] * L.amp_s[i], b = (float)kap[2 * i + 1] * L.amp_s[i];
+    const float a = kap[2 * i] * L.amp_s[i], b = kap[2 * i + 1] * L.amp_s[i];
     zr += cre * a - cim * b;
     zi += cre * b + cim * a;
-    hh += (cre * cre + cim * cim) * (vv ? (float)vv[i] : L.amp_k[i]);
+    hh += (cre * cre + cim * cim) * (vv ? vv[i] : L.amp_k[i]);
   }
   // with d_L marginalised the template is at 1 Mpc: zr, zi, hh are Z1, H1
   if (L.dist_marg) return distance_marg_logl(L, (double)zr, (double)zi, (double)hh);
