@@ -451,9 +451,9 @@ struct RowShared {
 // the weights in shared memory), a warp per 16 of the 256 hidden units: z1 and
 // z2 stay in the registers that the backward pass wants them in.
 // TRAIN false: outputs only.  1000 rows: about 9 us, of which 2.6 us until the
-// weights are there and 1.1 us for each 256 x 256 product (the shared memory
-// they are read from); 16 rows are the least that the product takes, so 63 SMs
-// work.
+// weights are there (taken in the order of their use, W2 in four groups: a step
+// 20.5 -> 19.9 us) and 1.1 us for each 256 x 256 product (the shared memory they
+// are read from); 16 rows are the least that the product takes, so 63 SMs work.
 template <bool TRAIN>
 __global__ void __launch_bounds__(kRowThreads) k_mlp_rows(RowArgs g) {
   extern __shared__ __align__(16) unsigned char s_raw[];
@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(kRowThreads) k_mlp_rows(RowArgs g) {
   chain_wait();
   for (int e = tid; e < kMlpInPad * (kMlpH / 8); e += kRowThreads)
     copy16(s.w1 + (e / (kMlpH / 8)) * kLdH + e % (kMlpH / 8) * 8, g.w1b + e * 8);
+  if (tid < kMlpH / 4) copy16(s.bias + 4 * tid, g.params + kMlpOffB1 + 4 * tid);
   const int tiles = mlp_rows(g.n) / 16;
   // lane addresses of the fragments: A [row][k]; B from [k][col] (transposed
   // on the way) and from [col][k]
@@ -474,23 +475,29 @@ __global__ void __launch_bounds__(kRowThreads) k_mlp_rows(RowArgs g) {
     const int r0 = 16 * tile;
     if (tid < 32) copy16(s.x + (tid >> 1) * kLdX + (tid & 1) * 8, g.xb + (size_t)r0 * kMlpInPad + tid * 8);
     copy_commit();
+    // the first tile's weights follow in the order of their use, a group each
     if (first) {
-      for (int e = tid; e < kMlpH * (kMlpH / 8); e += kRowThreads)
-        copy16(s.w2 + (e / (kMlpH / 8)) * kLdH + e % (kMlpH / 8) * 8, g.w2b + e * 8);
+#pragma unroll
+      for (int part = 0; part < 4; ++part) {
+        for (int e = part * (kMlpH / 4) * (kMlpH / 8) + tid; e < (part + 1) * (kMlpH / 4) * (kMlpH / 8); e += kRowThreads)
+          copy16(s.w2 + (e / (kMlpH / 8)) * kLdH + e % (kMlpH / 8) * 8, g.w2b + e * 8);
+        if (part == 0 && tid < kMlpH / 4) copy16(s.bias + kMlpH + 4 * tid, g.params + kMlpOffB2 + 4 * tid);
+        copy_commit();
+      }
       for (int e = tid; e < kMlpH * (kMlpOutPad / 8); e += kRowThreads)
         copy16(s.w3 + (e / (kMlpOutPad / 8)) * kLdO + e % (kMlpOutPad / 8) * 8, g.w3b + e * 8);
-      for (int e = tid; e < 2 * kMlpH + kMlpOutPad; e += kRowThreads)
-        s.bias[e] = e < kMlpH ? g.params[kMlpOffB1 + e]
-                              : e < 2 * kMlpH ? g.params[kMlpOffB2 + e - kMlpH]
-                                              : e < 2 * kMlpH + kMlpOut ? g.params[kMlpOffB3 + e - 2 * kMlpH] : 0.0f;
+      if (tid < kMlpOutPad / 4) copy16(s.bias + 2 * kMlpH + 4 * tid, g.params + kMlpOffB3 + 4 * tid);
+      copy_commit();
     }
-    copy_commit();
     float tgt = 0.0f;  // this lane's target of the warp's row: direction, then log-widths
     if (TRAIN && r0 + warp < g.n) {
       if (lane < kMlpIn) tgt = g.tdir[(size_t)(r0 + warp) * kMlpIn + lane];
       else if (lane < 2 * kMlpIn) tgt = g.tls[(size_t)(r0 + warp) * kMlpIn + lane - kMlpIn];
     }
-    copy_wait<1>();
+    if (first)
+      copy_wait<5>();
+    else
+      copy_wait<0>();
     __syncthreads();
     // Z1 = X W1 + b1
     float z1[2][4], z2[2][4];
@@ -532,19 +539,29 @@ __global__ void __launch_bounds__(kRowThreads) k_mlp_rows(RowArgs g) {
     mma_bf16_16816(z1[0], a, b);
     mma_bf16_16816(z1[1], a, b + 2);
     hidden(z1, s.bias, s.ha);
-    copy_wait<0>();
+    if (first) copy_wait<4>();
     __syncthreads();
     // Z2 = H1 W2 + b2
     if (TRAIN) put_rows(s.ha, g.h1b);
     zero(z2);
-#pragma unroll 4
-    for (int k0 = 0; k0 < kMlpH; k0 += 16) {
-      ldsm4<false>(a, s.ha + la * kLdH + k0 + lk);
-      ldsm4<true>(b, s.w2 + (k0 + la) * kLdH + c0 + lk);
-      mma_bf16_16816(z2[0], a, b);
-      mma_bf16_16816(z2[1], a, b + 2);
+#pragma unroll
+    for (int part = 0; part < 4; ++part) {
+      if (first && part > 0) {
+        if (part == 1) copy_wait<3>();
+        if (part == 2) copy_wait<2>();
+        if (part == 3) copy_wait<1>();
+        __syncthreads();
+      }
+#pragma unroll
+      for (int k0 = part * (kMlpH / 4); k0 < (part + 1) * (kMlpH / 4); k0 += 16) {
+        ldsm4<false>(a, s.ha + la * kLdH + k0 + lk);
+        ldsm4<true>(b, s.w2 + (k0 + la) * kLdH + c0 + lk);
+        mma_bf16_16816(z2[0], a, b);
+        mma_bf16_16816(z2[1], a, b + 2);
+      }
     }
     hidden(z2, s.bias + kMlpH, s.hb);
+    if (first) copy_wait<0>();
     __syncthreads();
     // O = H2 W3 + b3
     if (TRAIN) put_rows(s.hb, g.h2b);
@@ -699,7 +716,7 @@ __device__ __forceinline__ void take_gradient(const ColArgs& g, int p, float gr,
 // blocks, 4 columns each, come first: an FP64 add (or conversion) occupies a
 // scheduler for 64 cycles, so the 538 columns are spread over 135 SMs and
 // widened by integer instructions.  1000 rows: about 8 us.  A step of the two
-// kernels takes 20.5 us; products, epilogues, loss, column sums (one thread a
+// kernels takes 19.9 us; products, epilogues, loss, column sums (one thread a
 // column) and Adam as 16 kernels of a graph took 560 us.
 template <int STAGES>
 __global__ void __launch_bounds__(128 * kMlpMaxSplit) k_mlp_cols(ColArgs g) {
@@ -871,7 +888,7 @@ cudaError_t mlp_alloc(Mlp& M, int cap) {
   int dev = 0;
   A(cudaGetDevice(&dev));
   A(cudaDeviceGetAttribute(&M.sms, cudaDevAttrMultiProcessorCount, dev));
-  A(dalloc(M.params, kMlpParams));
+  A(dalloc(M.params, kMlpParams + 6));  // (the output biases are read as 32)
   A(dalloc(M.adam_m, kMlpParams));
   A(dalloc(M.adam_v, kMlpParams));
   A(dalloc(M.grad, kMlpParams));
