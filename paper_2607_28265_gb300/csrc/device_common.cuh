@@ -249,14 +249,6 @@ __device__ inline void antenna_fp_fx(const double* d, double ra, double dec, dou
   *fx = 2.0 * form(X, Y);
 }
 
-// Arrival time at a detector minus arrival at Earth's centre: -n.r / c.
-__device__ inline double geocentric_delay(const double* vertex, double ra, double dec, double gmst) {
-  double sl, cl, sd, cd;
-  sincos(ra - gmst, &sl, &cl);
-  sincos(dec, &sd, &cd);
-  return -(cd * cl * vertex[0] + cd * sl * vertex[1] + sd * vertex[2]) / kCSI;
-}
-
 // log I0(x) for x >= 0: power series sum_k (x^2/4)^k / (k!)^2 below 20, and
 // the large-argument expansion I0(x) ~ e^x / sqrt(2 pi x) sum_k ((2k-1)!!)^2 /
 // (k! (8x)^k) above (Abramowitz & Stegun 9.6.10, 9.7.1).  The series terms
@@ -391,40 +383,6 @@ __device__ inline void setup_projection(const LikeConst& L, const double* th, Ev
 __device__ inline void setup_amp_f32(const double* th, EvalRecord* rec) {
   const float rel = exp2f(0.8333333333f * log2f((float)th[0])) / (float)th[6];
   rec->amp = rec->valid ? (double)rel * amplitude_per_mpc(1.0) : 0.0;
-}
-
-__device__ inline void setup_projection_f32(const LikeConst& L, const double* th, EvalRecord* rec) {
-  float sl, cl, sd, cd, sp, cp;
-  sincosf((float)(th[9] - L.gmst), &sl, &cl);
-  sincosf((float)th[10], &sd, &cd);
-  sincosf((float)th[8], &sp, &cp);
-  const float east[3] = {-sl, cl, 0.0f};
-  const float north[3] = {-sd * cl, -sd * sl, cd};
-  float X[3], Y[3];
-  for (int k = 0; k < 3; ++k) {
-    X[k] = -cp * east[k] + sp * north[k];
-    Y[k] = sp * east[k] + cp * north[k];
-  }
-  const float ci = cosf((float)th[7]);
-  const float plus = 0.5f * (1.0f + ci * ci), cross = -ci;
-  float sph = 0.0f, cph = 1.0f;
-  if (!L.phase_marg) sincosf((float)th[12], &sph, &cph);
-  for (int i = 0; i < SWIG_MAX_DET; ++i) {
-    if (i >= L.n_det) {
-      rec->pre[i] = rec->pim[i] = 0.0;
-      continue;
-    }
-    float d[6];
-    for (int q = 0; q < 6; ++q) d[q] = L.dten_f[i][q];
-    auto form = [&d](const float* a, const float* b) {
-      return a[0] * (d[0] * b[0] + d[1] * b[1] + d[2] * b[2]) + a[1] * (d[1] * b[0] + d[3] * b[1] + d[4] * b[2]) +
-             a[2] * (d[2] * b[0] + d[4] * b[1] + d[5] * b[2]);
-    };
-    const float fp = form(X, X) - form(Y, Y), fx = 2.0f * form(X, Y);
-    const float re0 = fp * plus, im0 = fx * cross;
-    rec->pre[i] = (double)(re0 * cph - im0 * sph);
-    rec->pim[i] = (double)(re0 * sph + im0 * cph);
-  }
 }
 
 __device__ inline void setup_delays(const LikeConst& L, const double* th, EvalRecord* rec) {

@@ -448,8 +448,6 @@ __device__ inline double het_epilogue(const LikeConst& L, double Z_re, double Z_
   return Z_re + base_ll;
 }
 
-__host__ __device__ inline int het_chunks(int n_bins) { return (n_bins + 30) / 31; }
-
 // ---------------------------------------------------------------------------
 // Time pass of the time-marginalised likelihood.
 // ---------------------------------------------------------------------------

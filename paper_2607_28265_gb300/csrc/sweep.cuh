@@ -1,7 +1,6 @@
-// Bin-sweep device code shared by the batched likelihood kernels and the
-// persistent sampler: per-(theta, tile) double-float phase anchors and the
-// per-bin FP32 evaluation of kappa_i = sum_k D_i(k) exp(-2 pi i phi_i(k)) over
-// one slice, reduced by warp shuffles and the warp-group's shared memory.
+// Bin by bin: the FP64 sweep of the batched kernel and the FP64 sampler, and the
+// mixed-precision sweep (per-(theta, tile) double-float phase anchors, FP32 per
+// bin) that the folded evaluation falls back on outside its band.
 #pragma once
 
 #include "device_common.cuh"
