@@ -1419,6 +1419,7 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
       if (R[i].finished) continue;
       if ((rc = run_reset(ctxs[i], R[i]))) break;
       hd.push_back(chain_event(ctxs[i], R[i]));
+      hd.back().P.cta_prof = nullptr;  // (rows of one event's CTAs; this launch has more)
       idx.push_back(i);
     }
     if (rc || hd.empty()) break;
