@@ -823,10 +823,11 @@ int prepare_het(swig_ctx* c) {
   double* th_d = nullptr;
   double2* h_d = nullptr;
   std::vector<double2> h0((size_t)n_det * n);
+  const StreamDrain drain{c->stream};
   CUDA_TRY(c, cudaMalloc(&B.het_fid, sizeof(EvalRecord)));
   CUDA_TRY(c, cudaMalloc(&th_d, sizeof(th)));
   cudaError_t e = cudaMalloc(&h_d, sizeof(double2) * h0.size());
-  if (e == cudaSuccess) e = cudaMemcpy(th_d, th, sizeof(th), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(th_d, th, sizeof(th), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = launch_waveform(L, th_d, B.het_fid, h_d, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) e = cudaMemcpy(h0.data(), h_d, sizeof(double2) * h0.size(), cudaMemcpyDeviceToHost);
@@ -861,17 +862,18 @@ int prepare_het(swig_ctx* c) {
   // chunk anchor tables (kernels.h HetChunkRow)
   std::vector<float> ct, dfe;
   const int nc = het_chunk_tables(f, idx, nb, ct, dfe);
+  std::vector<float2> g, w;
+  const StreamDrain drain_tables{c->stream};
   CUDA_TRY(c, cudaMalloc(&B.het_chunk, sizeof(float) * ct.size()));
-  CUDA_TRY(c, cudaMemcpy(B.het_chunk, ct.data(), sizeof(float) * ct.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.het_chunk, ct.data(), sizeof(float) * ct.size(), cudaMemcpyHostToDevice, c->stream));
   c->h2d_bytes += sizeof(float) * ct.size();
   B.het_nc = nc;
   for (int i = 0; i < n_det; ++i) L.het_fid_iden[i] = 1.0 / (fid.cre[i] * fid.cre[i] + fid.cim[i] * fid.cim[i]);
   CUDA_TRY(c, cudaMalloc(&B.het_edge_basis, sizeof(float) * eb.size()));
   CUDA_TRY(c, cudaMalloc(&B.het_edge_f, sizeof(float) * ef.size()));
-  CUDA_TRY(c, cudaMemcpy(B.het_edge_basis, eb.data(), sizeof(float) * eb.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(B.het_edge_f, ef.data(), sizeof(float) * ef.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.het_edge_basis, eb.data(), sizeof(float) * eb.size(), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(B.het_edge_f, ef.data(), sizeof(float) * ef.size(), cudaMemcpyHostToDevice, c->stream));
   c->h2d_bytes += sizeof(float) * (eb.size() + ef.size());
-  std::vector<float2> g, w;
   if (L.tm_n > 0) {
     L.tm_M = 0;
     L.tm_pieces = L.tm_points = 0;
@@ -893,18 +895,20 @@ int prepare_het(swig_ctx* c) {
       // kNufftPiece (summed by one lane each), and the grid points with
       // entries (their pieces are combined in order)
       std::vector<int4> piece, point;
+      std::vector<float> wrow;
+      const StreamDrain drain_gather{c->stream};
       nufft_pieces(ptr, edge, L.tm_M, piece, point);
       L.tm_pieces = (int)piece.size();
       L.tm_points = (int)point.size();
       CUDA_TRY(c, cudaMalloc(&B.het_nu_piece, sizeof(int4) * std::max<size_t>(1, piece.size())));
       CUDA_TRY(c, cudaMalloc(&B.het_nu_point, sizeof(int4) * std::max<size_t>(1, point.size())));
       if (!piece.empty()) {
-        CUDA_TRY(c, cudaMemcpy(B.het_nu_piece, piece.data(), sizeof(int4) * piece.size(), cudaMemcpyHostToDevice));
-        CUDA_TRY(c, cudaMemcpy(B.het_nu_point, point.data(), sizeof(int4) * point.size(), cudaMemcpyHostToDevice));
+        CUDA_TRY(c, cudaMemcpyAsync(B.het_nu_piece, piece.data(), sizeof(int4) * piece.size(), cudaMemcpyHostToDevice, c->stream));
+        CUDA_TRY(c, cudaMemcpyAsync(B.het_nu_point, point.data(), sizeof(int4) * point.size(), cudaMemcpyHostToDevice, c->stream));
       }
       c->h2d_bytes += sizeof(int4) * (piece.size() + point.size());
       // their weights, entry i of 32 pieces in a row: the lanes take a piece each
-      std::vector<float> wrow((piece.size() + 31) / 32 * 32 * kNufftPiece, 0.0f);
+      wrow.assign((piece.size() + 31) / 32 * 32 * kNufftPiece, 0.0f);
       for (size_t p = 0; p < piece.size(); ++p)
         for (int i = 0; i < piece[p].y; ++i)
           wrow[(p / 32 * kNufftPiece + i) * 32 + p % 32] = wt[(size_t)piece[p].x + i];
@@ -913,20 +917,21 @@ int prepare_het(swig_ctx* c) {
       CUDA_TRY(c, cudaMalloc(&B.het_nu_corr, sizeof(float) * corr.size()));
       tw = nufft_stage_twiddles(tw, L.tm_M);
       CUDA_TRY(c, cudaMalloc(&B.het_nu_tw, sizeof(float2) * tw.size()));
-      CUDA_TRY(c, cudaMemcpy(B.het_nu_wt, wt.data(), sizeof(float) * wt.size(), cudaMemcpyHostToDevice));
-      CUDA_TRY(c, cudaMemcpy(B.het_nu_corr, corr.data(), sizeof(float) * corr.size(), cudaMemcpyHostToDevice));
-      CUDA_TRY(c, cudaMemcpy(B.het_nu_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice));
+      CUDA_TRY(c, cudaMemcpyAsync(B.het_nu_wt, wt.data(), sizeof(float) * wt.size(), cudaMemcpyHostToDevice, c->stream));
+      CUDA_TRY(c, cudaMemcpyAsync(B.het_nu_corr, corr.data(), sizeof(float) * corr.size(), cudaMemcpyHostToDevice, c->stream));
+      CUDA_TRY(c, cudaMemcpyAsync(B.het_nu_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, c->stream));
       c->h2d_bytes += sizeof(float) * (wt.size() + corr.size()) + sizeof(float2) * tw.size();
     }
     CUDA_TRY(c, cudaMalloc(&B.het_tm_w, sizeof(float2) * w.size()));
-    CUDA_TRY(c, cudaMemcpy(B.het_tm_w, w.data(), sizeof(float2) * w.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(B.het_tm_w, w.data(), sizeof(float2) * w.size(), cudaMemcpyHostToDevice, c->stream));
     c->h2d_bytes += sizeof(float2) * w.size();
   } else {
     het_tm_tables(a01, f, idx, nb, n_det, 0.0, g, w);
   }
   const std::vector<float4> ew = het_edge_weights(g, coefB, dfe, nb, nc, n_det);
+  const StreamDrain drain_weights{c->stream};
   CUDA_TRY(c, cudaMalloc(&B.het_ew, sizeof(float4) * ew.size()));
-  CUDA_TRY(c, cudaMemcpy(B.het_ew, ew.data(), sizeof(float4) * ew.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.het_ew, ew.data(), sizeof(float4) * ew.size(), cudaMemcpyHostToDevice, c->stream));
   c->h2d_bytes += sizeof(float4) * ew.size();
   for (int i = 0; i < n_det; ++i) {
     NSum b0;
@@ -1042,15 +1047,16 @@ int prepare_fold(swig_ctx* c) {
   std::vector<float> tab;
   fold_plan(c, c->L.n_det, chunks, tab);
   const std::vector<float2> x = fold_abscissae();
+  const StreamDrain drain{c->stream};
   FoldChunk* ck_d = nullptr;
   B.fold_nc = (int)chunks.size();
   CUDA_TRY(c, cudaMalloc(&B.fold_tab, sizeof(float) * tab.size()));
-  CUDA_TRY(c, cudaMemcpy(B.fold_tab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.fold_tab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMalloc(&B.fold_x, sizeof(float2) * x.size()));
-  CUDA_TRY(c, cudaMemcpy(B.fold_x, x.data(), sizeof(float2) * x.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.fold_x, x.data(), sizeof(float2) * x.size(), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMalloc(&B.fold_w, sizeof(float4) * 32 * c->L.n_det * chunks.size()));
   CUDA_TRY(c, cudaMalloc(&ck_d, sizeof(FoldChunk) * chunks.size()));
-  cudaError_t e = cudaMemcpy(ck_d, chunks.data(), sizeof(FoldChunk) * chunks.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpyAsync(ck_d, chunks.data(), sizeof(FoldChunk) * chunks.size(), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = launch_fold_weights(c->L, B, ck_d, c->stream);
   cudaFree(ck_d);
   if (e != cudaSuccess)
@@ -1149,6 +1155,7 @@ int prepare(swig_ctx* c) {
   std::vector<TileBasis> basis;
   if (prec == SWIG_PREC_MIXED) plan_tiles(c, tiles, basis);
   std::vector<int> slice_begin;
+  const StreamDrain drain{c->stream};
   int max_bins = 0;
   plan_slices(n, n_det, c->sm_count, tiles, slice_begin, &max_bins);
   int n_slices = (int)slice_begin.size() - 1;
@@ -1157,7 +1164,7 @@ int prepare(swig_ctx* c) {
 
   DeviceBuffers& B = c->B;
   CUDA_TRY(c, cudaMalloc(&B.slice_begin, sizeof(int) * (n_slices + 1)));
-  CUDA_TRY(c, cudaMemcpy(B.slice_begin, slice_begin.data(), sizeof(int) * (n_slices + 1), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.slice_begin, slice_begin.data(), sizeof(int) * (n_slices + 1), cudaMemcpyHostToDevice, c->stream));
   c->h2d_bytes += sizeof(int) * (n_slices + 1);
 
   if (prec == SWIG_PREC_MIXED) {
@@ -1166,20 +1173,21 @@ int prepare(swig_ctx* c) {
       const double s = 1.0 / L.inv_scale[i];
       for (int64_t k = 0; k < n; ++k) d32[i * n + k] = make_float2((float)(dre[i * n + k] * s), (float)(dim[i * n + k] * s));
     }
+    std::vector<int> bin_tile(n);
+    const StreamDrain drain_grid{c->stream};
     CUDA_TRY(c, cudaMalloc(&B.data32, sizeof(float2) * d32.size()));
-    CUDA_TRY(c, cudaMemcpy(B.data32, d32.data(), sizeof(float2) * d32.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(B.data32, d32.data(), sizeof(float2) * d32.size(), cudaMemcpyHostToDevice, c->stream));
     c->h2d_bytes += sizeof(float2) * d32.size() + sizeof(TileInfo) * tiles.size() + sizeof(TileBasis) * basis.size() +
                     sizeof(int) * n;
     L.n_tiles = (int)tiles.size();
-    std::vector<int> bin_tile(n);
     for (int t = 0; t < L.n_tiles; ++t)
       for (int k = tiles[t].k0; k < tiles[t].k0 + tiles[t].nbins; ++k) bin_tile[k] = t;
     CUDA_TRY(c, cudaMalloc(&B.tiles, sizeof(TileInfo) * tiles.size()));
-    CUDA_TRY(c, cudaMemcpy(B.tiles, tiles.data(), sizeof(TileInfo) * tiles.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(B.tiles, tiles.data(), sizeof(TileInfo) * tiles.size(), cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMalloc(&B.basis, sizeof(TileBasis) * basis.size()));
-    CUDA_TRY(c, cudaMemcpy(B.basis, basis.data(), sizeof(TileBasis) * basis.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(B.basis, basis.data(), sizeof(TileBasis) * basis.size(), cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMalloc(&B.bin_tile, sizeof(int) * n));
-    CUDA_TRY(c, cudaMemcpy(B.bin_tile, bin_tile.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(B.bin_tile, bin_tile.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
     B.max_slice_tiles = 1;
     for (int q = 0; q < n_slices; ++q)
       B.max_slice_tiles = std::max(B.max_slice_tiles, bin_tile[slice_begin[q + 1] - 1] - bin_tile[slice_begin[q]] + 1);
@@ -1190,10 +1198,11 @@ int prepare(swig_ctx* c) {
   } else {
     std::vector<double2> d64((size_t)n_det * n);
     for (size_t k = 0; k < d64.size(); ++k) d64[k] = make_double2(dre[k], dim[k]);
-    CUDA_TRY(c, cudaMalloc(&B.data64, sizeof(double2) * d64.size()));
-    CUDA_TRY(c, cudaMemcpy(B.data64, d64.data(), sizeof(double2) * d64.size(), cudaMemcpyHostToDevice));
-    c->h2d_bytes += sizeof(double2) * d64.size() + sizeof(double) * 3 * n;
     std::vector<double> ftab((size_t)3 * n);
+    const StreamDrain drain_grid{c->stream};
+    CUDA_TRY(c, cudaMalloc(&B.data64, sizeof(double2) * d64.size()));
+    CUDA_TRY(c, cudaMemcpyAsync(B.data64, d64.data(), sizeof(double2) * d64.size(), cudaMemcpyHostToDevice, c->stream));
+    c->h2d_bytes += sizeof(double2) * d64.size() + sizeof(double) * 3 * n;
     for (int64_t k = 0; k < n; ++k) {
       const double f = (double)(c->k_min + k) * c->df;
       ftab[3 * k] = 1.0 / std::cbrt(f);
@@ -1212,12 +1221,13 @@ int prepare(swig_ctx* c) {
   }
   // prior slots (defaults when no prior was set: every slot sampled uniform on [0,1])
   PriorSlot slots[SWIG_N_PARAMS];
+  const StreamDrain drain_prior{c->stream};
   for (int i = 0; i < SWIG_N_PARAMS; ++i) {
     const swig_param& p = c->params[i];
     slots[i] = c->prior_set ? make_prior_slot(p.kind, p.mode, p.lo, p.hi, p.value) : make_prior_slot(0, 0, 0.0, 1.0, 0.0);
   }
   CUDA_TRY(c, cudaMalloc(&B.prior, sizeof(slots)));
-  CUDA_TRY(c, cudaMemcpy(B.prior, slots, sizeof(slots), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(B.prior, slots, sizeof(slots), cudaMemcpyHostToDevice, c->stream));
   c->prepared_precision = prec;
   c->prepared_like = c->cfg_set ? c->cfg.likelihood : SWIG_LIKE_FULL;
   if (c->prepared_like == SWIG_LIKE_HET) {
@@ -1545,7 +1555,7 @@ int swig_inject(swig_ctx* c, const double* theta, double target_snr, const doubl
     if ((e = cudaMalloc(&rec_d, sizeof(EvalRecord)))) return e;
     if ((e = cudaMalloc(&h_d, sizeof(double2) * h.size()))) return e;
     for (int pass = 0; pass < 2; ++pass) {
-      if ((e = cudaMemcpy(th_d, th, sizeof(th), cudaMemcpyHostToDevice))) return e;
+      if ((e = cudaMemcpyAsync(th_d, th, sizeof(th), cudaMemcpyHostToDevice, c->stream))) return e;
       if ((e = launch_waveform(L, th_d, rec_d, h_d, c->stream))) return e;
       if ((e = cudaStreamSynchronize(c->stream))) return e;
       if ((e = cudaMemcpy(&rec, rec_d, sizeof(rec), cudaMemcpyDeviceToHost))) return e;

@@ -58,6 +58,15 @@ struct swig_ctx {
 };
 
 namespace swig {
+// Waits for a stream's copies at the end of a scope, before the host arrays
+// that they read (declared ahead of it) go: the preparation's uploads are queued
+// on the context's stream, ahead of the kernels that read them, and a copy of
+// pageable memory need not be staged where the device reads host memory itself.
+struct StreamDrain {
+  cudaStream_t stream;
+  ~StreamDrain() { cudaStreamSynchronize(stream); }
+};
+
 int prepare(swig_ctx* c);
 int ensure_scratch(swig_ctx* c, int n);
 int loglike_device(swig_ctx* c, const double* theta_dev, int64_t n, double* out_dev, cudaStream_t st);

@@ -878,7 +878,7 @@ cudaError_t launch_cols(Mlp& M, int n, int t, float lr, cudaStream_t st, long lo
 
 }  // namespace
 
-cudaError_t mlp_alloc(Mlp& M, int cap) {
+cudaError_t mlp_alloc(Mlp& M, int cap, cudaStream_t st) {
   mlp_free(M);
   cudaError_t e = cudaSuccess;
   auto A = [&](cudaError_t r) {
@@ -915,9 +915,10 @@ cudaError_t mlp_alloc(Mlp& M, int cap) {
   A(dalloc(M.row_loss, rows));
   A(dalloc(M.loss, 1));
   if (e == cudaSuccess) {
-    // padded rows/columns of the weight copies stay zero
-    A(cudaMemset(M.w1b, 0, sizeof(__nv_bfloat16) * kMlpInPad * kMlpH));
-    A(cudaMemset(M.w3b, 0, sizeof(__nv_bfloat16) * kMlpH * kMlpOutPad));
+    // padded rows/columns of the weight copies stay zero (on the stream of the
+    // kernels that write the others)
+    A(cudaMemsetAsync(M.w1b, 0, sizeof(__nv_bfloat16) * kMlpInPad * kMlpH, st));
+    A(cudaMemsetAsync(M.w3b, 0, sizeof(__nv_bfloat16) * kMlpH * kMlpOutPad, st));
   }
   if (e != cudaSuccess) {
     mlp_free(M);
@@ -1038,7 +1039,7 @@ int ensure_mlp(swig_ctx* c, int n) {
   if (n < 1 || n > 8192) return mfail(c, SWIG_E_ARG, "need 1 <= n <= 8192");
   MCUDA(cudaSetDevice(c->device));
   if (!c->mlp) c->mlp = new Mlp();
-  if (c->mlp->cap < n) MCUDA(mlp_alloc(*c->mlp, std::max(n, 1024)));
+  if (c->mlp->cap < n) MCUDA(mlp_alloc(*c->mlp, std::max(n, 1024), c->stream));
   return SWIG_OK;
 }
 
@@ -1058,7 +1059,7 @@ int upload_live(swig_ctx* c, const double* live_u, int64_t n, int d) {
 
 template <typename T>
 int upload(swig_ctx* c, T* dst, const T* src, size_t n) {
-  MCUDA(cudaMemcpy(dst, src, sizeof(T) * n, cudaMemcpyHostToDevice));
+  MCUDA(cudaMemcpyAsync(dst, src, sizeof(T) * n, cudaMemcpyHostToDevice, c->stream));
   c->h2d_bytes += sizeof(T) * n;
   return SWIG_OK;
 }
@@ -1106,7 +1107,7 @@ int swig_mlp_forward(swig_ctx* c, const float* params, const float* x_std, int64
   if ((rc = upload_params(c, params))) return rc;
   float* xd = nullptr;
   MCUDA(cudaMalloc(&xd, sizeof(float) * n * kMlpIn));
-  cudaError_t e = cudaMemcpy(xd, x_std, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpyAsync(xd, x_std, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = mlp_inputs(*c->mlp, xd, (int)n, c->stream, &c->n_launches);
   if (e == cudaSuccess) e = mlp_forward(*c->mlp, (int)n, c->stream, &c->n_launches);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1129,7 +1130,7 @@ int swig_mlp_loss_grad(swig_ctx* c, const float* params, const float* x_std, con
   if ((rc = upload(c, M.tls, tls, (size_t)n * kMlpIn))) return rc;
   float* xd = nullptr;
   MCUDA(cudaMalloc(&xd, sizeof(float) * n * kMlpIn));
-  cudaError_t e = cudaMemcpy(xd, x_std, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpyAsync(xd, x_std, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = mlp_inputs(M, xd, (int)n, c->stream, &c->n_launches);
   if (e == cudaSuccess) e = mlp_loss_grad(M, (int)n, d, c->stream, &c->n_launches);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -66,7 +66,7 @@ struct Mlp {
   int sms = 0;                    // SMs of the device
 };
 
-cudaError_t mlp_alloc(Mlp& M, int cap);
+cudaError_t mlp_alloc(Mlp& M, int cap, cudaStream_t st);
 void mlp_free(Mlp& M);
 // Philox-4x32-10 initial weights N(0, 1/fan_in), biases 0; resets Adam.
 cudaError_t mlp_init(Mlp& M, uint64_t seed, cudaStream_t st, long long* launches);

@@ -789,7 +789,7 @@ struct RunState {
   float learn_lr = 0.0f;
   int learn_steps = 0;
   std::vector<double> du, dl, dw;
-  NSGlobal gh;
+  NSGlobal gh, gl;  // after a launch; as uploaded before one (the copies read it)
   long long total_iters = 0;
   double persistent_ms = 0.0, learn_ms = 0.0;
   long long persistent_launches = 0, learn_rounds = 0;
@@ -834,6 +834,7 @@ int run_setup(swig_ctx* c, RunState& R) {
   int rc = prepare(c);
   if (rc) return rc;
   R.t_start = std::chrono::steady_clock::now();
+  const StreamDrain drain{c->stream};
   const bool het = c->prepared_like == SWIG_LIKE_HET;
   const bool mixed = !het && c->prepared_precision == SWIG_PREC_MIXED;
   R.het = het;
@@ -1018,10 +1019,11 @@ int run_setup(swig_ctx* c, RunState& R) {
     SCUDA(cudaMalloc(&st->lw, sizeof(double) * (m + 1)));
     SCUDA(cudaMalloc(&st->init_theta, sizeof(double) * m * SWIG_N_PARAMS));
     std::vector<double> harm(k + 1, 0.0), lw(m + 1, 0.0);
+    const StreamDrain drain_weights{c->stream};
     for (int j = 1; j <= k; ++j) harm[j] = harm[j - 1] + 1.0 / (double)(m - (j - 1));
     for (int n = 1; n <= m; ++n) lw[n] = std::log(-std::expm1(-1.0 / (double)n));
-    SCUDA(cudaMemcpy(st->harm, harm.data(), sizeof(double) * harm.size(), cudaMemcpyHostToDevice));
-    SCUDA(cudaMemcpy(st->lw, lw.data(), sizeof(double) * lw.size(), cudaMemcpyHostToDevice));
+    SCUDA(cudaMemcpyAsync(st->harm, harm.data(), sizeof(double) * harm.size(), cudaMemcpyHostToDevice, c->stream));
+    SCUDA(cudaMemcpyAsync(st->lw, lw.data(), sizeof(double) * lw.size(), cudaMemcpyHostToDevice, c->stream));
     st->P.harm = st->harm;
     st->P.lw = st->lw;
   }
@@ -1036,7 +1038,7 @@ int run_setup(swig_ctx* c, RunState& R) {
   st->P.learn_out = nullptr;
   if (R.learned) {
     if (!c->mlp) c->mlp = new Mlp();
-    if (c->mlp->cap < m) SCUDA(mlp_alloc(*c->mlp, std::max(m, 1024)));
+    if (c->mlp->cap < m) SCUDA(mlp_alloc(*c->mlp, std::max(m, 1024), c->stream));
   }
   if ((rc = ensure_scratch(c, std::max(m, k)))) return rc;  // FP64: records and partials of k requests
 
@@ -1055,7 +1057,7 @@ int run_setup(swig_ctx* c, RunState& R) {
     }
     SCUDA(e);
   }
-  NSGlobal g0;
+  NSGlobal& g0 = R.gl;
   std::memset(&g0, 0, sizeof(g0));
   g0.logx = 0.0;
   g0.logz = -INFINITY;
@@ -1081,7 +1083,7 @@ int run_setup(swig_ctx* c, RunState& R) {
 
 // Reset the per-launch counters of the NS state before a launch.
 int run_reset(swig_ctx* c, RunState& R) {
-  NSGlobal gl;
+  NSGlobal& gl = R.gl;
   SCUDA(cudaMemcpyAsync(&gl, R.st->P.g, sizeof(gl), cudaMemcpyDeviceToHost, c->stream));
   SCUDA(cudaStreamSynchronize(c->stream));
   gl.iters_launch = 0;
@@ -1160,7 +1162,7 @@ int run_finish(swig_ctx* c, RunState& R, swig_result* out) {
     double *du_d = nullptr, *th_d = nullptr;
     SCUDA(cudaMalloc(&du_d, sizeof(double) * std::max<size_t>(1, du.size())));
     SCUDA(cudaMalloc(&th_d, sizeof(double) * std::max<size_t>(1, c->out_theta.size())));
-    SCUDA(cudaMemcpy(du_d, du.data(), sizeof(double) * du.size(), cudaMemcpyHostToDevice));
+    SCUDA(cudaMemcpyAsync(du_d, du.data(), sizeof(double) * du.size(), cudaMemcpyHostToDevice, c->stream));
     k_dead_theta<<<(unsigned)((n_dead + 127) / 128), 128, 0, c->stream>>>(S, du_d, (int)n_dead, th_d);
     ++c->n_launches;
     if (L.dist_marg) {
@@ -1335,6 +1337,7 @@ int run_loop_single(swig_ctx* c, RunState& R) {
     void** args = chain ? chain_args : flow_args;
     cudaError_t e = cudaSuccess;
     ChainEvent hev;
+    const StreamDrain drain{c->stream};
     if (chain) {
       hev = chain_event(c, R);
       e = cudaMemcpyAsync(R.st->ev, &hev, sizeof(hev), cudaMemcpyHostToDevice, c->stream);
@@ -1412,6 +1415,9 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
   if (e == cudaSuccess) e = cudaEventCreate(&ev1);
   std::vector<ChainEvent> hd;
   std::vector<int> idx;
+  NSGlobal g0;
+  std::memset(&g0, 0, sizeof(g0));
+  const StreamDrain drain{c0->stream};
   while (e == cudaSuccess && rc == SWIG_OK) {
     hd.clear();
     idx.clear();
@@ -1427,8 +1433,6 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
       e = cudaStreamSynchronize(ctxs[i]->stream);
       if (e != cudaSuccess) break;
     }
-    NSGlobal g0;
-    std::memset(&g0, 0, sizeof(g0));
     // on the launch's stream, which does not wait for the default stream's copies
     if (e == cudaSuccess) e = cudaMemcpyAsync(gb, &g0, sizeof(g0), cudaMemcpyHostToDevice, c0->stream);
     if (e == cudaSuccess)

@@ -7,8 +7,11 @@
 // Ordering rules (CUDA programming guide, API synchronisation behaviour): a copy
 // of pageable memory or a memset on the default stream may return before it is
 // done, and a non-blocking stream does not wait for it; work on two streams has
-// no order until the host has waited for one of them.
+// no order until the host has waited for one of them; an asynchronous copy may read
+// its host array until then.
 #include <cuda_runtime.h>
+#include <sys/uio.h>
+#include <unistd.h>
 
 #include <cstdlib>
 #include <cstring>
@@ -16,12 +19,19 @@
 #include <mutex>
 #include <set>
 #include <string>
+#include <vector>
 
 #include "../paper_2607_28265_gb300/csrc/chain.h"
 
 using namespace swig;
 
 namespace {
+
+struct Source {  // of an asynchronous copy to the device
+  cudaStream_t stream;
+  const void* p;
+  std::vector<char> bytes;
+};
 
 struct Fake {
   std::mutex lock;
@@ -30,6 +40,7 @@ struct Fake {
   std::map<const void*, int> smem_limit;          // dynamic shared memory allowed
   std::map<const void*, size_t> vars;
   std::set<cudaStream_t> busy;                    // streams with work the host has not waited for
+  std::vector<Source> sources;
   std::map<std::string, long long> calls;
   std::string report;
   int sms = 152;
@@ -55,6 +66,24 @@ size_t room(const void* p) {
 
 void on_write(const char* what, const void* dst, size_t n) {
   if (n > room(dst)) F().note(std::string(what) + ": past the end of its allocation");
+}
+
+// The host has waited for st: the arrays that its copies read still have to be
+// what they were.
+void waited(cudaStream_t st) {
+  F().busy.erase(st);
+  std::vector<Source> left;
+  for (Source& s : F().sources) {
+    if (s.stream != st) {
+      left.push_back(std::move(s));
+      continue;
+    }
+    std::vector<char> now(s.bytes.size());
+    iovec to{now.data(), now.size()}, from{const_cast<void*>(s.p), now.size()};  // (fails where nothing is mapped)
+    if (process_vm_readv(getpid(), &to, 1, &from, 1, 0) != (ssize_t)now.size() || now != s.bytes)
+      F().note("cudaMemcpyAsync: host array gone before the copy was waited for");
+  }
+  F().sources.swap(left);
 }
 
 cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t shared, cudaStream_t st) {
@@ -219,6 +248,8 @@ RT(cudaError_t, cudaMemcpy, (void* dst, const void* src, size_t n, cudaMemcpyKin
 RT(cudaError_t, cudaMemcpyAsync, (void* dst, const void* src, size_t n, cudaMemcpyKind kind, cudaStream_t st)) {
   Guard g(F().lock);
   F().busy.insert(st);
+  const char* p = static_cast<const char*>(src);
+  if (kind == cudaMemcpyHostToDevice) F().sources.push_back({st, src, std::vector<char>(p, p + n)});
   return copy("cudaMemcpyAsync", dst, src, n, kind);
 }
 RT(cudaError_t, cudaMemset, (void* p, int v, size_t n)) {
@@ -242,13 +273,13 @@ RT(cudaError_t, cudaStreamCreateWithFlags, (cudaStream_t* s, unsigned)) {
 }
 RT(cudaError_t, cudaStreamDestroy, (cudaStream_t s)) {
   Guard g(F().lock);
-  F().busy.erase(s);
+  waited(s);
   std::free(s);
   return cudaSuccess;
 }
 RT(cudaError_t, cudaStreamSynchronize, (cudaStream_t s)) {
   Guard g(F().lock);
-  F().busy.erase(s);
+  waited(s);
   return cudaSuccess;
 }
 RT(cudaError_t, cudaStreamIsCapturing, (cudaStream_t, cudaStreamCaptureStatus* s)) {
@@ -269,7 +300,7 @@ RT(cudaError_t, cudaEventRecord, (cudaEvent_t e, cudaStream_t s)) {
 }
 RT(cudaError_t, cudaEventSynchronize, (cudaEvent_t e)) {  // (recorded behind all of its stream's work)
   Guard g(F().lock);
-  F().busy.erase(*(cudaStream_t*)e);
+  waited(*(cudaStream_t*)e);
   return cudaSuccess;
 }
 RT(cudaError_t, cudaEventElapsedTime_v2, (float* ms, cudaEvent_t, cudaEvent_t)) {

@@ -7,6 +7,7 @@ import os
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 import swig_inputs as si
@@ -72,3 +73,63 @@ def test_campaign_counters_stay_in_their_buffer(device, n_ev, nrep):
     assert not [r for r in _report(device) if "counters" in r or "past" in r]
     for c in ctxs:
         c.close()
+
+
+def _hazards(lib):
+    return [r for r in _report(lib) if "counters" not in r]
+
+
+@pytest.mark.parametrize("kind", ["mixed", "fp64", "het", "het_time"])
+def test_uploads_precede_the_kernels_that_read_them(device, kind):
+    """Preparation, a batch on another stream and a run: no kernel is launched
+    while a copy that it may read is under way, and no copy's host array goes
+    before the copy is done."""
+    extra = {"mixed": {}, "fp64": dict(precision=swig.PREC_FP64), "het": dict(het=True),
+             "het_time": dict(het=True, tmarg_nodes=256)}[kind]
+    ctx, th = _context(max_iter=4, **extra)
+    if kind == "het_time":
+        params = list(si.config1(nlive=200).params)
+        params[11] = si.Param(params[11].kind, params[11].lo, params[11].hi, si.MODE_MARG)
+        ctx.set_prior(params)
+    theta, out = np.tile(th, (100, 1)), np.empty(100)
+    device.fake_set(b"check streams", 1)
+    # (host arrays for device pointers: no kernel runs)
+    ctx.loglike_batch_dev(theta.ctypes.data, 100, out.ctypes.data, 0x1000)
+    device.cudaStreamSynchronize(ctypes.c_void_p(0x1000))
+    ctx.loglike_batch(theta)
+    ctx.run()
+    ctx.get_samples()
+    assert not _hazards(device)
+    ctx.close()
+
+
+def test_uploads_of_a_campaign(device):
+    ctxs = [_context(i)[0] for i in range(3)]
+    swig.run_batch(ctxs)
+    assert not _hazards(device)
+    for c in ctxs:
+        c.close()
+
+
+def test_uploads_of_the_learned_proposal(device):
+    ctx = swig.Context(0)
+    rng = np.random.default_rng(0)
+    params = ctx.mlp_init(1)
+    x, t, u = rng.standard_normal((40, 13)), rng.standard_normal((40, 13)), rng.random((40, 5))
+    ctx.mlp_forward(params, x)
+    ctx.mlp_loss_grad(params, x, t, t, 13)
+    ctx.mlp_targets(u)
+    ctx.mlp_train(u, params, 2, lr=1e-3)
+    assert not _hazards(device)
+    ctx.close()
+    ctx, _ = _context(proposal=swig.PROPOSAL_LEARNED, max_iter=4)
+    ctx.run()
+    assert not _hazards(device)
+    ctx.close()
+
+
+def test_uploads_of_an_injection(device):
+    ctx, th = _context()
+    ctx.inject(th, 1, target_snr=20.0)
+    assert not _hazards(device)
+    ctx.close()
