@@ -131,7 +131,7 @@ cudaError_t weights_launch(const FoldTables& F, const FoldChunk* chunks, int n_b
   cudaError_t e = cudaMalloc(&mom, sizeof(double) * (size_t)F.nc * kMomParts * 2 * NDET * kFoldNodes);
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(double) * (kFoldNodes * (kMomThreads + 1) + 2 * NDET * kMomThreads);
-  e = cudaFuncSetAttribute(k_fold_moments<NDET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_shared((const void*)k_fold_moments<NDET>);
   if (e == cudaSuccess) {
     k_fold_moments<NDET><<<dim3(F.nc, kMomParts), kMomThreads, smem, st>>>(F, chunks, n_bins, mom);
     k_fold_weights<NDET><<<dim3(F.nc, NDET), 32, 0, st>>>(F, chunks, n_bins, mom, w);
@@ -299,7 +299,7 @@ namespace {
 template <int NDET, bool RES>
 cudaError_t fold_launch_as(const LikeConst& L, const FoldTables& F, const EvalRecord* rec, int n, double* out,
                            cudaStream_t st, double* kappa_out, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_fold<NDET, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared((const void*)k_fold<NDET, RES>);
   if (e != cudaSuccess) return e;
   // the widest team that leaves no vector waiting for a second turn
   const int ctas = L.sm_count;

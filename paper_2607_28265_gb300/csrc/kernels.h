@@ -230,6 +230,12 @@ inline __host__ __device__ size_t fold_resident_bytes(int nc, int n_det) {
   return (size_t)nc * n_det * 32 * sizeof(float4) + sizeof(float) * FR_ROWS * fold_ld(nc);
 }
 
+// Lets kernel f take all the dynamic shared memory that a block of its device may
+// have.  The limit belongs to the function, not to a context or a launch, and
+// contexts may be used by several threads at once: every launch asks for the same
+// value, so that none lowers it between another's call and its launch.
+cudaError_t allow_shared(const void* f);
+
 // FP64 path: the basis functions at every bin, tab [NBASIS][n_bins] (f in row
 // B_ONE), from base [n_bins][3] (f^-1/3, f^1/3, ln f).
 cudaError_t launch_fp64_basis(const LikeConst& L, const double* base, double* tab, cudaStream_t st);

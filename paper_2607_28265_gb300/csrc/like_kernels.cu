@@ -11,6 +11,10 @@
 // follow.
 #include <cuda_runtime.h>
 
+#include <mutex>
+#include <utility>
+#include <vector>
+
 #include "kernels.h"
 #include "het.cuh"
 #include "sweep.cuh"
@@ -161,11 +165,34 @@ __global__ void __launch_bounds__(32 * kSetupWarps)
   }
 }
 
+cudaError_t allow_shared(const void* f) {
+  static std::mutex lock;
+  static std::vector<std::pair<const void*, int>> limits;  // (one architecture: the same on every device)
+  int most = -1;
+  {
+    const std::lock_guard<std::mutex> hold(lock);
+    for (const auto& l : limits)
+      if (l.first == f) most = l.second;
+  }
+  if (most < 0) {
+    int device = 0, optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, f);
+    if (e != cudaSuccess) return e;
+    most = optin - (int)a.sharedSizeBytes;
+    const std::lock_guard<std::mutex> hold(lock);
+    limits.emplace_back(f, most);
+  }
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // A kernel whose start overlaps the one before it on st (it waits for that one's
 // end before it reads its results).
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, size_t bytes, cudaStream_t st, A... args) {
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const cudaError_t e = bytes ? allow_shared((const void*)kern) : cudaSuccess;
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;

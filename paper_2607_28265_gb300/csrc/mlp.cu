@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "device_common.cuh"
+#include "kernels.h"
 #include "mlp.h"
 
 namespace swig {
@@ -839,7 +840,7 @@ cudaError_t dalloc(T*& p, size_t n) {
 // A launch whose set-up overlaps the kernel before it.
 template <typename Args>
 cudaError_t launch_chained(void (*kern)(Args), int grid, int threads, size_t smem, const Args& a, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared((const void*)kern);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

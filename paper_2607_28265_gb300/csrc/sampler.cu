@@ -1299,7 +1299,7 @@ ChainEvent chain_event(const swig_ctx* c, const RunState& R) {
 int run_loop_single(swig_ctx* c, RunState& R) {
   int rc = SWIG_OK;
   const bool chain = R.mixed || R.het;
-  SCUDA(cudaFuncSetAttribute(R.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R.smem));
+  SCUDA(allow_shared(R.kern));
   int per_sm = 0;
   SCUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, R.kern, R.threads, R.smem));
   if (per_sm < 1 || R.S.n_ctas > per_sm * c->sm_count)
@@ -1399,7 +1399,7 @@ int run_loop_multi(swig_ctx* const* ctxs, std::vector<RunState>& R, int i0, int 
   const int grid = std::min(c0->sm_count, (i1 - i0) * k);
   lay.n_ctas = std::max(grid, i1 - i0);
   void* kern = chain_kernel(n_det, CHAIN_FOLD);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(kern);
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kChainBlock, smem);
   if (e != cudaSuccess) return fail(c0, SWIG_E_CUDA, std::string("multi-event kernel set-up: ") + cudaGetErrorString(e));

@@ -133,3 +133,26 @@ def test_uploads_of_an_injection(device):
     ctx.inject(th, 1, target_snr=20.0)
     assert not _hazards(device)
     ctx.close()
+
+
+def test_contexts_do_not_lower_each_others_shared_memory_limit(device):
+    """The limit is the function's and contexts may run in several threads: calls
+    of different sizes, types and grids never lower it."""
+    def use(i, **kw):
+        ctx, th = _context(i, max_iter=2, **kw)
+        theta = np.tile(th, (400, 1))
+        for n in (400, 1, 160):
+            ctx.loglike_batch(theta[:n])
+        ctx.run()
+        ctx.close()
+
+    for het in (True, False):
+        use(0, het=het, nlive=2000)
+        use(1, het=het, nlive=200)
+    rng = np.random.default_rng(0)
+    ctx = swig.Context(0)
+    params = ctx.mlp_init(1)
+    for n in (2000, 40):
+        ctx.mlp_train(rng.random((n, 5)), params, 2, lr=1e-3)
+    ctx.close()
+    assert not _report(device)
