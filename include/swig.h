@@ -286,8 +286,10 @@ int swig_autotune(swig_ctx* ctx, int iters, double* out, int n);
  * appear once.  Stops at the first failure (that context's error). */
 int swig_run_batch(swig_ctx** ctxs, int n_ctx, swig_result* outs);
 /* Cap, in polling iterations of ~100 ns, on every spin-wait of the persistent
- * kernel (grid barriers).  Default 1e7.  A wait that reaches the cap makes
- * swig_run return SWIG_E_TIMEOUT instead of hanging. */
+ * kernel (grid barriers).  Default 1e7.  While CTAs wait for others' chains it
+ * caps the polls without progress of any chain, not the length of an iteration.
+ * A wait that reaches the cap makes swig_run return SWIG_E_TIMEOUT instead of
+ * hanging. */
 int swig_set_wait_limit(swig_ctx* ctx, long long spins);
 /* Counters of the last swig_run.  Phase timers measured on the device by the
  * first CTA of the persistent kernel: out[0] rounds, out[1] iteration-

@@ -424,7 +424,8 @@ __global__ void __launch_bounds__(kChainBlock, 1)
   if (tid == 0) s.event = -1;
   NSGlobal* g0 = ev[0].P.g;
   for (;;) {
-    if (!grid_sync(gb, lay.n_ctas, lay.spin_limit)) return;
+    // a CTA without a chain waits here for the longest one: as long as any advances
+    if (!grid_sync(gb, lay.n_ctas, lay.spin_limit, &gb->beat)) return;
     if (timer) {
       t1 = gtimer();
       g0->t_wait_sweep += t1 - t0;
@@ -514,7 +515,8 @@ __global__ void __launch_bounds__(kChainBlock, 1)
             if (have) finish_fold<NDET>(s, lane);
           if constexpr (MODE == CHAIN_HET)
             if (have) finish_het<NDET>(s, E.H, lane);
-          chain_control<NDET, MODE != CHAIN_FOLD>(s.L, s.S, P, w, c, it, logl_star, have, lane, prof);
+          if (lane == 0 && (guard & 7) == 0) atomicAdd(&gb->beat, 1u);
+          chain_control<NDET, MODE != CHAIN_FOLD>(s.L, s.S, P, w, c, it, logl_star, have, lane, prof, &gb->beat);
           if constexpr (MODE != CHAIN_HET_TM)
             if (lane == 0 && w.status == ROUND_EVAL && (w.fl & (BF_INTR | BF_TIDE))) s.e.base_ok = 0;
           if (lane == 0) {

@@ -481,11 +481,12 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
 
 // Warp 0 between two evaluations: apply the results (have: a round is pending,
 // its logL in w.ly), then advance to the next round that needs the CTA.
-// Projection-only blocks are evaluated here, a candidate per lane.
+// Projection-only blocks are evaluated here, a candidate per lane.  beat: raised
+// after eight of their steps (grid_sync).
 template <int NDET, bool HET>
 __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerConst& S, const SamplerPtrs& P,
                                               ChainWork& w, int c, long long it, double logl_star, bool have,
-                                              int lane, unsigned long long* prof) {
+                                              int lane, unsigned long long* prof, unsigned* beat) {
   ChainState& ch = w.ch;
   long long tk = clock64();
   auto lap = [&](int slot) {
@@ -513,6 +514,7 @@ __device__ __forceinline__ void chain_control(const LikeConst& L, const SamplerC
     if (S.block_free[ch.block]) {
       const int seen = chain_free_step<HET>(L, S, w, c, it, logl_star, lane);
       if (prof && lane == 0) prof[5] += seen;
+      if (lane == 0 && (guard & 7) == 7) atomicAdd(beat, 1u);
       lap(3);
       continue;
     }

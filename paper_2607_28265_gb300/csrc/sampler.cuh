@@ -86,6 +86,7 @@ struct NSGlobal {
   int n_dead;
   unsigned bar_count, bar_gen;
   int task;  // chain sampler: next chain of the iteration
+  unsigned beat;  // ... raised as any CTA's chain advances (every eight rounds, or steps)
   // phase timers of CTA 0 [ns, %globaltimer]: boundary, control, wait after
   // control, sweep, wait after sweep; and rounds
   unsigned long long t_bound, t_ctrl, t_wait_ctrl, t_sweep, t_wait_sweep, rounds;
@@ -145,9 +146,11 @@ __device__ __forceinline__ float chain_normal(const SamplerConst& S, ChainState&
 }
 
 // ---------------------------------------------------------------------------
-// Bounded grid barrier (all CTAs co-resident by cooperative launch).
+// Bounded grid barrier (all CTAs co-resident by cooperative launch).  beat
+// (optional): a count that the other CTAs raise as they work; the limit then
+// bounds the polls in which it stands still.
 // ---------------------------------------------------------------------------
-static __device__ bool grid_sync(NSGlobal* g, int n_ctas, long long limit) {
+static __device__ bool grid_sync(NSGlobal* g, int n_ctas, long long limit, const unsigned* beat = nullptr) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -161,7 +164,15 @@ static __device__ bool grid_sync(NSGlobal* g, int n_ctas, long long limit) {
       atomicAdd(&g->bar_gen, 1u);
     } else {
       long long spins = 0;
+      unsigned last = 0;
       while (*vgen == gen) {
+        if (beat) {
+          const unsigned now = *(const volatile unsigned*)beat;
+          if (now != last) {
+            last = now;
+            spins = 0;
+          }
+        }
         if (++spins > limit) {
           atomicCAS(&g->error, 0, SWIG_E_TIMEOUT);
           break;
