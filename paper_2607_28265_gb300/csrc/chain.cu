@@ -104,7 +104,7 @@ __device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, cons
     __syncthreads();
     if (threadIdx.x == 0) s.e.base_ok = 1;
   }
-  int panel = slots / na & ~31;  // whole turns, and a multiple of the groups
+  int panel = slots / na & ~31;  // whole turns
   if (slots / na >= F.nc) panel = F.nc;
   FoldAcc<NDET> acc[2];
   acc[0].clear();
@@ -132,11 +132,16 @@ __device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, cons
     }
     if (p < pairs) {
       const bool two = 2 * p + 1 < na;
-      const float* an0 = s_an + (2 * p * panel + g) * kFoldAnchor;
+      // the group takes the chunks whose number is g modulo G, whatever the panels
+      // (their length follows the launch's scratch; five groups do not divide it)
+      int g0 = g;
+      if (q0 > 0) g0 += (G - q0 % G) % G;
+      if (g0 >= G) g0 -= G;
+      const float* an0 = s_an + (2 * p * panel + g0) * kFoldAnchor;
       const float* an1 = an0 + panel * kFoldAnchor;
-      const float4* wq = W + (q0 + g) * NDET * 32 + lane;
+      const float4* wq = W + (q0 + g0) * NDET * 32 + lane;
       auto kind = [&](int q) { return __float_as_int(tab[FR_KIND * ld + q0 + q]); };
-      for (int q = g; q < np; q += G, wq += G * NDET * 32, an0 += G * kFoldAnchor, an1 += G * kFoldAnchor) {
+      for (int q = g0; q < np; q += G, wq += G * NDET * 32, an0 += G * kFoldAnchor, an1 += G * kFoldAnchor) {
         FoldNode<NDET> v;
         fold_load<NDET>(wq, kind(q), x0, s.e.x, lane, v);
         fold_chunk<NDET>(an0, q, v, acc[0]);
