@@ -25,7 +25,7 @@ struct ChainEval<NDET, CHAIN_FOLD> {
   FoldPair in[kCand / 2];
   FoldPair cur;               // the chain's current point
   int base_ok;                // its partial sums are formed
-  float sum[kCand][kChainWarps][2 * NDET];  // per group
+  float2 sum[kChainWarps][4 * NDET];  // of a warp's pair of candidates, double-float
   double tot[kCand][2 * NDET];
   double dir[kChainWarps][2 * NDET];  // bin by bin, per warp
 };
@@ -73,6 +73,26 @@ size_t chain_fixed_bytes(int n_det, int mode) {
   return (b + 15) & ~(size_t)15;
 }
 
+// Chunks that a lane adds in FP32 (fold.cuh kFoldBlock): a round's groups share the
+// chunks, so that blocks of 32 are beyond what the 128 s grid's 78 come to (20 for
+// each of four groups) and their sums stay out of the way of the chunks' loop (blocks
+// of 8, in registers: 12.77 -> 13.17 ms for 4 iterations).
+constexpr int kChainFoldBlock = 32;
+// A warp's sums over its pair of candidates to sum, or added to what is there.
+template <int NDET>
+__device__ __forceinline__ void fold_take_sums(const FoldAcc<NDET>* acc, bool add, float2* sum, int lane) {
+  fold_warp_sums<NDET, 2, 2>(acc, false, nullptr, lane, [&](int j, dfl v) {
+    if (add) v = df_add(v, dfl{sum[j].x, sum[j].y});
+    sum[j] = make_float2(v.hi, v.lo);
+  });
+}
+// The same out of the chunks' loop (by value: the accumulators stay in registers).
+template <int NDET>
+__device__ __noinline__ void fold_block_sums(FoldAcc<NDET> a, FoldAcc<NDET> b, bool add, float2* sum, int lane) {
+  const FoldAcc<NDET> acc[2] = {a, b};
+  fold_take_sums<NDET>(acc, add, sum, lane);
+}
+
 // Folded full-grid sums of the round's candidates, two at a time: anchors of a
 // panel of chunks (packed over the pair, quarter by quarter), then a (pair, group
 // of chunks) per warp, the chunks q = group, group + G, ..., the weights loaded
@@ -109,6 +129,8 @@ __device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, cons
   FoldAcc<NDET> acc[2];
   acc[0].clear();
   acc[1].clear();
+  int held = 0;           // chunks in the accumulators
+  bool blocks = false;    // earlier blocks' sums in s.e.sum
   const float2 x0 = s.e.x[lane];
   const int p = warp / G, g = warp - p * G;  // this warp's pair and group
   for (int q0 = 0; q0 < F.nc; q0 += panel) {
@@ -146,39 +168,30 @@ __device__ __forceinline__ void eval_fold(ChainShared<NDET, CHAIN_FOLD>& s, cons
         fold_load<NDET>(wq, kind(q), x0, s.e.x, lane, v);
         fold_chunk<NDET>(an0, q, v, acc[0]);
         if (two) fold_chunk<NDET>(an1, q, v, acc[1]);
+        if (++held == kChainFoldBlock) {  // warp-uniform; many chunks
+          fold_block_sums<NDET>(acc[0], acc[1], blocks, s.e.sum[warp], lane);
+          acc[0].clear();
+          acc[1].clear();
+          held = 0;
+          blocks = true;
+        }
       }
     }
     __syncthreads();
   }
-  if (p < pairs)
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      if (2 * p + j < na) {
-        const int k = w.list[2 * p + j];
-#pragma unroll
-        for (int i = 0; i < NDET; ++i) {
-          float re, im;
-          acc[j].total(i, re, im);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            re += __shfl_xor_sync(0xffffffffu, re, o);
-            im += __shfl_xor_sync(0xffffffffu, im, o);
-          }
-          if (lane == 0) {
-            s.e.sum[k][g][2 * i] = re;
-            s.e.sum[k][g][2 * i + 1] = im;
-          }
-        }
-      }
+  if (p < pairs) fold_take_sums<NDET>(acc, blocks, s.e.sum[warp], lane);
   __syncthreads();
   {  // the groups' sums (double-float, four threads a value), rounded once to FP64
     const int v = threadIdx.x >> 2, a = v / (2 * NDET), j = v - a * (2 * NDET), g0 = threadIdx.x & 3;
     const int k = a < na ? w.list[a] : 0;
     dfl t = {0.0f, 0.0f};
-    for (int r = g0; r < G; r += 4) t = df_add(t, dfl{s.e.sum[k][r][j], 0.0f});
+    for (int r = g0; r < G; r += 4) {
+      const float2 x = a < na ? s.e.sum[(a >> 1) * G + r][(a & 1) * 2 * NDET + j] : make_float2(0.0f, 0.0f);
+      t = df_accumulate(t, dfl{x.x, x.y});
+    }
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1)
-      t = df_add(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
+      t = df_accumulate(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
     if (a < na && g0 == 0) s.e.tot[k][j] = (double)t.hi + (double)t.lo;
   }
   for (int a = 0; a < na; ++a) {

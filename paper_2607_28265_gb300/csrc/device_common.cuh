@@ -72,6 +72,13 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   return fast_two_sum(s.hi, e);
 }
 
+// The same without the last renormalisation, for sums of a few terms: the high
+// words' chain is one addition a term, the low word collects their rounding.
+__device__ __forceinline__ dfl df_accumulate(dfl a, dfl b) {
+  const dfl s = two_sum(a.hi, b.hi);
+  return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
+}
+
 // Fractional part (nearest-integer reduction) of a double-float, returned as
 // a float in [-0.5, 0.5] plus rounding of the low word.
 __device__ __forceinline__ float df_frac(dfl a) {

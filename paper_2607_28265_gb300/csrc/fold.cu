@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
            double* __restrict__ kappa_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ FoldIn s_in[kFoldWarps];
-  __shared__ float s_sum[2 * NDET][kFoldWarps];
+  __shared__ float2 s_sum[2 * NDET][kFoldWarps];
   __shared__ double s_dir[2 * NDET][kFoldWarps];
   __shared__ int s_bad[kFoldWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -219,7 +219,9 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
     const bool valid = r.valid != 0;  // team-uniform
     team_sync(team, T);
     FoldAcc<NDET> acc;
+    FoldSum<NDET> sum;
     acc.clear();
+    sum.hi.clear();
     if (valid)
       for (int base = 0; base < F.nc; base += panel) {
         const int np = min(panel, F.nc - base);
@@ -240,30 +242,22 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
         for (int q = tid; q < np; q += 32 * T)
           if (!fold_in_band<NDET>(tab, ld, an + q * kFoldAnchor, q, base + q)) s_bad[team] = 1;
         const float* aq = an + tw * kFoldAnchor;
-        for (int q = tw; q < np; q += 2 * T, wq += 2 * T * NDET * 32, aq += 2 * T * kFoldAnchor) {
-          if (q + T < np) fold_load<NDET>(wq + T * NDET * 32, kind(q + T), x0, s_x, lane, v1);
-          fold_chunk<NDET>(aq, q, v0, acc);
-          if (q + T < np) {
-            if (q + 2 * T < np) fold_load<NDET>(wq + 2 * T * NDET * 32, kind(q + 2 * T), x0, s_x, lane, v0);
-            fold_chunk<NDET>(aq + T * kFoldAnchor, q + T, v1, acc);
+        for (int q = tw; q < np;) {
+          const int end = min(np, q + kFoldBlock * T);
+          for (; q < end; q += 2 * T, wq += 2 * T * NDET * 32, aq += 2 * T * kFoldAnchor) {
+            if (q + T < np) fold_load<NDET>(wq + T * NDET * 32, kind(q + T), x0, s_x, lane, v1);
+            fold_chunk<NDET>(aq, q, v0, acc);
+            if (q + T < np) {
+              if (q + 2 * T < np) fold_load<NDET>(wq + 2 * T * NDET * 32, kind(q + 2 * T), x0, s_x, lane, v0);
+              fold_chunk<NDET>(aq + T * kFoldAnchor, q + T, v1, acc);
+            }
           }
+          if (F.nc > kFoldBlock * T) sum.take(acc);
         }
         team_sync(team, T);
       }
-#pragma unroll
-    for (int i = 0; i < NDET; ++i) {
-      float re, im;
-      acc.total(i, re, im);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, o);
-        im += __shfl_xor_sync(0xffffffffu, im, o);
-      }
-      if (lane == 0) {
-        s_sum[2 * i][warp] = re;
-        s_sum[2 * i + 1][warp] = im;
-      }
-    }
+    fold_warp_sums<NDET, 1, 1>(&acc, F.nc > kFoldBlock * T, &sum.hi, lane,
+                               [&](int j, dfl v) { s_sum[j][warp] = make_float2(v.hi, v.lo); });
     team_sync(team, T);
     const bool bad = valid && s_bad[team];  // team-uniform
     if (bad) {
@@ -275,18 +269,22 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
       team_sync(team, T);
     }
     if (tw == 0) {
-      // the warps' sums in warp order (double-float), component j on lane j
-      double kapc = 0.0;
-      if (lane < 2 * NDET) {
-        if (bad) {
+      // the warps' sums (double-float, four lanes a component), component j on lane j
+      const int j = lane & 7;
+      dfl t = {0.0f, 0.0f};
+      if (j < 2 * NDET)
+        for (int w = lane >> 3; w < T; w += 4)
+          t = df_accumulate(t, dfl{s_sum[j][warp + w].x, s_sum[j][warp + w].y});
+#pragma unroll
+      for (int o = 8; o < 32; o <<= 1)
+        t = df_accumulate(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
+      double kapc = lane < 2 * NDET ? (double)t.hi + (double)t.lo : 0.0;
+      if (bad) {
+        kapc = 0.0;
+        if (lane < 2 * NDET)
           for (int w = 0; w < T; ++w) kapc += s_dir[lane][warp + w];
-        } else {
-          dfl t = {0.0f, 0.0f};
-          for (int w = 0; w < T; ++w) t = df_add(t, dfl{s_sum[lane][warp + w], 0.0f});
-          kapc = (double)t.hi + (double)t.lo;
-        }
+        __syncwarp();
       }
-      __syncwarp();
       const double ll = loglike_epilogue_warp<NDET>(L, r, kapc, lane);
       if (lane == 0) out[th] = ll;
       if (kappa_out && lane < 2 * SWIG_MAX_DET) kappa_out[(size_t)th * 2 * SWIG_MAX_DET + lane] = kapc;
