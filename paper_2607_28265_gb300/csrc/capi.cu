@@ -396,6 +396,8 @@ std::vector<float2> fold_abscissae() {
 void free_scratch(DeviceBuffers& B) {
   dfree(B.rec);
   dfree(B.partials64);
+  if (B.strays) cudaFree(B.strays);
+  B.strays = nullptr;
   dfree(B.theta);
   dfree(B.out);
   dfree(B.u);
@@ -990,6 +992,7 @@ int ensure_scratch(swig_ctx* c, int n) {
   // sampler's request slots (at most 4096): up to 4 per (theta, slice)
   const size_t units = (size_t)c->L.n_slices * 4 * std::min(cap, 4096);
   CUDA_TRY(c, cudaMalloc(&B.partials64, sizeof(double) * kPartialStride * units));
+  if (B.fold_nc > 0) CUDA_TRY(c, cudaMalloc(&B.strays, fold_strays_bytes(cap, c->L.n_slices)));
   CUDA_TRY(c, cudaMalloc(&B.theta, sizeof(double) * SWIG_N_PARAMS * cap));
   CUDA_TRY(c, cudaMalloc(&B.out, sizeof(double) * cap));
   CUDA_TRY(c, cudaMalloc(&B.u, sizeof(double) * SWIG_N_PARAMS * cap));

@@ -2,6 +2,8 @@
 // batched evaluation.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "fold.cuh"
 #include "kernels.h"
 
@@ -177,15 +179,259 @@ __device__ __forceinline__ void team_sync(int team, int T) {
     named_barrier(1 + team, 32 * T);
 }
 
+// The strays of a batch, vectors far from the prior box that the node weights do
+// not serve, are summed bin by bin by the CTAs that are left: a slice of the grid for
+// two strays per warp, on packed FP32.  Few strays: units by ticket, a warp each.  32
+// or more: a slice and up to 128 strays per CTA, the slice's tables in shared memory
+// for all.  The warp that finishes a stray's last slice adds its partial sums in FP64
+// and writes the result.
+//
+// Every stray is summed whatever the others do: the CTA that is the last to have
+// decided its vectors knows how many there are and takes units until none is left.
+// The others wait for that only to help, where they know of a stray when they are
+// done, so that a batch without strays waits for nothing: a CTA asks with its last
+// decision, ahead of that vector's epilogue.
+//
+// A pair over a slice of 1,700 bins and three detectors is bound by the sines (a
+// quarter of a warp per clock) and the issue slots about alike.  One GB300, 128 s
+// grid, three detectors: one stray among 1000 vectors 31 -> 63 us (by the team that met
+// it, one or two warps, 965; any 1000 vectors summed over all bins 667), a stray by
+// itself 47 us (174; 66), 100 strays 136 us (177; 135), 1000 strays 877 us (1440;
+// 667), 4099 on the 256 s grid 4.32 ms (10.3; 4.74).
+constexpr int kStrayCtas = 16;   // CTAs of a small batch at least: a warp per slice of one stray
+constexpr int kStrayTiles = 18;  // tiles whose anchors, of two strays, a warp holds
+constexpr int kStrayGroup = 128;
+
+// The strays once all CTAs with vectors have decided them, or -1 after so many polls
+// (0.7 us each).
+__device__ __forceinline__ int strays_known(const FoldStrays& S, int ctas, int polls, int polls_stray) {
+  for (int p = 0;; ++p) {
+    const unsigned long long c = *(const volatile unsigned long long*)S.ctl;
+    if ((int)(unsigned)c >= ctas) return (int)(c >> 32);
+    if (p >= (c >> 32 ? polls_stray : polls)) return -1;
+    __nanosleep(100);
+  }
+}
+
+// sweep_warp_mixed for two vectors: bins lo .. hi - 1 of a slice that starts at bin b0,
+// row: StrayRow of the tiles from tile0 on.  re, im - jm: the lane's sums.
+struct StrayRow {
+  f2 an[kAnchorStride];  // the anchors (compute_anchor)
+  int k0, end;           // the tile's bins
+  float inv_T, pad;
+};
+static_assert(kStrayTiles * sizeof(StrayRow) <= kFoldSlots * kFoldAnchor * sizeof(float) / kFoldWarps,
+              "a warp's share of the anchors");
+
+template <int NDET>
+__device__ __forceinline__ void sweep_warp_pair(const float2* data, int stride, const int* tile, int b0, int lo, int hi,
+                                                const StrayRow* row, int tile0, const f2* shift, int lane, f2* re,
+                                                f2* im, f2* jm) {
+  using O = PkOps<2>;
+  const f2 magic = O::all(12582912.0f), nmagic = O::all(-12582912.0f), none = O::all(-1.0f);
+  const auto off = [&](f2 v) { return f2_fma(f2_add(f2_add(v, magic), nmagic), none, v); };  // (see round_nearest)
+  StrayRow a;
+  a.end = -1;
+  const auto phase = [&](float x) {
+    const float u = x * a.inv_T;
+    const f2 u2 = O::all(u), x2 = O::all(x);
+    f2 p = a.an[2 + kNumPoly];
+#pragma unroll
+    for (int m = kNumPoly - 2; m >= 0; --m) p = f2_fma(p, u2, a.an[3 + m]);
+    p = f2_mul(p, O::all(u * u));
+    return f2_add(off(f2_mul(x2, a.an[1])), f2_add(a.an[0], f2_fma(x2, a.an[2], p)));
+  };
+  const auto add = [&](float x, f2 p, int k) {
+    const f2 x2 = O::all(x);
+#pragma unroll
+    for (int i = 0; i < NDET; ++i) {
+      const f2 ph = f2_mul(off(f2_add(p, f2_fma(x2, shift[i], a.an[3 + kNumPoly + i]))), O::all(6.283185307179586f));
+      float pa, pb, sa, ca, sb, cb;
+      f2_split(ph, pa, pb);
+      __sincosf(pa, &sa, &ca);
+      __sincosf(pb, &sb, &cb);
+      const f2 c2 = f2_make(ca, cb), s2 = f2_make(sa, sb);
+      const float2 d = data[i * stride + k];
+      const f2 dx = O::all(d.x), dy = O::all(d.y);
+      re[i] = f2_fma(dx, c2, f2_fma(dy, s2, re[i]));
+      im[i] = f2_fma(dy, c2, im[i]);
+      jm[i] = f2_fma(dx, s2, jm[i]);
+    }
+  };
+  for (int k = lo + lane; k < hi;) {
+    if (k >= a.end) {
+      a = row[tile[k] - tile0];
+      a.k0 -= b0;
+      a.end -= b0;
+    }
+    const float x = (float)(k - a.k0);
+    const f2 p = phase(x);
+    if (k + 32 < min(hi, a.end)) {  // two bins of a tile at a time
+      const f2 q = phase(x + 32.0f);
+      add(x, p, k);
+      add(x + 32.0f, q, k + 32);
+      k += 64;
+    } else {
+      add(x, p, k);
+      k += 32;
+    }
+  }
+}
+
+// A slice's tables where a warp reads them: data and tile indices of the bins from b0
+// on, tiles from t0 on.
+struct StraySlice {
+  const float2* data;
+  int stride;
+  const int* tile;
+  int b0;
+  const TileInfo* tiles;
+  const TileBasis* basis;
+  int t0;
+};
+inline __host__ __device__ size_t stray_slice_bytes(int n_det, int bins, int tiles) {
+  return (sizeof(float2) * n_det + sizeof(int)) * (size_t)bins + (sizeof(TileInfo) + sizeof(TileBasis)) * (size_t)tiles;
+}
+
+// Strays i and i + 1 over one slice by a warp; row: the warp's share of the anchors.
+template <int NDET>
+__device__ __forceinline__ void stray_unit(const LikeConst& L, const FoldTables& F, const EvalRecord* rec,
+                                           const FoldStrays& S, int strays, int slice, int i, const StraySlice& T,
+                                           StrayRow* row, int lane, double* out, double* kappa_out) {
+  const bool two = i + 1 < strays;
+  const EvalRecord* r = &rec[__ldcg(&S.list[two ? i + (lane & 1) : i])];  // even lanes', odd lanes'
+  const int k0 = F.slice_begin[slice], k1 = F.slice_begin[slice + 1];
+  const int t1 = T.tile[k1 - 1 - T.b0] + 1;
+  const float sh = lane < 2 * NDET ? (float)(L.df * r->tau[lane >> 1]) : 0.0f;
+  f2 shift[NDET], re[NDET], im[NDET], jm[NDET];
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) {
+    shift[d] = f2_make(__shfl_sync(0xffffffffu, sh, 2 * d), __shfl_sync(0xffffffffu, sh, 2 * d + 1));
+    re[d] = im[d] = jm[d] = 0ull;
+  }
+  for (int t = T.tile[k0 - T.b0]; t < t1; t += kStrayTiles) {
+    const int nt = min(kStrayTiles, t1 - t);
+    __syncwarp();
+    for (int q = lane; q < 2 * nt; q += 32) {
+      const int at = t - T.t0 + (q >> 1);
+      const TileInfo ti = T.tiles[at];
+      float an[kAnchorStride];
+      compute_anchor(NDET, ti, T.basis[at], *r, an);
+      StrayRow& w = row[q >> 1];
+#pragma unroll
+      for (int m = 0; m < kAnchorStride; ++m) reinterpret_cast<float*>(&w.an[m])[q & 1] = an[m];
+      if (!(q & 1)) w.k0 = ti.k0, w.end = ti.k0 + ti.nbins, w.inv_T = ti.inv_T;
+    }
+    __syncwarp();
+    const int lo = max(k0, row[0].k0), hi = min(k1, row[nt - 1].end);
+    sweep_warp_pair<NDET>(T.data, T.stride, T.tile, T.b0, lo - T.b0, hi - T.b0, row, t, shift, lane, re, im, jm);
+  }
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) im[d] = pk_sub<2>(im[d], jm[d]);
+#pragma unroll
+  for (int d = 0; d < NDET; ++d)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      re[d] = f2_add(re[d], __shfl_xor_sync(0xffffffffu, re[d], o));
+      im[d] = f2_add(im[d], __shfl_xor_sync(0xffffffffu, im[d], o));
+    }
+  float* p[2] = {S.part + (size_t)i * L.n_slices * kPartialStride, S.part + (size_t)(i + 1) * L.n_slices * kPartialStride};
+#pragma unroll
+  for (int j = 0; j < 2 * NDET; ++j) {
+    float a, b;
+    f2_split(j & 1 ? im[j / 2] : re[j / 2], a, b);
+    if (lane == j) __stcg(&p[0][slice * kPartialStride + j], a);
+    if (lane == j && two) __stcg(&p[1][slice * kPartialStride + j], b);
+  }
+  __threadfence();
+  __syncwarp();
+  int last = 0;
+  if (lane < 2 && i + lane < strays) last = atomicAdd(&S.done[i + lane], 1) == L.n_slices - 1;
+  const unsigned done = __ballot_sync(0xffffffffu, last);
+  if (!done) return;
+  __threadfence();
+#pragma unroll 1
+  for (int e = 0; e < 2; ++e) {
+    if (!((done >> e) & 1u)) continue;
+    double acc[2 * NDET];
+#pragma unroll
+    for (int j = 0; j < 2 * NDET; ++j) acc[j] = 0.0;
+    const float* q = S.part + (size_t)(i + e) * L.n_slices * kPartialStride;
+    for (int s = lane; s < L.n_slices; s += 32)
+#pragma unroll
+      for (int j = 0; j < 2 * NDET; ++j) acc[j] += (double)__ldcg(&q[s * kPartialStride + j]);
+    double kapc = 0.0;
+#pragma unroll
+    for (int j = 0; j < 2 * NDET; ++j) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+      if (lane == j) kapc = acc[j];
+    }
+    const int th = __ldcg(&S.list[i + e]);
+    const double ll = loglike_epilogue_warp<NDET>(L, rec[th], kapc, lane);
+    if (lane == 0) out[th] = ll;
+    if (kappa_out && lane < 2 * SWIG_MAX_DET) kappa_out[(size_t)th * 2 * SWIG_MAX_DET + lane] = kapc;
+  }
+}
+
+// s_slice: room for the tables of a slice of cap bins and tiles (cap.x 0: none).
+template <int NDET>
+__device__ __noinline__ void fold_strays(const LikeConst& L, const FoldTables& F, const EvalRecord* rec,
+                                         const FoldStrays& S, int strays, StrayRow* row, float2* s_slice, int2 cap,
+                                         int lane, double* out, double* kappa_out) {
+  __shared__ int s_unit;
+  const int warp = threadIdx.x >> 5, pairs = (strays + 1) / 2;
+  StraySlice T = {F.data, L.n_bins, F.bin_tile, 0, F.tiles, F.basis, 0};
+  if (pairs < kFoldWarps || cap.x == 0) {
+    for (;;) {
+      int u = 0;
+      if (lane == 0) u = atomicAdd(&S.ctl[2], 1);
+      u = __shfl_sync(0xffffffffu, u, 0);
+      if (u >= pairs * L.n_slices) return;
+      stray_unit<NDET>(L, F, rec, S, strays, u / pairs, 2 * (u % pairs), T, row, lane, out, kappa_out);
+    }
+  }
+  int* s_tile = reinterpret_cast<int*>(s_slice + (size_t)NDET * cap.x);
+  TileBasis* s_basis = reinterpret_cast<TileBasis*>(s_tile + cap.x);
+  TileInfo* s_info = reinterpret_cast<TileInfo*>(s_basis + cap.y);
+  T.data = s_slice, T.stride = cap.x, T.tile = s_tile, T.tiles = s_info, T.basis = s_basis;
+  const int groups = (strays + kStrayGroup - 1) / kStrayGroup;
+  for (int held = -1;;) {
+    __syncthreads();  // the previous unit's tables have been read
+    if (threadIdx.x == 0) s_unit = atomicAdd(&S.ctl[2], 1);
+    __syncthreads();
+    const int slice = s_unit / groups, first = (s_unit - slice * groups) * kStrayGroup;
+    if (slice >= L.n_slices) return;
+    if (slice != held) {
+      T.b0 = F.slice_begin[slice];
+      const int nb = F.slice_begin[slice + 1] - T.b0;
+      T.t0 = F.bin_tile[T.b0];
+      const int nt = F.bin_tile[T.b0 + nb - 1] + 1 - T.t0;
+      for (int d = 0; d < NDET; ++d)
+        for (int k = threadIdx.x; k < nb; k += blockDim.x) s_slice[d * cap.x + k] = F.data[(size_t)d * L.n_bins + T.b0 + k];
+      for (int k = threadIdx.x; k < nb; k += blockDim.x) s_tile[k] = F.bin_tile[T.b0 + k];
+      const float* from = reinterpret_cast<const float*>(F.basis + T.t0);
+      for (int k = threadIdx.x; k < nt * (int)(sizeof(TileBasis) / sizeof(float)); k += blockDim.x)
+        reinterpret_cast<float*>(s_basis)[k] = from[k];
+      for (int k = threadIdx.x; k < nt; k += blockDim.x) s_info[k] = F.tiles[T.t0 + k];
+      __syncthreads();
+      held = slice;
+    }
+    const int end = min(strays, first + kStrayGroup);
+    for (int i = first + 2 * warp; i < end; i += 2 * kFoldWarps)
+      stray_unit<NDET>(L, F, rec, S, strays, slice, i, T, row, lane, out, kappa_out);
+  }
+}
+
 template <int NDET, bool RES>
 __global__ void __launch_bounds__(32 * kFoldWarps, 1)
     k_fold(LikeConst L, FoldTables F, const EvalRecord* __restrict__ rec, int n, int T, double* __restrict__ out,
-           double* __restrict__ kappa_out) {
-  extern __shared__ __align__(16) unsigned char smem[];
+           double* __restrict__ kappa_out, FoldStrays S, int2 slice_cap) {
+  // (16 bytes off a line, as the static arrays left it, 1000 vectors took 31.0 us for 27.5)
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ FoldIn s_in[kFoldWarps];
   __shared__ float2 s_sum[2 * NDET][kFoldWarps];
-  __shared__ double s_dir[2 * NDET][kFoldWarps];
-  __shared__ int s_bad[kFoldWarps];
+  __shared__ int s_bad[kFoldWarps], s_left, s_met, s_strays;  // (strays: teams at work, strays met, all known)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int team = warp / T, tw = warp - team * T, tid = 32 * tw + lane;  // within the team
   const int teams = kFoldWarps / T, panel = min(128, kFoldSlots / teams);
@@ -194,22 +440,31 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
   const float4* w = F.w;
   const float* tab = F.tab;
   const int ld = F.ld;
+  const bool idle = blockIdx.x * teams >= n;  // here to help with strays
   if (RES) {
     float4* s_w = reinterpret_cast<float4*>(s_x + 32 * kFoldKinds);
     float4* s_t = s_w + F.nc * NDET * 32;
     const float4* g_t = reinterpret_cast<const float4*>(F.tab);
-    for (int k = threadIdx.x; k < FR_ROWS * ld / 4; k += blockDim.x) cp_async16(s_t + k, g_t + k);
-    for (int k = threadIdx.x; k < F.nc * NDET * 32; k += blockDim.x) cp_async16(s_w + k, F.w + k);
+    if (!idle) {
+      for (int k = threadIdx.x; k < FR_ROWS * ld / 4; k += blockDim.x) cp_async16(s_t + k, g_t + k);
+      for (int k = threadIdx.x; k < F.nc * NDET * 32; k += blockDim.x) cp_async16(s_w + k, F.w + k);
+    }
     w = s_w;
     tab = reinterpret_cast<const float*>(s_t);
   }
   for (int k = threadIdx.x; k < 32 * kFoldKinds; k += blockDim.x) s_x[k] = F.x[k];
+  if (threadIdx.x == 0) {
+    s_left = min(teams, n - (int)blockIdx.x * teams);
+    s_met = 0;
+    s_strays = 0;
+  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   // the set-up kernel's records, while this one's start overlapped its end
   asm volatile("griddepcontrol.wait;" ::: "memory");
   float* an = s_anchor + team * panel * kFoldAnchor;
   const float2 x0 = s_x[lane];
+  unsigned long long seen = 0;  // CTAs done deciding, strays << 32, with this one: of the thread that reported it
   for (int th = blockIdx.x * teams + team; th < n; th += gridDim.x * teams) {
     const EvalRecord& r = rec[th];
     team_sync(team, T);  // the previous vector's shared memory has been read
@@ -259,16 +514,19 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
     fold_warp_sums<NDET, 1, 1>(&acc, F.nc > kFoldBlock * T, &sum.hi, lane,
                                [&](int j, dfl v) { s_sum[j][warp] = make_float2(v.hi, v.lo); });
     team_sync(team, T);
-    const bool bad = valid && s_bad[team];  // team-uniform
-    if (bad) {
-      double v[2 * NDET];
-      fold_direct<NDET>(L, F, r, tw, T, lane, an + tw * kAnchorStride, v);
-      if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < 2 * NDET; ++j) s_dir[j][warp] = v[j];
-      team_sync(team, T);
+    const bool stray = valid && s_bad[team];  // team-uniform
+    if (tid == 0) {
+      if (stray) {
+        S.list[atomicAdd(&S.ctl[3], 1)] = th;
+        __threadfence();
+        atomicAdd(&s_met, 1);
+      }
+      if (th + gridDim.x * teams >= n && (teams == 1 || atomicSub(&s_left, 1) == 1)) {
+        const unsigned long long mine = 1 + ((unsigned long long)*(volatile int*)&s_met << 32);
+        seen = atomicAdd(reinterpret_cast<unsigned long long*>(S.ctl), mine) + mine;
+      }
     }
-    if (tw == 0) {
+    if (tw == 0 && !stray) {
       // the warps' sums (double-float, four lanes a component), component j on lane j
       const int j = lane & 7;
       dfl t = {0.0f, 0.0f};
@@ -278,17 +536,28 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1)
 #pragma unroll
       for (int o = 8; o < 32; o <<= 1)
         t = df_accumulate(t, dfl{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
-      double kapc = lane < 2 * NDET ? (double)t.hi + (double)t.lo : 0.0;
-      if (bad) {
-        kapc = 0.0;
-        if (lane < 2 * NDET)
-          for (int w = 0; w < T; ++w) kapc += s_dir[lane][warp + w];
-        __syncwarp();
-      }
+      const double kapc = lane < 2 * NDET ? (double)t.hi + (double)t.lo : 0.0;
       const double ll = loglike_epilogue_warp<NDET>(L, r, kapc, lane);
       if (lane == 0) out[th] = ll;
       if (kappa_out && lane < 2 * SWIG_MAX_DET) kappa_out[(size_t)th * 2 * SWIG_MAX_DET + lane] = kapc;
     }
+  }
+  // all strays if this CTA was the last to decide, -1 if there are some so far
+  const int ctas = min((int)gridDim.x, (n + teams - 1) / teams);
+  if (seen) s_strays = (int)(unsigned)seen == ctas ? (int)(seen >> 32) : seen >> 32 ? -1 : 0;
+  __syncthreads();
+  int strays = s_strays;
+  if (strays < 0 || idle) {  // block-uniform
+    __syncthreads();
+    if (threadIdx.x == 0) s_strays = strays_known(S, ctas, idle ? 40 : 0, 200);
+    __syncthreads();
+    strays = s_strays;
+  }
+  if (strays > 0) {
+    __threadfence();  // the list, behind the count
+    fold_strays<NDET>(L, F, rec, S, strays,
+                      reinterpret_cast<StrayRow*>(s_anchor + warp * (kFoldSlots * kFoldAnchor / kFoldWarps)),
+                      reinterpret_cast<float2*>(smem + fold_fixed_bytes()), slice_cap, lane, out, kappa_out);
   }
 }
 
@@ -296,14 +565,22 @@ namespace {
 
 template <int NDET, bool RES>
 cudaError_t fold_launch_as(const LikeConst& L, const FoldTables& F, const EvalRecord* rec, int n, double* out,
-                           cudaStream_t st, double* kappa_out, size_t smem) {
+                           cudaStream_t st, double* kappa_out, const FoldStrays& S, int2 slice_cap, size_t smem) {
   cudaError_t e = allow_shared((const void*)k_fold<NDET, RES>);
   if (e != cudaSuccess) return e;
   // the widest team that leaves no vector waiting for a second turn
   const int ctas = L.sm_count;
   int T = kFoldWarps;
   while (T > 1 && (long long)n * T > (long long)ctas * kFoldWarps) T /= 2;
-  const int teams = kFoldWarps / T, need = (n + teams - 1) / teams;
+  // a small batch gets CTAs to help with strays (one among up to 100: 47 us, 227
+  // without them; without strays they change nothing)
+  const int teams = kFoldWarps / T, need = std::max(3 * ((n + teams - 1) / teams), kStrayCtas);
+  // room for a slice's tables, over the weights or beside the anchors
+  const size_t slice = fold_fixed_bytes() + stray_slice_bytes(NDET, slice_cap.x, slice_cap.y);
+  if (slice <= 220 * 1024)
+    smem = std::max(smem, slice);
+  else
+    slice_cap = make_int2(0, 0);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(need < ctas ? need : ctas);
   cfg.blockDim = dim3(32 * kFoldWarps);
@@ -314,17 +591,19 @@ cudaError_t fold_launch_as(const LikeConst& L, const FoldTables& F, const EvalRe
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_fold<NDET, RES>, L, F, rec, n, T, out, kappa_out);
+  return cudaLaunchKernelEx(&cfg, k_fold<NDET, RES>, L, F, rec, n, T, out, kappa_out, S, slice_cap);
 }
 
 template <int NDET>
 cudaError_t fold_launch(const LikeConst& L, const DeviceBuffers& B, int n, double* out, cudaStream_t st,
                         double* kappa_out) {
   const FoldTables F = fold_tables(B);
+  const FoldStrays S = fold_strays_at(B.strays, n);
+  const int2 slice = make_int2(B.max_slice_bins, B.max_slice_tiles);
   const size_t fixed = fold_fixed_bytes(), res = fixed + fold_resident_bytes(F.nc, NDET);
   if (n > L.sm_count && res <= 220 * 1024)
-    return fold_launch_as<NDET, true>(L, F, B.rec, n, out, st, kappa_out, res);
-  return fold_launch_as<NDET, false>(L, F, B.rec, n, out, st, kappa_out, fixed);
+    return fold_launch_as<NDET, true>(L, F, B.rec, n, out, st, kappa_out, S, slice, res);
+  return fold_launch_as<NDET, false>(L, F, B.rec, n, out, st, kappa_out, S, slice, fixed);
 }
 
 }  // namespace

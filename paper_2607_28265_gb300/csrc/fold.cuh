@@ -22,7 +22,8 @@
 //
 // An evaluation checks its own bandwidth and Taylor remainder on every chunk
 // against the bound the weights were made for; a parameter vector outside
-// (one far from the prior box) is summed bin by bin instead (fold_direct).
+// (one far from the prior box) is summed bin by bin instead: in a batch by all
+// its CTAs (fold.cu fold_strays), in the sampler by the chain's (fold_direct).
 #pragma once
 
 #include "packed.cuh"
@@ -410,7 +411,7 @@ __device__ __forceinline__ void fold_chunk(const float* __restrict__ an, int sw,
   }
 }
 
-// Bin by bin (rare): tiles first, first + stride, ... of the grid by one warp
+// Bin by bin (rare, the sampler): tiles first, first + stride, ... of the grid by one warp
 // from global memory, with the tile anchors of the direct sum (sweep.cuh);
 // row: kAnchorStride floats of the warp's own in shared memory.  Lane sums in
 // FP64 across tiles; every lane returns the warp's totals.

@@ -148,12 +148,34 @@ struct FoldTables {
   const float* tab;   // [FR_ROWS][ld]
   const float4* w;    // [nc][n_det][32] node weights (+x re, -x re, +x im, -x im)
   const float2* x;    // [kFoldKinds][32] the lanes' node abscissae (hi, lo)
-  // bin by bin (fold_direct)
+  // bin by bin (fold_direct, fold_strays)
   const float2* data;
   const TileInfo* tiles;
   const TileBasis* basis;
   const int* bin_tile;
+  const int* slice_begin;
 };
+
+// Vectors of a batch that the node weights do not serve (fold.cu fold_strays), in
+// the scratch of the batch; the set-up kernel clears ctl and done.
+struct FoldStrays {
+  int* ctl;     // [4] vectors decided, strays among them (one 64-bit count), units taken, list entries
+  int* list;    // [n] the strays
+  int* done;    // [n] slices summed of stray i
+  float* part;  // [n][n_slices][kPartialStride] their sums
+};
+inline size_t fold_strays_bytes(int n, int n_slices) {
+  return sizeof(int) * (4 + 2 * (size_t)n) + sizeof(float) * kPartialStride * (size_t)n_slices * n + 16;
+}
+inline FoldStrays fold_strays_at(void* p, int n) {
+  FoldStrays s;
+  s.ctl = static_cast<int*>(p);
+  s.list = s.ctl + 4;
+  s.done = s.list + n;
+  const size_t off = (sizeof(int) * (4 + 2 * (size_t)n) + 15) / 16 * 16;
+  s.part = reinterpret_cast<float*>(static_cast<char*>(p) + off);
+  return s;
+}
 
 // Device buffers owned by a context (all allocated with cudaMalloc).
 struct DeviceBuffers {
@@ -193,6 +215,7 @@ struct DeviceBuffers {
   int cap = 0;
   EvalRecord* rec = nullptr;     // [cap]
   double* partials64 = nullptr;  // [cap][n_slices][kPartialStride]
+  void* strays = nullptr;        // FoldStrays of cap vectors (mixed, full grid)
   double* theta = nullptr;       // [cap][13] staging for host calls
   double* out = nullptr;         // [cap]
   double* u = nullptr;           // [cap][13]
@@ -222,7 +245,8 @@ inline HetTmLayout het_tm_layout(const LikeConst& L, const DeviceBuffers& B) {
 
 inline __host__ __device__ int fold_ld(int nc) { return (nc + 3) & ~3; }
 inline __host__ __device__ FoldTables fold_tables(const DeviceBuffers& B) {
-  return {B.fold_nc, fold_ld(B.fold_nc), B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile};
+  return {B.fold_nc, fold_ld(B.fold_nc), B.fold_tab, B.fold_w, B.fold_x, B.data32, B.tiles, B.basis, B.bin_tile,
+          B.slice_begin};
 }
 
 // Bytes of the weights and table (weights first) in shared memory.
@@ -276,8 +300,8 @@ cudaError_t launch_time_draw(const LikeConst& L, const DeviceBuffers& B, const f
 cudaError_t launch_prior_transform(const PriorSlot* slots, int n_sampled, const double* u, int n, double* theta,
                                    cudaStream_t st, SkyFrame sky);
 
-// Dynamic shared memory of the mixed sweep: data (float2 per detector and
-// bin) plus the tile index of each bin of the slice.
+// Shared memory that a slice of the bins is planned for (plan_slices): data (float2
+// per detector and bin) plus the tile index of each bin.
 inline size_t sweep_smem_bytes(int n_det, int slice_bins) {
   return (size_t)slice_bins * (n_det * sizeof(float2) + sizeof(int));
 }

@@ -34,7 +34,7 @@ namespace swig {
 constexpr int kSetupWarps = 8;
 
 __global__ void __launch_bounds__(32 * kSetupWarps)
-    k_setup(LikeConst L, const double* __restrict__ theta, int n, EvalRecord* __restrict__ rec) {
+    k_setup(LikeConst L, const double* __restrict__ theta, int n, EvalRecord* __restrict__ rec, FoldStrays strays) {
   __shared__ double s_th[SWIG_N_PARAMS][33];
   __shared__ double s_m[8][32];      // MassTerms, in EvalRecord::mterm's order
   __shared__ double s_sc[8][32];     // sines and cosines of RA - GMST, Dec, 2 psi, phi_c
@@ -44,6 +44,10 @@ __global__ void __launch_bounds__(32 * kSetupWarps)
   // a dependent kernel may start; it waits for this grid's end before it
   // reads a record (griddepcontrol.wait)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (strays.ctl && blockIdx.y == 0 && warp == kSetupWarps - 1) {
+    if (i < n) strays.done[i] = 0;
+    if (blockIdx.x == 0 && lane < 4) strays.ctl[lane] = 0;
+  }
   for (int e = threadIdx.x; e < 32 * SWIG_N_PARAMS; e += blockDim.x) {
     const int v = e / SWIG_N_PARAMS, j = e - v * SWIG_N_PARAMS;
     double x = i0 + v < n ? theta[(size_t)i0 * SWIG_N_PARAMS + e] : 1.0;
@@ -208,8 +212,9 @@ cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, size_t byte
 }
 
 // k_setup of n vectors.
-static void launch_setup(const LikeConst& L, const double* theta, int n, EvalRecord* rec, cudaStream_t st) {
-  k_setup<<<dim3((n + 31) / 32, 2), 32 * kSetupWarps, 0, st>>>(L, theta, n, rec);
+static void launch_setup(const LikeConst& L, const double* theta, int n, EvalRecord* rec, cudaStream_t st,
+                         const FoldStrays& strays = {}) {
+  k_setup<<<dim3((n + 31) / 32, 2), 32 * kSetupWarps, 0, st>>>(L, theta, n, rec, strays);
 }
 
 template <int NDET>
@@ -677,7 +682,7 @@ __global__ void k_prior_transform(const PriorSlot* __restrict__ slots, int n_sam
 cudaError_t launch_loglike_mixed(const LikeConst& L, const DeviceBuffers& B, const double* theta, int n,
                                  double* out, cudaStream_t st, double* kappa_out) {
   if (n <= 0) return cudaSuccess;
-  launch_setup(L, theta, n, B.rec, st);
+  launch_setup(L, theta, n, B.rec, st, fold_strays_at(B.strays, n));
   return launch_fold(L, B, n, out, st, kappa_out);
 }
 

@@ -69,7 +69,7 @@ extern "C" int swig_loglike_batch_noalloc(swig_ctx* c, const double* theta_dev, 
   // Capacity first, so that no size below is formed from an unchecked n.  The
   // per-vector bytes are this entry point's stated budget (a record, an anchor
   // per tile and four partial sums per slice); the folded evaluation uses the
-  // record alone.
+  // record and, of a stray, a partial sum per slice.
   const size_t per_theta = sizeof(EvalRecord) + sizeof(float) * kAnchorStride * (size_t)c->L.n_tiles +
                            sizeof(float) * kPartialStride * (size_t)c->L.n_slices * 4;
   const int64_t cap = (int64_t)((kNoAllocScratchBytes - 3 * 256) / per_theta);
@@ -86,10 +86,11 @@ extern "C" int swig_loglike_batch_noalloc(swig_ctx* c, const double* theta_dev, 
     c->err = std::string("scratch set-up: ") + cudaGetErrorString(e);
     return SWIG_E_CUDA;
   }
-  // The scratch holds the set-up records, each written earlier in the same
-  // call that reads it, so nothing needs clearing.
+  // The scratch holds the set-up records and the strays' sums, each written
+  // earlier in the same call that reads it, so nothing needs clearing.
   DeviceBuffers B = c->B;
   B.rec = static_cast<EvalRecord*>(base);
+  B.strays = static_cast<char*>(base) + (sizeof(EvalRecord) * (size_t)n + 255) / 256 * 256;
   B.cap = (int)n;
   e = launch_loglike_mixed(c->L, B, theta_dev, (int)n, out_logl_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) {

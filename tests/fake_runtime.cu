@@ -109,6 +109,19 @@ cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t sha
       for (int d = 0; d < SWIG_MAX_DET; ++d) r[i].cre[d] = 1.0;
     }
   }
+  if (name.find("6k_foldI") != std::string::npos) {
+    const LikeConst& L = *static_cast<LikeConst*>(args[0]);
+    const int n = *static_cast<int*>(args[3]);
+    const FoldStrays& S = *static_cast<FoldStrays*>(args[7]);
+    if (room(*static_cast<void**>(args[2])) < sizeof(EvalRecord) * n) F().note("k_fold's records: past the end");
+    if (room(S.ctl) < 16 || room(S.list) < 4 * (size_t)n || room(S.done) < 4 * (size_t)n ||
+        room(S.part) < sizeof(float) * kPartialStride * L.n_slices * n)
+      F().note("k_fold's strays: past the end");
+    if ((const char*)S.ctl < *static_cast<char**>(args[2]) + sizeof(EvalRecord) * n &&
+        (const char*)S.ctl >= *static_cast<char**>(args[2]))
+      F().note("k_fold's strays: over the records");
+    if ((size_t)S.part % 16) F().note("k_fold's strays: alignment");
+  }
   if (name.find("k_ns_chain") != std::string::npos) {
     const ChainEvent* ev = *static_cast<ChainEvent**>(args[0]);
     const int n_ev = *static_cast<int*>(args[1]);

@@ -156,3 +156,21 @@ def test_contexts_do_not_lower_each_others_shared_memory_limit(device):
         ctx.mlp_train(rng.random((n, 5)), params, 2, lr=1e-3)
     ctx.close()
     assert not _report(device)
+
+
+@pytest.mark.parametrize("n", [1, 37, 300, 5000, 16384, 20000])
+def test_scratch_of_a_batch_holds_its_strays(device, n):
+    """Records, list, counts and partial sums of any batch lie in its scratch, also
+    in the fixed one of the entry point that does not allocate."""
+    ctx, th = _context()
+    theta, out = np.tile(th, (n, 1)), np.empty(n)
+    ctx.loglike_batch(theta)
+    cap = n
+    try:
+        ctx.loglike_batch_noalloc(theta.ctypes.data, n, out.ctypes.data, 0x1000)
+    except swig.SwigError as e:
+        cap = int(str(e).split(" parameter vectors")[0].split()[-1])
+        ctx.loglike_batch_noalloc(theta.ctypes.data, cap, out.ctypes.data, 0x1000)
+    assert cap >= min(n, 100)
+    assert not _report(device)
+    ctx.close()
