@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -1270,6 +1271,59 @@ int loglike_device(swig_ctx* c, const double* theta_dev, int64_t n, double* out_
 
 }  // namespace swig
 
+namespace {
+
+// Vectors of a host batch that goes through mapped memory.
+constexpr int kPinnedVectors = 64;
+
+// Mapped host memory of such a batch (7 KB).  To allocate and free it takes 245 us,
+// more than a short event's few evaluations gain by it, so that contexts leave it to
+// later ones: at most kPinnedKept blocks, for any device.
+constexpr size_t kPinnedKept = 16;
+struct PinnedPool {
+  std::mutex lock;
+  std::vector<double*> kept;
+};
+PinnedPool& pinned_pool() {
+  static PinnedPool* p = new PinnedPool;  // (not destroyed: contexts may outlive static objects)
+  return *p;
+}
+double* take_pinned() {
+  PinnedPool& pool = pinned_pool();
+  double* p = nullptr;
+  for (;;) {
+    {
+      const std::lock_guard<std::mutex> hold(pool.lock);
+      if (pool.kept.empty()) break;
+      p = pool.kept.back();
+      pool.kept.pop_back();
+    }
+    // (a device reset in between has freed it)
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost) return p;
+    cudaGetLastError();
+  }
+  if (cudaHostAlloc(&p, sizeof(double) * (SWIG_N_PARAMS + 1) * kPinnedVectors,
+                    cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess)
+    return p;
+  cudaGetLastError();
+  return nullptr;
+}
+void give_pinned(double* p) {
+  if (!p) return;
+  PinnedPool& pool = pinned_pool();
+  {
+    const std::lock_guard<std::mutex> hold(pool.lock);
+    if (pool.kept.size() < kPinnedKept) {
+      pool.kept.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
+}  // namespace
+
 // ===========================================================================
 // C-ABI
 // ===========================================================================
@@ -1316,7 +1370,7 @@ void swig_destroy(swig_ctx* c) {
   swig_mlp_release(c);
   free_problem(c->B);
   free_scratch(c->B);
-  if (c->pinned) cudaFreeHost(c->pinned);
+  give_pinned(c->pinned);
   if (c->stream && c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -1456,9 +1510,6 @@ int swig_set_sampler(swig_ctx* c, const swig_sampler_cfg* cfg) {
   return SWIG_OK;
 }
 
-// Vectors of a host batch that goes through mapped memory.
-constexpr int kPinnedVectors = 64;
-
 int swig_loglike_batch(swig_ctx* c, const double* theta, int64_t n, double* out_logl) {
   if (!c) return SWIG_E_ARG;
   if (n == 0) return SWIG_OK;
@@ -1468,11 +1519,7 @@ int swig_loglike_batch(swig_ctx* c, const double* theta, int64_t n, double* out_
   // A small batch goes through mapped host memory, which the set-up reads and
   // the evaluation writes over the link: two copies less to queue and wait for
   // (one vector: 36.2 -> 29.3 us; a larger batch's copies are a small part of it).
-  if (n <= kPinnedVectors && !c->pinned &&
-      cudaHostAlloc(&c->pinned, sizeof(double) * (SWIG_N_PARAMS + 1) * kPinnedVectors, cudaHostAllocMapped) != cudaSuccess) {
-    cudaGetLastError();
-    c->pinned = nullptr;
-  }
+  if (n <= kPinnedVectors && !c->pinned) c->pinned = take_pinned();
   if (n <= kPinnedVectors && c->pinned) {
     double* res = c->pinned + SWIG_N_PARAMS * kPinnedVectors;
     std::memcpy(c->pinned, theta, sizeof(double) * SWIG_N_PARAMS * n);

@@ -39,6 +39,7 @@ struct Fake {
   std::map<const void*, std::string> names;       // kernels by their host stub
   std::map<const void*, int> smem_limit;          // dynamic shared memory allowed
   std::map<const void*, size_t> vars;
+  std::set<const void*> hosts;                    // page-locked host allocations
   std::set<cudaStream_t> busy;                    // streams with work the host has not waited for
   std::vector<Source> sources;
   std::map<std::string, long long> calls;
@@ -162,7 +163,8 @@ int fake_report(char* out, int n) {
   return (int)F().report.size();
 }
 // Clears what was noted and counted; what: "sms" (of the device), "capturing",
-// "check streams" are settings, anything else a count to read.
+// "check streams" are settings, "forget hosts" frees page-locked memory as a device
+// reset does, anything else is a count to read.
 void fake_reset() {
   Guard g(F().lock);
   F().report.clear();
@@ -170,6 +172,7 @@ void fake_reset() {
 }
 long long fake_get(const char* what) {
   Guard g(F().lock);
+  if (std::string(what) == "hosts") return (long long)F().hosts.size();
   if (std::string(what) == "blocks") return (long long)F().blocks.size();
   return F().calls[what];
 }
@@ -177,6 +180,8 @@ void fake_set(const char* what, int v) {
   Guard g(F().lock);
   if (std::string(what) == "sms")
     F().sms = v;
+  else if (std::string(what) == "forget hosts")
+    F().hosts.clear();
   else if (std::string(what) == "capturing")
     F().capturing = v != 0;
   else
@@ -244,9 +249,13 @@ RT(cudaError_t, cudaHostAlloc, (void** p, size_t n, unsigned)) {
   Guard g(F().lock);
   F().calls["cudaHostAlloc"] += 1;
   *p = std::calloc(1, n);
+  F().hosts.insert(*p);
   return cudaSuccess;
 }
 RT(cudaError_t, cudaFreeHost, (void* p)) {
+  Guard g(F().lock);
+  F().calls["cudaFreeHost"] += 1;
+  if (!F().hosts.erase(p)) F().note("cudaFreeHost: not an allocation");
   std::free(p);
   return cudaSuccess;
 }
@@ -351,6 +360,12 @@ RT(cudaError_t, cudaFuncSetAttribute, (const void* f, cudaFuncAttribute, int v))
 }
 RT(cudaError_t, cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags, (int* n, const void*, int, size_t, unsigned)) {
   *n = 1;
+  return cudaSuccess;
+}
+RT(cudaError_t, cudaPointerGetAttributes, (cudaPointerAttributes* a, const void* p)) {
+  Guard g(F().lock);
+  std::memset(a, 0, sizeof(*a));
+  a->type = F().hosts.count(p) ? cudaMemoryTypeHost : room(p) ? cudaMemoryTypeDevice : cudaMemoryTypeUnregistered;
   return cudaSuccess;
 }
 RT(cudaError_t, cudaGetSymbolAddress, (void** p, const void* var)) {

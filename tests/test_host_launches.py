@@ -174,3 +174,28 @@ def test_scratch_of_a_batch_holds_its_strays(device, n):
     assert cap >= min(n, 100)
     assert not _report(device)
     ctx.close()
+
+
+def test_a_context_per_event_reuses_the_mapped_memory(device):
+    """Small host batches of contexts made one after another page-lock memory once,
+    not in each one's first call; what is kept is bounded, and dropped where a device
+    reset has freed it."""
+    def once(ctx, th):
+        ctx.loglike_batch(th[None])
+        ctx.close()
+
+    once(*_context())
+    device.fake_reset()
+    for i in range(5):
+        once(*_context(i))
+    assert device.fake_get(b"cudaHostAlloc") == 0 and device.fake_get(b"cudaFreeHost") == 0
+    many = [_context(i % 3) for i in range(30)]
+    for ctx, th in many:
+        ctx.loglike_batch(th[None])
+    for ctx, _ in many:
+        ctx.close()
+    assert device.fake_get(b"hosts") <= 16
+    device.fake_set(b"forget hosts", 1)
+    once(*_context())
+    assert device.fake_get(b"hosts") == 1
+    assert not _report(device)
