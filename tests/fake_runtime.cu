@@ -172,6 +172,11 @@ void fake_reset() {
 }
 long long fake_get(const char* what) {
   Guard g(F().lock);
+  if (std::string(what) == "bytes") {
+    long long n = 0;
+    for (const auto& b : F().blocks) n += (long long)b.second;
+    return n;
+  }
   if (std::string(what) == "hosts") return (long long)F().hosts.size();
   if (std::string(what) == "blocks") return (long long)F().blocks.size();
   return F().calls[what];

@@ -199,3 +199,15 @@ def test_a_context_per_event_reuses_the_mapped_memory(device):
     once(*_context())
     assert device.fake_get(b"hosts") == 1
     assert not _report(device)
+
+
+@pytest.mark.parametrize("het", [False, True])
+def test_small_batches_hold_no_scratch_of_the_fp64_path(device, het):
+    """A new event's first call pays for what it allocates: the partial sums per slice
+    of the FP64 path (256 vectors x 31 slices x 4 x 64 bytes) are not among it."""
+    ctx, th = _context(het=het)
+    ctx.loglike_batch(th[None])
+    held = device.fake_get(b"bytes")
+    ctx.close()
+    assert held - device.fake_get(b"bytes") < 256 * 31 * 4 * 64
+    assert not _report(device)
