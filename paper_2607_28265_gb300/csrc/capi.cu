@@ -1305,7 +1305,14 @@ static int batch_chunk(const swig_ctx* c) {
 }
 
 int loglike_device(swig_ctx* c, const double* theta_dev, int64_t n, double* out_dev, cudaStream_t st) {
-  const int chunk = batch_chunk(c);
+  int chunk = batch_chunk(c);
+  // a capture cannot allocate: once the scratch serves 4096 vectors, a longer batch is
+  // recorded in pieces of what it serves
+  if (std::min<int64_t>(n, chunk) > c->B.cap && c->B.cap >= 4096) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) chunk = c->B.cap;
+  }
   for (int64_t off = 0; off < n; off += chunk) {
     const int m = (int)std::min<int64_t>(chunk, n - off);
     int rc = ensure_scratch(c, m);

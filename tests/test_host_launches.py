@@ -211,3 +211,20 @@ def test_small_batches_hold_no_scratch_of_the_fp64_path(device, het):
     ctx.close()
     assert held - device.fake_get(b"bytes") < 256 * 31 * 4 * 64
     assert not _report(device)
+
+
+@pytest.mark.parametrize("kind", ["mixed", "fp64", "het"])
+def test_a_long_batch_is_captured_after_a_batch_of_4096(device, kind):
+    """Nothing is allocated or freed under capture: the batch is recorded in pieces
+    that the scratch serves."""
+    ctx, th = _context(**{"mixed": {}, "fp64": dict(precision=swig.PREC_FP64), "het": dict(het=True)}[kind])
+    theta, out = np.tile(th, (20000, 1)), np.empty(20000)
+    ctx.loglike_batch(theta[:4500])
+    device.fake_reset()
+    device.fake_set(b"capturing", 1)
+    try:
+        ctx.loglike_batch_dev(theta.ctypes.data, 20000, out.ctypes.data, 0x1000)
+    finally:
+        device.fake_set(b"capturing", 0)
+    assert device.fake_get(b"cudaMalloc") == 0 and device.fake_get(b"cudaFree") == 0
+    ctx.close()
