@@ -1205,8 +1205,8 @@ int prepare(swig_ctx* c) {
   {
     const double a1 = std::sqrt(5.0 / 24.0) * std::pow(kPi, -2.0 / 3.0) * std::pow(kMtsunS, 5.0 / 6.0) * kCSI / kMpcM;
     for (int i = 0; i < n_det; ++i) {
-      L.amp_s[i] = (float)(L.inv_scale[i] * a1);
-      L.amp_k[i] = (float)(L.K[i] * a1 * a1);
+      L.amp_s[i] = L.inv_scale[i] * a1;
+      L.amp_k[i] = L.K[i] * a1 * a1;
       L.amp1 = a1;
     }
   }

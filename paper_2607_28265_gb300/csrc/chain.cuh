@@ -55,7 +55,8 @@ struct ChainWork {
   int status;
   int bad[kCand];            // folded sums: outside the band, summed bin by bin
   // projection-only steps: a lane's theta, the current point's sums
-  float fth[2 * kFreeRungs][SWIG_N_PARAMS], fkap[2 * SWIG_MAX_DET], fvv[SWIG_MAX_DET];
+  float fth[2 * kFreeRungs][SWIG_N_PARAMS];
+  float2 fkap[2 * SWIG_MAX_DET], fvv[SWIG_MAX_DET];  // free_loglike's, (hi, lo)
 };
 
 enum { ROUND_EVAL = 0, ROUND_DONE = 1 };
@@ -371,14 +372,18 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
   float* th = w.fth[row];
   {
     // rounded once, a value per lane
-    const double x = lane < SWIG_N_PARAMS                        ? ch.th[lane]
-                     : lane < SWIG_N_PARAMS + 2 * SWIG_MAX_DET   ? ch.kap[lane - SWIG_N_PARAMS]
-                     : lane < SWIG_N_PARAMS + 3 * SWIG_MAX_DET   ? ch.vv[lane - SWIG_N_PARAMS - 2 * SWIG_MAX_DET]
-                                                                 : 0.0;
-    const float f = (float)x;
-    if (lane >= SWIG_N_PARAMS && lane < SWIG_N_PARAMS + 2 * SWIG_MAX_DET) w.fkap[lane - SWIG_N_PARAMS] = f;
-    if (lane >= SWIG_N_PARAMS + 2 * SWIG_MAX_DET && lane < SWIG_N_PARAMS + 3 * SWIG_MAX_DET)
-      w.fvv[lane - SWIG_N_PARAMS - 2 * SWIG_MAX_DET] = f;
+    const int j = lane - SWIG_N_PARAMS, i = j - 2 * SWIG_MAX_DET;
+    double x = 0.0;
+    if (j < 0)
+      x = ch.th[lane];
+    else if (i < 0)
+      x = ch.kap[j] * L.amp_s[j >> 1];
+    else if (i < SWIG_MAX_DET)
+      x = HET ? ch.vv[i] : L.amp_k[i];
+    const dfl v = df_from_double(x);
+    const float f = v.hi;
+    if (j >= 0 && i < 0) w.fkap[j] = make_float2(v.hi, v.lo);
+    if (i >= 0 && i < SWIG_MAX_DET) w.fvv[i] = make_float2(v.hi, v.lo);
 #pragma unroll
     for (int s = 0; s < SWIG_N_PARAMS; ++s) {
       const float v = __shfl_sync(0xffffffffu, f, s);
@@ -398,7 +403,7 @@ __device__ __forceinline__ int chain_free_step(const LikeConst& L, const Sampler
         if (in) th[slot] = (float)prior_slot_inverse_f32(S.prior[slot], v);
       }
     inside = __ballot_sync(0xffffffffu, in);
-    if (in) ly = free_loglike_f32(L, th, w.fkap, HET ? w.fvv : nullptr);
+    if (in) ly = free_loglike(L, th, w.fkap, w.fvv);
     ok = __ballot_sync(0xffffffffu, in && ly > logl_star);
     __syncwarp();
   };

@@ -87,11 +87,11 @@ struct LikeConst {
   double DD;                     // sum_i <d_i|d_i>
   double inv_scale[SWIG_MAX_DET];  // data scale folded into C_i
   double rscale[SWIG_MAX_DET];     // its reciprocal
-  // FP32-friendly constants for projection-only evaluations:
+  // constants of projection-only evaluations:
   // amp_s = inv_scale * A1, amp_k = K * A1^2 with A1 the SPA amplitude of
   // Mc = 1 Msun at 1 Mpc, so C_i kappa_i and |C_i|^2 K_i stay O(1..1e6).
-  float amp_s[SWIG_MAX_DET];
-  float amp_k[SWIG_MAX_DET];
+  double amp_s[SWIG_MAX_DET];
+  double amp_k[SWIG_MAX_DET];
   double amp1;  // A1 itself
   double dten[SWIG_MAX_DET][6];  // detector tensor xx xy xz yy yz zz
   float dten_f[SWIG_MAX_DET][6];  // the same rounded, and gmst, for the FP32 projections
