@@ -12,8 +12,8 @@
 //
 // Measured (one GB300, first iterations of the 128 s three-detector run, nlive
 // 1000, nrep 100): 4 iterations 145 ms with one candidate at a time across all
-// SMs (a request to every SM's slice of the grid, control on one warp), 12.3 ms
-// here; heterodyned, 8 iterations 133 -> 35.6 ms.  1.3 candidates are evaluated
+// SMs (a request to every SM's slice of the grid, control on one warp), 12.9 ms
+// here; heterodyned, 8 iterations 133 -> 38.9 ms.  1.3 candidates are evaluated
 // per candidate used; with fewer per round the latencies dominate.
 //
 // A round costs its latency once: the set-up's FP64 chains (64 cycles an

@@ -14,11 +14,11 @@
 // (the lowest frequencies) the nodes are the bins themselves.  The 128 s
 // three-detector grid's 259,585 bins become about 80 chunks of 64 nodes.
 //
-// Bound: the SFU (two results per node and detector, 78 x 64 x 3 nodes instead
-// of 778,755 bins) and the FP32 issue slots beside it.  Batched, against the
-// direct sum over every bin (one GB300): 1000 vectors on the 128 s grid 84 us
-// (668), 4099 on the 256 s grid 253 us (4.74 ms), one vector 63 us with the
-// host copies (91); the error against FP64 is the same or smaller.
+// Bound: the FP32 issue slots, with the SFU beside them (two results per node and
+// detector, 78 x 64 x 3 nodes instead of 778,755 bins).  Batched, against the direct
+// sum over every bin (one GB300): 1000 vectors on the 128 s grid 31 us (668), 4099 on
+// the 256 s grid 88 us (4.74 ms), one vector 30 us with the host's part (90); the
+// error against FP64 is that of the direct sum (kFoldBlock).
 //
 // An evaluation checks its own bandwidth and Taylor remainder on every chunk
 // against the bound the weights were made for; a parameter vector outside

@@ -912,8 +912,9 @@ int run_setup(swig_ctx* c, RunState& R) {
   S.flow_parts = c->cfg.flow_parts > 0 ? c->cfg.flow_parts : SWIG_FLOW_PARTS;
   // chain sampler: candidates per round (chain.cuh).  Four rungs per end and
   // two draws unless a smaller launch shape is asked for (first iterations of the
-  // 128 s run, ms: (rungs, draws) = (4, 2) 16.0, (4, 3) 16.4, (4, 4) 16.7, (4, 8)
-  // 18.3, (3, 3) 17.8, (2, 4) 19.8; heterodyned 45.8, 46.9, 47.5, 52.9, 49.8, 55.8); with t_c marginalised
+  // 128 s run, ms: (rungs, draws) = (4, 2) 12.8, (4, 3) 13.1, (4, 4) 13.3, (4, 8)
+  // 13.6, (3, 3) 14.4, (2, 4) 16.5; heterodyned 38.8, 39.1, 38.9, 40.2, 42.2, 47.9);
+  // with t_c marginalised
   // an evaluation costs as much as a round's latency: one at a time
   const int shape = c->cfg.flow_parts;
   S.spec_out = L.tm_n > 0 ? 1 : shape >= 3 ? 1 : shape == 2 ? 2 : 4;

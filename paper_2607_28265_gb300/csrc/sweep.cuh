@@ -1,6 +1,7 @@
 // Bin by bin: the FP64 sweep of the batched kernel and the FP64 sampler, and the
 // mixed-precision sweep (per-(theta, tile) double-float phase anchors, FP32 per
-// bin) that the folded evaluation falls back on outside its band.
+// bin) that the folded evaluation falls back on outside its band (in the sampler;
+// batches sum two vectors at a time, fold.cu).
 #pragma once
 
 #include "device_common.cuh"
